@@ -23,6 +23,7 @@
 //   pull (Eq 4 lane-wise, masking + early exit + operand reuse): every vertex with
 //     an unvisited lane ORs V of its in-neighbours (V is the state before this
 //     level) and stops as soon as every unvisited lane is covered; new = acc & ~V.
+//     Long rows are deferred and spread over the whole grid.
 // New lanes get depth L + 1.  Depths are not stored as they are found (2-byte
 // stores scattered over S rows leave partial sectors that are evicted and merged
 // again level after level): a depth below 16 is recorded as bits in four per-vertex
@@ -43,7 +44,7 @@ constexpr int kMsThreads = 512;
 // chooses it (blocks_per_sm >= 3) and the autotuner times both.
 constexpr int kMsOcc = 2;
 constexpr int kMsOccLean = 3;
-constexpr int kMsProbe = 8;  // default in-neighbours a lane scans alone before the warp takes over
+constexpr int kMsProbe = 8;  // default a.probe: a long row is deferred after four times as many in-neighbours
 constexpr int kMsPlanes = 4;  // depth bit planes: bit p of depths below 16
 
 struct MsArgs {
@@ -74,6 +75,7 @@ struct MsArgs {
     int32_t* status;
     float alpha;
     int32_t mode, trace_cap, symmetric, probe;
+    int32_t group;  // warp lanes that hold a vertex's words (a power of two)
     unsigned long long timeout_ns;
 };
 
@@ -128,185 +130,531 @@ __device__ __forceinline__ void record_depth(const MsArgs& a, int32_t v, int32_t
 }
 
 // After the last level: every (lane, vertex) entry of the output rows, once.  A warp
-// takes 32 consecutive vertices and one lane word; for each of the word's lanes the 32
-// entries are one coalesced store.  Lanes never visited get -1; lanes found at depth
-// 16 or more were stored when found and are left alone.
-__device__ __forceinline__ void emit_depths(const MsArgs& a) {
-    const int lane = threadIdx.x & 31;
-    const long long gwarp = ((long long)blockIdx.x * kMsThreads + threadIdx.x) >> 5;
-    const long long nwarps = ((long long)gridDim.x * kMsThreads) >> 5;
-    const int32_t nvb = (a.n + 31) >> 5;
-    const int32_t wl = (a.S + 63) >> 6;  // words holding real lanes
-    const long long items = (long long)nvb * wl;
-    for (long long it = gwarp; it < items; it += nwarps) {
-        const int32_t vb = (int32_t)(it / wl), w = (int32_t)(it - (long long)vb * wl);
-        const int32_t v = (vb << 5) + lane;
-        const bool ok = v < a.n;
-        const size_t iv = (size_t)(ok ? v : 0) * a.W + w;
-        const unsigned long long vis = ok ? a.V[iv] : 0ull;
-        const unsigned long long p0 = ok ? a.P[0][iv] : 0ull, p1 = ok ? a.P[1][iv] : 0ull;
-        const unsigned long long p2 = ok ? a.P[2][iv] : 0ull, p3 = ok ? a.P[3][iv] : 0ull;
-        const unsigned long long any = p0 | p1 | p2 | p3;
-        const int nb = a.S - w * 64 < 64 ? a.S - w * 64 : 64;
-        for (int b = 0; b < nb; ++b) {
-            if (!ok) continue;
+// takes 128 consecutive vertices and 32 rows (half a lane word), four vertices a lane,
+// and each row's 128 entries leave together: four entries of a lane are one 8- or
+// 16-byte store where the rows allow it (aligned, a full group), else four stores whose
+// 32 lanes are consecutive.  Lanes never visited get -1; lanes found at depth 16 or more
+// were stored when found and are left alone (emit_rows_mixed).
+//
+// Bound by the stores: S rows of n entries, written once, many rows at a time.  With 32
+// vertices a warp (one 64- or 128-byte piece of a row per store, ten instructions an
+// entry) the RMAT-20 batch of 1,000 int16 rows spent 2.0 ms here and the RMAT-21 batch of
+// 64 int32 rows 0.25 ms; now 0.8 and 0.14 ms, of which 0.31 and 0.08 are the rows' 2.1 and
+// 0.54 GB at the measured copy rate.
+constexpr int kEmitV = 4;               // vertices a lane
+constexpr int kEmitTile = 32 * kEmitV;  // vertices a warp
+
+// Bits 0..3 of x as the low bits of bytes 0..3.
+__device__ __forceinline__ uint32_t spread4(uint32_t x) { return ((x & 0xfu) * 0x00204081u) & 0x01010101u; }
+
+// Byte-wise selection of (lo, hi) with sign replication (selector bit 3 of a nibble).
+__device__ __forceinline__ uint32_t prmt_sext(uint32_t lo, uint32_t hi, uint32_t sel) {
+    uint32_t r;
+    asm("prmt.b32 %0, %1, %2, %3;" : "=r"(r) : "r"(lo), "r"(hi), "r"(sel));
+    return r;
+}
+
+// The address of entry 0 of output row b.
+__device__ __forceinline__ char* depth_row(const MsArgs& a, int32_t b) {
+    if (a.rows) return static_cast<char*>(a.rows[b]);
+    return static_cast<char*>(a.depth) + (size_t)b * (size_t)a.n * (a.depth16 ? 2u : 4u);
+}
+
+// One group's half word when some lane of it was found at depth 16 or more, or is its own
+// source: entry by entry, a row's 32 consecutive entries per store.
+__device__ __noinline__ void emit_rows_mixed(const MsArgs& a, int32_t g, int32_t h, int nrows) {
+    for (int j = 0; j < kEmitV; ++j) {
+        const int32_t v = g * kEmitTile + 32 * j + (threadIdx.x & 31);
+        if (v >= a.n) continue;
+        const size_t iw = (size_t)v * a.W * 2 + h;
+        const uint32_t vis = reinterpret_cast<const uint32_t*>(a.V)[iw];
+        uint32_t p[kMsPlanes];
+#pragma unroll
+        for (int q = 0; q < kMsPlanes; ++q) p[q] = reinterpret_cast<const uint32_t*>(a.P[q])[iw];
+        for (int b = 0; b < nrows; ++b) {
             int32_t d = -1;
-            if ((vis >> b) & 1ull) {
-                if (!((any >> b) & 1ull) && __ldg(a.src + w * 64 + b) != v) continue;  // deep: already stored
-                d = (int32_t)(((p0 >> b) & 1ull) | (((p1 >> b) & 1ull) << 1) | (((p2 >> b) & 1ull) << 2) |
-                              (((p3 >> b) & 1ull) << 3));
+            if ((vis >> b) & 1u) {
+                d = (int32_t)(((p[0] >> b) & 1u) | (((p[1] >> b) & 1u) << 1) | (((p[2] >> b) & 1u) << 2) |
+                              (((p[3] >> b) & 1u) << 3));
+                if (d == 0 && __ldg(a.src + 32 * h + b) != v) continue;  // deep: already stored
             }
-            store_depth(a, w * 64 + b, v, d);
+            store_depth(a, 32 * h + b, v, d);
         }
     }
+}
+
+// One half word of a group: the lane's visited and plane bits of vertices v + stride * j.
+struct EmitBits {
+    uint32_t vis[kEmitV], p[kMsPlanes][kEmitV];
+};
+
+// Writes the rows of one half word (rows 32 h + lane's row address in `row`).
+__device__ __forceinline__ void emit_half(const MsArgs& a, const EmitBits& e, char* row, int nrows, int32_t v,
+                                          bool wide) {
+    for (int b = 0; b < nrows; b += 4) {
+        // byte r of d[j]: depth of (row b + r, vertex j), 0xff where it was never visited
+        uint32_t d[kEmitV];
+#pragma unroll
+        for (int j = 0; j < kEmitV; ++j)
+            d[j] = (spread4(e.p[0][j] >> b) | (spread4(e.p[1][j] >> b) << 1) | (spread4(e.p[2][j] >> b) << 2) |
+                    (spread4(e.p[3][j] >> b) << 3)) |
+                   ~(spread4(e.vis[j] >> b) * 0xffu);
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            char* const rp = reinterpret_cast<char*>(
+                __shfl_sync(0xffffffffu, (unsigned long long)reinterpret_cast<uintptr_t>(row), b + r));
+            if (b + r >= nrows) continue;
+            if (a.depth16) {
+                const uint32_t sel = 0xc480u + 0x1111u * r;  // bytes r, sign of r, 4 + r, its sign
+                const uint32_t lo = prmt_sext(d[0], d[1], sel), hi = prmt_sext(d[2], d[3], sel);
+                int16_t* const o = reinterpret_cast<int16_t*>(rp) + v;
+                if (wide) {
+                    *reinterpret_cast<uint2*>(o) = make_uint2(lo, hi);
+                } else {
+                    if (v < a.n) o[0] = (int16_t)lo;
+                    if (v + 32 < a.n) o[32] = (int16_t)(lo >> 16);
+                    if (v + 64 < a.n) o[64] = (int16_t)hi;
+                    if (v + 96 < a.n) o[96] = (int16_t)(hi >> 16);
+                }
+            } else {
+                const uint32_t sel = 0x8880u + 0x1111u * r;  // byte r, its sign three times
+                int32_t* const o = reinterpret_cast<int32_t*>(rp) + v;
+                const int32_t x0 = (int32_t)prmt_sext(d[0], 0u, sel), x1 = (int32_t)prmt_sext(d[1], 0u, sel);
+                const int32_t x2 = (int32_t)prmt_sext(d[2], 0u, sel), x3 = (int32_t)prmt_sext(d[3], 0u, sel);
+                if (wide) {
+                    *reinterpret_cast<int4*>(o) = make_int4(x0, x1, x2, x3);
+                } else {
+                    if (v < a.n) o[0] = x0;
+                    if (v + 32 < a.n) o[32] = x1;
+                    if (v + 64 < a.n) o[64] = x2;
+                    if (v + 96 < a.n) o[96] = x3;
+                }
+            }
+        }
+    }
+}
+
+// W >= 4: the block stages 128 vertices x 8 words of V and the planes in shared memory
+// (16-byte loads, 64 consecutive bytes a vertex), one array of 128 32-bit halves per half
+// word, and each of its 16 warps writes the rows of one half.  Loading a half straight
+// from the vertex-major words would touch 32 lines with every load (stride 8 W bytes).
+constexpr int kEmitWords = 8;
+constexpr int kEmitPad = kEmitTile + 2;  // staging writes 8 vertices x 4 halves: distinct banks
+constexpr int kEmitSmem = (1 + kMsPlanes) * 2 * kEmitWords * kEmitPad * 4;  // bytes
+static_assert(kMsThreads / 32 == 2 * kEmitWords, "one warp per half word of the staged tile");
+
+// smem: kEmitSmem bytes (16-byte aligned), used by the block from here on.
+template <bool kStaged>
+__device__ __forceinline__ void emit_depths(const MsArgs& a, uint32_t* smem) {
+    const int lane = threadIdx.x & 31;
+    const int wib = threadIdx.x >> 5;
+    const int32_t ngroups = (a.n + kEmitTile - 1) / kEmitTile;
+    const int32_t nhalf = (a.S + 31) >> 5;  // half words holding real lanes
+    const uint32_t esz = a.depth16 ? 2u : 4u;
+    // staged: a block takes a tile of 16 halves; else a warp takes one half
+    const int32_t per = kStaged ? 2 * kEmitWords : 1;
+    const int32_t ntile = (nhalf + per - 1) / per;
+    const long long items = (long long)ngroups * ntile;
+    const long long first = kStaged ? blockIdx.x : (((long long)blockIdx.x * kMsThreads + threadIdx.x) >> 5);
+    const long long nstep = kStaged ? gridDim.x : (((long long)gridDim.x * kMsThreads) >> 5);
+    for (long long it = first; it < items; it += nstep) {
+        const int32_t g = (int32_t)(it / ntile);
+        const int32_t h0 = (int32_t)(it - (long long)g * ntile) * per;
+        if (kStaged) {
+            __syncthreads();  // the last tile has been read
+            const int32_t w0 = h0 >> 1;
+            for (int i = threadIdx.x; i < (1 + kMsPlanes) * kEmitTile * (kEmitWords / 2); i += kMsThreads) {
+                const int q = i / (kEmitTile * (kEmitWords / 2)), r = i - q * (kEmitTile * (kEmitWords / 2));
+                const int vl = r / (kEmitWords / 2), c = r - vl * (kEmitWords / 2);  // vertex, pair of words
+                const int32_t v = g * kEmitTile + vl, w = w0 + 2 * c;
+                uint4 x = make_uint4(0u, 0u, 0u, 0u);
+                if (v < a.n && w < a.W)
+                    x = *reinterpret_cast<const uint4*>((q == 0 ? a.V : a.P[q - 1]) + (size_t)v * a.W + w);
+                uint32_t* const o = smem + (q * 2 * kEmitWords + 4 * c) * kEmitPad + vl;
+                o[0] = x.x;
+                o[kEmitPad] = x.y;
+                o[2 * kEmitPad] = x.z;
+                o[3 * kEmitPad] = x.w;
+            }
+            __syncthreads();
+        }
+        const int32_t h = kStaged ? h0 + wib : h0;
+        if (h >= nhalf) continue;
+        const int nrows = a.S - 32 * h < 32 ? a.S - 32 * h : 32;
+        char* const row = depth_row(a, 32 * h + (lane < nrows ? lane : 0));  // lane r: row 32 h + r
+        const bool wide = __all_sync(0xffffffffu, (reinterpret_cast<uintptr_t>(row) & (kEmitV * esz - 1)) == 0) &&
+                          (long long)(g + 1) * kEmitTile <= a.n;
+        const int32_t stride = wide ? 1 : 32, vl = wide ? kEmitV * lane : lane;
+        const int32_t v = g * kEmitTile + vl;
+        EmitBits e;
+        uint32_t deep = 0u;
+#pragma unroll
+        for (int j = 0; j < kEmitV; ++j) {
+            const int32_t vj = v + stride * j;
+            if (kStaged) {
+                const uint32_t* const sp = smem + wib * kEmitPad + vl + stride * j;
+                e.vis[j] = sp[0];
+#pragma unroll
+                for (int q = 0; q < kMsPlanes; ++q) e.p[q][j] = sp[(q + 1) * 2 * kEmitWords * kEmitPad];
+            } else {
+                const size_t iw = (size_t)(vj < a.n ? vj : 0) * a.W * 2 + h;  // 32-bit half of the word
+                e.vis[j] = vj < a.n ? reinterpret_cast<const uint32_t*>(a.V)[iw] : 0u;
+#pragma unroll
+                for (int q = 0; q < kMsPlanes; ++q)
+                    e.p[q][j] = vj < a.n ? reinterpret_cast<const uint32_t*>(a.P[q])[iw] : 0u;
+            }
+            deep |= e.vis[j] & ~(e.p[0][j] | e.p[1][j] | e.p[2][j] | e.p[3][j]);
+        }
+        if (__any_sync(0xffffffffu, deep != 0u))
+            emit_rows_mixed(a, g, h, nrows);
+        else
+            emit_half(a, e, row, nrows, v, wide);
+    }
+}
+
+// ---------------------------------------------------------------- lane-word groups
+
+// A vertex's W lane words are handled by a group of a.group consecutive warp lanes,
+// WL words a lane (one 8- or 16-byte access): W = 1 is one lane and one word, W = 16
+// eight lanes whose 16-byte loads make one 128-byte line per vertex.  W above 64 goes
+// through the group in chunks of 64 words.
+template <int WL>
+struct Words {
+    unsigned long long x[WL];
+    __device__ __forceinline__ bool any() const {
+        unsigned long long o = 0ull;
+#pragma unroll
+        for (int j = 0; j < WL; ++j) o |= x[j];
+        return o != 0ull;
+    }
+};
+
+template <int WL>
+__device__ __forceinline__ Words<WL> ld_words(const unsigned long long* p) {
+    Words<WL> r;
+    if (WL == 2) {
+        const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(p);
+        r.x[0] = t.x;
+        r.x[WL - 1] = t.y;
+    } else {
+        r.x[0] = *p;
+    }
+    return r;
+}
+
+template <int WL>
+__device__ __forceinline__ void st_words(unsigned long long* p, const Words<WL>& w) {
+    if (WL == 2)
+        *reinterpret_cast<ulonglong2*>(p) = make_ulonglong2(w.x[0], w.x[WL - 1]);
+    else
+        *p = w.x[0];
+}
+
+template <int WL>
+__device__ __forceinline__ Words<WL> zero_words() {
+    Words<WL> r;
+#pragma unroll
+    for (int j = 0; j < WL; ++j) r.x[j] = 0ull;
+    return r;
+}
+
+// The calling lane's place in its group.
+struct Group {
+    int size, sub, first;  // lanes, this lane's index, warp lane of index 0
+    uint32_t mask;         // the group's lanes
+    __device__ __forceinline__ explicit Group(int n) {
+        const int lane = threadIdx.x & 31;
+        size = n;
+        sub = lane & (n - 1);
+        first = lane & ~(n - 1);
+        mask = (n == 32 ? 0xffffffffu : (1u << n) - 1u) << first;
+    }
+    __device__ __forceinline__ bool any(bool p) const { return (__ballot_sync(0xffffffffu, p) & mask) != 0u; }
+    __device__ __forceinline__ bool all(bool p) const { return (__ballot_sync(0xffffffffu, p) & mask) == mask; }
+};
+
+// Records depth d for this lane's new words nw of vertex v (one writer per word); was: its
+// words of V before.  With two words a lane the planes are not zeroed at the start: the
+// first lanes found in a word write all four of its plane words.
+template <int WL>
+__device__ __forceinline__ void record_words(const MsArgs& a, int32_t v, int32_t w, const Words<WL>& nw,
+                                             const Words<WL>& was, int32_t d) {
+    if (!nw.any()) return;
+    const size_t iv = (size_t)v * a.W + w;
+    if (WL == 2) {
+        const bool fresh = (nw.x[0] && !was.x[0]) || (nw.x[WL - 1] && !was.x[WL - 1]);
+        const int32_t bits = d < 16 ? d : 0;
+#pragma unroll
+        for (int p = 0; p < kMsPlanes; ++p) {
+            const bool set = (bits >> p) & 1;
+            if (!set && !fresh) continue;
+            Words<WL> t = was.any() ? ld_words<WL>(a.P[p] + iv) : zero_words<WL>();
+#pragma unroll
+            for (int j = 0; j < WL; ++j) t.x[j] = (was.x[j] ? t.x[j] : 0ull) | (set ? nw.x[j] : 0ull);
+            st_words<WL>(a.P[p] + iv, t);
+        }
+        if (d < 16) return;
+    }
+#pragma unroll
+    for (int j = 0; j < WL; ++j) record_depth(a, v, w + j, nw.x[j], d, false);
 }
 
 // ---------------------------------------------------------------- pull level
 
-template <int CW>
-__device__ __forceinline__ void ms_pull(const MsArgs& a, int32_t L, unsigned long long* Fn, Stage& st, Acc& acc) {
+constexpr int kMsUnroll = 4;        // in-neighbours a group ORs per step (loads in flight)
+constexpr int32_t kMsLongRow = 64;   // in-edges left after the probe beyond which a row is deferred
+constexpr int32_t kMsChunk = 512;   // in-edges of a deferred row a warp takes at a time
+constexpr int32_t kMsCheck = 128;   // ... between two tests whether they cover the row (a power of two)
+
+// Rows of a pull level left to the grid: vertex, first in-edge left, ascending prefix
+// of their chunk counts.
+struct MsLong {
+    int32_t* row;
+    int32_t* k;
+    int32_t* base;
+};
+
+// Every vertex with an unvisited lane ORs V of its in-neighbours (V as of the level's
+// start), kMsUnroll at a time, until all its unvisited lanes are covered.  A warp lists
+// the open vertices of 32 of its bitmap words in shared memory and its groups take them
+// one after another, each going on to the next as soon as its own is settled, so a long
+// row holds up nobody else's.  A row that is still open after 4 a.probe in-neighbours with
+// more than kMsLongRow left is deferred: its chunks are spread over all warps
+// (ms_pull_long) and it is settled after that (ms_finalize).
+//
+// Bound by the gathers of V (W words per examined in-neighbour, mostly L2).  A lane per
+// row with its V words in 32-byte chunks, and one warp for a long row, had made the first
+// pull level of the RMAT-20 batch of 1,000 sources 7.1 ms: every gather touched 32 rows at
+// once and a hub row held one warp for milliseconds.  Now 0.76 ms (31.4M in-neighbours x
+// 128 B, 5.3 TB/s).  kMsLongRow 64, 128 and 512 give that level 0.76, 0.78 and 1.0 ms;
+// deferring after 8 instead of 32 in-neighbours costs the RMAT-21 batch of 64 5 %, and
+// kMsChunk 256 instead of 512 6 % (more of a row's chunks run before one covers it).
+template <int WL>
+__device__ __forceinline__ void ms_pull(const MsArgs& a, int32_t L, int32_t c0, unsigned long long* Fn, uint32_t* Tn,
+                                        uint16_t* list, const MsLong& lr, bool defer, Stage& st, Acc& acc) {
     const int lane = threadIdx.x & 31;
     const int gwarp = (int)((blockIdx.x * kMsThreads + threadIdx.x) >> 5);
     const int nwarps = (int)((gridDim.x * kMsThreads) >> 5);
-    const int32_t ntiles = (a.n + 31) >> 5;
-    for (int32_t tile = gwarp; tile < ntiles; tile += nwarps) {
-        const int32_t v = (tile << 5) + lane;
-        const uint32_t todo = v < a.n ? (a.nz_in[tile] & ~a.D[tile]) : 0u;
-        if (__ballot_sync(0xffffffffu, (todo >> lane) & 1u) == 0u) continue;
-        const bool mine = (todo >> lane) & 1u;
-        int32_t beg = 0, end = 0;
+    const Group gr(a.group);
+    const int32_t w = c0 + WL * gr.sub;
+    const bool wok = w < a.W;
+    const bool one = a.W <= WL * gr.size;  // one chunk: a row is settled in one go
+    const uint32_t chunks256 = (uint32_t)(a.W + 3) >> 2;
+    Words<WL> lm;
+#pragma unroll
+    for (int j = 0; j < WL; ++j) lm.x[j] = wok ? lane_mask(a.S, w + j) : 0ull;
+    for (long long wb = gwarp; wb < a.nwords; wb += 32ll * nwarps) {
+        const long long tw = wb + (long long)lane * nwarps;
+        uint32_t m = tw < a.nwords ? (a.nz_in[tw] & ~a.D[tw]) : 0u;
+        const uint32_t cnt = __popc(m);
+        const uint32_t incl = warp_inclusive_sum(cnt);
+        const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);
+        if (total == 0u) continue;
+        __syncwarp();
+        for (uint32_t at = incl - cnt; m; m &= m - 1) list[at++] = (uint16_t)((lane << 5) + __ffs(m) - 1);
+        __syncwarp();
+        uint32_t next = 0;
+        int32_t v = -1, k = 0, end = 0, lim = 0;
+        int32_t u[kMsUnroll] = {-1, -1, -1, -1};  // the in-neighbours of this step; the next step's are loaded meanwhile
         bool sink = false;
-        if (mine) {
-            beg = __ldg(a.in_ptr + v);
-            end = __ldg(a.in_ptr + v + 1);
-            sink = !a.symmetric && __ldg(a.out_ptr + v + 1) == __ldg(a.out_ptr + v);
-        }
-        // A vertex without out-edges is nobody's in-neighbour, so no other row reads
-        // its V during this level: its new lanes are committed in place (it never
-        // joins the active list, which holds vertices with out-edges only).
-        bool any_new = false, full = true;
-        for (int32_t c = 0; c < a.W; c += CW) {
-            unsigned long long unv[CW], accw[CW];
-            bool pend = false;
+        Words<WL> unv = zero_words<WL>(), ac = zero_words<WL>();
+        for (;;) {
+            const uint32_t need = __ballot_sync(0xffffffffu, v < 0 && gr.sub == 0);
+            if (need) {
+                const uint32_t idx = next + __popc(need & ((1u << gr.first) - 1u));
+                if (v < 0 && idx < total) {
+                    const uint32_t off = list[idx];
+                    v = (int32_t)((wb + (long long)(off >> 5) * nwarps) << 5) + (int32_t)(off & 31u);
+                    k = __ldg(a.in_ptr + v);
+                    end = __ldg(a.in_ptr + v + 1);
+                    lim = end - k > 4 * a.probe + kMsLongRow ? k + 4 * a.probe : end;
+                    sink = !a.symmetric && __ldg(a.out_ptr + v + 1) == __ldg(a.out_ptr + v);
+                    unv = wok ? ld_words<WL>(a.V + (size_t)v * a.W + w) : zero_words<WL>();
 #pragma unroll
-            for (int j = 0; j < CW; ++j) {
-                unv[j] = mine ? (~a.V[(size_t)v * a.W + c + j] & lane_mask(a.S, c + j)) : 0ull;
-                accw[j] = 0ull;
-                pend |= unv[j] != 0ull;
-            }
-            unsigned long long exam = 0;
-            // lane probes: up to a.probe in-neighbours, two loads in flight
-            int32_t k = beg;
-            bool covered = !pend;
-            const int32_t lim = end < beg + a.probe ? end : beg + a.probe;
-            while (!covered && k < lim) {
-                const bool two = k + 1 < lim;
-                const int32_t u0 = __ldg(a.in_col + k);
-                const int32_t u1 = two ? __ldg(a.in_col + k + 1) : u0;
-                covered = true;
-#pragma unroll
-                for (int j = 0; j < CW; ++j) {
-                    accw[j] |= a.V[(size_t)u0 * a.W + c + j] | a.V[(size_t)u1 * a.W + c + j];
-                    covered &= (accw[j] & unv[j]) == unv[j];
-                }
-                k += two ? 2 : 1;
-                exam += two ? 2u : 1u;
-            }
-            // long rows: the whole warp ORs 32 in-neighbours at a time and stops once
-            // every unvisited lane of the chunk is covered (warp OR-reduction)
-            uint32_t wpend = __ballot_sync(0xffffffffu, !covered && k < end);
-            while (wpend) {
-                const int t = __ffs(wpend) - 1;
-                wpend &= wpend - 1;
-                const int32_t kt = __shfl_sync(0xffffffffu, k, t);
-                const int32_t et = __shfl_sync(0xffffffffu, end, t);
-                unsigned long long ut[CW], wa[CW];
-#pragma unroll
-                for (int j = 0; j < CW; ++j) {
-                    ut[j] = __shfl_sync(0xffffffffu, unv[j], t);
-                    wa[j] = __shfl_sync(0xffffffffu, accw[j], t);
-                }
-                unsigned long long tx = 0;
-                for (int32_t kk = kt; kk < et; kk += 32) {
-                    const int32_t idx = kk + lane;
-                    unsigned long long x[CW];
-                    if (idx < et) {
-                        const int32_t u = __ldg(a.in_col + idx);
-#pragma unroll
-                        for (int j = 0; j < CW; ++j) x[j] = a.V[(size_t)u * a.W + c + j];
-                    } else {
-#pragma unroll
-                        for (int j = 0; j < CW; ++j) x[j] = 0ull;
+                    for (int j = 0; j < WL; ++j) {
+                        unv.x[j] = ~unv.x[j] & lm.x[j];
+                        ac.x[j] = 0ull;
                     }
-                    bool cov = true;
 #pragma unroll
-                    for (int j = 0; j < CW; ++j) {
-                        const uint32_t lo = __reduce_or_sync(0xffffffffu, (uint32_t)x[j]);
-                        const uint32_t hi = __reduce_or_sync(0xffffffffu, (uint32_t)(x[j] >> 32));
-                        wa[j] |= ((unsigned long long)hi << 32) | lo;
-                        cov &= (wa[j] & ut[j]) == ut[j];
-                    }
-                    tx += (unsigned long long)(et - kk < 32 ? et - kk : 32);
-                    if (cov) break;
+                    for (int t = 0; t < kMsUnroll; ++t) u[t] = k + t < end ? __ldg(a.in_col + k + t) : -1;
                 }
-                if (lane == t) {
+                next += __popc(need);
+            }
+            if (__ballot_sync(0xffffffffu, v >= 0) == 0u) break;
+            Words<WL> x[kMsUnroll];
 #pragma unroll
-                    for (int j = 0; j < CW; ++j) accw[j] = wa[j];
-                    exam += tx;
+            for (int t = 0; t < kMsUnroll; ++t)
+                x[t] = u[t] >= 0 && wok ? ld_words<WL>(a.V + (size_t)u[t] * a.W + w) : zero_words<WL>();
+            const int32_t left = end - k;
+            k += kMsUnroll;
+#pragma unroll
+            for (int t = 0; t < kMsUnroll; ++t) u[t] = v >= 0 && k + t < end ? __ldg(a.in_col + k + t) : -1;
+            bool cov = true;
+#pragma unroll
+            for (int j = 0; j < WL; ++j) {
+#pragma unroll
+                for (int t = 0; t < kMsUnroll; ++t) ac.x[j] |= x[t].x[j];
+                cov &= (ac.x[j] & unv.x[j]) == unv.x[j];
+            }
+            const bool covered = gr.all(cov);
+            if (v >= 0 && gr.sub == 0) acc.exam += chunks256 * (uint32_t)(left < kMsUnroll ? left : kMsUnroll);
+            const bool done = v >= 0 && (covered || k >= end);
+            const bool put_off = defer && v >= 0 && !done && k >= lim && lim != end;
+            if (!__any_sync(0xffffffffu, done || put_off)) continue;
+            Words<WL> nw;
+#pragma unroll
+            for (int j = 0; j < WL; ++j) nw.x[j] = done || put_off ? ac.x[j] & unv.x[j] : 0ull;
+            const bool any_new = gr.any(nw.any());
+            const bool full = gr.all(!done || (nw.x[0] == unv.x[0] && nw.x[WL - 1] == unv.x[WL - 1]));
+            // F_next is zero before the level: only words with new lanes are written
+            if (nw.any()) {
+                const size_t iv = (size_t)v * a.W + w;
+                if (done && sink) {
+                    // nobody's in-neighbour: no other row reads its V, and it never joins the active list
+                    Words<WL> t = ld_words<WL>(a.V + iv);
+#pragma unroll
+                    for (int j = 0; j < WL; ++j) t.x[j] |= nw.x[j];
+                    st_words<WL>(a.V + iv, t);
+                } else {
+                    st_words<WL>(Fn + iv, nw);
+                }
+                if (done) {
+#pragma unroll
+                    for (int j = 0; j < WL; ++j) acc.n_new += (uint32_t)__popcll(nw.x[j]);
+                    Words<WL> was;
+#pragma unroll
+                    for (int j = 0; j < WL; ++j) was.x[j] = ~unv.x[j] & lm.x[j];
+                    record_words<WL>(a, v, w, nw, was, L + 1);
                 }
             }
-            acc.exam += exam;
-#pragma unroll
-            for (int j = 0; j < CW; ++j) {
-                const unsigned long long nw = accw[j] & unv[j];
-                if (mine) Fn[(size_t)v * a.W + c + j] = nw;
-                if (sink) {
-                    a.V[(size_t)v * a.W + c + j] |= nw;
-                    full &= unv[j] == nw;
+            bool take = done && gr.sub == 0 && any_new && !sink;
+            if (done && sink && full && one && gr.sub == 0) atomicOr(a.D + (v >> 5), 1u << (v & 31));
+            if (!one && take) take = !(atomicOr(Tn + (v >> 5), 1u << (v & 31)) & (1u << (v & 31)));
+            st.put(take, v);
+            const uint32_t dm = __ballot_sync(0xffffffffu, put_off && gr.sub == 0);
+            if (dm) {
+                const uint32_t nch = put_off && gr.sub == 0 ? (uint32_t)(end - k + kMsChunk - 1) / kMsChunk : 0u;
+                const uint32_t inc = warp_inclusive_sum(nch);
+                const uint32_t tot = __shfl_sync(0xffffffffu, inc, 31);
+                unsigned long long old = 0ull;
+                if (lane == 0)
+                    old = atomicAdd(&st.cout->huge, ((unsigned long long)tot << 32) | (unsigned long long)__popc(dm));
+                old = __shfl_sync(0xffffffffu, old, 0);
+                if (put_off && gr.sub == 0) {
+                    const uint32_t slot = (uint32_t)old + __popc(dm & lanemask_lt());
+                    lr.row[slot] = v;
+                    lr.k[slot] = k;
+                    lr.base[slot] = (int32_t)((uint32_t)(old >> 32) + inc - nch);
                 }
-                any_new |= nw != 0ull;
-                acc.n_new += (uint32_t)__popcll(nw);
-                if (mine) record_depth(a, v, c + j, nw, L + 1, false);
             }
+            if (done || put_off) v = -1;
         }
-        if (sink && full) atomicOr(a.D + (v >> 5), 1u << (v & 31));
-        st.put(any_new && !sink, v);
     }
     st.flush();
 }
 
+// The deferred rows' chunks, round-robin over the warps: the groups of a warp take
+// kMsUnroll in-neighbours each per step, their results are ORed together and folded into
+// F_next (which already holds what the probe found).  A chunk of a row that is covered by
+// then is skipped.
+template <int WL>
+__device__ __forceinline__ void ms_pull_long(const MsArgs& a, unsigned long long* Fn, const MsLong& lr,
+                                             int32_t entries, int32_t chunks, Acc& acc) {
+    const int gwarp = (int)((blockIdx.x * kMsThreads + threadIdx.x) >> 5);
+    const int nwarps = (int)((gridDim.x * kMsThreads) >> 5);
+    const Group gr(a.group);
+    const int32_t w = WL * gr.sub;
+    const bool wok = w < a.W;
+    const int32_t step = kMsUnroll * (32 / gr.size);
+    const uint32_t chunks256 = (uint32_t)(a.W + 3) >> 2;
+    for (int32_t c = gwarp; c < chunks; c += nwarps) {
+        const int32_t e = warp_find_entry(lr.base, entries, c);
+        const int32_t v = lr.row[e];
+        const int32_t rend = __ldg(a.in_ptr + v + 1);
+        const int32_t beg = lr.k[e] + (c - lr.base[e]) * kMsChunk;
+        const int32_t end = rend - beg < kMsChunk ? rend : beg + kMsChunk;
+        const size_t iv = (size_t)v * a.W + w;
+        Words<WL> unv = zero_words<WL>(), ac = zero_words<WL>();
+        if (wok) {
+            const Words<WL> vis = ld_words<WL>(a.V + iv);
+#pragma unroll
+            for (int j = 0; j < WL; ++j)  // what the row still misses (the fold of another chunk may have come in)
+                unv.x[j] = ~(vis.x[j] | __ldcg(Fn + iv + j)) & lane_mask(a.S, w + j);
+        }
+        if (!__any_sync(0xffffffffu, unv.any())) continue;
+        int32_t k0 = beg;
+        const int32_t kofs = kMsUnroll * (gr.first / gr.size);
+        int32_t u[kMsUnroll];  // the group's in-neighbours of this step; the next step's are loaded meanwhile
+#pragma unroll
+        for (int t = 0; t < kMsUnroll; ++t) u[t] = k0 + kofs + t < end ? __ldg(a.in_col + k0 + kofs + t) : -1;
+        while (k0 < end) {
+            Words<WL> x[kMsUnroll];
+#pragma unroll
+            for (int t = 0; t < kMsUnroll; ++t)
+                x[t] = u[t] >= 0 && wok ? ld_words<WL>(a.V + (size_t)u[t] * a.W + w) : zero_words<WL>();
+            k0 += step;
+#pragma unroll
+            for (int t = 0; t < kMsUnroll; ++t) u[t] = k0 + kofs + t < end ? __ldg(a.in_col + k0 + kofs + t) : -1;
+#pragma unroll
+            for (int j = 0; j < WL; ++j)
+#pragma unroll
+                for (int t = 0; t < kMsUnroll; ++t) ac.x[j] |= x[t].x[j];
+            if (k0 < end && ((k0 - beg) & (kMsCheck - 1)) != 0) continue;
+            bool cov = true;
+#pragma unroll
+            for (int j = 0; j < WL; ++j) {
+                for (int o = gr.size; o < 32; o <<= 1) ac.x[j] |= __shfl_xor_sync(0xffffffffu, ac.x[j], o);
+                cov &= (ac.x[j] & unv.x[j]) == unv.x[j];
+            }
+            if (__all_sync(0xffffffffu, cov)) break;
+        }
+        if ((threadIdx.x & 31) == 0) acc.exam += chunks256 * (uint32_t)((k0 < end ? k0 : end) - beg);
+        if (gr.first == 0)
+#pragma unroll
+            for (int j = 0; j < WL; ++j)
+                if (ac.x[j] & unv.x[j]) atomicOr(Fn + iv + j, ac.x[j] & unv.x[j]);
+    }
+}
+
 // V |= F for the vertices found by the pull level; mark vertices with all lanes visited.
-template <int CW>
+template <int WL>
 __device__ __forceinline__ void ms_pull_commit(const MsArgs& a, const int32_t* list, uint32_t count,
                                                const unsigned long long* Fn) {
-    const long long gtid = (long long)blockIdx.x * kMsThreads + threadIdx.x;
-    const long long gstride = (long long)gridDim.x * kMsThreads;
-    for (long long k = gtid; k < count; k += gstride) {
-        const int32_t v = list[k];
-        bool full = true;
-        for (int32_t w = 0; w < a.W; ++w) {
-            const unsigned long long x = a.V[(size_t)v * a.W + w] | Fn[(size_t)v * a.W + w];
-            a.V[(size_t)v * a.W + w] = x;
-            full &= (x & lane_mask(a.S, w)) == lane_mask(a.S, w);
+    const Group gr(a.group);
+    const int per = 32 / gr.size;  // vertices a warp takes at a time
+    const long long gwarp = ((long long)blockIdx.x * kMsThreads + threadIdx.x) >> 5;
+    const long long nwarps = ((long long)gridDim.x * kMsThreads) >> 5;
+    for (long long b = gwarp * per; b < count; b += nwarps * per) {  // warp-uniform
+        const long long i = b + gr.first / gr.size;
+        const int32_t v = i < count ? list[i] : -1;
+        bool full = v >= 0;
+        for (int32_t w = WL * gr.sub; v >= 0 && w < a.W; w += WL * gr.size) {
+            const size_t iv = (size_t)v * a.W + w;
+            Words<WL> x = ld_words<WL>(a.V + iv);
+            const Words<WL> f = ld_words<WL>(Fn + iv);
+#pragma unroll
+            for (int j = 0; j < WL; ++j) {
+                x.x[j] |= f.x[j];
+                full &= (x.x[j] & lane_mask(a.S, w + j)) == lane_mask(a.S, w + j);
+            }
+            if (f.any()) st_words<WL>(a.V + iv, x);
         }
-        if (full) atomicOr(a.D + (v >> 5), 1u << (v & 31));
+        if (gr.all(full) && gr.sub == 0) atomicOr(a.D + (v >> 5), 1u << (v & 31));
     }
 }
 
 // ---------------------------------------------------------------- push level
 
-// One phase: each edge (u, v) of the active list claims the lanes F_cur[u] & ~V[v]
+// W == 1, one phase: each edge (u, v) of the active list claims the lanes F_cur[u] & ~V[v]
 // with an atomicOr on V[v]; the lanes it gained (not set before) are new at level
 // L + 1 and this edge is their only claimant, so it writes their depth and ORs them
-// into F_next[v]; the first edge to gain anything at v lists v (for W == 1 the
-// previous F_next word tells, otherwise the T_next bit).  One-word batches claim
-// without probing V[v] first (a dependent load per edge costs more than the extra
-// atomics); wider ones probe, which only saves reductions (bits are only ever set).
-template <int CW>
-__device__ __forceinline__ void ms_push(const MsArgs& a, int32_t L, const int32_t* q, const int32_t* qp,
-                                        const int32_t* qd, uint32_t qcount, uint32_t qedges,
-                                        const unsigned long long* Fc, unsigned long long* Fn, uint32_t* Tn, Stage& st,
-                                        Acc& acc) {
+// into F_next[v]; the first edge to gain anything at v (the previous F_next word tells)
+// lists v.  It claims without probing V[v] first (a dependent load per edge costs more
+// than the extra atomics).
+__device__ __forceinline__ void ms_push_one(const MsArgs& a, int32_t L, const int32_t* q, const int32_t* qp,
+                                            const int32_t* qd, uint32_t qcount, uint32_t qedges,
+                                            const unsigned long long* Fc, unsigned long long* Fn, Stage& st,
+                                            Acc& acc) {
     const int gwarp = (int)((blockIdx.x * kMsThreads + threadIdx.x) >> 5);
     const int nwarps = (int)((gridDim.x * kMsThreads) >> 5);
     const int32_t E = (int32_t)qedges;
@@ -325,121 +673,194 @@ __device__ __forceinline__ void ms_push(const MsArgs& a, int32_t L, const int32_
             for (int t = 0; t < kPushIlp; ++t) {
                 const int32_t u = ps.u[t], v = ps.v[t];
                 bool first = false;
-                if (CW > 1 && u >= 0 && !((a.D[v >> 5] >> (v & 31)) & 1u)) {
-                    // wide batch: accumulate, finalised after the barrier
-                    bool touched = false;
-                    for (int32_t c = 0; c < a.W; c += CW) {
-#pragma unroll
-                        for (int j = 0; j < CW; ++j) {
-                            const size_t iu = (size_t)u * a.W + c + j, iv = (size_t)v * a.W + c + j;
-                            const unsigned long long cand = Fc[iu] & ~a.V[iv];
-                            if (cand) {
-                                atomicOr(Fn + iv, cand);  // result unused: a reduction
-                                touched = true;
-                            }
-                        }
-                    }
-                    if (touched) first = !(atomicOr(Tn + (v >> 5), 1u << (v & 31)) & (1u << (v & 31)));
-                } else if (CW == 1 && u >= 0 && !((a.D[v >> 5] >> (v & 31)) & 1u)) {
-                    bool any = false;
-                    for (int32_t c = 0; c < a.W; c += CW) {
-#pragma unroll
-                        for (int j = 0; j < CW; ++j) {
-                            const size_t iu = (size_t)u * a.W + c + j, iv = (size_t)v * a.W + c + j;
-                            const unsigned long long cand = Fc[iu];
-                            if (!cand) continue;
-                            const unsigned long long old = atomicOr(a.V + iv, cand);
-                            const unsigned long long gained = cand & ~old;
-                            if (!gained) continue;
-                            if (a.W == 1) {
-                                first |= atomicOr(Fn + iv, gained) == 0ull;
-                                if (((old | cand) & full0) == full0) atomicOr(a.D + (v >> 5), 1u << (v & 31));
-                            } else {
-                                atomicOr(Fn + iv, gained);  // result unused: a reduction; T_next lists v
-                            }
-                            any = true;
+                if (u >= 0 && !((a.D[v >> 5] >> (v & 31)) & 1u)) {
+                    const unsigned long long cand = Fc[u];
+                    if (cand) {
+                        const unsigned long long old = atomicOr(a.V + v, cand);
+                        const unsigned long long gained = cand & ~old;
+                        if (gained) {
+                            first = atomicOr(Fn + v, gained) == 0ull;
+                            if (((old | cand) & full0) == full0) atomicOr(a.D + (v >> 5), 1u << (v & 31));
                             acc.n_new += (uint32_t)__popcll(gained);
-                            record_depth(a, v, c + j, gained, L + 1, true);
+                            record_depth(a, v, 0, gained, L + 1, true);
                         }
                     }
-                    (void)any;
                 }
-                if (CW == 1) {
-                    st.put(first, v);
-                } else {
-                    // warp-aggregated append to the touched list
-                    const int lane = threadIdx.x & 31;
-                    const uint32_t m = __ballot_sync(0xffffffffu, first);
-                    if (m) {
-                        unsigned long long base_pos = 0;
-                        if (lane == 0) base_pos = atomicAdd(&st.cout->list, (unsigned long long)__popc(m));
-                        base_pos = __shfl_sync(0xffffffffu, base_pos, 0);
-                        if (first) a.tlist[base_pos + __popc(m & lanemask_lt())] = v;
-                    }
-                }
+                st.put(first, v);
             }
         }
     }
-    if (CW == 1) st.flush();
+    st.flush();
 }
 
-// Wide push levels, after the barrier: new = F_next & ~V for the touched vertices;
-// V |= new, F_next = new, depth, "all lanes" map; the touched ones with new lanes
-// form the next active list.  Every T_next bit belongs to a touched vertex, so the
-// words are cleared whole (racing writers all store zero).
-template <int CW>
-__device__ __forceinline__ void ms_push_finalize(const MsArgs& a, int32_t L, uint32_t count, unsigned long long* Fn,
-                                                 uint32_t* Tn, Stage& st, Acc& acc) {
-    const long long gtid = (long long)blockIdx.x * kMsThreads + threadIdx.x;
-    const long long gstride = (long long)gridDim.x * kMsThreads;
-    const long long rounds = ((long long)count + gstride - 1) / gstride;
-    for (long long r = 0; r < rounds; ++r) {  // warp-uniform trip count: st.put needs all lanes
-        const long long k = r * gstride + gtid;
-        const bool mine = k < count;
-        const int32_t v = mine ? a.tlist[k] : 0;
-        bool any_new = false, full = true;
-        if (mine) {
-            for (int32_t w = 0; w < a.W; ++w) {
-                const size_t idx = (size_t)v * a.W + w;
-                const unsigned long long vv = a.V[idx];
-                const unsigned long long nw = Fn[idx] & ~vv & lane_mask(a.S, w);
-                a.V[idx] = vv | nw;
-                Fn[idx] = nw;
-                full &= ((vv | nw) & lane_mask(a.S, w)) == lane_mask(a.S, w);
-                acc.n_new += (uint32_t)__popcll(nw);
-                any_new |= nw != 0ull;
-                record_depth(a, v, w, nw, L + 1, false);
+// Wide batches, first phase: a warp takes 32 edges (u, v) of the active list and its
+// groups OR F_cur[u] & ~V[v] into F_next[v] with reductions, one edge a group and
+// kMsUnroll in flight; a touched v is listed once (the T_next bit).  The probe of V[v]
+// only saves reductions (bits are only ever set).  A lane per edge walking its W words
+// instead touched 32 rows with every load: level 0 of the RMAT-20 batch of 1,000 sources
+// (55.7K edges), with the zeroing of the state, 276 us, now 128.
+template <int WL>
+__device__ __forceinline__ void ms_push_wide(const MsArgs& a, const int32_t* q, const int32_t* qp, const int32_t* qd,
+                                             uint32_t qcount, uint32_t qedges, const unsigned long long* Fc,
+                                             unsigned long long* Fn, uint32_t* Tn, StageBuf* sb, LevelCtr* cout) {
+    const int lane = threadIdx.x & 31;
+    const int gwarp = (int)((blockIdx.x * kMsThreads + threadIdx.x) >> 5);
+    const int nwarps = (int)((gridDim.x * kMsThreads) >> 5);
+    const Group gr(a.group);
+    const int per = 32 / gr.size;  // edges the warp's groups take at a time
+    const int32_t E = (int32_t)qedges;
+    int32_t chunk = (int32_t)(((long long)E + nwarps - 1) / nwarps);
+    chunk = chunk < 32 ? 32 : ((chunk + 31) / 32) * 32;
+    int staged = 0;  // touched vertices waiting in sb (warp-uniform)
+    auto publish = [&]() {
+        __syncwarp();
+        unsigned long long pos = 0ull;
+        if (lane == 0) pos = atomicAdd(&cout->list, (unsigned long long)staged);
+        pos = __shfl_sync(0xffffffffu, pos, 0);
+        for (int i = lane; i < staged; i += 32) a.tlist[pos + i] = sb->v[i];
+        staged = 0;
+        __syncwarp();
+    };
+    for (long long e0l = (long long)gwarp * chunk; e0l < E; e0l += (long long)nwarps * chunk) {
+        const int32_t e0 = (int32_t)e0l;
+        const int32_t e1 = E - e0 > chunk ? e0 + chunk : E;
+        PushCursorT<1> cur_;
+        cur_.k = warp_find_entry(qp, (int32_t)qcount, e0);
+        cur_.wlast = -1;
+        for (int32_t base = e0; base < e1; base += 32) {
+            const PushStepT<1> ps = cur_.gather(a.out_col, q, qp, qd, qcount, base, e1);
+            const int32_t v = ps.v[0];
+            const int32_t u = ps.u[0] >= 0 && !((a.D[v >> 5] >> (v & 31)) & 1u) ? ps.u[0] : -1;
+            bool touched = false;
+            for (int32_t w = WL * gr.sub; w - WL * gr.sub < a.W; w += WL * gr.size) {
+                for (int j0 = 0; j0 < gr.size; j0 += kMsUnroll) {
+                    int32_t vv[kMsUnroll];
+                    Words<WL> f[kMsUnroll], x[kMsUnroll];
+#pragma unroll
+                    for (int t = 0; t < kMsUnroll; ++t) {
+                        const int e = (j0 + t) * per + gr.first / gr.size;  // the group's edge (a lane of the warp)
+                        const int32_t uu = __shfl_sync(0xffffffffu, u, e & 31);
+                        vv[t] = __shfl_sync(0xffffffffu, v, e & 31);
+                        const bool ok = j0 + t < gr.size && uu >= 0 && w < a.W;
+                        f[t] = ok ? ld_words<WL>(Fc + (size_t)uu * a.W + w) : zero_words<WL>();
+                        x[t] = ok ? ld_words<WL>(a.V + (size_t)vv[t] * a.W + w) : zero_words<WL>();
+                    }
+#pragma unroll
+                    for (int t = 0; t < kMsUnroll; ++t) {
+                        bool hit = false;
+#pragma unroll
+                        for (int j = 0; j < WL; ++j) {
+                            const unsigned long long cand = f[t].x[j] & ~x[t].x[j];
+                            if (cand) {
+                                atomicOr(Fn + (size_t)vv[t] * a.W + w + j, cand);  // result unused: a reduction
+                                hit = true;
+                            }
+                        }
+                        const uint32_t hm = __ballot_sync(0xffffffffu, hit);
+                        // this lane's edge was taken by group lane % per in round lane / per
+                        const uint32_t gm = gr.size == 32 ? 0xffffffffu : (1u << gr.size) - 1u;
+                        if (lane / per == j0 + t) touched |= ((hm >> ((lane % per) * gr.size)) & gm) != 0u;
+                    }
+                }
             }
-            Tn[v >> 5] = 0u;
-            if (full) atomicOr(a.D + (v >> 5), 1u << (v & 31));
+            const bool first = touched && !(atomicOr(Tn + (v >> 5), 1u << (v & 31)) & (1u << (v & 31)));
+            const uint32_t fm = __ballot_sync(0xffffffffu, first);
+            if (fm) {
+                if (staged + __popc(fm) > kStage) publish();
+                if (first) sb->v[staged + __popc(fm & lanemask_lt())] = v;
+                staged += __popc(fm);
+            }
         }
-        st.put(mine && any_new, v);
+    }
+    if (staged) publish();
+}
+
+// Vertices whose F_next words were gathered by several warps (a wide push level's touched
+// ones, a pull level's deferred rows), after a barrier: new = F_next & ~V; V |= new,
+// F_next = new, depth, "all lanes" map; those with new lanes join the next active list.
+// Every T_next bit belongs to a touched vertex, so the words are cleared whole (racing
+// writers all store zero).
+template <int WL>
+__device__ __forceinline__ void ms_finalize(const MsArgs& a, int32_t L, const int32_t* list, uint32_t count,
+                                            unsigned long long* Fn, uint32_t* Tn, Stage& st, Acc& acc) {
+    const Group gr(a.group);
+    const int per = 32 / gr.size;
+    const long long gwarp = ((long long)blockIdx.x * kMsThreads + threadIdx.x) >> 5;
+    const long long nwarps = ((long long)gridDim.x * kMsThreads) >> 5;
+    for (long long b = gwarp * per; b < count; b += nwarps * per) {  // warp-uniform: st.put needs all lanes
+        const long long i = b + gr.first / gr.size;
+        const int32_t v = i < count ? list[i] : -1;
+        bool any_new = false, full = v >= 0;
+        for (int32_t w = WL * gr.sub; v >= 0 && w < a.W; w += WL * gr.size) {
+            const size_t iv = (size_t)v * a.W + w;
+            Words<WL> x = ld_words<WL>(a.V + iv);
+            const Words<WL> was = x, f = ld_words<WL>(Fn + iv);
+            Words<WL> nw;
+            bool changed = false;
+#pragma unroll
+            for (int j = 0; j < WL; ++j) {
+                const unsigned long long lm = lane_mask(a.S, w + j);
+                nw.x[j] = f.x[j] & ~x.x[j] & lm;
+                changed |= nw.x[j] != f.x[j];
+                x.x[j] |= nw.x[j];
+                full &= (x.x[j] & lm) == lm;
+                acc.n_new += (uint32_t)__popcll(nw.x[j]);
+            }
+            if (changed) st_words<WL>(Fn + iv, nw);
+            if (nw.any()) st_words<WL>(a.V + iv, x);
+            any_new |= nw.any();
+            record_words<WL>(a, v, w, nw, was, L + 1);
+        }
+        const bool allfull = gr.all(full);
+        any_new = gr.any(any_new);
+        if (v >= 0 && gr.sub == 0) {
+            Tn[v >> 5] = 0u;
+            if (allfull) atomicOr(a.D + (v >> 5), 1u << (v & 31));
+        }
+        st.put(v >= 0 && gr.sub == 0 && any_new, v);
     }
     st.flush();
 }
 
 // Clear F_{(L+2) mod 3} and T_{(L+2) mod 3} for the active list of level L - 1:
 // those buffers were last read at level L - 1 and are written again at level L + 1.
+template <int WL>
 __device__ __forceinline__ void ms_clear_prev(const MsArgs& a, const int32_t* ids, uint32_t count,
                                               unsigned long long* F, uint32_t* T) {
-    const long long gtid = (long long)blockIdx.x * kMsThreads + threadIdx.x;
-    const long long gstride = (long long)gridDim.x * kMsThreads;
-    for (long long k = gtid; k < count; k += gstride) {
-        const int32_t v = ids[k];
-        for (int32_t w = 0; w < a.W; ++w) F[(size_t)v * a.W + w] = 0ull;
-        T[v >> 5] = 0u;  // every bit of T_{(L+2) mod 3} belongs to that list: racing writers all store zero
+    const Group gr(a.group);
+    const int per = 32 / gr.size;
+    const long long gwarp = ((long long)blockIdx.x * kMsThreads + threadIdx.x) >> 5;
+    const long long nwarps = ((long long)gridDim.x * kMsThreads) >> 5;
+    for (long long b = gwarp * per; b < count; b += nwarps * per) {
+        const long long i = b + gr.first / gr.size;
+        if (i >= count) continue;
+        const int32_t v = ids[i];
+        for (int32_t w = WL * gr.sub; w < a.W; w += WL * gr.size)
+            st_words<WL>(F + (size_t)v * a.W + w, zero_words<WL>());
+        // every bit of T_{(L+2) mod 3} belongs to that list: racing writers all store zero
+        if (gr.sub == 0) T[v >> 5] = 0u;
     }
 }
 
 // ---------------------------------------------------------------- kernel
 
-template <int CW, int kOcc>
-__global__ void __launch_bounds__(kMsThreads, kOcc) ms_bfs_kernel(MsArgs a) {
+template <int WL, int kOcc>
+__global__ void __launch_bounds__(kMsThreads, kOcc) ms_bfs_kernel(const __grid_constant__ MsArgs a) {
     const long long gtid = (long long)blockIdx.x * kMsThreads + threadIdx.x;
     // an error of an earlier launch not yet read by the host: this launch does nothing
     const int pending = threadIdx.x == 0 ? ld_volatile_i32(a.status + ST_ERROR) : 0;
     const long long gstride = (long long)gridDim.x * kMsThreads;
-    __shared__ StageBuf stage_mem[kMsThreads / 32];
+    // per warp: staged vertices, open rows of a pull level; after the last level the
+    // emission's staging area
+    struct WarpMem {
+        StageBuf stage;
+        uint16_t open_list[1024];
+    };
+    union BlockMem {
+        WarpMem warp[kMsThreads / 32];
+        uint32_t emit[WL == 2 ? kEmitSmem / 4 : 1];
+    };
+    __shared__ __align__(16) BlockMem mem;
     __shared__ unsigned long long lvl[6];
     __shared__ unsigned long long acc_mem[kMsThreads / 32][4];
     const int wib = threadIdx.x >> 5;
@@ -453,8 +874,9 @@ __global__ void __launch_bounds__(kMsThreads, kOcc) ms_bfs_kernel(MsArgs a) {
         a.Fb[0][i] = 0ull;
         a.Fb[1][i] = 0ull;
         a.Fb[2][i] = 0ull;
+        if (WL == 1)
 #pragma unroll
-        for (int p = 0; p < kMsPlanes; ++p) a.P[p][i] = 0ull;
+            for (int p = 0; p < kMsPlanes; ++p) a.P[p][i] = 0ull;
     }
     for (long long w = gtid; w < a.nwords; w += gstride) {
         a.D[w] = 0u;
@@ -476,12 +898,15 @@ __global__ void __launch_bounds__(kMsThreads, kOcc) ms_bfs_kernel(MsArgs a) {
     for (long long b = gtid; b < a.S; b += gstride) {
         const int32_t s = a.src[b];
         atomicOr(a.V + (size_t)s * a.W + (b >> 6), 1ull << (b & 63));  // depth 0: no plane bit
+        if (WL == 2)
+#pragma unroll
+            for (int p = 0; p < kMsPlanes; ++p) a.P[p][(size_t)s * a.W + (b >> 6)] = 0ull;
     }
     if (!grid_barrier(barc, gridDim.x, bar_round, a.status, a.timeout_ns)) return;
     // F = V for the (distinct) source vertices; they form the first active list
     {
         Acc acc0;
-        Stage st{stage_mem + wib, 0, a.ctr + 0, a.ids[0], a.qp[0], a.qd[0], a.out_ptr, a.in_ptr, 1, 0, &acc0};
+        Stage st{&mem.warp[wib].stage, 0, a.ctr + 0, a.ids[0], a.qp[0], a.qd[0], a.out_ptr, a.in_ptr, 1, 0, &acc0};
         const long long rounds = ((long long)a.S + gstride - 1) / gstride;
         for (long long r = 0; r < rounds; ++r) {
             const long long b = r * gstride + gtid;
@@ -525,18 +950,24 @@ __global__ void __launch_bounds__(kMsThreads, kOcc) ms_bfs_kernel(MsArgs a) {
             return;
         }
         Acc acc;
-        Stage st{stage_mem + wib, 0, cout, a.ids[r1], a.qp[p1], a.qd[p1], a.out_ptr, a.in_ptr, 1, 0, &acc};
-        ms_clear_prev(a, a.ids[r2], prev_count, a.Fb[r2], a.Tb[r2]);
+        Stage st{&mem.warp[wib].stage, 0, cout, a.ids[r1], a.qp[p1], a.qd[p1], a.out_ptr, a.in_ptr, 1, 0, &acc};
+        ms_clear_prev<WL>(a, a.ids[r2], prev_count, a.Fb[r2], a.Tb[r2]);
+        const MsLong lr{a.tlist, a.qp[p0], a.qd[p0]};  // a pull level does not read the queue's prefix
         if (dir == GBX_DIR_PUSH) {
-            ms_push<CW>(a, L, a.ids[r0], a.qp[p0], a.qd[p0], qcount, qedges, a.Fb[r0], a.Fb[r1], a.Tb[r1], st, acc);
-            if (CW > 1) {
+            if (WL == 1) {
+                ms_push_one(a, L, a.ids[r0], a.qp[p0], a.qd[p0], qcount, qedges, a.Fb[r0], a.Fb[r1], st, acc);
+            } else {
+                ms_push_wide<WL>(a, a.ids[r0], a.qp[p0], a.qd[p0], qcount, qedges, a.Fb[r0], a.Fb[r1], a.Tb[r1],
+                                 &mem.warp[wib].stage, cout);
                 if (!grid_barrier(barc, gridDim.x, bar_round, a.status, a.timeout_ns)) return;
                 if (threadIdx.x == 0) lvl[5] = ld_volatile_u64(&cout->list);
                 __syncthreads();
-                ms_push_finalize<CW>(a, L, (uint32_t)lvl[5], a.Fb[r1], a.Tb[r1], st, acc);
+                ms_finalize<WL>(a, L, a.tlist, (uint32_t)lvl[5], a.Fb[r1], a.Tb[r1], st, acc);
             }
         } else {
-            ms_pull<CW>(a, L, a.Fb[r1], st, acc);
+            const bool one = a.W <= WL * a.group;  // one chunk of words: long rows can be deferred
+            for (int32_t c0 = 0; c0 < a.W; c0 += WL * a.group)
+                ms_pull<WL>(a, L, c0, a.Fb[r1], a.Tb[r1], mem.warp[wib].open_list, lr, one, st, acc);
         }
         block_add_counts<kMsThreads / 32>(acc_mem, acc.n_new, acc.mf, acc.exam, 0ull, &cout->n_new, &cout->mf_new,
                                           &cout->e_exam, nullptr);
@@ -544,15 +975,34 @@ __global__ void __launch_bounds__(kMsThreads, kOcc) ms_bfs_kernel(MsArgs a) {
         if (threadIdx.x == 0) {
             lvl[0] = ld_volatile_u64(&cout->n_new);
             lvl[1] = ld_volatile_u64(&cout->mf_new);
+            lvl[2] = ld_volatile_u64(&cout->huge);
             lvl[3] = ld_volatile_u64(&cout->e_exam);
             lvl[4] = ld_volatile_u64(&cout->q);
         }
         __syncthreads();
+        if (dir == GBX_DIR_PULL && lvl[2] != 0ull) {  // the level deferred long rows: the grid takes them now
+            const uint32_t rows = (uint32_t)lvl[2];
+            Acc acc2;
+            Stage st2{&mem.warp[wib].stage, 0, cout, a.ids[r1], a.qp[p1], a.qd[p1], a.out_ptr, a.in_ptr, 1, 0, &acc2};
+            ms_pull_long<WL>(a, a.Fb[r1], lr, (int32_t)rows, (int32_t)(lvl[2] >> 32), acc2);
+            if (!grid_barrier(barc, gridDim.x, bar_round, a.status, a.timeout_ns)) return;
+            ms_finalize<WL>(a, L, lr.row, rows, a.Fb[r1], a.Tb[r1], st2, acc2);
+            block_add_counts<kMsThreads / 32>(acc_mem, acc2.n_new, acc2.mf, acc2.exam, 0ull, &cout->n_new,
+                                              &cout->mf_new, &cout->e_exam, nullptr);
+            if (!grid_barrier(barc, gridDim.x, bar_round, a.status, a.timeout_ns)) return;
+            if (threadIdx.x == 0) {
+                lvl[0] = ld_volatile_u64(&cout->n_new);
+                lvl[1] = ld_volatile_u64(&cout->mf_new);
+                lvl[3] = ld_volatile_u64(&cout->e_exam);
+                lvl[4] = ld_volatile_u64(&cout->q);
+            }
+            __syncthreads();
+        }
         qv = lvl[4];
         if (dir == GBX_DIR_PULL) {
             // V |= F for the vertices the pull found (their new lanes were kept apart so the
             // level read V as it was before it started)
-            ms_pull_commit<CW>(a, a.ids[r1], (uint32_t)qv, a.Fb[r1]);
+            ms_pull_commit<WL>(a, a.ids[r1], (uint32_t)qv, a.Fb[r1]);
             if (!grid_barrier(barc, gridDim.x, bar_round, a.status, a.timeout_ns)) return;
         }
         const long long n_new = (long long)lvl[0];
@@ -573,7 +1023,10 @@ __global__ void __launch_bounds__(kMsThreads, kOcc) ms_bfs_kernel(MsArgs a) {
         }
         if (n_new == 0) {
             if (gtid == 0) a.status[ST_LEVELS] = L + 1;
-            emit_depths(a);
+            if (WL == 2 && a.W >= 4)
+                emit_depths<true>(a, mem.emit);
+            else
+                emit_depths<false>(a, mem.emit);
             return;
         }
         if (L + 1 >= a.n) {
@@ -626,17 +1079,17 @@ int64_t ms_scratch_bytes(int32_t n, int32_t S) {
     return (4ll + kMsPlanes) * 8ll * (int64_t)n * ((w_raw + cw - 1) / cw * cw) + 4ll * ((int64_t)n + 1);
 }
 
-template <int CW, int kOcc>
+template <int WL, int kOcc>
 static gbx_status ms_launch(Graph* G, const MsArgs& a0, int blocks, int per_sm_cap, cudaStream_t s) {
     int per_sm = 0;
-    GBX_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ms_bfs_kernel<CW, kOcc>, kMsThreads, 0));
+    GBX_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ms_bfs_kernel<WL, kOcc>, kMsThreads, 0));
     GBX_CHECK(per_sm >= 1, GBX_ERR_CUDA, "batched BFS kernel cannot be resident");
     if (per_sm_cap > 0 && per_sm_cap < per_sm) per_sm = per_sm_cap;
     const int full = per_sm * G->num_sms;
     const int nb = blocks > 1 ? (full / blocks > 0 ? full / blocks : 1) : full;  // a 1/blocks share of the GPU
     MsArgs a = a0;
     void* args[] = {&a};
-    GBX_CUDA_TRY(cudaLaunchCooperativeKernel((const void*)ms_bfs_kernel<CW, kOcc>, dim3(nb), dim3(kMsThreads), args, 0,
+    GBX_CUDA_TRY(cudaLaunchCooperativeKernel((const void*)ms_bfs_kernel<WL, kOcc>, dim3(nb), dim3(kMsThreads), args, 0,
                                              s));
     return GBX_OK;
 }
@@ -698,9 +1151,9 @@ gbx_status ms_run(Graph* G, Workspace& w, int32_t S, const int32_t* src_dev, voi
     const bool lean = blocks <= 1 && d.blocks_per_sm >= kMsOccLean && cw <= 2;
     const int cap = lean ? 0 : d.blocks_per_sm;
     gbx_status st;
-    if (cw == 4)
-        st = ms_launch<4, kMsOcc>(G, a, blocks, cap, s);
-    else if (cw == 2)
+    a.group = 1;
+    while (2 * a.group < W && a.group < 32) a.group *= 2;
+    if (W > 1)
         st = lean ? ms_launch<2, kMsOccLean>(G, a, blocks, cap, s) : ms_launch<2, kMsOcc>(G, a, blocks, cap, s);
     else
         st = lean ? ms_launch<1, kMsOccLean>(G, a, blocks, cap, s) : ms_launch<1, kMsOcc>(G, a, blocks, cap, s);

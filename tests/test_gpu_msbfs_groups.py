@@ -1,0 +1,55 @@
+"""GPU parity of the batched BFS where its lane-word groups can go wrong: every group
+width (W = 1, 2, 4, 8, 12, 36 words and, above 64 words, two chunks), ragged last words,
+rows long enough to be deferred to the whole grid (in-degrees of about 5,700 and 7,800),
+directed graphs with vertices nobody leaves, odd vertex counts (output rows that no
+vector store fits) and depths on both sides of 16.  Depths equal the oracle's exactly."""
+import numpy as np
+import pytest
+
+import oracle
+import synth
+from paper_1804_03327_gb300 import gbx
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+_cache = {}
+
+
+def graph(name):
+    if name not in _cache:
+        if name == "chain":  # a path with a dense end: depths 0 .. 40 in one batch
+            k = 40
+            a, b = np.triu_indices(30, 1)
+            s = np.concatenate([np.arange(k), k + a]).astype(np.int32)
+            d = np.concatenate([np.arange(1, k + 1), k + b]).astype(np.int32)
+            n, directed = k + 30 + 3, False
+        else:
+            directed = name == "hubs-directed"
+            n, s, d = synth.rmat_edges(13, 8, seed=21)
+            hs, hd = [s], [d]
+            for h, p in ((0, 0.7), (1, 0.95)):
+                v = np.flatnonzero(synth.vertex_set(n, p, seed=6, stream=h + 1)).astype(np.int32)
+                hs.append(v if directed else np.full(len(v), h, np.int32))
+                hd.append(np.full(len(v), h, np.int32) if directed else v)
+            s, d, n = np.concatenate(hs), np.concatenate(hd), n + 3
+        _cache[name] = (n, s, d, oracle.graph(n, s, d, symmetrize=not directed),
+                        gbx.graph_build(n, s, d, symmetrize=not directed))
+    return _cache[name]
+
+
+@pytest.mark.parametrize("name", ["hubs", "hubs-directed", "chain"])
+@pytest.mark.parametrize("S", [3, 64, 66, 130, 500, 700, 2100, 4200])
+@pytest.mark.parametrize("direction", [gbx.DIR_AUTO, gbx.DIR_PUSH, gbx.DIR_PULL])
+def test_lane_groups(name, S, direction):
+    n, s, d, og, g = graph(name)
+    pool = synth.sources(n, s, d, 64, seed=S)
+    srcs = pool[np.arange(S) % len(pool)]  # repeated sources: the oracle runs each once
+    dtype = torch.int16 if S % 4 else torch.int32
+    depth = torch.full((S, n), 77, dtype=dtype, device="cuda")
+    gbx.bfs_batch(g, srcs, depth, gbx.desc_init(direction=direction))
+    gbx.graph_sync(g)
+    want = {int(v): oracle.bfs(og, int(v))[0] for v in pool[: min(S, len(pool))]}
+    got = depth.cpu().numpy().astype(np.int32)
+    for b, v in enumerate(srcs):
+        assert np.array_equal(got[b], want[int(v)]), (b, int(v))
