@@ -22,6 +22,7 @@
 // barrier instead of kernel launches.
 #include <atomic>
 
+#include "bfs_cluster.cuh"
 #include "frontier.cuh"
 #include "gbx_internal.cuh"
 
@@ -64,6 +65,7 @@ struct BfsArgs {
     GridBar* bar;
     LevelRec* trace;
     int32_t* status;
+    const ClHandoff* ho;  // kResume: what the cluster kernel left
     float alpha, beta;
     int32_t heuristic, mode, early_exit, masking, operand_reuse, symmetric, need_indeg, need_deg, trace_cap, probe,
         tile_words;
@@ -707,30 +709,6 @@ __device__ __forceinline__ void bitmap_to_queue(const BfsArgs& a, int vcur, Stag
     st.flush_block<kBfsThreads / 32>(bsm);
 }
 
-// out[i] = fill for all i < n except out[special] = special_value; 16-byte stores when aligned.
-__device__ __forceinline__ void fill_outputs(int32_t* out, int32_t n, int32_t fill, int32_t special,
-                                             int32_t special_value, long long gtid, long long gstride) {
-    if ((reinterpret_cast<uintptr_t>(out) & 15u) == 0) {
-        const long long n4 = n >> 2;
-        int4* o4 = reinterpret_cast<int4*>(out);
-        for (long long q = gtid; q < n4; q += gstride) {
-            int4 v = make_int4(fill, fill, fill, fill);
-            const long long b = q << 2;
-            if (special >= b && special < b + 4) {
-                const int r = (int)(special - b);
-                if (r == 0) v.x = special_value;
-                if (r == 1) v.y = special_value;
-                if (r == 2) v.z = special_value;
-                if (r == 3) v.w = special_value;
-            }
-            o4[q] = v;
-        }
-        for (long long i = (n4 << 2) + gtid; i < n; i += gstride) out[i] = i == special ? special_value : fill;
-    } else {
-        for (long long i = gtid; i < n; i += gstride) out[i] = i == special ? special_value : fill;
-    }
-}
-
 struct LoopState {
     unsigned long long qv;  // queue of the next level: entries (low 32 bits), out-degree sum (high 32)
     long long nf, mf, mu;   // |F_L|, out-edges of F_L, in-edges of the rows unvisited before level L
@@ -799,7 +777,9 @@ __device__ __forceinline__ void level_end(const BfsArgs& a, int32_t L, int dir, 
 // expect full row scans (no early exit, or pull on every level); with the
 // direction rule and early exit a pull level rarely meets a long row without a
 // parent, and those runs keep the kernel without that phase (fewer registers).
-template <bool kTrace, bool kHuge>
+// kResume: the search goes on where bfs_cluster_kernel handed it over (outputs and
+// bitmap initialised, the frontier in q[1] and hfirst), or returns at once if it ended there.
+template <bool kTrace, bool kHuge, bool kResume>
 __global__ void __launch_bounds__(kBfsThreads, kBfsMinBlocks) bfs_kernel(BfsArgs a) {
     const long long gtid = (long long)blockIdx.x * kBfsThreads + threadIdx.x;
     const long long gstride = (long long)gridDim.x * kBfsThreads;
@@ -811,34 +791,38 @@ __global__ void __launch_bounds__(kBfsThreads, kBfsMinBlocks) bfs_kernel(BfsArgs
     // its claims (the source's out-neighbours, all new) write no outputs, so the outputs
     // are initialised during level 0 instead, hidden behind its latency, and level 1
     // starts by stamping the source's out-neighbours (depth 1, parent s).
-    const bool fill_in_level0 = a.mode != GBX_DIR_PULL;
-    if (!fill_in_level0) {
-        fill_outputs(a.depth, a.n, -1, s, 0, gtid, gstride);
-        if (a.parent) fill_outputs(a.parent, a.n, -1, s, s, gtid, gstride);
+    const bool fill_in_level0 = !kResume && a.mode != GBX_DIR_PULL;
+    if (!kResume && !fill_in_level0) {
+        fill_i32(a.depth, a.n, -1, s, 0, gtid, gstride);
+        if (a.parent) fill_i32(a.parent, a.n, -1, s, s, gtid, gstride);
     }
-    for (long long w = gtid; w < a.nwords; w += gstride) a.vis[0][w] = w == (s >> 5) ? 1u << (s & 31) : 0u;
+    if (!kResume)
+        for (long long w = gtid; w < a.nwords; w += gstride) a.vis[0][w] = w == (s >> 5) ? 1u << (s & 31) : 0u;
     const int32_t s_rs = __ldg(a.out_ptr + s);
     const int32_t s_od = __ldg(a.out_ptr + s + 1) - s_rs;
     const int32_t s_id = __ldg(a.in_ptr + s + 1) - __ldg(a.in_ptr + s);
     if (gtid == 0) {
-        if (s_od > 0) {
-            a.q[0][0] = s;
-            a.qp[0][0] = 0;
-            a.qd[0][0] = s_rs;
-        }
         LevelCtr z = {};
         a.ctr[1] = z;
         a.ctr[2] = z;
-        z.q = s_od > 0 ? (((unsigned long long)s_od << 32) | 1ull) : 0ull;
-        z.n_new = 1;
-        z.mf_new = (unsigned long long)s_od;
+        if (!kResume) {
+            if (s_od > 0) {
+                a.q[0][0] = s;
+                a.qp[0][0] = 0;
+                a.qd[0][0] = s_rs;
+            }
+            z.q = s_od > 0 ? (((unsigned long long)s_od << 32) | 1ull) : 0ull;
+            z.n_new = 1;
+            z.mf_new = (unsigned long long)s_od;
+            a.status[ST_LEVELS] = 0;
+        }
         a.ctr[0] = z;
-        a.status[ST_LEVELS] = 0;
         a.bar->count[a.bar_parity ^ 1u] = 0u;  // the next launch's counter
     }
     unsigned int* barc = a.bar->count + a.bar_parity;
     unsigned int bar_round = 0;
     if (__syncthreads_or(pending)) return;
+    if (kResume && a.ho->done) return;
     if (!grid_barrier(barc, gridDim.x, bar_round, a.status, a.timeout_ns)) return;
 
     __shared__ StageBuf stage_mem[kBfsThreads / 32];
@@ -863,7 +847,29 @@ __global__ void __launch_bounds__(kBfsThreads, kBfsMinBlocks) bfs_kernel(BfsArgs
     __syncthreads();
     int dir = a.mode == GBX_DIR_PULL ? DIR_PULL : DIR_PUSH;
     int cur = 0, vcur = 0;
-    for (int32_t L = 0;; ++L) {
+    int32_t L0 = 0;
+    if (kResume) {  // the handed-over frontier as a queue with its degree prefix
+        L0 = a.ho->level;
+        const int32_t listed = a.ho->listed, count = listed + a.ho->spilled;
+        Acc acc;
+        Stage st{stage_mem + wib, 0, a.ctr + L0 % 3, a.q[0], a.qp[0], a.qd[0], a.out_ptr, a.in_ptr, 0, 0, &acc};
+        for (long long b = (gtid >> 5) << 5; b < count; b += gstride) {
+            const long long i = b + (threadIdx.x & 31);
+            st.put(i < count, i < listed ? a.q[1][i] : (i < count ? a.hfirst[i - listed] : 0));
+        }
+        st.flush_block<kBfsThreads / 32>(stage_sum);
+        if (!grid_barrier(barc, gridDim.x, bar_round, a.status, a.timeout_ns)) return;
+        if (threadIdx.x == 0) {
+            ls.qv = ld_volatile_u64(&a.ctr[L0 % 3].q);
+            ls.nf = a.ho->frontier;
+        }
+        __syncthreads();
+        // Section 6.3's rule on the level before
+        if (a.mode == GBX_DIR_AUTO && (double)a.ho->frontier / (double)a.n > (double)a.alpha &&
+            a.ho->frontier > a.ho->before)
+            dir = DIR_PULL;
+    }
+    for (int32_t L = L0;; ++L) {
         LevelCtr* cout = a.ctr + ((L + 1) % 3);
         if (gtid == 0) {
             LevelCtr z = {};
@@ -879,8 +885,8 @@ __global__ void __launch_bounds__(kBfsThreads, kBfsMinBlocks) bfs_kernel(BfsArgs
             const bool first = L == 0 && fill_in_level0;
             push_level(a, L, cur, vcur, qcount, qedges, st, stage_sum, acc, !first);
             if (first) {
-                fill_outputs(a.depth, a.n, -1, s, 0, gtid, gstride);
-                if (a.parent) fill_outputs(a.parent, a.n, -1, s, s, gtid, gstride);
+                fill_i32(a.depth, a.n, -1, s, 0, gtid, gstride);
+                if (a.parent) fill_i32(a.parent, a.n, -1, s, s, gtid, gstride);
             }
             appended = true;
         } else {
@@ -979,8 +985,9 @@ static gbx_status check_desc(const gbx_desc* d) {
 
 static gbx_status bfs_geometry(Graph* G) {
     if (G->bfs_blocks > 0) return GBX_OK;  // blocks per SM that fit (cached per graph)
-    const void* fns[] = {(const void*)bfs_kernel<false, false>, (const void*)bfs_kernel<true, false>,
-                         (const void*)bfs_kernel<false, true>, (const void*)bfs_kernel<true, true>};
+    const void* fns[] = {(const void*)bfs_kernel<false, false, false>, (const void*)bfs_kernel<true, false, false>,
+                         (const void*)bfs_kernel<false, true, false>, (const void*)bfs_kernel<true, true, false>,
+                         (const void*)bfs_kernel<false, false, true>};
     int per_sm = 1 << 30;
     for (const void* fn : fns) {
         int b = 0;
@@ -1037,10 +1044,22 @@ static gbx_status launch_bfs(Graph* G, int32_t source, int32_t* depth, int32_t* 
     a.probe = d.pull_probe > 0 ? (d.pull_probe + 3) / 4 * 4 : kProbe;
     a.timeout_ns = wait_timeout_ns();
     a.bar_parity = G->ws.bar_parity;
+    a.ho = G->ws.handoff;
     void* args[] = {&a};
     const bool huge = !d.early_exit || d.direction == GBX_DIR_PULL;
-    const void* fn = d.trace ? (huge ? (const void*)bfs_kernel<true, true> : (const void*)bfs_kernel<true, false>)
-                             : (huge ? (const void*)bfs_kernel<false, true> : (const void*)bfs_kernel<false, false>);
+    const void* fn = d.trace ? (huge ? (const void*)bfs_kernel<true, true, false> : (const void*)bfs_kernel<true, false, false>)
+                             : (huge ? (const void*)bfs_kernel<false, true, false>
+                                     : (const void*)bfs_kernel<false, false, false>);
+    bool cluster = false;
+    GBX_TRY(cluster_bfs_wanted(G, d, &cluster));
+    if (cluster) {
+        bool complete = false;
+        GBX_TRY(cluster_bfs_launch(G, source, depth, parent, s, &complete));
+        G->ws.last_stream = s;
+        G->ws.last_traced = 0;
+        if (complete) return GBX_OK;
+        fn = (const void*)bfs_kernel<false, false, true>;
+    }
     const int per_sm = d.blocks_per_sm > 0 && d.blocks_per_sm < G->bfs_blocks ? d.blocks_per_sm : G->bfs_blocks;
     a.tile_words = pull_tile_words(G->nwords, (long long)per_sm * G->num_sms * (kBfsThreads / 32));
     GBX_CUDA_TRY(cudaLaunchCooperativeKernel(fn, dim3(per_sm * G->num_sms), dim3(kBfsThreads), args, 0, s));

@@ -69,6 +69,16 @@ struct GridBar {
     unsigned int pad[30];
 };
 
+// What the cluster kernel of the single-source BFS leaves for the grid-wide one.
+struct ClHandoff {
+    int32_t done;      // nothing is left to do
+    int32_t level;     // the level the search goes on with
+    int32_t listed;    // its frontier: entries of ws.q[1] ...
+    int32_t spilled;   // ... and of ws.list
+    int32_t frontier;  // their number
+    int32_t before;    // size of the frontier one level up
+};
+
 // Device-side trace record (mirrors gbx_level; nu / nu_nz filled on the host).
 struct LevelRec {
     int32_t direction;
@@ -96,6 +106,7 @@ struct Workspace {
     LevelRec* trace = nullptr;                                // kTraceCap records
     int32_t* status = nullptr;                                // ST_WORDS ints
     int32_t* flag = nullptr;                                  // small device scratch (mxv decisions)
+    ClHandoff* handoff = nullptr;                             // cluster BFS -> grid-wide BFS
     unsigned int bar_parity = 0;  // counter of GridBar the next persistent launch uses
     // batched multi-source BFS scratch (allocated on first use, grown as needed)
     unsigned long long* msV = nullptr;                     // visited lanes [n][W]
@@ -158,6 +169,8 @@ struct Graph {
     cudaEvent_t ev_done[2] = {nullptr, nullptr};
     cudaEvent_t ev_copied[2] = {nullptr, nullptr};
     int bfs_blocks = 0;  // BFS launch geometry
+    int cluster_blocks = 0;  // ... blocks of the cluster kernel (0: not asked yet, -1: none fits)
+    int32_t max_out_degree = 0;
     // gbx_mxv launch sequences captured as CUDA graphs (keyed by the call's buffers and descriptor)
     cudaStream_t mxv_cap_stream = nullptr;
     struct MxvCache* mxv_cache = nullptr;

@@ -97,6 +97,15 @@ __global__ void nonzero_rows_kernel(const int32_t* __restrict__ row_ptr, int32_t
     if ((threadIdx.x & 31) == 0) bm[i >> 5] = word;
 }
 
+// *out = the length of the longest row (*out starts at 0).
+__global__ void max_row_kernel(const int32_t* __restrict__ row_ptr, int32_t n, int32_t* out) {
+    int32_t m = 0;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+        m = max(m, row_ptr[i + 1] - row_ptr[i]);
+    m = __reduce_max_sync(0xffffffffu, m);
+    if ((threadIdx.x & 31) == 0) atomicMax(out, m);
+}
+
 static unsigned grid_for(int64_t work) { return (unsigned)std::max<int64_t>(1, std::min<int64_t>((work + 255) / 256, 152 * 32)); }
 
 // Sort the K keys and produce CSR (row_ptr, col) in freshly allocated device memory.
@@ -169,6 +178,7 @@ void workspace_release(Workspace& w) {
     f(w.trace);
     f(w.status);
     f(w.flag);
+    f(w.handoff);
     f(w.msV);
     for (auto& p : w.msF) f(p);
     f(w.msP);
@@ -230,6 +240,7 @@ static gbx_status workspace_alloc_all(Workspace& w, int32_t n) {
     GBX_CUDA_TRY(cudaMemset(w.status, 0, sizeof(int32_t) * ST_WORDS));
     GBX_CUDA_TRY(cudaMalloc((void**)&w.flag, sizeof(int32_t) * 64));
     GBX_CUDA_TRY(cudaMemset(w.flag, 0, sizeof(int32_t) * 64));
+    GBX_CUDA_TRY(cudaMalloc((void**)&w.handoff, sizeof(ClHandoff)));
     w.n_cap = n;  // only once every buffer exists
     return GBX_OK;
 }
@@ -345,7 +356,10 @@ static gbx_status build_impl(Graph* g, int32_t n, int64_t m, const int32_t* src,
         GBX_CUDA_TRY(cudaMalloc((void**)&g->next_out, sizeof(int4) * ((size_t)n + 1)));
         next_neighbours_kernel<<<grid_for(n), 256, 0, s>>>(g->out_ptr, g->out_col, n, g->next_out);
     }
+    int32_t* const longest = g->ws.flag + 10;  // zero since the workspace was made
+    max_row_kernel<<<grid_for(n), 256, 0, s>>>(g->out_ptr, n, longest);
     GBX_CUDA_TRY(cudaGetLastError());
+    GBX_CUDA_TRY(cudaMemcpyAsync(&g->max_out_degree, longest, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
     GBX_CUDA_TRY(cudaStreamSynchronize(s));
     return GBX_OK;
 }
