@@ -55,6 +55,8 @@ struct MsArgs {
     const int32_t* in_ptr;
     const int32_t* in_col;
     const uint32_t* nz_in;
+    const int32_t* first_out;
+    const int4* next_out;
     unsigned long long* V;
     unsigned long long* Fb[3];  // rotating found-lane buffers
     unsigned long long* P[4];   // depth bit planes (see record_depth)
@@ -431,7 +433,8 @@ struct MsLong {
 // kMsChunk 256 instead of 512 6 % (more of a row's chunks run before one covers it).
 template <int WL>
 __device__ __forceinline__ void ms_pull(const MsArgs& a, int32_t L, int32_t c0, unsigned long long* Fn, uint32_t* Tn,
-                                        uint16_t* list, const MsLong& lr, bool defer, Stage& st, Acc& acc) {
+                                        uint16_t* list, const MsLong& lr, bool defer, Stage& st,
+                                        unsigned long long* bsm, Acc& acc) {
     const int lane = threadIdx.x & 31;
     const int gwarp = (int)((blockIdx.x * kMsThreads + threadIdx.x) >> 5);
     const int nwarps = (int)((gridDim.x * kMsThreads) >> 5);
@@ -550,7 +553,7 @@ __device__ __forceinline__ void ms_pull(const MsArgs& a, int32_t L, int32_t c0, 
             if (done || put_off) v = -1;
         }
     }
-    st.flush();
+    st.flush_block<kMsThreads / 32>(bsm);
 }
 
 // The deferred rows' chunks, round-robin over the warps: the groups of a warp take
@@ -654,7 +657,7 @@ __device__ __forceinline__ void ms_pull_commit(const MsArgs& a, const int32_t* l
 __device__ __forceinline__ void ms_push_one(const MsArgs& a, int32_t L, const int32_t* q, const int32_t* qp,
                                             const int32_t* qd, uint32_t qcount, uint32_t qedges,
                                             const unsigned long long* Fc, unsigned long long* Fn, Stage& st,
-                                            Acc& acc) {
+                                            unsigned long long* bsm, Acc& acc) {
     const int gwarp = (int)((blockIdx.x * kMsThreads + threadIdx.x) >> 5);
     const int nwarps = (int)((gridDim.x * kMsThreads) >> 5);
     const int32_t E = (int32_t)qedges;
@@ -690,7 +693,168 @@ __device__ __forceinline__ void ms_push_one(const MsArgs& a, int32_t L, const in
             }
         }
     }
-    st.flush();
+    st.flush_block<kMsThreads / 32>(bsm);
+}
+
+// A level's next active list without degrees: vertices staged per warp, published with one
+// atomic per full stage and one per block at the end.
+struct IdStage {
+    StageBuf* sb;
+    int cnt;  // warp-uniform
+    LevelCtr* cout;
+    int32_t* ids;
+
+    __device__ __forceinline__ void write(unsigned long long at) {
+        __syncwarp();
+        for (int i = threadIdx.x & 31; i < cnt; i += 32) ids[(uint32_t)at + i] = sb->v[i];
+        __syncwarp();
+        cnt = 0;
+    }
+    __device__ __forceinline__ void put(bool take, int32_t v) {
+        const uint32_t m = __ballot_sync(0xffffffffu, take);
+        if (!m) return;
+        if (cnt + __popc(m) > kStage) {
+            unsigned long long at = 0ull;
+            if ((threadIdx.x & 31) == 0) at = atomicAdd(&cout->q, (unsigned long long)cnt);
+            write(__shfl_sync(0xffffffffu, at, 0));
+        }
+        if (take) sb->v[cnt + __popc(m & lanemask_lt())] = v;
+        cnt += __popc(m);
+    }
+    template <int kWarps>
+    __device__ __forceinline__ void flush_block(unsigned long long* bsm) {
+        const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+        if (lane == 0) bsm[w] = (unsigned long long)cnt;
+        __syncthreads();
+        if (w == 0) {
+            const uint32_t own = lane < kWarps ? (uint32_t)bsm[lane] : 0u;
+            const uint32_t inc = warp_inclusive_sum(own);
+            unsigned long long at = 0ull;
+            if (lane == 31 && inc) at = atomicAdd(&cout->q, (unsigned long long)inc);
+            at = __shfl_sync(0xffffffffu, at, 31);
+            if (lane < kWarps) bsm[lane] = at + inc - own;
+        }
+        __syncthreads();
+        write(bsm[w]);
+    }
+};
+
+// W == 1 on a mesh (a symmetric graph whose rows are short): ms_push_one without the queue's
+// degree prefix.  Four lanes take a vertex and read its first five neighbours from the dense
+// first-entry and next-entries arrays; a warp has up to kMsMeshIlp x 8 vertices in flight and
+// the level's work is spread over all warps before one takes more than 8.  The degrees (the
+// direction rule and the trace want their sum) are loaded when a vertex is claimed and added
+// a step later.
+//
+// A mesh level (the 1024 x 1024 grid, 64 sources: 2,000 levels of about 30K active vertices)
+// is bound by its chain of dependent round trips: list, neighbours, claim, F_next, list slot,
+// barrier; the prefix search, the queue's row starts, the probe of D and the degrees of the
+// flush are off it, and one atomic per block instead of one per warp reserves the list slots.
+// A level 11.7 -> 8.5 us on the whole GPU (the batch 23.8 -> 18.4 ms); on the quarter that a
+// server slot gets 14 -> 11 us.
+constexpr int kMsMeshIlp = 4;
+constexpr int32_t kMsMeshDegree = 32;  // longest row of a mesh
+
+__device__ __forceinline__ bool ms_mesh_gain(const MsArgs& a, int32_t L, int32_t v, unsigned long long cand,
+                                             unsigned long long old, unsigned long long was, char* const* rows,
+                                             Acc& acc) {
+    const unsigned long long gained = cand & ~old;
+    if (!gained) return false;
+    const unsigned long long full0 = lane_mask(a.S, 0);
+    if (((old | cand) & full0) == full0) atomicOr(a.D + (v >> 5), 1u << (v & 31));
+    acc.n_new += (uint32_t)__popcll(gained);
+    if (L + 1 < 16) {
+        record_depth(a, v, 0, gained, L + 1, true);
+    } else {
+        for (unsigned long long m = gained; m; m &= m - 1) {
+            char* const r = rows[__ffsll((long long)m) - 1];
+            if (a.depth16)
+                reinterpret_cast<int16_t*>(r)[v] = (int16_t)(L + 1);
+            else
+                reinterpret_cast<int32_t*>(r)[v] = L + 1;
+        }
+    }
+    return was == 0ull;  // the first edge to gain a lane at v lists it
+}
+
+// rows: the output rows' addresses (shared memory).
+__device__ __forceinline__ void ms_push_mesh(const MsArgs& a, int32_t L, const int32_t* ids, uint32_t qcount,
+                                             const unsigned long long* Fc, unsigned long long* Fn, char* const* rows,
+                                             IdStage& st, unsigned long long* bsm, Acc& acc) {
+    constexpr int K = kMsMeshIlp;
+    const int lane = threadIdx.x & 31, j = lane & 3;
+    const uint32_t gwarp = (uint32_t)((blockIdx.x * kMsThreads + threadIdx.x) >> 5);
+    const uint32_t nwarps = (uint32_t)((gridDim.x * kMsThreads) >> 5);
+    const uint32_t steps = (qcount + 8u * nwarps - 1u) / (8u * nwarps);  // steps of 8 vertices a warp has
+    const uint32_t per = 8u * (steps < (uint32_t)K ? (steps ? steps : 1u) : (uint32_t)K);
+    int32_t da[K], db[K];
+#pragma unroll
+    for (int k = 0; k < K; ++k) da[k] = db[k] = 0;
+    for (unsigned long long base = (unsigned long long)gwarp * per; base < qcount;
+         base += (unsigned long long)nwarps * per) {
+        int32_t u[K], w[K];
+        unsigned long long f[K], old[K], was[K];
+        bool more = false;
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            const uint32_t o = 8u * k + (lane >> 2);
+            u[k] = o < per && base + o < qcount ? ids[base + o] : -1;
+        }
+#pragma unroll
+        for (int k = 0; k < K; ++k) acc.mf += (uint32_t)(db[k] - da[k]);
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            w[k] = -1;
+            f[k] = 0ull;
+            if (u[k] < 0) continue;
+            f[k] = Fc[u[k]];
+            if (j == 0) {
+                w[k] = __ldg(a.first_out + u[k]);
+            } else if (j < 3) {
+                w[k] = __ldg(reinterpret_cast<const int32_t*>(a.next_out + u[k]) + (j - 1));
+            } else {
+                const int2 x = __ldg(reinterpret_cast<const int2*>(a.next_out + u[k]) + 1);
+                w[k] = x.x;
+                more |= x.y >= 0;
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < K; ++k) old[k] = w[k] >= 0 ? atomicOr(a.V + w[k], f[k]) : ~0ull;
+#pragma unroll
+        for (int k = 0; k < K; ++k) was[k] = (f[k] & ~old[k]) ? atomicOr(Fn + w[k], f[k] & ~old[k]) : ~0ull;
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            const bool first = ms_mesh_gain(a, L, w[k], f[k], old[k], was[k], rows, acc);
+            da[k] = first ? __ldg(a.out_ptr + w[k]) : 0;
+            db[k] = first ? __ldg(a.out_ptr + w[k] + 1) : 0;
+            st.put(first, w[k]);
+        }
+        if (__any_sync(0xffffffffu, more)) {  // rows of more than four entries: the rest, four lanes each
+#pragma unroll
+            for (int k = 0; k < K; ++k) {
+                int32_t x = 0, end = 0;
+                if (u[k] >= 0) {
+                    x = __ldg(a.out_ptr + u[k]) + 4 + j;
+                    end = __ldg(a.out_ptr + u[k] + 1);
+                }
+                for (; __any_sync(0xffffffffu, x < end); x += 4) {
+                    bool first = false;
+                    int32_t v = 0;
+                    if (x < end) {
+                        v = __ldg(a.out_col + x);
+                        const unsigned long long o = atomicOr(a.V + v, f[k]);
+                        const unsigned long long p = (f[k] & ~o) ? atomicOr(Fn + v, f[k] & ~o) : ~0ull;
+                        first = ms_mesh_gain(a, L, v, f[k], o, p, rows, acc);
+                        if (first) acc.mf += (uint32_t)(__ldg(a.out_ptr + v + 1) - __ldg(a.out_ptr + v));
+                    }
+                    st.put(first, v);
+                }
+            }
+        }
+    }
+    st.flush_block<kMsThreads / 32>(bsm);
+#pragma unroll
+    for (int k = 0; k < K; ++k) acc.mf += (uint32_t)(db[k] - da[k]);
 }
 
 // Wide batches, first phase: a warp takes 32 edges (u, v) of the active list and its
@@ -782,7 +946,8 @@ __device__ __forceinline__ void ms_push_wide(const MsArgs& a, const int32_t* q, 
 // writers all store zero).
 template <int WL>
 __device__ __forceinline__ void ms_finalize(const MsArgs& a, int32_t L, const int32_t* list, uint32_t count,
-                                            unsigned long long* Fn, uint32_t* Tn, Stage& st, Acc& acc) {
+                                            unsigned long long* Fn, uint32_t* Tn, Stage& st, unsigned long long* bsm,
+                                            Acc& acc) {
     const Group gr(a.group);
     const int per = 32 / gr.size;
     const long long gwarp = ((long long)blockIdx.x * kMsThreads + threadIdx.x) >> 5;
@@ -819,7 +984,7 @@ __device__ __forceinline__ void ms_finalize(const MsArgs& a, int32_t L, const in
         }
         st.put(v >= 0 && gr.sub == 0 && any_new, v);
     }
-    st.flush();
+    st.flush_block<kMsThreads / 32>(bsm);
 }
 
 // Clear F_{(L+2) mod 3} and T_{(L+2) mod 3} for the active list of level L - 1:
@@ -844,7 +1009,8 @@ __device__ __forceinline__ void ms_clear_prev(const MsArgs& a, const int32_t* id
 
 // ---------------------------------------------------------------- kernel
 
-template <int WL, int kOcc>
+// kMesh (WL = 1): push levels run ms_push_mesh.
+template <int WL, int kOcc, bool kMesh = false>
 __global__ void __launch_bounds__(kMsThreads, kOcc) ms_bfs_kernel(const __grid_constant__ MsArgs a) {
     const long long gtid = (long long)blockIdx.x * kMsThreads + threadIdx.x;
     // an error of an earlier launch not yet read by the host: this launch does nothing
@@ -861,6 +1027,7 @@ __global__ void __launch_bounds__(kMsThreads, kOcc) ms_bfs_kernel(const __grid_c
         uint32_t emit[WL == 2 ? kEmitSmem / 4 : 1];
     };
     __shared__ __align__(16) BlockMem mem;
+    __shared__ unsigned long long stage_sum[kMsThreads / 32];  // per-warp queue ranges of a block flush
     __shared__ unsigned long long lvl[6];
     __shared__ unsigned long long acc_mem[kMsThreads / 32][4];
     const int wib = threadIdx.x >> 5;
@@ -929,6 +1096,8 @@ __global__ void __launch_bounds__(kMsThreads, kOcc) ms_bfs_kernel(const __grid_c
         const int32_t s = a.src[b];
         a.Tb[0][s >> 5] = 0u;  // racing writers all store zero
     }
+    __shared__ char* row_mem[kMesh ? 64 : 1];  // the output rows' addresses
+    if (kMesh && threadIdx.x < 64) row_mem[threadIdx.x] = depth_row(a, (int)threadIdx.x < a.S ? threadIdx.x : 0);
     if (threadIdx.x == 0) lvl[4] = ld_volatile_u64(&a.ctr[0].q);
     if (!grid_barrier(barc, gridDim.x, bar_round, a.status, a.timeout_ns)) return;
     unsigned long long qv = lvl[4];
@@ -941,7 +1110,7 @@ __global__ void __launch_bounds__(kMsThreads, kOcc) ms_bfs_kernel(const __grid_c
             LevelCtr z = {};
             a.ctr[(L + 2) % 3] = z;
         }
-        const uint32_t qcount = (uint32_t)qv, qedges = (uint32_t)(qv >> 32);
+        const uint32_t qcount = (uint32_t)qv, qedges = (uint32_t)(qv >> 32);  // active vertices, their out-edges
         // direction for the whole batch: pull once the active edges exceed alpha * nnz
         int dir = a.mode;
         if (dir == GBX_DIR_AUTO) dir = (double)qedges > (double)a.alpha * (double)a.nnz ? GBX_DIR_PULL : GBX_DIR_PUSH;
@@ -954,20 +1123,24 @@ __global__ void __launch_bounds__(kMsThreads, kOcc) ms_bfs_kernel(const __grid_c
         ms_clear_prev<WL>(a, a.ids[r2], prev_count, a.Fb[r2], a.Tb[r2]);
         const MsLong lr{a.tlist, a.qp[p0], a.qd[p0]};  // a pull level does not read the queue's prefix
         if (dir == GBX_DIR_PUSH) {
-            if (WL == 1) {
-                ms_push_one(a, L, a.ids[r0], a.qp[p0], a.qd[p0], qcount, qedges, a.Fb[r0], a.Fb[r1], st, acc);
+            if (kMesh) {
+                IdStage ist{&mem.warp[wib].stage, 0, cout, a.ids[r1]};
+                ms_push_mesh(a, L, a.ids[r0], qcount, a.Fb[r0], a.Fb[r1], row_mem, ist, stage_sum, acc);
+            } else if (WL == 1) {
+                ms_push_one(a, L, a.ids[r0], a.qp[p0], a.qd[p0], qcount, qedges, a.Fb[r0], a.Fb[r1], st,
+                            stage_sum, acc);
             } else {
                 ms_push_wide<WL>(a, a.ids[r0], a.qp[p0], a.qd[p0], qcount, qedges, a.Fb[r0], a.Fb[r1], a.Tb[r1],
                                  &mem.warp[wib].stage, cout);
                 if (!grid_barrier(barc, gridDim.x, bar_round, a.status, a.timeout_ns)) return;
                 if (threadIdx.x == 0) lvl[5] = ld_volatile_u64(&cout->list);
                 __syncthreads();
-                ms_finalize<WL>(a, L, a.tlist, (uint32_t)lvl[5], a.Fb[r1], a.Tb[r1], st, acc);
+                ms_finalize<WL>(a, L, a.tlist, (uint32_t)lvl[5], a.Fb[r1], a.Tb[r1], st, stage_sum, acc);
             }
         } else {
             const bool one = a.W <= WL * a.group;  // one chunk of words: long rows can be deferred
             for (int32_t c0 = 0; c0 < a.W; c0 += WL * a.group)
-                ms_pull<WL>(a, L, c0, a.Fb[r1], a.Tb[r1], mem.warp[wib].open_list, lr, one, st, acc);
+                ms_pull<WL>(a, L, c0, a.Fb[r1], a.Tb[r1], mem.warp[wib].open_list, lr, one, st, stage_sum, acc);
         }
         block_add_counts<kMsThreads / 32>(acc_mem, acc.n_new, acc.mf, acc.exam, 0ull, &cout->n_new, &cout->mf_new,
                                           &cout->e_exam, nullptr);
@@ -986,7 +1159,7 @@ __global__ void __launch_bounds__(kMsThreads, kOcc) ms_bfs_kernel(const __grid_c
             Stage st2{&mem.warp[wib].stage, 0, cout, a.ids[r1], a.qp[p1], a.qd[p1], a.out_ptr, a.in_ptr, 1, 0, &acc2};
             ms_pull_long<WL>(a, a.Fb[r1], lr, (int32_t)rows, (int32_t)(lvl[2] >> 32), acc2);
             if (!grid_barrier(barc, gridDim.x, bar_round, a.status, a.timeout_ns)) return;
-            ms_finalize<WL>(a, L, lr.row, rows, a.Fb[r1], a.Tb[r1], st2, acc2);
+            ms_finalize<WL>(a, L, lr.row, rows, a.Fb[r1], a.Tb[r1], st2, stage_sum, acc2);
             block_add_counts<kMsThreads / 32>(acc_mem, acc2.n_new, acc2.mf, acc2.exam, 0ull, &cout->n_new,
                                               &cout->mf_new, &cout->e_exam, nullptr);
             if (!grid_barrier(barc, gridDim.x, bar_round, a.status, a.timeout_ns)) return;
@@ -999,6 +1172,7 @@ __global__ void __launch_bounds__(kMsThreads, kOcc) ms_bfs_kernel(const __grid_c
             __syncthreads();
         }
         qv = lvl[4];
+        if (kMesh && dir == GBX_DIR_PUSH) qv |= lvl[1] << 32;  // a mesh push lists without the degrees
         if (dir == GBX_DIR_PULL) {
             // V |= F for the vertices the pull found (their new lanes were kept apart so the
             // level read V as it was before it started)
@@ -1079,17 +1253,17 @@ int64_t ms_scratch_bytes(int32_t n, int32_t S) {
     return (4ll + kMsPlanes) * 8ll * (int64_t)n * ((w_raw + cw - 1) / cw * cw) + 4ll * ((int64_t)n + 1);
 }
 
-template <int WL, int kOcc>
+template <int WL, int kOcc, bool kMesh = false>
 static gbx_status ms_launch(Graph* G, const MsArgs& a0, int blocks, int per_sm_cap, cudaStream_t s) {
     int per_sm = 0;
-    GBX_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ms_bfs_kernel<WL, kOcc>, kMsThreads, 0));
+    GBX_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ms_bfs_kernel<WL, kOcc, kMesh>, kMsThreads, 0));
     GBX_CHECK(per_sm >= 1, GBX_ERR_CUDA, "batched BFS kernel cannot be resident");
     if (per_sm_cap > 0 && per_sm_cap < per_sm) per_sm = per_sm_cap;
     const int full = per_sm * G->num_sms;
     const int nb = blocks > 1 ? (full / blocks > 0 ? full / blocks : 1) : full;  // a 1/blocks share of the GPU
     MsArgs a = a0;
     void* args[] = {&a};
-    GBX_CUDA_TRY(cudaLaunchCooperativeKernel((const void*)ms_bfs_kernel<WL, kOcc>, dim3(nb), dim3(kMsThreads), args, 0,
+    GBX_CUDA_TRY(cudaLaunchCooperativeKernel((const void*)ms_bfs_kernel<WL, kOcc, kMesh>, dim3(nb), dim3(kMsThreads), args, 0,
                                              s));
     return GBX_OK;
 }
@@ -1116,6 +1290,8 @@ gbx_status ms_run(Graph* G, Workspace& w, int32_t S, const int32_t* src_dev, voi
     a.in_ptr = G->in_ptr;
     a.in_col = G->in_col;
     a.nz_in = G->nz_in;
+    a.first_out = G->first_out;
+    a.next_out = G->next_out;
     a.V = w.msV;
     for (int k = 0; k < 3; ++k) a.Fb[k] = w.msF[k];
     for (int k = 0; k < kMsPlanes; ++k) a.P[k] = w.msP + (size_t)k * (size_t)G->n * (size_t)W;
@@ -1155,6 +1331,8 @@ gbx_status ms_run(Graph* G, Workspace& w, int32_t S, const int32_t* src_dev, voi
     while (2 * a.group < W && a.group < 32) a.group *= 2;
     if (W > 1)
         st = lean ? ms_launch<2, kMsOccLean>(G, a, blocks, cap, s) : ms_launch<2, kMsOcc>(G, a, blocks, cap, s);
+    else if (!lean && G->symmetric && G->max_out_degree <= kMsMeshDegree)
+        st = ms_launch<1, kMsOcc, true>(G, a, blocks, cap, s);
     else
         st = lean ? ms_launch<1, kMsOccLean>(G, a, blocks, cap, s) : ms_launch<1, kMsOcc>(G, a, blocks, cap, s);
     if (st != GBX_OK) return st;

@@ -53,3 +53,31 @@ def test_lane_groups(name, S, direction):
     got = depth.cpu().numpy().astype(np.int32)
     for b, v in enumerate(srcs):
         assert np.array_equal(got[b], want[int(v)]), (b, int(v))
+
+
+@pytest.mark.parametrize("w,h", [(1, 1), (3, 1), (1, 700), (37, 41), (300, 211)])
+@pytest.mark.parametrize("S", [1, 31, 64])
+@pytest.mark.parametrize("k", [0, 3, 16])
+def test_mesh_batches(w, h, S, k):
+    """One lane word on graphs of short rows (the push without a degree prefix): grids, and
+    rings joined to the k next vertices (rows of 2k entries: beyond the five of the dense
+    arrays, up to the 32 that make a mesh), in every direction, int16 and int32 rows."""
+    n, s, d = synth.grid_edges(w, h, p_delete=0.02, seed=h)
+    if k:
+        n = w * h + 40
+        s = np.repeat(np.arange(n, dtype=np.int32), k)
+        d = ((s + np.tile(np.arange(1, k + 1, dtype=np.int32), n)) % n).astype(np.int32)
+    og, g = oracle.graph(n, s, d), gbx.graph_build(n, s, d)
+    srcs = (np.arange(S) * 7919 % n).astype(np.int32)
+    want = {int(v): oracle.bfs(og, int(v))[0] for v in set(srcs[:16])}
+    for direction, alpha in ((gbx.DIR_AUTO, 1e30), (gbx.DIR_AUTO, 0.01), (gbx.DIR_PUSH, 0.0), (gbx.DIR_PULL, 0.0)):
+        for dtype in (torch.int16, torch.int32):
+            depth = torch.full((S, n), 55, dtype=dtype, device="cuda")
+            gbx.bfs_batch(g, srcs, depth, gbx.desc_init(direction=direction, alpha=alpha))
+            gbx.graph_sync(g)
+            tr = gbx.bfs_batch_trace(g)
+            got = depth.cpu().numpy().astype(np.int32)
+            for b in range(min(S, 16)):
+                assert np.array_equal(got[b], want[int(srcs[b])]), (direction, b)
+            assert tr["n_new"].sum() == np.sum(got > 0) and np.all(tr["mf"][1:] == tr["mf_new"][:-1])
+    g.free()
