@@ -344,6 +344,9 @@ gbx_status gbx_bfs_trace(gbx_graph* g, gbx_level* levels, int32_t cap, int32_t* 
  * device float[n]: dist[source] = 0, +inf where unreachable.  Every relaxation
  * is one binary32 addition; for non-negative weights the result is, per vertex,
  * the smallest left-to-right rounded path sum, independent of the schedule.
+ * On a graph whose rows have at most 32 entries, with no negative weight, an
+ * untraced run that is not forced to pull relaxes the vertices near the source
+ * first instead of all improved ones (the distances are the same).
  * A negative cycle ends in GBX_ERR_OVERFLOW after n iterations (reported by
  * gbx_graph_sync).  One persistent cooperative launch, asynchronous on
  * `stream`; desc->blocks_per_sm >= 3 selects a register-lean build at three

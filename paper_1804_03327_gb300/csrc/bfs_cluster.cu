@@ -30,6 +30,7 @@
 // Every level pushes.  Section 6.3's rule would pull on some levels of a small graph; depths
 // do not depend on it, and the traced kernel (which reports the schedule) follows the rule.
 #include "bfs_cluster.cuh"
+#include "cluster.cuh"
 
 #include <algorithm>
 
@@ -67,66 +68,6 @@ struct ClArgs {
     int32_t shared_bm;  // the visited bitmap is in shared memory (block r: words w with w mod blocks = r)
 };
 
-__device__ __forceinline__ uint32_t cluster_rank() {
-    uint32_t r;
-    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-__device__ __forceinline__ uint32_t cluster_size() {
-    uint32_t r;
-    asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
-    return r;
-}
-__device__ __forceinline__ void cluster_barrier() {
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-// The address of shared variable p in block `rank` of the cluster.
-__device__ __forceinline__ uint32_t remote_smem(const void* p, uint32_t rank) {
-    uint32_t a;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;"
-                 : "=r"(a)
-                 : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
-    return a;
-}
-__device__ __forceinline__ void st_remote(uint32_t a, int32_t v) {
-    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
-}
-// Stores v at a (another block's or this one's shared memory) and counts its bytes on the
-// mbarrier at m of the same block.
-__device__ __forceinline__ void st_async(uint32_t a, int32_t v, uint32_t m) {
-    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.u32 [%0], %1, [%2];" ::"r"(a), "r"(v),
-                 "r"(m)
-                 : "memory");
-}
-__device__ __forceinline__ void mbar_init(unsigned long long* m, uint32_t count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"((uint32_t)__cvta_generic_to_shared(m)), "r"(count)
-                 : "memory");
-}
-__device__ __forceinline__ void mbar_expect(unsigned long long* m, uint32_t bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"((uint32_t)__cvta_generic_to_shared(m)),
-                 "r"(bytes)
-                 : "memory");
-}
-__device__ __forceinline__ bool mbar_try(unsigned long long* m, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"((uint32_t)__cvta_generic_to_shared(m)), "r"(parity)
-        : "memory");
-    return ok != 0u;
-}
-__device__ __forceinline__ int32_t ld_remote(uint32_t a) {
-    int32_t v;
-    asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
-    return v;
-}
-__device__ __forceinline__ uint32_t or_remote(uint32_t a, uint32_t v) {
-    uint32_t old;
-    asm volatile("atom.shared::cluster.or.b32 %0, [%1], %2;" : "=r"(old) : "r"(a), "r"(v) : "memory");
-    return old;
-}
-
 // Outputs and visited bitmap of a new search (Algorithm 1, lines 2-5), by threads
 // [tid, stride) of the launch.
 __device__ __forceinline__ void cl_fill(const ClArgs& a, long long tid, long long stride) {
@@ -150,7 +91,7 @@ struct ClSmem {
     int32_t beg[kClThreads];
     int32_t own[kClThreads];
     unsigned long long bar[2];  // mbarriers of the queue lengths, by level parity
-    int32_t counts[2][16];      // every block's queue length, by level parity
+    int32_t counts[2][kClusterMax];      // every block's queue length, by level parity
     int32_t cnt[2];             // entries in q[.]
     int32_t lcnt[2];            // entries in lq, by level parity
     int32_t abort;              // a block's wait ran out
@@ -297,14 +238,8 @@ __device__ __forceinline__ void cl_take(const ClArgs& a, ClSmem& sm, const ClSha
             int32_t parent = -1;
             bool near = true;
             if (part.share) {
-                int32_t o = 0;  // the block whose queue holds the entry
-#pragma unroll
-                for (int s = 8; s > 0; s >>= 1) {
-                    const int32_t y = __shfl_sync(0xffffffffu, part.inc, o + s - 1);
-                    if (part.g0 + i >= y) o += s;
-                }
-                const int32_t y = __shfl_sync(0xffffffffu, part.inc, o > 0 ? o - 1 : 0);
-                const int32_t x = part.g0 + i - (o > 0 ? y : 0);
+                int32_t o, x;
+                cluster_locate(part.inc, part.g0 + i, o, x);
                 if (i < part.m) {
                     near = x < kClNear;
                     u[k] = ld_remote(remote_smem(&sm.q[p][x], (uint32_t)o));
@@ -383,7 +318,7 @@ __global__ void __launch_bounds__(kClThreads, 1) bfs_cluster_kernel(const __grid
         sm.cnt[0] = sm.cnt[1] = sm.lcnt[0] = sm.lcnt[1] = 0;
         if (rank == 0) a.ho->spilled = 0;
     }
-    if (t < 16) sm.counts[0][t] = t == 0 ? 1 : 0;
+    if (t < kClusterMax) sm.counts[0][t] = t == 0 ? 1 : 0;
     if (a.shared_bm) {
         const int32_t sw = a.source >> 5;
         for (int32_t i = t; rank + (i << cs.shift) < a.nwords; i += kClThreads)
@@ -461,24 +396,9 @@ __global__ void __launch_bounds__(kClThreads, 1) bfs_cluster_kernel(const __grid
             st_async(remote_smem(&sm.counts[np][rank], (uint32_t)t), sm.cnt[np], remote_smem(&sm.bar[np], (uint32_t)t));
         if (t == 0) mbar_expect(&sm.bar[np], 4u * (uint32_t)C);
         last = total;
-        bool ok = true;
-        if (t < 32) {  // bounded wait, by the first warp
-            ok = mbar_try(&sm.bar[np], (uint32_t)(L >> 1) & 1u);
-            for (unsigned long long t0 = 0ull; !ok; ok = mbar_try(&sm.bar[np], (uint32_t)(L >> 1) & 1u)) {
-                const unsigned long long now = global_timer_ns();
-                if (t0 == 0ull) t0 = now;
-                if (now - t0 > a.timeout_ns) break;
-            }
-        }
-        if (!__syncthreads_and(ok)) {
-            // gives up: tells every block, which sees it at its next cluster barrier (its own wait
-            // runs out, or it is at a shared level); nobody touches another block after that one
-            if (t < C) st_remote(remote_smem(&sm.abort, (uint32_t)t), 1);
-            if (t == 0) {
-                atomicCAS(a.status + ST_ERROR, 0, (int)GBX_ERR_TIMEOUT);
-                a.ho->done = 1;
-            }
-            cluster_barrier();
+        if (!mbar_wait_block(&sm.bar[np], (uint32_t)(L >> 1) & 1u, a.timeout_ns)) {
+            if (t == 0) a.ho->done = 1;
+            cluster_give_up(&sm.abort, C, a.status);
             return;
         }
     }
@@ -491,27 +411,7 @@ static size_t cl_smem(int32_t bm_words) { return sizeof(ClSmem) + sizeof(uint32_
 
 static gbx_status cl_geometry(Graph* G) {
     if (G->cluster_blocks != 0) return GBX_OK;
-    const size_t smem = cl_smem(kClBmWords);
-    GBX_CUDA_TRY(cudaFuncSetAttribute(bfs_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    int best = -1;  // none fits: the grid-wide kernel does every level
-    if (cudaFuncSetAttribute(bfs_cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess)
-        for (int c = 16; c >= 8 && best < 0; c >>= 1) {
-            cudaLaunchConfig_t cfg = {};
-            cfg.gridDim = dim3(c);
-            cfg.blockDim = dim3(kClThreads);
-            cfg.dynamicSmemBytes = smem;
-            cudaLaunchAttribute at[1];
-            at[0].id = cudaLaunchAttributeClusterDimension;
-            at[0].val.clusterDim.x = c;
-            at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-            cfg.attrs = at;
-            cfg.numAttrs = 1;
-            int k = 0;
-            if (cudaOccupancyMaxActiveClusters(&k, bfs_cluster_kernel, &cfg) == cudaSuccess && k >= 1) best = c;
-        }
-    cudaGetLastError();  // a size that does not fit is no error of this call
-    G->cluster_blocks = best;
-    return GBX_OK;
+    return cluster_fit((const void*)bfs_cluster_kernel, kClThreads, cl_smem(kClBmWords), &G->cluster_blocks);
 }
 
 // Which searches start in the cluster: those of graphs whose levels stay small.
@@ -566,18 +466,9 @@ gbx_status cluster_bfs_launch(Graph* G, int32_t source, int32_t* depth, int32_t*
         cl_fill_kernel<<<blocks, 512, 0, s>>>(a);
         GBX_CUDA_TRY(cudaGetLastError());
     }
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(G->cluster_blocks);
-    cfg.blockDim = dim3(kClThreads);
-    cfg.dynamicSmemBytes = cl_smem(a.shared_bm ? bm_words : 0);
-    cfg.stream = s;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = G->cluster_blocks;
-    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    GBX_CUDA_TRY(cudaLaunchKernelEx(&cfg, bfs_cluster_kernel, a));
+    void* args[] = {&a};
+    GBX_TRY(cluster_launch((const void*)bfs_cluster_kernel, G->cluster_blocks, kClThreads,
+                           cl_smem(a.shared_bm ? bm_words : 0), args, s));
     return GBX_OK;
 }
 

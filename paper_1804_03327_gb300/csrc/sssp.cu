@@ -13,6 +13,7 @@
 // (rounding is monotonic), so the result does not depend on the schedule.
 #include "frontier.cuh"
 #include "gbx_internal.cuh"
+#include "sssp_cluster.cuh"
 
 namespace gbx {
 
@@ -46,6 +47,7 @@ struct SsspArgs {
     GridBar* bar;
     LevelRec* trace;
     int32_t* status;
+    const ClHandoff* ho;  // kResume: what the cluster kernel left
     float alpha, beta;
     int32_t mode, trace_cap;
     unsigned long long timeout_ns;
@@ -355,17 +357,21 @@ __device__ __forceinline__ void sssp_stamp_to_queue(const SsspArgs& a, int32_t L
     st.flush();
 }
 
-template <bool kTrace, int kOcc>
+// kResume: returns at once if sssp_cluster_kernel finished the search; else its distances
+// (each that of a path) are finished, starting with a pull of every row.
+template <bool kTrace, int kOcc, bool kResume = false>
 __global__ void __launch_bounds__(kSsspThreads, kOcc) sssp_kernel(SsspArgs a) {
     const long long gtid = (long long)blockIdx.x * kSsspThreads + threadIdx.x;
     const long long gstride = (long long)gridDim.x * kSsspThreads;
     const int32_t s = a.source;
     const int pending = threadIdx.x == 0 ? ld_volatile_i32(a.status + ST_ERROR) : 0;
     unsigned long long t_mark = kTrace && gtid == 0 ? global_timer_ns() : 0ull;
-    for (long long i = gtid; i < a.n; i += gstride) {
-        a.dist[i] = i == s ? 0.0f : INFINITY;
-        a.stamp[i] = 0;
-    }
+    const bool finished = kResume && a.ho->done;
+    if (!finished)
+        for (long long i = gtid; i < a.n; i += gstride) {
+            if (!kResume) a.dist[i] = i == s ? 0.0f : INFINITY;
+            a.stamp[i] = 0;
+        }
     const int32_t s_rs = __ldg(a.out_ptr + s);
     const int32_t s_od = __ldg(a.out_ptr + s + 1) - s_rs;
     if (gtid == 0) {
@@ -379,12 +385,12 @@ __global__ void __launch_bounds__(kSsspThreads, kOcc) sssp_kernel(SsspArgs a) {
         a.ctr[2] = z;
         z.q = s_od > 0 ? (((unsigned long long)s_od << 32) | 1ull) : 0ull;
         a.ctr[0] = z;
-        a.status[ST_LEVELS] = 0;
+        if (!kResume) a.status[ST_LEVELS] = 0;
         a.bar->count[a.bar_parity ^ 1u] = 0u;
     }
     unsigned int* barc = a.bar->count + a.bar_parity;
     unsigned int bar_round = 0;
-    if (__syncthreads_or(pending)) return;
+    if (__syncthreads_or(pending) || finished) return;
     if (!grid_barrier(barc, gridDim.x, bar_round, a.status, a.timeout_ns)) return;
 
     __shared__ StageBuf stage_mem[kSsspThreads / 32];
@@ -395,7 +401,7 @@ __global__ void __launch_bounds__(kSsspThreads, kOcc) sssp_kernel(SsspArgs a) {
     if ((threadIdx.x & 31) < 4) pull_sm[wib].occ[threadIdx.x & 31] = 0u;
     __syncwarp();
     unsigned long long qv = s_od > 0 ? (((unsigned long long)s_od << 32) | 1ull) : 0ull;
-    int dir = a.mode == GBX_DIR_PULL ? GBX_DIR_PULL : GBX_DIR_PUSH;
+    int dir = kResume || a.mode == GBX_DIR_PULL ? GBX_DIR_PULL : GBX_DIR_PUSH;
     int cur = 0;
     long long nf = 1, mf = s_od;
     for (int32_t L = 0;; ++L) {
@@ -426,7 +432,7 @@ __global__ void __launch_bounds__(kSsspThreads, kOcc) sssp_kernel(SsspArgs a) {
         const long long n_new = (long long)lvl[0];
         long long mf_new = (long long)lvl[1];
         qv = lvl[3];
-        int next = dir;
+        int next = kResume && a.mode == GBX_DIR_PUSH ? GBX_DIR_PUSH : dir;
         if (a.mode == GBX_DIR_AUTO && n_new > 0) {
             const double r_new = (double)n_new / (double)a.n;
             if (dir == GBX_DIR_PUSH) {
@@ -528,10 +534,19 @@ extern "C" gbx_status gbx_sssp(gbx_graph* g, int32_t source, float* dist, const 
     a.trace_cap = kTraceCap;
     a.timeout_ns = wait_timeout_ns();
     a.bar_parity = w.bar_parity;
-    const bool lean = d.blocks_per_sm >= kSsspOccLean;
+    a.ho = w.handoff;
+    bool cluster = false;
+    GBX_TRY(sssp_cluster_wanted(G, d, &cluster));
+    const bool lean = d.blocks_per_sm >= kSsspOccLean && !cluster;
     const void* fn = lean ? (d.trace ? (const void*)sssp_kernel<true, kSsspOccLean>
                                      : (const void*)sssp_kernel<false, kSsspOccLean>)
                           : (d.trace ? (const void*)sssp_kernel<true, kSsspOcc> : (const void*)sssp_kernel<false, kSsspOcc>);
+    if (cluster) {
+        fn = (const void*)sssp_kernel<false, kSsspOcc, true>;
+        GBX_TRY(sssp_cluster_launch(G, source, dist, s));
+        w.last_stream = s;
+        w.last_traced = 0;
+    }
     int per_sm = 0;
     GBX_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kSsspThreads, 0));
     GBX_CHECK(per_sm >= 1, GBX_ERR_CUDA, "SSSP kernel cannot be resident");

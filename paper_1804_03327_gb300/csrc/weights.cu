@@ -6,6 +6,7 @@
 #include <cmath>
 
 #include "gbx_internal.cuh"
+#include "sssp_cluster.cuh"
 
 namespace gbx {
 
@@ -117,6 +118,7 @@ extern "C" gbx_status gbx_graph_set_weights(gbx_graph* g, int64_t m, const int32
     if (!on_device)
         for (int64_t e = 0; e < m; ++e) GBX_CHECK(std::isfinite(w[e]), GBX_ERR_INVALID_VALUE, "weights must be finite");
     const int64_t nnz = G->nnz;
+    G->sp_step = -1.0f;  // the mesh records are of the old weights until the new ones are in
     if (!G->out_val) {  // both orientations or neither: a half-made pair would leave in_val null
         const size_t bytes = sizeof(float) * (size_t)(nnz > 0 ? nnz : 1);
         float* ov = nullptr;
@@ -177,7 +179,7 @@ extern "C" gbx_status gbx_graph_set_weights(gbx_graph* g, int64_t m, const int32
     GBX_CUDA_TRY(cudaStreamSynchronize(s));
     GBX_CHECK(hbad != 1, GBX_ERR_INVALID_INDEX, "a vertex outside [0, n) or a weight that is not finite");
     GBX_CHECK(hbad != 2, GBX_ERR_INVALID_VALUE, "a pair that the graph does not store (built from another edge list?)");
-    return GBX_OK;
+    return sssp_cluster_prepare(G, s);
 }
 
 extern "C" gbx_status gbx_graph_copy_weights(const gbx_graph* g, int32_t transpose, float* dst) {
