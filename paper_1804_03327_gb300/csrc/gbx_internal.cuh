@@ -107,6 +107,9 @@ struct Workspace {
     int32_t* status = nullptr;                                // ST_WORDS ints
     int32_t* flag = nullptr;                                  // small device scratch (mxv decisions)
     ClHandoff* handoff = nullptr;                             // cluster BFS -> grid-wide BFS
+    uint32_t* mx_bm[3] = {nullptr, nullptr, nullptr};         // gbx_mxv's u, mask and result bitmaps (one block),
+    LevelCtr* mx_ctr = nullptr;                               // and its queue counter: zero between calls ...
+    bool mx_dirty = false;                                    // ... unless a call was not issued whole
     unsigned int bar_parity = 0;  // counter of GridBar the next persistent launch uses
     // batched multi-source BFS scratch (allocated on first use, grown as needed)
     unsigned long long* msV = nullptr;                     // visited lanes [n][W]
@@ -175,13 +178,7 @@ struct Graph {
     void* sp_rec = nullptr;     // records of the first four out-edges: int4[n], float4[n]
     float sp_step = -1.0f;      // step of the near-far threshold (negative: not used)
     int sp_cluster_blocks = 0;  // as cluster_blocks
-    // gbx_mxv launch sequences captured as CUDA graphs (keyed by the call's buffers and descriptor)
-    cudaStream_t mxv_cap_stream = nullptr;
-    struct MxvCache* mxv_cache = nullptr;
 };
-
-// Releases the captured gbx_mxv graphs of G (mxv.cu).
-void mxv_cache_release(Graph* G);
 
 // ---------------------------------------------------------------- primitives (prims.cu)
 
@@ -336,24 +333,6 @@ inline gbx_status check_graph(const gbx_graph* g) {
 
 inline Graph* as_impl(gbx_graph* g) { return reinterpret_cast<Graph*>(g); }
 inline const Graph* as_impl(const gbx_graph* g) { return reinterpret_cast<const Graph*>(g); }
-
-// The row-based masked matvec of gbx_mxv (mxv.cu), also launched by the
-// allocation-free entry point (noalloc.cu).  It must be launched with
-// kMxvThreads threads per block: its shared tile is sized from that constant.
-constexpr int kMxvThreads = 256;
-
-// Per-call counters of gbx_mxv (desc.trace): [0] rows computed by pull, [1]
-// entries examined by pull, [2] nonzeros of u expanded by push, [3] edges expanded.
-struct MxvStats {
-    unsigned long long rows, exam, ucount, edges, pad[4];
-};
-
-__global__ void __launch_bounds__(kMxvThreads)
-    mxv_pull_kernel(const int32_t* __restrict__ ptr, const int32_t* __restrict__ col, const int32_t* __restrict__ first,
-                    const int4* __restrict__ next, const uint32_t* __restrict__ nzrows, const uint32_t* __restrict__ multi,
-                    const uint32_t* __restrict__ ubm,
-                    const uint32_t* __restrict__ pass, uint32_t* __restrict__ R, int32_t nwords, int early_exit,
-                    const int32_t* flag, MxvStats* stats, int32_t* huge, int32_t* huge_next, int32_t* huge_count);
 
 // Batched BFS internals (msbfs.cu), shared with the server.
 gbx_status ms_reserve(Workspace& w, int32_t n, int32_t S, cudaStream_t s);

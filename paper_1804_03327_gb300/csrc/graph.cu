@@ -179,6 +179,8 @@ void workspace_release(Workspace& w) {
     f(w.status);
     f(w.flag);
     f(w.handoff);
+    f(w.mx_bm[0]);
+    f(w.mx_ctr);
     f(w.msV);
     for (auto& p : w.msF) f(p);
     f(w.msP);
@@ -218,7 +220,6 @@ static void graph_release(Graph* g) {
         if (g->ev_copied[i]) cudaEventDestroy(g->ev_copied[i]);
     }
     if (g->copy_stream) cudaStreamDestroy(g->copy_stream);
-    mxv_cache_release(g);
     delete g;
 }
 
@@ -242,6 +243,12 @@ static gbx_status workspace_alloc_all(Workspace& w, int32_t n) {
     GBX_CUDA_TRY(cudaMalloc((void**)&w.flag, sizeof(int32_t) * 64));
     GBX_CUDA_TRY(cudaMemset(w.flag, 0, sizeof(int32_t) * 64));
     GBX_CUDA_TRY(cudaMalloc((void**)&w.handoff, sizeof(ClHandoff)));
+    GBX_CUDA_TRY(cudaMalloc((void**)&w.mx_bm[0], sizeof(uint32_t) * 3 * nw));
+    GBX_CUDA_TRY(cudaMemset(w.mx_bm[0], 0, sizeof(uint32_t) * 3 * nw));
+    w.mx_bm[1] = w.mx_bm[0] + nw;
+    w.mx_bm[2] = w.mx_bm[1] + nw;
+    GBX_CUDA_TRY(cudaMalloc((void**)&w.mx_ctr, sizeof(LevelCtr)));
+    GBX_CUDA_TRY(cudaMemset(w.mx_ctr, 0, sizeof(LevelCtr)));
     w.n_cap = n;  // only once every buffer exists
     return GBX_OK;
 }

@@ -6,171 +6,364 @@
 // (Algorithm 2 without the break), push expands the columns of u's finite
 // entries and folds them into w with an atomic minimum (Eq 5 / Algorithm 3's
 // reduction, done in place).  All sums are binary32.
+//
+// A call is three kernels, four under AUTO (a push then needs a queue first): mask and u, the
+// matvec, the rows a pull deferred.  The scratch is that of the Boolean operator (mxv.cu),
+// left zero.
+#include <algorithm>
 #include <cmath>
 
+#include "frontier.cuh"
 #include "gbx_internal.cuh"
+#include "mxv.cuh"
 
 namespace gbx {
 
-constexpr int kMpThreads = 256;
+constexpr int kMpUnroll = 4;          // entries a lane has in flight
+constexpr int32_t kMpChunk = 1024;    // entries of a deferred row a warp takes at a time
 
-__device__ __forceinline__ bool mp_enabled(const int32_t* flag, int want) { return !flag || *flag == want; }
+struct MpArgs {
+    int32_t n, nwords;
+    MxvVec mask;
+    uint32_t invert;
+    int32_t accum, dir, group;
+    float alpha;
+    const float* u;
+    float* w;
+    const int32_t* pull_ptr;
+    const int32_t* pull_col;
+    const float* pull_val;
+    const int32_t* push_ptr;
+    const int32_t* push_col;
+    const float* push_val;
+    uint32_t* ubm;
+    uint32_t* pass;
+    LevelCtr* ctr;  // q: the push queue; n_new: finite entries of u; huge: deferred rows and their chunks
+    int32_t* q[2];  // [0] the push queue, [1] deferred rows: row, next entry, prefix of the chunk counts
+    int32_t* qp[2];
+    int32_t* qd[2];
+    int32_t nothing;
+};
 
-__device__ __forceinline__ bool mp_pass(const uint32_t* pass, int32_t i) {
-    return !pass || ((pass[i >> 5] >> (i & 31)) & 1u);
+__device__ __forceinline__ int mp_dir(const MpArgs& a) {
+    if (a.dir != GBX_DIR_AUTO) return a.dir;
+    return (double)(int32_t)a.ctr->n_new / (double)a.n <= (double)a.alpha ? GBX_DIR_PUSH : GBX_DIR_PULL;
 }
 
-// bm bit i = u[i] is finite (an entry of u)
-__global__ void mp_finite_bitmap_kernel(const float* __restrict__ u, int32_t n, uint32_t* __restrict__ bm) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t n32 = ((int64_t)n + 31) & ~(int64_t)31;
-    if (i - (threadIdx.x & 31) >= n32) return;
-    const bool fin = i < n && u[i] < INFINITY;
-    const uint32_t word = __ballot_sync(0xffffffffu, fin);
-    if ((threadIdx.x & 31) == 0) bm[i >> 5] = word;
+__device__ __forceinline__ bool mp_pass(const MpArgs& a, int32_t i) {
+    return a.mask.format < 0 || (((a.pass[i >> 5] ^ a.invert) >> (i & 31)) & 1u);
 }
 
-__global__ void mp_degrees_kernel(const int32_t* __restrict__ ptr, const int32_t* __restrict__ list,
-                                  const int32_t* count_dev, int32_t n, int32_t* __restrict__ deg, const int32_t* flag) {
-    if (!mp_enabled(flag, GBX_DIR_PUSH)) return;
-    const int32_t count = min(*count_dev, n);
-    for (int32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < count; k += gridDim.x * blockDim.x) {
-        const int32_t u = list[k];
-        deg[k] = ptr[u + 1] - ptr[u];
-    }
+__device__ __forceinline__ Stage mp_stage(const MpArgs& a, StageBuf* sb, Acc* acc) {
+    return Stage{sb + (threadIdx.x >> 5), 0, a.ctr, a.q[0], a.qp[0], a.qd[0], a.push_ptr, a.push_ptr, 0, 0, acc};
 }
 
-// Push: w(i) <- min(w(i), a(j, i) + u(j)) for every entry of the columns of u's
-// finite entries j, rows that pass the mask only.  w was set to +inf (or keeps
-// w_old with accumulate) beforehand.  Each thread takes gathered positions
-// grid-stride and finds its column by binary search of the degree prefix.
-__global__ void __launch_bounds__(kMpThreads)
-    mp_push_kernel(const int32_t* __restrict__ ptr, const int32_t* __restrict__ col, const float* __restrict__ val,
-                   const int32_t* __restrict__ list, const int32_t* count_dev, int32_t n,
-                   const int32_t* __restrict__ pre, const float* __restrict__ u, const uint32_t* __restrict__ pass,
-                   float* w, const int32_t* flag) {
-    if (!mp_enabled(flag, GBX_DIR_PUSH)) return;
-    const int32_t count = min(*count_dev, n);
-    if (count <= 0) return;
-    const int64_t E = pre[count];
-    for (int64_t e = (int64_t)blockIdx.x * kMpThreads + threadIdx.x; e < E; e += (int64_t)gridDim.x * kMpThreads) {
-        int32_t lo = 0, hi = count;  // largest k with pre[k] <= e (pre[0] = 0)
-        while (hi - lo > 1) {
-            const int32_t mid = lo + ((hi - lo) >> 1);
-            if (pre[mid] <= e)
-                lo = mid;
-            else
-                hi = mid;
-        }
-        const int32_t j = list[lo];
-        const int64_t idx = (int64_t)ptr[j] + (e - pre[lo]);
-        const int32_t i = col[idx];
-        if (!mp_pass(pass, i)) continue;
-        const float x = u[j] + val[idx];
-        if (x < w[i]) atomic_min_f32(w + i, x);
-    }
-}
-
-__global__ void mp_prepare_kernel(float* __restrict__ w, int32_t n, int accum, const int32_t* flag) {
-    if (!mp_enabled(flag, GBX_DIR_PUSH) || accum) return;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        w[i] = INFINITY;
-}
-
-// Pull: a warp takes 32 consecutive rows, a lane each; rows with more than 32
-// entries are then reduced by the whole warp, one after another.
-__global__ void __launch_bounds__(kMpThreads)
-    mp_pull_kernel(const int32_t* __restrict__ ptr, const int32_t* __restrict__ col, const float* __restrict__ val,
-                   int32_t n, const float* __restrict__ u, const uint32_t* __restrict__ pass, float* __restrict__ w,
-                   int accum, const int32_t* flag) {
-    if (!mp_enabled(flag, GBX_DIR_PULL)) return;
+// The mask as a bitmap; u's finite entries as the push queue (dir == PUSH) or as a bitmap and
+// their number (AUTO); w = +inf where a push without accumulation starts from that.
+__global__ void __launch_bounds__(kMxvThreads) mp_prep_kernel(const __grid_constant__ MpArgs a) {
+    __shared__ StageBuf sb[kMxvThreads / 32];
+    __shared__ unsigned long long bsm[kMxvThreads / 32];
+    __shared__ unsigned long long csm[kMxvThreads / 32][4];
     const int lane = threadIdx.x & 31;
-    const int64_t nwarps = ((int64_t)gridDim.x * kMpThreads) >> 5;
-    const int64_t ntiles = ((int64_t)n + 31) >> 5;
-    for (int64_t tile = ((int64_t)blockIdx.x * kMpThreads + threadIdx.x) >> 5; tile < ntiles; tile += nwarps) {
-        const int64_t i64 = (tile << 5) + lane;
-        const bool in_range = i64 < n;
-        const int32_t i = (int32_t)i64;
-        const bool ps = in_range && mp_pass(pass, i);
-        int32_t beg = 0, end = 0;
-        if (ps) {
-            beg = ptr[i];
-            end = ptr[i + 1];
+    const int64_t gtid = (int64_t)blockIdx.x * kMxvThreads + threadIdx.x, gs = (int64_t)gridDim.x * kMxvThreads;
+    if (gtid == 0) a.ctr->huge = 0ull;
+    if (a.mask.format == GBX_DENSE) {
+        for (int64_t w = gtid; w < a.nwords; w += gs)
+            a.pass[w] = pack_word(static_cast<const uint8_t*>(a.mask.data), a.n, (int32_t)w);
+    } else if (a.mask.format == GBX_SPARSE) {
+        const int32_t* list = static_cast<const int32_t*>(a.mask.data);
+        const int32_t count = min(*a.mask.count, a.mask.cap);
+        for (int64_t i = gtid; i < count; i += gs) {
+            const int32_t v = list[i];
+            if (v >= 0 && v < a.n) atomicOr(a.pass + (v >> 5), 1u << (v & 31));
         }
-        float t = INFINITY;
-        const bool longrow = end - beg > 32;
-        if (!longrow)
-            for (int32_t k = beg; k < end; ++k) t = fminf(t, val[k] + u[col[k]]);
-        uint32_t pend = __ballot_sync(0xffffffffu, longrow);
-        while (pend) {
-            const int owner = __ffs(pend) - 1;
-            pend &= pend - 1;
-            const int32_t b = __shfl_sync(0xffffffffu, beg, owner);
-            const int32_t e = __shfl_sync(0xffffffffu, end, owner);
-            float m = INFINITY;
-            for (int32_t k = b + lane; k < e; k += 32) m = fminf(m, val[k] + u[col[k]]);
+    }
+    if (a.dir == GBX_DIR_PULL && !a.nothing) return;
+    if ((a.dir == GBX_DIR_PUSH || a.nothing) && !a.accum)
+        for (int64_t i = gtid; i < a.n; i += gs) a.w[i] = INFINITY;
+    if (a.nothing) return;
+    Acc acc;
+    Stage st = mp_stage(a, sb, &acc);
+    uint32_t cnt = 0;
+    for (int64_t b = gtid - lane; b < a.n; b += gs) {  // warp-uniform
+        const int32_t i = (int32_t)b + lane;
+        const bool fin = i < a.n && a.u[i] < INFINITY;
+        if (a.dir == GBX_DIR_PUSH) {
+            st.put(fin, i);
+        } else {
+            const uint32_t word = __ballot_sync(0xffffffffu, fin);
+            if (lane == 0) a.ubm[b >> 5] = word;
+            cnt += fin ? 1u : 0u;
+        }
+    }
+    if (a.dir == GBX_DIR_PUSH) st.flush_block<kMxvThreads / 32>(bsm);
+    block_add_counts<kMxvThreads / 32>(csm, cnt, 0ull, 0ull, 0ull, &a.ctr->n_new, nullptr, nullptr, nullptr);
+}
+
+// Push: w(i) <- min(w(i), a(j, i) + u(j)) for every entry of the columns of u's finite
+// entries j, rows that pass the mask only; the edges are split evenly over all warps.
+__device__ __forceinline__ void mp_push(const MpArgs& a) {
+    const unsigned long long qv = a.ctr->q;
+    const uint32_t qcount = (uint32_t)qv;
+    const int32_t E = (int32_t)(qv >> 32);
+    const int gwarp = (int)((blockIdx.x * kMxvThreads + threadIdx.x) >> 5);
+    const int nwarps = (int)((gridDim.x * kMxvThreads) >> 5);
+    constexpr int kStep = 32 * kMpUnroll;
+    int32_t chunk = (int32_t)(((long long)E + nwarps - 1) / nwarps);
+    chunk = chunk <= 32 ? 32 : ((chunk + kStep - 1) / kStep) * kStep;
+    for (long long e0l = (long long)gwarp * chunk; e0l < E; e0l += (long long)nwarps * chunk) {
+        const int32_t e0 = (int32_t)e0l;
+        const int32_t e1 = E - e0 > chunk ? e0 + chunk : E;
+        PushCursorT<kMpUnroll> cur;
+        cur.k = warp_find_entry(a.qp[0], (int32_t)qcount, e0);
+        cur.wlast = -1;
+        for (int32_t base = e0; base < e1; base += kStep) {
+            const PushStepT<kMpUnroll> ps = cur.gather(a.push_col, a.q[0], a.qp[0], a.qd[0], qcount, base, e1);
+            float x[kMpUnroll], old[kMpUnroll];
+            bool ok[kMpUnroll];
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) m = fminf(m, __shfl_xor_sync(0xffffffffu, m, o));
-            if (lane == owner) t = m;
-        }
-        if (in_range) {
-            const float old = accum ? w[i] : INFINITY;
-            w[i] = ps ? fminf(old, t) : old;
+            for (int t = 0; t < kMpUnroll; ++t) {
+                const bool in = ps.u[t] >= 0;
+                x[t] = in ? a.u[ps.u[t]] + a.push_val[ps.k[t]] : INFINITY;
+                old[t] = in ? a.w[ps.v[t]] : 0.0f;
+                ok[t] = in && mp_pass(a, ps.v[t]);
+            }
+#pragma unroll
+            for (int t = 0; t < kMpUnroll; ++t)  // a stale w only costs an atomic: w falls
+                if (ok[t] && x[t] < old[t]) atomic_min_f32(a.w + ps.v[t], x[t]);
         }
     }
 }
 
-__global__ void mp_decide_kernel(const int32_t* count_dev, int32_t n, float alpha, int32_t* flag) {
-    const double r = (double)(*count_dev) / (double)n;
-    *flag = r <= (double)alpha ? GBX_DIR_PUSH : GBX_DIR_PULL;
+// Pull: groups of a.group lanes take a row each, kMpUnroll entries a lane in flight, and go on to
+// the next row as soon as their own is done.  A warp's row offsets come 32 rows at a time,
+// the next 32 loaded ahead.  A row with more than 64 steps left is deferred: mp_last_kernel
+// spreads its chunks over all warps.
+//
+// Bound by the gathers of u (4 bytes of a 32-byte L2 sector per entry).  A lane per row of up to
+// 32 entries, one load at a time, and a warp for each longer row had taken 316 us on a
+// directed graph of 700,001 rows and 11.2M entries whose longest rows hold tens of thousands
+// (the whole call 358 us, now 141).  The group is 8 lanes from 12 entries a row on, 4 from 6, else 1: rows shorter
+// than the group's step leave lanes idle, longer ones take several dependent steps.
+__device__ __forceinline__ void mp_pull(const MpArgs& a) {
+    const int lane = threadIdx.x & 31;
+    const int G = a.group, sub = lane & (G - 1), first = lane & ~(G - 1);
+    const int32_t nwarps = (int32_t)((gridDim.x * kMxvThreads) >> 5);
+    const int32_t ntiles = a.nwords;
+    int32_t tile = (int32_t)((blockIdx.x * kMxvThreads + threadIdx.x) >> 5);
+    const int32_t kLong = 64 * kMpUnroll * G;
+    // a tile's rows: lane l holds row 32 tile + l
+    auto load = [&](int32_t t, int32_t& b, int32_t& e) {
+        const int64_t i = ((int64_t)t << 5) + lane;
+        b = e = 0;
+        if (t < ntiles && i < a.n && mp_pass(a, (int32_t)i)) {
+            b = __ldg(a.pull_ptr + i);
+            e = __ldg(a.pull_ptr + i + 1);
+        }
+    };
+    int32_t b0, e0, b1, e1;
+    load(tile, b0, e0);
+    load(tile + nwarps, b1, e1);
+    int32_t base = -1;   // first row of the tile in b0 / e0 that is being handed out
+    uint32_t open = 0;   // its rows not yet handed out
+    int32_t v = -1, k = 0, end = 0;
+    float m = INFINITY;
+    for (;;) {
+        const uint32_t need = __ballot_sync(0xffffffffu, v < 0 && sub == 0);
+        if (need && !open && tile < ntiles) {  // the next tile; its rows without entries are settled here
+            open = __ballot_sync(0xffffffffu, e0 > b0);
+            base = tile << 5;
+            if (e0 == b0 && base + lane < a.n && !a.accum) a.w[base + lane] = INFINITY;
+        }
+        if (need && open) {
+            // the r-th group without a row takes the r-th open one
+            const int r = __popc(need & ((1u << first) - 1u));
+            const int nth = (int)__fns(open, 0, r + 1);
+            const bool got = v < 0 && nth >= 0 && nth < 32;
+            const int32_t nb = __shfl_sync(0xffffffffu, b0, got ? nth : 0);
+            const int32_t ne = __shfl_sync(0xffffffffu, e0, got ? nth : 0);
+            const uint32_t taken = __ballot_sync(0xffffffffu, got && sub == 0);
+            if (got) {
+                v = base + nth;
+                k = nb;
+                end = ne;
+                m = INFINITY;
+            }
+            for (int c = __popc(taken); c > 0; --c) open &= open - 1;
+            if (!open) {
+                tile += nwarps;
+                b0 = b1;
+                e0 = e1;
+                load(tile + nwarps, b1, e1);
+            }
+        } else if (need && tile < ntiles) {  // a tile without open rows
+            tile += nwarps;
+            b0 = b1;
+            e0 = e1;
+            load(tile + nwarps, b1, e1);
+            if (__popc(need) * G == 32) continue;
+        }
+        if (__ballot_sync(0xffffffffu, v >= 0) == 0u) {
+            if (tile >= ntiles) break;
+            continue;
+        }
+        // one step of every group: G * kMpUnroll entries
+        int32_t c[kMpUnroll];
+        float x[kMpUnroll];
+#pragma unroll
+        for (int t = 0; t < kMpUnroll; ++t) {
+            const int32_t e = k + sub + G * t;
+            const bool in = v >= 0 && e < end;
+            c[t] = in ? __ldg(a.pull_col + e) : -1;
+            x[t] = in ? __ldg(a.pull_val + e) : INFINITY;
+        }
+#pragma unroll
+        for (int t = 0; t < kMpUnroll; ++t)
+            if (c[t] >= 0) m = fminf(m, x[t] + __ldg(a.u + c[t]));
+        k += G * kMpUnroll;
+        const bool done = v >= 0 && k >= end;
+        const bool defer = v >= 0 && end - k > kLong;
+        if (!__any_sync(0xffffffffu, done || defer)) continue;
+        float t = m;
+        for (int o = 1; o < G; o <<= 1) t = fminf(t, __shfl_xor_sync(0xffffffffu, t, o));
+        if ((done || defer) && sub == 0) {
+            if (a.accum) t = fminf(t, a.w[v]);
+            a.w[v] = t;
+        }
+        const uint32_t dm = __ballot_sync(0xffffffffu, defer && sub == 0);
+        if (dm) {
+            const uint32_t nch = defer && sub == 0 ? (uint32_t)(end - k + kMpChunk - 1) / kMpChunk : 0u;
+            const uint32_t inc = warp_inclusive_sum(nch);
+            const uint32_t tot = __shfl_sync(0xffffffffu, inc, 31);
+            unsigned long long old = 0ull;
+            if (lane == 0)
+                old = atomicAdd(&a.ctr->huge, ((unsigned long long)tot << 32) | (unsigned long long)__popc(dm));
+            old = __shfl_sync(0xffffffffu, old, 0);
+            if (defer && sub == 0) {
+                const uint32_t slot = (uint32_t)old + __popc(dm & lanemask_lt());
+                a.q[1][slot] = v;
+                a.qp[1][slot] = k;
+                a.qd[1][slot] = (int32_t)((uint32_t)(old >> 32) + inc - nch);
+            }
+        }
+        if (done || defer) v = -1;
+    }
 }
 
-gbx_status mxv_minplus(Graph* G, float* w, const uint32_t* pass_bm, bool nothing_passes, const float* u,
-                       const gbx_desc& d, cudaStream_t s) {
-    const int32_t n = G->n;
-    GBX_CHECK(G->out_val != nullptr, GBX_ERR_INVALID_VALUE,
-              "the (min, +) semiring needs edge weights (gbx_graph_set_weights)");
-    const int32_t* pull_ptr = d.transpose ? G->in_ptr : G->out_ptr;
-    const int32_t* pull_col = d.transpose ? G->in_col : G->out_col;
-    const float* pull_val = d.transpose ? G->in_val : G->out_val;
-    const int32_t* push_ptr = d.transpose ? G->out_ptr : G->in_ptr;
-    const int32_t* push_col = d.transpose ? G->out_col : G->in_col;
-    const float* push_val = d.transpose ? G->out_val : G->in_val;
-    const unsigned int grid = (unsigned)G->num_sms * 8u;
-    if (nothing_passes) {
-        // every row fails the mask: w keeps w_old (accumulate) or becomes +inf
-        if (!d.accum) mp_prepare_kernel<<<grid, kMpThreads, 0, s>>>(w, n, 0, nullptr);
-        GBX_CUDA_TRY(cudaGetLastError());
-        return GBX_OK;
-    }
-    const int dir = d.direction;
-    const bool want_push = dir != GBX_DIR_PULL;
-    const bool want_pull = dir != GBX_DIR_PUSH;
-    uint32_t* ubm = G->ws.bm[0];
-    int32_t* list = G->ws.list;
-    int32_t* count = G->ws.flag + 0;
-    int32_t* dflag = G->ws.flag + 1;
-    const int32_t* flag = nullptr;
-    if (want_push) {
-        const int64_t n32 = ((int64_t)n + 31) & ~(int64_t)31;
-        mp_finite_bitmap_kernel<<<div_up(n32, 256), 256, 0, s>>>(u, n, ubm);
-        GBX_TRY(bitmap_to_list(ubm, n, list, count, G->ws.qd[0], G->ws.scan_tmp, s));
-        if (dir == GBX_DIR_AUTO) {
-            mp_decide_kernel<<<1, 1, 0, s>>>(count, n, d.alpha, dflag);
-            flag = dflag;
+// Pull, push, or -- AUTO found u sparse -- the queue (and w = +inf) for mp_push_kernel.
+__global__ void __launch_bounds__(kMxvThreads, 6) mp_main_kernel(const __grid_constant__ MpArgs a) {
+    __shared__ StageBuf sb[kMxvThreads / 32];
+    __shared__ unsigned long long bsm[kMxvThreads / 32];
+    if (mp_dir(a) == GBX_DIR_PULL) {
+        mp_pull(a);
+    } else if (a.dir == GBX_DIR_PUSH) {
+        mp_push(a);
+    } else {
+        const int lane = threadIdx.x & 31;
+        const int64_t gtid = (int64_t)blockIdx.x * kMxvThreads + threadIdx.x, gs = (int64_t)gridDim.x * kMxvThreads;
+        if (!a.accum)
+            for (int64_t i = gtid; i < a.n; i += gs) a.w[i] = INFINITY;
+        Acc acc;
+        Stage st = mp_stage(a, sb, &acc);
+        for (int64_t w0 = gtid - lane; w0 < a.nwords; w0 += gs) {
+            const uint32_t mine = w0 + lane < a.nwords ? a.ubm[w0 + lane] : 0u;
+            uint32_t todo = __ballot_sync(0xffffffffu, mine != 0u);
+            while (todo) {
+                const int j = __ffs(todo) - 1;
+                todo &= todo - 1;
+                const uint32_t word = __shfl_sync(0xffffffffu, mine, j);
+                st.put((word >> lane) & 1u, (int32_t)((w0 + j) << 5) + lane);
+            }
         }
-        int32_t* deg = G->ws.q[0];
-        int32_t* pre = G->ws.qp[0];
-        mp_degrees_kernel<<<grid, 256, 0, s>>>(push_ptr, list, count, n, deg, flag);
-        GBX_TRY(exclusive_scan_i32(deg, pre, n, count, G->ws.scan_tmp, s));
-        mp_prepare_kernel<<<grid, kMpThreads, 0, s>>>(w, n, d.accum ? 1 : 0, flag);
-        mp_push_kernel<<<grid, kMpThreads, 0, s>>>(push_ptr, push_col, push_val, list, count, n, pre, u, pass_bm, w,
-                                                   flag);
+        st.flush_block<kMxvThreads / 32>(bsm);
     }
-    if (want_pull)
-        mp_pull_kernel<<<grid, kMpThreads, 0, s>>>(pull_ptr, pull_col, pull_val, n, u, pass_bm, w, d.accum ? 1 : 0,
-                                                   flag);
+}
+
+__global__ void __launch_bounds__(kMxvThreads) mp_push_kernel(const __grid_constant__ MpArgs a) {
+    if (mp_dir(a) == GBX_DIR_PUSH) mp_push(a);
+}
+
+// The chunks of the rows a pull deferred, and the scratch left zero for the next call.
+__global__ void __launch_bounds__(kMxvThreads) mp_last_kernel(const __grid_constant__ MpArgs a) {
+    const int lane = threadIdx.x & 31;
+    const int64_t gtid = (int64_t)blockIdx.x * kMxvThreads + threadIdx.x, gs = (int64_t)gridDim.x * kMxvThreads;
+    const unsigned long long huge = a.ctr->huge;
+    const int32_t entries = (int32_t)(uint32_t)huge, chunks = (int32_t)(huge >> 32);
+    for (int64_t c = gtid >> 5; c < chunks; c += gs >> 5) {
+        const int32_t h = warp_find_entry(a.qd[1], entries, c);
+        const int32_t v = a.q[1][h];
+        const int32_t rend = __ldg(a.pull_ptr + v + 1);
+        const int32_t beg = a.qp[1][h] + (int32_t)(c - a.qd[1][h]) * kMpChunk;
+        const int32_t end = rend - beg < kMpChunk ? rend : beg + kMpChunk;
+        float m = INFINITY;
+        for (int32_t k = beg + lane; k < end; k += 32 * kMpUnroll) {
+            int32_t j[kMpUnroll];
+            float x[kMpUnroll];
+#pragma unroll
+            for (int t = 0; t < kMpUnroll; ++t) {
+                const bool in = k + 32 * t < end;
+                j[t] = in ? __ldg(a.pull_col + k + 32 * t) : -1;
+                x[t] = in ? __ldg(a.pull_val + k + 32 * t) : INFINITY;
+            }
+#pragma unroll
+            for (int t = 0; t < kMpUnroll; ++t)
+                if (j[t] >= 0) m = fminf(m, x[t] + __ldg(a.u + j[t]));
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) m = fminf(m, __shfl_xor_sync(0xffffffffu, m, o));
+        if (lane == 0 && m < a.w[v]) atomic_min_f32(a.w + v, m);
+    }
+    for (int64_t w = gtid; w < a.nwords; w += gs) {
+        a.ubm[w] = 0u;
+        if (a.mask.format >= 0) a.pass[w] = 0u;
+    }
+    if (gtid == 0) {
+        a.ctr->q = 0ull;
+        a.ctr->n_new = 0ull;
+    }
+}
+
+gbx_status mxv_scratch(Graph* G, cudaStream_t s);
+
+gbx_status mxv_minplus(Graph* G, float* w, const MxvVec& mask, const float* u, const gbx_desc& d, cudaStream_t s) {
+    MpArgs a;
+    a.n = G->n;
+    a.nwords = G->nwords;
+    a.mask = mask;
+    a.invert = d.mask_complement ? 0xffffffffu : 0u;
+    a.accum = d.accum ? 1 : 0;
+    a.dir = d.direction;
+    a.group = G->nnz > 12ll * G->n ? 8 : (G->nnz > 6ll * G->n ? 4 : 1);
+    a.alpha = d.alpha;
+    a.u = u;
+    a.w = w;
+    a.pull_ptr = d.transpose ? G->in_ptr : G->out_ptr;
+    a.pull_col = d.transpose ? G->in_col : G->out_col;
+    a.pull_val = d.transpose ? G->in_val : G->out_val;
+    a.push_ptr = d.transpose ? G->out_ptr : G->in_ptr;
+    a.push_col = d.transpose ? G->out_col : G->in_col;
+    a.push_val = d.transpose ? G->out_val : G->in_val;
+    a.ubm = G->ws.mx_bm[0];
+    a.pass = G->ws.mx_bm[1];
+    a.ctr = G->ws.mx_ctr;
+    for (int i = 0; i < 2; ++i) {
+        a.q[i] = G->ws.q[i];
+        a.qp[i] = G->ws.qp[i];
+        a.qd[i] = G->ws.qd[i];
+    }
+    a.nothing = mask.format < 0 && d.mask_complement;
+    const unsigned grid = (unsigned)G->num_sms * 6u;
+    const unsigned small = std::max(1u, std::min(div_up(a.n, kMxvThreads), (unsigned)G->num_sms * 4u));
+    GBX_TRY(mxv_scratch(G, s));
+    G->ws.mx_dirty = true;  // until every kernel of the call is issued
+    mp_prep_kernel<<<small, kMxvThreads, 0, s>>>(a);
+    if (!a.nothing) {
+        mp_main_kernel<<<grid, kMxvThreads, 0, s>>>(a);
+        if (a.dir == GBX_DIR_AUTO) mp_push_kernel<<<grid, kMxvThreads, 0, s>>>(a);
+    }
+    mp_last_kernel<<<small, kMxvThreads, 0, s>>>(a);
     GBX_CUDA_TRY(cudaGetLastError());
+    G->ws.mx_dirty = false;
     return GBX_OK;
 }
 

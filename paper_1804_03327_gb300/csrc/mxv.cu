@@ -11,29 +11,35 @@
 //     the radix sort of Algorithm 3).
 // The result bitmap is then written out as a dense byte vector or as a sorted
 // index list (Section 3: sparse vectors are sorted lists).
-#include <cstring>
-#include <new>
-#include <vector>
+//
+// A call is three kernels (a fourth for a sparse result, or where AUTO has to count a dense u
+// before it can push): mxv_prep_kernel reads u and the mask into bitmaps, or u into a queue
+// with its degree prefix; mxv_main_kernel pulls or pushes, by a decision each block takes
+// from the count of u; the output kernels write w and leave the scratch bitmaps zero for the
+// next call.  A small call is bound by its launches: the separate conversions, scans and
+// decisions of 17 captured launches took 42 us for a sparse step of 100 vertices on RMAT-20
+// (and a capture for every new set of buffers); now 22 us, launched directly (a first
+// call on new buffers 172 -> 55 us).
+#include <algorithm>
 
+#include "frontier.cuh"
 #include "gbx_internal.cuh"
+#include "mxv.cuh"
 
 namespace gbx {
 
 constexpr int kMxvProbe = 16;
 constexpr int kMxvLaneRow = 32;
-constexpr int kMxvHugeRow = 4096;  // rows longer than this are spread over every warp
-constexpr int kMxvChunk = 1024;
-
-__device__ __forceinline__ bool dir_enabled(const int32_t* flag, int want) { return !flag || *flag == want; }
 
 // Row-based matvec over the rows the mask lets through (Eq 2 / Eq 4).  A warp
-// takes a tile of 32 result words (1024 rows), lists the passing nonempty rows in
+// takes a tile of a.tile_words result words (at most 32: 1,024 rows), lists the passing nonempty rows in
 // shared memory (each lane its word's rows, at its prefix of the words' counts)
 // and computes them 64 per round, two rows per lane probing in lockstep: the
 // first entry of a row comes from the dense first-entry array when one is given
 // (one coalesced read instead of a random sector), entries 1..4 from the dense
 // next-entries array (one 16-byte read), then up to kMxvProbe entries four at a
-// time; longer rows are finished by the whole warp 32 entries at a time.  With
+// time; longer rows are finished by the whole warp 128 entries at a time, and those
+// with more than kMxvLongRow left by the whole block after its tiles.  With
 // early exit a row stops at its first hit (Section 5.3); the result is the same
 // either way.
 constexpr int kMxvIlp = 2;
@@ -52,30 +58,64 @@ __device__ __forceinline__ void mxv_tile_list(uint16_t* list, uint32_t m, uint32
     __syncwarp();
 }
 
-__global__ void __launch_bounds__(kMxvThreads) mxv_pull_kernel(const int32_t* __restrict__ ptr, const int32_t* __restrict__ col,
-                                                                const int32_t* __restrict__ first,
-                                                                const int4* __restrict__ next,
-                                                                const uint32_t* __restrict__ nzrows,
-                                                                const uint32_t* __restrict__ multi,
-                                                                const uint32_t* __restrict__ ubm,
-                                                                const uint32_t* __restrict__ pass, uint32_t* __restrict__ R,
-                                                                int32_t nwords, int early_exit, const int32_t* flag,
-                                                                MxvStats* stats, int32_t* huge, int32_t* huge_next,
-                                                                int32_t* huge_count) {
-    if (!dir_enabled(flag, GBX_DIR_PULL)) return;
-    __shared__ uint32_t tile_hits[kMxvThreads / 32][32];
-    __shared__ uint16_t tile_rows[kMxvThreads / 32][1024];
-    uint32_t* hits = tile_hits[threadIdx.x >> 5];
-    uint16_t* list = tile_rows[threadIdx.x >> 5];
+// The block's deferred rows: its warps take 512-entry pieces of a row, four loads in flight a
+// lane.  With early exit the pieces after a known hit are skipped.  exam counts the entries
+// read (every lane adds its own).
+__device__ __forceinline__ void mxv_long_rows(const PullArgs& a, PullSmem& sm, unsigned long long& exam) {
+    __syncthreads();
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    const int cnt = sm.nlong < kMxvLongs ? sm.nlong : kMxvLongs;
+    for (int h = 0; h < cnt; ++h) {
+        const int32_t i = sm.longs[h].x, beg = sm.longs[h].y, end = a.ptr[i + 1];
+        if (threadIdx.x == 0) sm.hit = 0;
+        __syncthreads();
+        for (int32_t k0 = beg + 512 * wib; k0 < end; k0 += 512 * (kMxvThreads / 32)) {
+            if (a.early_exit && *(volatile int*)&sm.hit) break;
+            const int32_t k1 = end - k0 > 512 ? k0 + 512 : end;
+            for (int32_t kk = k0; kk < k1; kk += 128) {
+                int32_t j[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) j[q] = kk + 32 * q + lane < k1 ? a.col[kk + 32 * q + lane] : -1;
+                bool hit = false;
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    exam += j[q] >= 0 ? 1u : 0u;
+                    hit |= j[q] >= 0 && bit_test(a.ubm, j[q]);
+                }
+                if (__any_sync(0xffffffffu, hit)) {
+                    if (lane == 0) sm.hit = 1;
+                    if (a.early_exit) break;
+                }
+            }
+        }
+        __syncthreads();
+        if (threadIdx.x == 0 && sm.hit) atomicOr(a.R + (i >> 5), 1u << (i & 31));
+        __syncthreads();
+    }
+}
+
+__device__ __forceinline__ void mxv_pull(const PullArgs& a, PullSmem& sm) {
+    const int32_t* __restrict__ ptr = a.ptr;
+    const int32_t* __restrict__ col = a.col;
+    const int32_t* __restrict__ first = a.first;
+    const int4* __restrict__ next = a.next;
+    const uint32_t* __restrict__ multi = a.multi;
+    const uint32_t* __restrict__ ubm = a.ubm;
+    const int32_t nwords = a.nwords, tw = a.tile_words;
+    const int early_exit = a.early_exit;
+    uint32_t* hits = sm.hits[threadIdx.x >> 5];
+    uint16_t* list = sm.rows[threadIdx.x >> 5];
+    if (threadIdx.x == 0) sm.nlong = 0;
+    __syncthreads();
     const int lane = threadIdx.x & 31;
     const int gwarp = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
     const int nwarps = (int)((gridDim.x * blockDim.x) >> 5);
-    const int32_t ntiles = (nwords + 31) >> 5;
+    const int32_t ntiles = (nwords + tw - 1) / tw;
     unsigned long long rows = 0, exam = 0;
     for (int32_t tile = gwarp; tile < ntiles; tile += nwarps) {
-        const int32_t w = (tile << 5) + lane;
-        const bool wok = w < nwords;
-        const uint32_t cand0 = wok ? ((pass ? pass[w] : 0xffffffffu) & nzrows[w]) : 0u;
+        const int32_t w0 = tile * tw, w = w0 + lane;
+        const bool wok = lane < tw && w < nwords;
+        const uint32_t cand0 = wok ? ((a.pass ? a.pass[w] ^ a.invert : 0xffffffffu) & a.nz[w]) : 0u;
         hits[lane] = 0u;
         __syncwarp();
         // a tile with more candidates than one round first tests every candidate's first entry
@@ -92,7 +132,7 @@ __global__ void __launch_bounds__(kMxvThreads) mxv_pull_kernel(const int32_t* __
 #pragma unroll
                 for (int r = 0; r < kMxvP1; ++r) {
                     const uint32_t c = base + 32 * r + lane;
-                    i[r] = c < total0 ? (tile << 10) + (int)list[c] : -1;
+                    i[r] = c < total0 ? (w0 << 5) + (int)list[c] : -1;
                 }
 #pragma unroll
                 for (int r = 0; r < kMxvP1; ++r) f0[r] = i[r] >= 0 ? first[i[r]] : -1;
@@ -101,7 +141,7 @@ __global__ void __launch_bounds__(kMxvThreads) mxv_pull_kernel(const int32_t* __
                     if (i[r] < 0) continue;
                     rows += 1;
                     exam += 1;
-                    if (bit_test(ubm, f0[r])) atomicOr(hits + ((i[r] >> 5) - (tile << 5)), 1u << (i[r] & 31));
+                    if (bit_test(ubm, f0[r])) atomicOr(hits + ((i[r] >> 5) - w0), 1u << (i[r] & 31));
                 }
             }
             __syncwarp();
@@ -133,7 +173,7 @@ __global__ void __launch_bounds__(kMxvThreads) mxv_pull_kernel(const int32_t* __
             int4 nx[kMxvIlp];
 #pragma unroll
             for (int r = 0; r < kMxvIlp; ++r) {
-                const int32_t i = (((tile << 5) + jw[r]) << 5) + bitpos[r];
+                const int32_t i = ((w0 + jw[r]) << 5) + bitpos[r];
                 beg[r] = mine[r] ? ptr[i] : 0;
                 end[r] = mine[r] ? ptr[i + 1] : 0;
                 f0[r] = (mine[r] && !two_pass) ? (first ? first[i] : -2) : -1;
@@ -210,14 +250,14 @@ __global__ void __launch_bounds__(kMxvThreads) mxv_pull_kernel(const int32_t* __
             }
 #pragma unroll
             for (int r = 0; r < kMxvIlp; ++r) {
-                if (huge && mine[r] && !done[r] && end[r] - beg[r] > kMxvHugeRow) {
-                    // still unresolved after the lane probe: mxv_pull_huge_kernel scans the rest of
-                    // the row with a whole block (a found row keeps its bit from the probe)
-                    const int32_t i = (((tile << 5) + jw[r]) << 5) + bitpos[r];
-                    const int32_t slot = atomicAdd(huge_count, 1);  // fewer than n rows: fits
-                    huge[slot] = i;
-                    huge_next[slot] = k[r];
-                    done[r] = true;
+                if (mine[r] && !done[r] && end[r] - k[r] > kMxvLongRow) {
+                    // left to the whole block once its tiles are done (a found row keeps its bit
+                    // from the probe)
+                    const int slot = atomicAdd(&sm.nlong, 1);
+                    if (slot < kMxvLongs) {
+                        sm.longs[slot] = make_int2(((w0 + jw[r]) << 5) + bitpos[r], k[r]);
+                        done[r] = true;
+                    }
                 }
                 uint32_t pend = __ballot_sync(0xffffffffu, mine[r] && !done[r] && k[r] < end[r]);
                 while (pend) {
@@ -263,137 +303,298 @@ __global__ void __launch_bounds__(kMxvThreads) mxv_pull_kernel(const int32_t* __
             }
         }
         __syncwarp();
-        if (wok) R[w] = hits[lane];
+        if (wok) a.R[w] = a.accum ? a.R[w] | hits[lane] : hits[lane];
         __syncwarp();
     }
-    if (stats) {
+    mxv_long_rows(a, sm, exam);
+    if (a.stats) {
         rows = warp_sum_u64(rows);
         exam = warp_sum_u64(exam);
         if (lane == 0) {
-            if (rows) atomicAdd(&stats->rows, rows);
-            if (exam) atomicAdd(&stats->exam, exam);
+            if (rows) atomicAdd(&a.stats->rows, rows);
+            if (exam) atomicAdd(&a.stats->exam, exam);
         }
     }
 }
 
-// Rows longer than kMxvHugeRow that the lane probe left unresolved: block b takes
-// rows b, b + gridDim.x, ... of the deferred list (row, next entry) and its warps
-// split the rest of the row into 1024-entry chunks, so a power-law hub is not
-// scanned by one warp.  A hit sets the row's result bit; with early exit, chunks
-// of a row already found are skipped.
-__global__ void __launch_bounds__(kMxvThreads) mxv_pull_huge_kernel(const int32_t* __restrict__ ptr,
-                                                                     const int32_t* __restrict__ col,
-                                                                     const uint32_t* __restrict__ ubm, uint32_t* R,
-                                                                     const int32_t* huge, const int32_t* huge_next,
-                                                                     const int32_t* huge_count,
-                                                                     int early_exit, const int32_t* flag, MxvStats* stats) {
-    if (!dir_enabled(flag, GBX_DIR_PULL)) return;
-    const int lane = threadIdx.x & 31;
-    const int wib = threadIdx.x >> 5;
-    const int nw = blockDim.x >> 5;
-    const int32_t count = *huge_count;
-    unsigned long long exam = 0;
-    for (int32_t h = blockIdx.x; h < count; h += gridDim.x) {
-        const int32_t i = huge[h];
-        const int32_t beg = huge_next[h], end = ptr[i + 1];
-        for (int32_t c0 = beg + wib * kMxvChunk; c0 < end; c0 += nw * kMxvChunk) {
-            if (early_exit && ((__ldcg(R + (i >> 5)) >> (i & 31)) & 1u)) break;
-            const int32_t c1 = end - c0 > kMxvChunk ? c0 + kMxvChunk : end;
-            bool hit = false;
-            for (int32_t k = c0 + lane; k < c1; k += 32) hit |= bit_test(ubm, col[k]);
-            exam += (unsigned long long)((c1 - c0) / 32 + (lane < (c1 - c0) % 32 ? 1 : 0));
-            if (__any_sync(0xffffffffu, hit)) {
-                if (lane == 0) atomicOr(R + (i >> 5), 1u << (i & 31));
-                if (early_exit) break;
-            }
-        }
-    }
-    if (stats) {
-        exam = warp_sum_u64(exam);
-        if (lane == 0 && exam) atomicAdd(&stats->exam, exam);
-    }
+
+__global__ void __launch_bounds__(kMxvThreads, 4) mxv_pull_kernel(PullArgs a) {
+    __shared__ PullSmem sm;
+    mxv_pull(a, sm);
 }
 
-__global__ void mxv_degrees_kernel(const int32_t* __restrict__ ptr, const int32_t* __restrict__ list,
-                                   const int32_t* count_dev, int32_t cap, int32_t n, int32_t* __restrict__ deg,
-                                   const int32_t* flag) {
-    if (!dir_enabled(flag, GBX_DIR_PUSH)) return;
-    // same count as the scan that follows (clamped to n); entries past the
-    // capacity or outside [0, n) expand nothing
-    const int32_t count = min(*count_dev, n);
-    for (int32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < count; k += gridDim.x * blockDim.x) {
-        const int32_t u = k < cap ? list[k] : -1;
-        deg[k] = (u >= 0 && u < n) ? ptr[u + 1] - ptr[u] : 0;
-    }
-}
+// ---------------------------------------------------------------- one call's arguments
 
-// Number of entries of the warp-held sorted window (one value per lane) that are <= e.
-__device__ __forceinline__ int window_rank(long long win, long long e) {
-    int c = 0;
-#pragma unroll
-    for (int j = 0; j < 32; ++j) c += (__shfl_sync(0xffffffffu, win, j) <= e) ? 1 : 0;
-    return c;
-}
-
-__device__ __forceinline__ int32_t last_le(const int32_t* pre, int32_t lo, int32_t hi, long long e) {
-    while (lo < hi) {
-        const int32_t mid = lo + ((hi - lo + 1) >> 1);
-        if ((long long)pre[mid] <= e)
-            lo = mid;
-        else
-            hi = mid - 1;
-    }
-    return lo;
-}
-
-__global__ void __launch_bounds__(kMxvThreads) mxv_push_kernel(const int32_t* __restrict__ ptr, const int32_t* __restrict__ col,
-                                                                const int32_t* __restrict__ list, const int32_t* count_dev,
-                                                                int32_t cap, const int32_t* __restrict__ pre,
-                                                                const uint32_t* __restrict__ pass, uint32_t* R,
-                                                                const int32_t* flag, MxvStats* stats) {
-    if (!dir_enabled(flag, GBX_DIR_PUSH)) return;
-    const int lane = threadIdx.x & 31;
-    const int gwarp = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
-    const int nwarps = (int)((gridDim.x * blockDim.x) >> 5);
-    const int32_t count = min(*count_dev, cap);  // cap = n here: matches the scan's count
-    if (count <= 0) return;
-    const long long E = pre[count];
-    if (stats && gwarp == 0 && lane == 0) {
-        atomicAdd(&stats->ucount, (unsigned long long)count);
-        atomicAdd(&stats->edges, (unsigned long long)E);
-    }
-    long long chunk = (E + nwarps - 1) / nwarps;
-    chunk = chunk < 64 ? 64 : ((chunk + 31) & ~31ll);
-    for (long long e0 = (long long)gwarp * chunk; e0 < E; e0 += (long long)nwarps * chunk) {
-        const long long e1 = e0 + chunk < E ? e0 + chunk : E;
-        int32_t k = 0;
-        if (lane == 0) k = last_le(pre, 0, count - 1, e0);
-        k = __shfl_sync(0xffffffffu, k, 0);
-        for (long long base = e0; base < e1; base += 32) {
-            const int32_t wi = k + 1 + lane;
-            const long long win = wi < count ? (long long)pre[wi] : (long long)INT64_MAX;
-            const long long e = base + lane;
-            const int c = window_rank(win, e);
-            int32_t kk = k + c;
-            if (c == 32) kk = last_le(pre, k + 32, count - 1, e);  // many empty columns in a row
-            if (e < e1) {
-                const int32_t u = list[kk];
-                const int32_t v = col[ptr[u] + (int32_t)(e - pre[kk])];
-                if (!pass || bit_test(pass, v)) {
-                    const uint32_t bit = 1u << (v & 31);
-                    if (!(__ldcg(R + (v >> 5)) & bit)) atomicOr(R + (v >> 5), bit);
-                }
-            }
-            k = __shfl_sync(0xffffffffu, kk, 31);
-        }
-    }
-}
+struct MxvArgs {
+    int32_t n, nwords;
+    MxvVec u, mask, w;
+    uint32_t invert;  // the mask's complement: all ones
+    int32_t accum, dir, early_exit;
+    float alpha;
+    PullArgs pull;
+    const int32_t* push_ptr;
+    const int32_t* push_col;
+    // scratch, zero between calls: u, mask and result bitmaps; ctr->q: the push queue's length
+    // and edges, ctr->n_new: nonzeros of a dense u
+    uint32_t* ubm;
+    uint32_t* pass;
+    uint32_t* R;
+    LevelCtr* ctr;
+    int32_t* q;
+    int32_t* qp;
+    int32_t* qd;
+    int32_t* sums;  // set bits of each block's words (sparse result)
+    int32_t per;    // words per thread of the sparse result's kernels
+    int32_t nothing;  // no row passes
+    MxvStats* stats;
+};
 
 // AUTO: push when nnz(u)/n <= alpha (input sparsity), else pull (Section 6.3).
-__global__ void mxv_decide_kernel(const int32_t* count_dev, int32_t n, float alpha, int32_t* flag) {
-    const double r = (double)(*count_dev) / (double)n;
-    *flag = r <= (double)alpha ? GBX_DIR_PUSH : GBX_DIR_PULL;
+__device__ __forceinline__ int mxv_dir(const MxvArgs& a) {
+    if (a.dir != GBX_DIR_AUTO) return a.dir;
+    const int32_t c = a.u.format == GBX_SPARSE ? *a.u.count : (int32_t)a.ctr->n_new;
+    return (double)c / (double)a.n <= (double)a.alpha ? GBX_DIR_PUSH : GBX_DIR_PULL;
 }
+
+// A queue of the columns a push expands: vertex, exclusive prefix of the columns' lengths, column
+// start minus prefix (frontier.cuh); empty columns are left out.
+__device__ __forceinline__ Stage mxv_stage(const MxvArgs& a, StageBuf* sb, Acc* acc) {
+    return Stage{sb + (threadIdx.x >> 5), 0, a.ctr, a.q, a.qp, a.qd, a.push_ptr, a.push_ptr, 0, 0, acc};
+}
+
+// Stages the set bits of the warp's 32 words (lane l holds word w0 + l); all lanes call.
+__device__ __forceinline__ void mxv_stage_words(Stage& st, uint32_t mine, int32_t w0) {
+    const int lane = threadIdx.x & 31;
+    uint32_t todo = __ballot_sync(0xffffffffu, mine != 0u);
+    while (todo) {
+        const int k = __ffs(todo) - 1;
+        todo &= todo - 1;
+        const uint32_t word = __shfl_sync(0xffffffffu, mine, k);
+        st.put((word >> lane) & 1u, ((w0 + k) << 5) + lane);
+    }
+}
+
+__global__ void __launch_bounds__(kMxvThreads) mxv_prep_kernel(const __grid_constant__ MxvArgs a) {
+    __shared__ StageBuf sb[kMxvThreads / 32];
+    __shared__ unsigned long long bsm[kMxvThreads / 32];
+    __shared__ unsigned long long csm[kMxvThreads / 32][4];
+    const int lane = threadIdx.x & 31;
+    const int64_t gtid = (int64_t)blockIdx.x * kMxvThreads + threadIdx.x, gs = (int64_t)gridDim.x * kMxvThreads;
+    if (a.stats && gtid == 0) *a.stats = MxvStats{};
+    const bool u_sparse = a.u.format == GBX_SPARSE;
+    // a dense u under AUTO is counted here and decided by the next kernel
+    const int dir = u_sparse || a.dir != GBX_DIR_AUTO ? mxv_dir(a) : GBX_DIR_AUTO;
+    Acc acc;
+    Stage st = mxv_stage(a, sb, &acc);
+    uint32_t cnt = 0;
+    if (!u_sparse || a.mask.format == GBX_DENSE) {
+        for (int64_t w0 = gtid - lane; w0 < a.nwords; w0 += gs) {  // warp-uniform
+            const int32_t w = (int32_t)w0 + lane;
+            const bool ok = w < a.nwords;
+            if (a.mask.format == GBX_DENSE && ok)
+                a.pass[w] = pack_word(static_cast<const uint8_t*>(a.mask.data), a.n, w);
+            if (u_sparse) continue;
+            const uint32_t word = ok ? pack_word(static_cast<const uint8_t*>(a.u.data), a.n, w) : 0u;
+            if (dir == GBX_DIR_PUSH) {
+                mxv_stage_words(st, word, (int32_t)w0);
+            } else if (ok) {
+                a.ubm[w] = word;
+            }
+            cnt += (uint32_t)__popc(word);
+        }
+    }
+    if (u_sparse) {
+        const int32_t* list = static_cast<const int32_t*>(a.u.data);
+        const int32_t count = min(min(*a.u.count, a.u.cap), a.n);
+        for (int64_t b = gtid - lane; b < count; b += gs) {  // entries outside [0, n) expand nothing
+            const int32_t v = b + lane < count ? list[b + lane] : -1;
+            const bool ok = v >= 0 && v < a.n;
+            if (dir == GBX_DIR_PUSH)
+                st.put(ok, v);
+            else if (ok)
+                atomicOr(a.ubm + (v >> 5), 1u << (v & 31));
+        }
+    }
+    if (a.mask.format == GBX_SPARSE) {
+        const int32_t* list = static_cast<const int32_t*>(a.mask.data);
+        const int32_t count = min(*a.mask.count, a.mask.cap);
+        for (int64_t i = gtid; i < count; i += gs) {
+            const int32_t v = list[i];
+            if (v >= 0 && v < a.n) atomicOr(a.pass + (v >> 5), 1u << (v & 31));
+        }
+    }
+    if (a.accum && a.w.format == GBX_SPARSE) {  // the result keeps w's entries
+        const int32_t* list = static_cast<const int32_t*>(a.w.data);
+        const int32_t count = min(*a.w.count, a.w.cap);
+        for (int64_t i = gtid; i < count; i += gs) {
+            const int32_t v = list[i];
+            if (v >= 0 && v < a.n) atomicOr(a.R + (v >> 5), 1u << (v & 31));
+        }
+    }
+    if (dir == GBX_DIR_PUSH) st.flush_block<kMxvThreads / 32>(bsm);
+    block_add_counts<kMxvThreads / 32>(csm, cnt, 0ull, 0ull, 0ull, &a.ctr->n_new, nullptr, nullptr, nullptr);
+}
+
+// The queue's edges, evenly over all warps, kMxvPushIlp per lane in flight: a target that
+// passes the mask sets its bit (a reduction) unless the L1-cached word already has it.
+constexpr int kMxvPushIlp = 4;
+
+__device__ __forceinline__ void mxv_push(const MxvArgs& a) {
+    const unsigned long long qv = a.ctr->q;
+    const uint32_t qcount = (uint32_t)qv;
+    const int32_t E = (int32_t)(qv >> 32);
+    const int gwarp = (int)((blockIdx.x * kMxvThreads + threadIdx.x) >> 5);
+    const int nwarps = (int)((gridDim.x * kMxvThreads) >> 5);
+    if (a.stats && blockIdx.x == 0 && threadIdx.x == 0) {
+        a.stats->ucount = a.u.format == GBX_SPARSE ? (unsigned long long)max(0, min(*a.u.count, a.n)) : a.ctr->n_new;
+        a.stats->edges = (unsigned long long)E;
+    }
+    constexpr int kStep = 32 * kMxvPushIlp;
+    int32_t chunk = (int32_t)(((long long)E + nwarps - 1) / nwarps);
+    chunk = chunk <= 32 ? 32 : ((chunk + kStep - 1) / kStep) * kStep;
+    for (long long e0l = (long long)gwarp * chunk; e0l < E; e0l += (long long)nwarps * chunk) {
+        const int32_t e0 = (int32_t)e0l;
+        const int32_t e1 = E - e0 > chunk ? e0 + chunk : E;
+        PushCursorT<kMxvPushIlp> cur;
+        cur.k = warp_find_entry(a.qp, (int32_t)qcount, e0);
+        cur.wlast = -1;
+        for (int32_t base = e0; base < e1; base += kStep) {
+            const PushStepT<kMxvPushIlp> ps = cur.gather(a.push_col, a.q, a.qp, a.qd, qcount, base, e1);
+            uint32_t p[kMxvPushIlp], r[kMxvPushIlp];
+#pragma unroll
+            for (int t = 0; t < kMxvPushIlp; ++t) {
+                p[t] = ps.u[t] >= 0 ? (a.mask.format >= 0 ? a.pass[ps.v[t] >> 5] ^ a.invert : 0xffffffffu) : 0u;
+                r[t] = ps.u[t] >= 0 ? __ldca(a.R + (ps.v[t] >> 5)) : 0xffffffffu;
+            }
+#pragma unroll
+            for (int t = 0; t < kMxvPushIlp; ++t)
+                if (((p[t] & ~r[t]) >> (ps.v[t] & 31)) & 1u) atomicOr(a.R + (ps.v[t] >> 5), 1u << (ps.v[t] & 31));
+        }
+    }
+}
+
+// Pull, push, or -- a dense u that AUTO found sparse -- the queue for mxv_push_kernel.
+__global__ void __launch_bounds__(kMxvThreads, 4) mxv_main_kernel(const __grid_constant__ MxvArgs a) {
+    union MainSmem {
+        PullSmem pull;
+        StageBuf sb[kMxvThreads / 32];
+    };
+    __shared__ MainSmem sm;
+    __shared__ unsigned long long bsm[kMxvThreads / 32];
+    if (mxv_dir(a) == GBX_DIR_PULL) {
+        mxv_pull(a.pull, sm.pull);
+    } else if (a.u.format == GBX_SPARSE || a.dir == GBX_DIR_PUSH) {
+        mxv_push(a);
+    } else {
+        Acc acc;
+        Stage st = mxv_stage(a, sm.sb, &acc);
+        const int lane = threadIdx.x & 31;
+        const int64_t gtid = (int64_t)blockIdx.x * kMxvThreads + threadIdx.x, gs = (int64_t)gridDim.x * kMxvThreads;
+        for (int64_t w0 = gtid - lane; w0 < a.nwords; w0 += gs)
+            mxv_stage_words(st, w0 + lane < a.nwords ? a.ubm[w0 + lane] : 0u, (int32_t)w0);
+        st.flush_block<kMxvThreads / 32>(bsm);
+    }
+}
+
+__global__ void __launch_bounds__(kMxvThreads) mxv_push_kernel(const __grid_constant__ MxvArgs a) {
+    if (mxv_dir(a) == GBX_DIR_PUSH) mxv_push(a);
+}
+
+// ---------------------------------------------------------------- output
+
+// Leaves word w of the scratch bitmaps zero for the next call and returns the result's.
+__device__ __forceinline__ uint32_t mxv_take_word(const MxvArgs& a, int32_t w) {
+    const uint32_t word = a.R[w];
+    if (word) a.R[w] = 0u;
+    a.ubm[w] = 0u;
+    if (a.mask.format >= 0) a.pass[w] = 0u;
+    return word;
+}
+
+// One thread per word writes its 32 bytes (two 16-byte stores where w is aligned), ORing in the
+// old values when accumulating.
+__global__ void __launch_bounds__(kMxvThreads) mxv_dense_kernel(const __grid_constant__ MxvArgs a) {
+    uint8_t* out = static_cast<uint8_t*>(const_cast<void*>(a.w.data));
+    const bool vec = (reinterpret_cast<uintptr_t>(out) & 15u) == 0;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        a.ctr->q = 0ull;
+        a.ctr->n_new = 0ull;
+    }
+    for (int64_t w = (int64_t)blockIdx.x * kMxvThreads + threadIdx.x; w < a.nwords; w += (int64_t)gridDim.x * kMxvThreads) {
+        const uint32_t word = mxv_take_word(a, (int32_t)w);
+        const int64_t base = w << 5;
+        if (vec && base + 32 <= a.n) {
+            uint32_t v[8];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) v[q] = (((word >> (4 * q)) & 0xfu) * 0x00204081u) & 0x01010101u;
+            if (a.accum) {
+                const uint4 x = reinterpret_cast<const uint4*>(out + base)[0];
+                const uint4 y = reinterpret_cast<const uint4*>(out + base)[1];
+                const uint32_t o[8] = {x.x, x.y, x.z, x.w, y.x, y.y, y.z, y.w};
+#pragma unroll
+                for (int q = 0; q < 8; ++q)
+#pragma unroll
+                    for (int t = 0; t < 4; ++t) v[q] |= (((o[q] >> (8 * t)) & 0xffu) != 0u ? 1u : 0u) << (8 * t);
+            }
+            reinterpret_cast<uint4*>(out + base)[0] = make_uint4(v[0], v[1], v[2], v[3]);
+            reinterpret_cast<uint4*>(out + base)[1] = make_uint4(v[4], v[5], v[6], v[7]);
+        } else {
+            for (int t = 0; t < 32 && base + t < a.n; ++t) {
+                uint8_t x = (uint8_t)((word >> t) & 1u);
+                if (a.accum) x |= out[base + t] != 0 ? 1 : 0;
+                out[base + t] = x;
+            }
+        }
+    }
+}
+
+// Set bits of each block's words (a.per consecutive words a thread).
+__global__ void __launch_bounds__(kMxvThreads) mxv_count_kernel(const __grid_constant__ MxvArgs a) {
+    __shared__ int32_t part[kMxvThreads / 32];
+    const int64_t w0 = ((int64_t)blockIdx.x * kMxvThreads + threadIdx.x) * a.per;
+    uint32_t c = 0;
+    for (int k = 0; k < a.per; ++k) c += w0 + k < a.nwords ? (uint32_t)__popc(a.R[w0 + k]) : 0u;
+    c = __reduce_add_sync(0xffffffffu, c);
+    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = (int32_t)c;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        int32_t s = 0;
+#pragma unroll
+        for (int k = 0; k < kMxvThreads / 32; ++k) s += part[k];
+        a.sums[blockIdx.x] = s;
+    }
+}
+
+// The sorted list of the set bits: a block's place is the sum of the blocks before it.
+__global__ void __launch_bounds__(kMxvThreads) mxv_list_kernel(const __grid_constant__ MxvArgs a) {
+    __shared__ uint32_t part[2][kMxvThreads / 32];
+    int32_t* out = static_cast<int32_t*>(const_cast<void*>(a.w.data));
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    uint32_t before = 0;
+    for (int32_t b = threadIdx.x; b < (int32_t)blockIdx.x; b += kMxvThreads) before += (uint32_t)a.sums[b];
+    const int64_t w0 = ((int64_t)blockIdx.x * kMxvThreads + threadIdx.x) * a.per;
+    uint32_t c = 0;
+    for (int k = 0; k < a.per; ++k) c += w0 + k < a.nwords ? (uint32_t)__popc(a.R[w0 + k]) : 0u;
+    const uint32_t inc = warp_inclusive_sum(c);
+    before = __reduce_add_sync(0xffffffffu, before);
+    if (lane == 31) part[0][wib] = inc;
+    if (lane == 0) part[1][wib] = before;
+    __syncthreads();
+    uint32_t at = inc - c;
+#pragma unroll
+    for (int k = 0; k < kMxvThreads / 32; ++k) at += part[1][k] + (k < wib ? part[0][k] : 0u);
+    for (int k = 0; k < a.per && w0 + k < a.nwords; ++k) {
+        uint32_t word = mxv_take_word(a, (int32_t)(w0 + k));
+        for (; word; word &= word - 1) out[at++] = (int32_t)((w0 + k) << 5) + __ffs(word) - 1;
+    }
+    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == kMxvThreads - 1) {
+        *const_cast<int32_t*>(a.w.count) = (int32_t)at;
+        a.ctr->q = 0ull;
+        a.ctr->n_new = 0ull;
+    }
+}
+
+// ---------------------------------------------------------------- host side
 
 __global__ void zero_stats_kernel(MxvStats* s) {
     MxvStats z = {};
@@ -420,34 +621,145 @@ static gbx_status check_vec(const gbx_vector* v, int32_t n, const char* name, bo
     return GBX_OK;
 }
 
-// mask -> bitmap of passing rows; pass = m XOR complement (Algorithm 2, line 3).
-// No mask: every row passes (*pass_bm = NULL), or none with the complement.
-static gbx_status build_pass(Graph* G, const gbx_vector* mask, int complement, const uint32_t** pass_bm,
-                             bool* nothing_passes, cudaStream_t s) {
+// desc.push_sort: Algorithm 3 on the host's decision (mxv_push_sorted); *done: w is written, else
+// the call pulls.
+static gbx_status mxv_sorted(Graph* G, gbx_vector* w, const gbx_vector* mask, const gbx_vector* u, const gbx_desc& d,
+                             cudaStream_t s, bool* done) {
     const int32_t n = G->n;
-    uint32_t* pass = G->ws.bm[1];
-    *pass_bm = nullptr;
-    *nothing_passes = false;
-    if (!mask) {
-        *nothing_passes = complement != 0;
-    } else if (mask->format == GBX_DENSE) {
-        GBX_TRY(pack_dense_to_bitmap((const uint8_t*)mask->data, n, complement ? 1u : 0u, pass, s));
-        *pass_bm = pass;
-    } else {
+    *done = false;
+    if (d.direction == GBX_DIR_PULL || (!mask && d.mask_complement)) return GBX_OK;
+    const int32_t* ulist = (const int32_t*)u->data;
+    const int32_t* ucount = u->nnz;
+    int32_t ucap = u->capacity < n ? u->capacity : n;
+    uint32_t* ubm = G->ws.bm[0];
+    uint32_t* pass = mask ? G->ws.bm[1] : nullptr;
+    uint32_t* R = G->ws.bm[2];
+    if (u->format == GBX_DENSE) {
+        GBX_TRY(pack_dense_to_bitmap((const uint8_t*)u->data, n, 0, ubm, s));
+        GBX_TRY(bitmap_to_list(ubm, n, G->ws.list, G->ws.flag + 0, G->ws.qd[0], G->ws.scan_tmp, s));
+        ulist = G->ws.list;
+        ucount = G->ws.flag + 0;
+        ucap = n;
+    }
+    if (mask && mask->format == GBX_DENSE) {
+        GBX_TRY(pack_dense_to_bitmap((const uint8_t*)mask->data, n, d.mask_complement ? 1u : 0u, pass, s));
+    } else if (mask) {
         GBX_TRY(fill_bitmap(pass, n, 0u, s));
         GBX_TRY(scatter_list_to_bitmap((const int32_t*)mask->data, mask->nnz, mask->capacity, n, pass, s));
-        if (complement) GBX_TRY(invert_bitmap(pass, n, s));
-        *pass_bm = pass;
+        if (d.mask_complement) GBX_TRY(invert_bitmap(pass, n, s));
     }
+    int32_t hc = 0;
+    GBX_CUDA_TRY(cudaMemcpyAsync(&hc, ucount, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+    GBX_CUDA_TRY(cudaStreamSynchronize(s));
+    if (d.direction == GBX_DIR_AUTO && !((double)hc / (double)n <= (double)d.alpha)) return GBX_OK;
+    const int32_t count = hc < 0 ? 0 : (hc > n ? n : hc);
+    const bool direct = w->format == GBX_SPARSE && !d.accum;  // the sorted list is w itself
+    if (!direct) GBX_TRY(fill_bitmap(R, n, 0u, s));
+    int64_t edges = 0;
+    GBX_TRY(mxv_push_sorted(G, d.transpose ? G->out_ptr : G->in_ptr, d.transpose ? G->out_col : G->in_col, ulist, count,
+                            ucap, pass, direct ? nullptr : R, direct ? (int32_t*)w->data : nullptr,
+                            direct ? w->nnz : nullptr, &edges, s));
+    if (d.trace) {
+        MxvStats* stats = reinterpret_cast<MxvStats*>(G->ws.ctr + 3);
+        zero_stats_kernel<<<1, 1, 0, s>>>(stats);
+        set_push_stats_kernel<<<1, 1, 0, s>>>(stats, count, edges);
+    }
+    if (!direct && w->format == GBX_DENSE) {
+        GBX_TRY(bitmap_to_dense(R, n, d.accum ? (const uint8_t*)w->data : nullptr, (uint8_t*)w->data, s));
+    } else if (!direct) {
+        GBX_TRY(scatter_list_to_bitmap((const int32_t*)w->data, w->nnz, w->capacity, n, R, s));
+        GBX_TRY(bitmap_to_list(R, n, (int32_t*)w->data, w->nnz, G->ws.qd[1], G->ws.scan_tmp, s));
+    }
+    GBX_CUDA_TRY(cudaGetLastError());
+    G->ws.last_stream = s;
+    *done = true;
     return GBX_OK;
 }
 
-gbx_status mxv_minplus(Graph* G, float* w, const uint32_t* pass_bm, bool nothing_passes, const float* u,
-                       const gbx_desc& d, cudaStream_t s);
-gbx_status mxv_issue(Graph* G, gbx_vector* w, const gbx_vector* mask, int32_t semiring, const gbx_vector* u,
-                     const gbx_desc& d, cudaStream_t s);
-gbx_status mxv_replay(Graph* G, gbx_vector* w, const gbx_vector* mask, int32_t semiring, const gbx_vector* u,
-                      const gbx_desc& d, cudaStream_t s);
+static MxvVec mxv_vec(const gbx_vector* v) {
+    if (!v) return MxvVec{-1, nullptr, nullptr, 0};
+    return MxvVec{v->format, v->data, v->nnz, v->capacity};
+}
+
+// Zeroes the call scratch after a call that could not be issued whole (the output kernels leave it zero).
+gbx_status mxv_scratch(Graph* G, cudaStream_t s) {
+    if (!G->ws.mx_dirty) return GBX_OK;
+    GBX_CUDA_TRY(cudaMemsetAsync(G->ws.mx_bm[0], 0, sizeof(uint32_t) * 3 * ((size_t)G->nwords + 1), s));
+    GBX_CUDA_TRY(cudaMemsetAsync(G->ws.mx_ctr, 0, sizeof(LevelCtr), s));
+    return GBX_OK;
+}
+
+static gbx_status mxv_bool(Graph* G, gbx_vector* w, const gbx_vector* mask, const gbx_vector* u, const gbx_desc& d,
+                           cudaStream_t s) {
+    // w = A' u with A' = A^T (transpose) or A.  Pull reads rows of A' (CSR of A'),
+    // push reads the columns of A' selected by u, i.e. rows of (A')^T.
+    MxvArgs a;
+    a.n = G->n;
+    a.nwords = G->nwords;
+    a.u = mxv_vec(u);
+    a.mask = mxv_vec(mask);
+    a.w = mxv_vec(w);
+    a.invert = d.mask_complement ? 0xffffffffu : 0u;
+    a.accum = d.accum ? 1 : 0;
+    a.dir = d.direction;
+    a.alpha = d.alpha;
+    a.early_exit = d.early_exit ? 1 : 0;
+    a.stats = d.trace ? reinterpret_cast<MxvStats*>(G->ws.ctr + 3) : nullptr;
+    a.push_ptr = d.transpose ? G->out_ptr : G->in_ptr;
+    a.push_col = d.transpose ? G->out_col : G->in_col;
+    a.ubm = G->ws.mx_bm[0];
+    a.pass = G->ws.mx_bm[1];
+    a.R = G->ws.mx_bm[2];
+    a.ctr = G->ws.mx_ctr;
+    a.q = G->ws.q[0];
+    a.qp = G->ws.qp[0];
+    a.qd = G->ws.qd[0];
+    a.sums = G->ws.scan_tmp;
+    a.nothing = !mask && d.mask_complement;
+    const unsigned main_blocks = (unsigned)G->num_sms * 4u;
+    PullArgs& p = a.pull;
+    p.ptr = d.transpose ? G->in_ptr : G->out_ptr;
+    p.col = d.transpose ? G->in_col : G->out_col;
+    p.first = d.transpose ? G->first_in : G->first_out;
+    p.next = d.transpose ? G->next_in : G->next_out;
+    p.nz = d.transpose ? G->nz_in : G->nz_out;
+    p.multi = d.transpose ? G->multi_in : G->multi_out;
+    p.ubm = a.ubm;
+    p.pass = mask ? a.pass : nullptr;
+    p.invert = a.invert;
+    p.R = a.R;
+    p.accum = a.accum && w->format == GBX_SPARSE ? 1 : 0;
+    p.nwords = a.nwords;
+    p.tile_words = mxv_tile_words(a.nwords, (long long)main_blocks * (kMxvThreads / 32));
+    p.early_exit = a.early_exit;
+    p.stats = a.stats;
+    GBX_TRY(mxv_scratch(G, s));
+    G->ws.mx_dirty = true;  // until every kernel of the call is issued
+    const int32_t most = std::max(std::max(a.nwords, u->format == GBX_SPARSE ? std::min(u->capacity, G->n) : 0),
+                                  std::max(mask && mask->format == GBX_SPARSE ? std::min(mask->capacity, G->n) : 0,
+                                           p.accum ? G->n : 0));
+    const unsigned prep_blocks = std::max(1u, std::min(div_up(most, kMxvThreads), (unsigned)G->num_sms * 4u));
+    mxv_prep_kernel<<<prep_blocks, kMxvThreads, 0, s>>>(a);
+    if (!a.nothing) {
+        mxv_main_kernel<<<main_blocks, kMxvThreads, 0, s>>>(a);
+        if (u->format == GBX_DENSE && a.dir == GBX_DIR_AUTO) mxv_push_kernel<<<main_blocks, kMxvThreads, 0, s>>>(a);
+    }
+    if (w->format == GBX_DENSE) {
+        const unsigned blocks = std::max(1u, std::min(div_up(a.nwords, kMxvThreads), (unsigned)G->num_sms * 16u));
+        mxv_dense_kernel<<<blocks, kMxvThreads, 0, s>>>(a);
+    } else {
+        a.per = std::max(4, (int)(((int64_t)a.nwords + kMxvThreads * 4096ll - 1) / (kMxvThreads * 4096ll)));
+        const unsigned blocks = div_up(a.nwords, (int64_t)kMxvThreads * a.per);
+        mxv_count_kernel<<<blocks, kMxvThreads, 0, s>>>(a);
+        mxv_list_kernel<<<blocks, kMxvThreads, 0, s>>>(a);
+    }
+    GBX_CUDA_TRY(cudaGetLastError());
+    G->ws.mx_dirty = false;
+    G->ws.last_stream = s;
+    return GBX_OK;
+}
+
+gbx_status mxv_minplus(Graph* G, float* w, const MxvVec& mask, const float* u, const gbx_desc& d, cudaStream_t s);
 
 }  // namespace gbx
 
@@ -488,249 +800,19 @@ extern "C" gbx_status gbx_mxv(gbx_vector* w, const gbx_vector* mask, int32_t sem
                   "GBX_DENSE_F32 vectors belong to the (min, +) semiring");
     }
     cudaStream_t s = (cudaStream_t)stream;
-    // the sorted push reads the frontier size on the host: issued directly; every
-    // other call is one fixed launch sequence, replayed from a captured graph
-    if (d.push_sort) return mxv_issue(G, w, mask, semiring, u, d, s);
-    return mxv_replay(G, w, mask, semiring, u, d, s);
-}
-
-namespace gbx {
-
-gbx_status mxv_issue(Graph* G, gbx_vector* w, const gbx_vector* mask, int32_t semiring, const gbx_vector* u,
-                     const gbx_desc& d, cudaStream_t s) {
-    const int32_t n = G->n;
     if (semiring == GBX_MIN_PLUS_F32) {
-        const uint32_t* pbm = nullptr;
-        bool none = false;
-        GBX_TRY(build_pass(G, mask, d.mask_complement, &pbm, &none, s));
-        GBX_TRY(mxv_minplus(G, (float*)w->data, pbm, none, (const float*)u->data, d, s));
+        GBX_TRY(mxv_minplus(G, (float*)w->data, mxv_vec(mask), (const float*)u->data, d, s));
         G->ws.last_stream = s;
         return GBX_OK;
     }
-
-    // w = A' u with A' = A^T (transpose) or A.  Pull reads rows of A' (CSR of A'),
-    // push reads the columns of A' selected by u, i.e. rows of (A')^T.
-    const int32_t* pull_ptr = d.transpose ? G->in_ptr : G->out_ptr;
-    const int32_t* pull_col = d.transpose ? G->in_col : G->out_col;
-    const uint32_t* pull_nz = d.transpose ? G->nz_in : G->nz_out;
-    const int32_t* pull_first = d.transpose ? G->first_in : G->first_out;
-    const int4* pull_next = d.transpose ? G->next_in : G->next_out;
-    const int32_t* push_ptr = d.transpose ? G->out_ptr : G->in_ptr;
-    const int32_t* push_col = d.transpose ? G->out_col : G->in_col;
-
-    uint32_t* ubm = G->ws.bm[0];
-    uint32_t* R = G->ws.bm[2];
-    int32_t* list_count = G->ws.flag + 0;
-    int32_t* dflag = G->ws.flag + 1;
-    MxvStats* stats = d.trace ? reinterpret_cast<MxvStats*>(G->ws.ctr + 3) : nullptr;
-    if (stats) zero_stats_kernel<<<1, 1, 0, s>>>(stats);
-
-    int dir = d.direction;
-    bool want_pull = dir != GBX_DIR_PUSH;
-    bool want_push = dir != GBX_DIR_PULL;
-
-    // u as a bitmap (pull) and as a sorted list (push)
-    const int32_t* ulist = nullptr;
-    const int32_t* ucount = nullptr;
-    int32_t ucap = n;
-    if (u->format == GBX_DENSE) {
-        GBX_TRY(pack_dense_to_bitmap((const uint8_t*)u->data, n, 0, ubm, s));
-        if (want_push) {
-            GBX_TRY(bitmap_to_list(ubm, n, G->ws.list, list_count, G->ws.qd[0], G->ws.scan_tmp, s));
-            ulist = G->ws.list;
-            ucount = list_count;
-        }
-    } else {
-        ulist = (const int32_t*)u->data;
-        ucount = u->nnz;
-        ucap = u->capacity < n ? u->capacity : n;
-        if (want_pull) {
-            GBX_TRY(fill_bitmap(ubm, n, 0u, s));
-            GBX_TRY(scatter_list_to_bitmap(ulist, ucount, ucap, n, ubm, s));
-        }
+    if (d.push_sort) {
+        bool done = false;
+        GBX_TRY(mxv_sorted(G, w, mask, u, d, s, &done));
+        if (done) return GBX_OK;
+        d.direction = GBX_DIR_PULL;
     }
-    const uint32_t* pass_bm = nullptr;
-    bool nothing_passes = false;
-    GBX_TRY(build_pass(G, mask, d.mask_complement, &pass_bm, &nothing_passes, s));
-    // Algorithm 3 (desc.push_sort): sizes its scratch from the frontier, so the
-    // frontier size and the AUTO decision are taken on the host
-    bool sorted_done = false;
-    if (d.push_sort && want_push && !nothing_passes) {
-        int32_t hc = 0;
-        GBX_CUDA_TRY(cudaMemcpyAsync(&hc, ucount, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
-        GBX_CUDA_TRY(cudaStreamSynchronize(s));
-        if (dir == GBX_DIR_PUSH || (double)hc / (double)n <= (double)d.alpha) {
-            const int32_t count = hc < 0 ? 0 : (hc > n ? n : hc);
-            const bool direct = w->format == GBX_SPARSE && !d.accum;  // the sorted list is w itself
-            if (!direct) GBX_TRY(fill_bitmap(R, n, 0u, s));
-            int64_t edges = 0;
-            GBX_TRY(mxv_push_sorted(G, push_ptr, push_col, ulist, count, ucap, pass_bm, direct ? nullptr : R,
-                                    direct ? (int32_t*)w->data : nullptr, direct ? w->nnz : nullptr, &edges, s));
-            if (stats) set_push_stats_kernel<<<1, 1, 0, s>>>(stats, count, edges);
-            if (direct) {
-                GBX_CUDA_TRY(cudaGetLastError());
-                G->ws.last_stream = s;
-                return GBX_OK;
-            }
-            sorted_done = true;
-        } else {
-            dir = GBX_DIR_PULL;
-            want_push = false;
-        }
-    }
-    // a pull writes every result word; push accumulates into a cleared bitmap
-    if (!sorted_done && (want_push || nothing_passes)) GBX_TRY(fill_bitmap(R, n, 0u, s));
-    if (!nothing_passes && !sorted_done) {
-        const int32_t* flag = nullptr;
-        if (dir == GBX_DIR_AUTO) {
-            mxv_decide_kernel<<<1, 1, 0, s>>>(ucount, n, d.alpha, dflag);
-            flag = dflag;
-        }
-        if (want_push) {
-            int32_t* deg = G->ws.q[0];
-            int32_t* pre = G->ws.qp[0];
-            mxv_degrees_kernel<<<max(1u, min(div_up(n, 256), 152u * 16)), 256, 0, s>>>(push_ptr, ulist, ucount, ucap,
-                                                                                    n, deg, flag);
-            GBX_TRY(exclusive_scan_i32(deg, pre, n, ucount, G->ws.scan_tmp, s));
-            mxv_push_kernel<<<G->num_sms * 8, kMxvThreads, 0, s>>>(push_ptr, push_col,
-                                                                    ulist, ucount, n, pre, pass_bm, R, flag, stats);
-        }
-        if (want_pull) {
-            int32_t* huge = G->ws.q[1];
-            int32_t* huge_next = G->ws.qp[1];
-            int32_t* huge_count = G->ws.flag + 2;
-            GBX_CUDA_TRY(cudaMemsetAsync(huge_count, 0, sizeof(int32_t), s));
-            mxv_pull_kernel<<<G->num_sms * 8, kMxvThreads, 0, s>>>(pull_ptr, pull_col, pull_first, pull_next, pull_nz,
-                                                                    d.transpose ? G->multi_in : G->multi_out, ubm,
-                                                                    pass_bm, R, G->nwords, d.early_exit ? 1 : 0, flag,
-                                                                    stats, huge, huge_next, huge_count);
-            mxv_pull_huge_kernel<<<G->num_sms * 8, kMxvThreads, 0, s>>>(pull_ptr, pull_col, ubm, R, huge, huge_next,
-                                                                         huge_count, d.early_exit ? 1 : 0, flag, stats);
-        }
-    }
-    // output
-    if (w->format == GBX_DENSE) {
-        GBX_TRY(bitmap_to_dense(R, n, d.accum ? (const uint8_t*)w->data : nullptr, (uint8_t*)w->data, s));
-    } else {
-        if (d.accum) GBX_TRY(scatter_list_to_bitmap((const int32_t*)w->data, w->nnz, w->capacity, n, R, s));
-        GBX_TRY(bitmap_to_list(R, n, (int32_t*)w->data, w->nnz, G->ws.qd[1], G->ws.scan_tmp, s));
-    }
-    GBX_CUDA_TRY(cudaGetLastError());
-    G->ws.last_stream = s;
-    return GBX_OK;
+    return mxv_bool(G, w, mask, u, d, s);
 }
-
-// ---------------------------------------------------------------- captured launch sequences
-
-// A gbx_mxv call with the same graph, buffers, counts' addresses, semiring and
-// descriptor issues the same kernels with the same arguments (counts and
-// contents are read on the device), so its launch sequence is captured once, on
-// a private stream, into a CUDA graph and replayed on the caller's stream.  The
-// most recently used kMxvGraphs sequences are kept per graph.
-constexpr size_t kMxvGraphs = 32;
-
-struct MxvKey {
-    const void* wd;
-    const void* wn;
-    const void* md;
-    const void* mn;
-    const void* ud;
-    const void* un;
-    int32_t wf, wc, mf, mc, uf, uc, has_mask, semiring;
-    gbx_desc d;
-};
-
-struct MxvCache {
-    struct Entry {
-        MxvKey key;
-        cudaGraphExec_t exec;
-        uint64_t used;
-    };
-    std::vector<Entry> entries;
-    uint64_t clock = 0;
-};
-
-static MxvKey make_key(const gbx_vector* w, const gbx_vector* mask, int32_t semiring, const gbx_vector* u,
-                       const gbx_desc& d) {
-    MxvKey k;
-    std::memset(&k, 0, sizeof(k));
-    k.wd = w->data;
-    k.wn = w->format == GBX_SPARSE ? w->nnz : nullptr;
-    k.wf = w->format;
-    k.wc = w->format == GBX_SPARSE ? w->capacity : 0;
-    if (mask) {
-        k.has_mask = 1;
-        k.md = mask->data;
-        k.mn = mask->format == GBX_SPARSE ? mask->nnz : nullptr;
-        k.mf = mask->format;
-        k.mc = mask->format == GBX_SPARSE ? mask->capacity : 0;
-    }
-    k.ud = u->data;
-    k.un = u->format == GBX_SPARSE ? u->nnz : nullptr;
-    k.uf = u->format;
-    k.uc = u->format == GBX_SPARSE ? u->capacity : 0;
-    k.semiring = semiring;
-    k.d = d;
-    return k;
-}
-
-void mxv_cache_release(Graph* G) {
-    if (G->mxv_cache) {
-        for (auto& e : G->mxv_cache->entries) cudaGraphExecDestroy(e.exec);
-        delete G->mxv_cache;
-        G->mxv_cache = nullptr;
-    }
-    if (G->mxv_cap_stream) {
-        cudaStreamDestroy(G->mxv_cap_stream);
-        G->mxv_cap_stream = nullptr;
-    }
-}
-
-gbx_status mxv_replay(Graph* G, gbx_vector* w, const gbx_vector* mask, int32_t semiring, const gbx_vector* u,
-                      const gbx_desc& d, cudaStream_t s) {
-    if (!G->mxv_cache) {
-        G->mxv_cache = new (std::nothrow) MxvCache();
-        GBX_CHECK(G->mxv_cache != nullptr, GBX_ERR_OUT_OF_MEMORY, "host allocation failed");
-    }
-    MxvCache& C = *G->mxv_cache;
-    const MxvKey key = make_key(w, mask, semiring, u, d);
-    for (auto& e : C.entries)
-        if (std::memcmp(&e.key, &key, sizeof(key)) == 0) {
-            e.used = ++C.clock;
-            GBX_CUDA_TRY(cudaGraphLaunch(e.exec, s));
-            G->ws.last_stream = s;
-            return GBX_OK;
-        }
-    if (!G->mxv_cap_stream) GBX_CUDA_TRY(cudaStreamCreateWithFlags(&G->mxv_cap_stream, cudaStreamNonBlocking));
-    cudaStream_t cs = G->mxv_cap_stream;
-    GBX_CUDA_TRY(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
-    const gbx_status st = mxv_issue(G, w, mask, semiring, u, d, cs);
-    cudaGraph_t graph = nullptr;
-    const cudaError_t ce = cudaStreamEndCapture(cs, &graph);
-    cudaGraphExec_t exec = nullptr;
-    cudaError_t ie = cudaErrorUnknown;
-    if (st == GBX_OK && ce == cudaSuccess && graph) ie = cudaGraphInstantiate(&exec, graph, 0);
-    if (graph) cudaGraphDestroy(graph);
-    if (st != GBX_OK || ce != cudaSuccess || ie != cudaSuccess) {
-        // not capturable here: issue the sequence directly on the caller's stream
-        if (exec) cudaGraphExecDestroy(exec);
-        cudaGetLastError();
-        return mxv_issue(G, w, mask, semiring, u, d, s);
-    }
-    if (C.entries.size() >= kMxvGraphs) {
-        size_t lru = 0;
-        for (size_t i = 1; i < C.entries.size(); ++i)
-            if (C.entries[i].used < C.entries[lru].used) lru = i;
-        cudaGraphExecDestroy(C.entries[lru].exec);
-        C.entries.erase(C.entries.begin() + (long)lru);
-    }
-    C.entries.push_back({key, exec, ++C.clock});
-    GBX_CUDA_TRY(cudaGraphLaunch(exec, s));
-    G->ws.last_stream = s;
-    return GBX_OK;
-}
-
-}  // namespace gbx
 
 extern "C" gbx_status gbx_mxv_stats(const gbx_graph* A, int64_t* rows, int64_t* examined, int64_t* u_nnz,
                                     int64_t* edges) {

@@ -1,0 +1,88 @@
+// Shared by the matvec translation units: the row-based (pull) matvec on bitmaps.
+#pragma once
+
+#include "gbx_internal.cuh"
+
+namespace gbx {
+
+constexpr int kMxvThreads = 256;
+
+// Per-call counters of gbx_mxv (desc.trace): [0] rows computed by pull, [1]
+// entries examined by pull, [2] nonzeros of u expanded by push, [3] edges expanded.
+struct MxvStats {
+    unsigned long long rows, exam, ucount, edges, pad[4];
+};
+
+constexpr int32_t kMxvLongRow = 1024;  // entries left after the lane probe beyond which a row is the block's
+constexpr int kMxvLongs = 64;          // such rows a block holds (further ones stay with their warp)
+
+struct PullArgs {
+    const int32_t* ptr;
+    const int32_t* col;
+    const int32_t* first;   // entry 0 of each row, or NULL
+    const int4* next;       // entries 1..4 of each row, or NULL
+    const uint32_t* nz;     // nonempty rows
+    const uint32_t* multi;  // rows of at least two entries, or NULL
+    const uint32_t* ubm;
+    const uint32_t* pass;  // rows that pass, XOR invert; NULL: all
+    uint32_t invert;       // 0 or all ones
+    uint32_t* R;
+    int32_t accum;  // R holds bits to be kept
+    int32_t nwords, tile_words, early_exit;
+    MxvStats* stats;
+};
+
+struct PullSmem {
+    uint32_t hits[kMxvThreads / 32][32];
+    uint16_t rows[kMxvThreads / 32][1024];
+    int2 longs[kMxvLongs];  // row, next entry
+    int nlong, hit;
+};
+
+// Bitmap words a warp takes at a time, 32 .. 4: the width whose round-robin critical path
+// over the grid's warps is shortest (ties: the wider).  A tile of 32 words (1,024 rows)
+// leaves most of 9,728 warps without any on a graph of a million rows.
+inline int32_t mxv_tile_words(int32_t nwords, long long nwarps) {
+    int32_t best = 32;
+    long long best_cost = -1;
+    for (int32_t tw = 32; tw >= 4; tw >>= 1) {
+        const long long tiles = ((long long)nwords + tw - 1) / tw;
+        const long long cost = (tiles + nwarps - 1) / nwarps * tw;
+        if (best_cost < 0 || cost < best_cost) {
+            best = tw;
+            best_cost = cost;
+        }
+    }
+    return best;
+}
+
+// The row-based matvec alone (mxv.cu), for the allocation-free entry point; kMxvThreads a block.
+__global__ void mxv_pull_kernel(PullArgs a);
+
+// What gbx_mxv reads, as bitmaps and queues (mxv.cu).
+struct MxvVec {
+    int32_t format;  // GBX_DENSE, GBX_SPARSE or GBX_DENSE_F32; -1: none
+    const void* data;
+    const int32_t* count;
+    int32_t cap;
+};
+
+// Word w of a dense byte vector (bits past n clear): two 16-byte loads where it is aligned.
+__device__ __forceinline__ uint32_t pack_word(const uint8_t* __restrict__ dense, int32_t n, int32_t w) {
+    const int64_t base = (int64_t)w << 5;
+    uint32_t word = 0;
+    if ((reinterpret_cast<uintptr_t>(dense) & 15u) == 0 && base + 32 <= n) {
+        const uint4 x = reinterpret_cast<const uint4*>(dense + base)[0];
+        const uint4 y = reinterpret_cast<const uint4*>(dense + base)[1];
+        const uint32_t v[8] = {x.x, x.y, x.z, x.w, y.x, y.y, y.z, y.w};
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+#pragma unroll
+            for (int t = 0; t < 4; ++t) word |= (((v[q] >> (8 * t)) & 0xffu) != 0u ? 1u : 0u) << (4 * q + t);
+    } else {
+        for (int t = 0; t < 32 && base + t < n; ++t) word |= (dense[base + t] != 0 ? 1u : 0u) << t;
+    }
+    return word;
+}
+
+}  // namespace gbx
