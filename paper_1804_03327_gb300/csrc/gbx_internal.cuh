@@ -95,6 +95,7 @@ constexpr int kTraceCap = 1 << 16;
 // another, so several batches of the same graph can run at once.
 struct Workspace {
     int32_t n_cap = 0;  // vertices the buffers below hold
+    void* slab = nullptr;  // the one allocation that holds them, up to the batched scratch
     uint32_t* bm[4] = {nullptr, nullptr, nullptr, nullptr};  // n-bit bitmaps
     int32_t* q[2] = {nullptr, nullptr};                       // frontier queues
     int32_t* qp[2] = {nullptr, nullptr};                      // out-degree prefix per entry
@@ -126,7 +127,11 @@ struct Workspace {
     int last_traced = 0;
 };
 
-gbx_status workspace_alloc(Workspace& w, int32_t n);
+// The zero-initialised parts are cleared on s: the workspace's first user has to be ordered after that.
+gbx_status workspace_alloc(Workspace& w, int32_t n, cudaStream_t s);
+
+// Entries allocated past the end of out_col and in_col: a whole 32-byte sector can be read anywhere.
+constexpr int64_t kColPad = 8;
 void workspace_release(Workspace& w);
 
 struct Graph {
@@ -136,6 +141,7 @@ struct Graph {
     int32_t symmetric = 0;
     int device = 0;
     int num_sms = 0;
+    void* slab = nullptr;  // one allocation: the arrays below whose size follows from n (not out_col, in_col)
     // CSR of A (out-edges) and of A^T (in-edges); in_* alias out_* when symmetric.
     int32_t* out_ptr = nullptr;
     int32_t* out_col = nullptr;
@@ -192,10 +198,13 @@ size_t scan_tmp_ints(int64_t count_max);
 gbx_status exclusive_scan_i32(const int32_t* in, int32_t* out, int64_t count_max, const int32_t* count_dev,
                               int32_t* tmp, cudaStream_t s);
 
-// Stable LSD radix sort of 64-bit keys on the low `bits` bits; result in *keys (buffers swapped as needed).
-gbx_status radix_sort_u64(unsigned long long** keys, unsigned long long** alt, int64_t n, int bits, cudaStream_t s);
+// Stable LSD radix sort of 64-bit keys on the low `bits` bits; result in *keys (buffers swapped as
+// needed).  tmp needs radix_tmp_ints(n) ints.
+size_t radix_tmp_ints(int64_t n);
+gbx_status radix_sort_u64(unsigned long long** keys, unsigned long long** alt, int64_t n, int bits, int32_t* tmp,
+                          cudaStream_t s);
 // The same for 32-bit keys (the key-only sort of Algorithm 3's multiway merge).
-gbx_status radix_sort_u32(uint32_t** keys, uint32_t** alt, int64_t n, int bits, cudaStream_t s);
+gbx_status radix_sort_u32(uint32_t** keys, uint32_t** alt, int64_t n, int bits, int32_t* tmp, cudaStream_t s);
 
 struct Graph;
 // Column-based matvec as Algorithm 3 (mxv_sort.cu): the columns of u's `count`

@@ -12,16 +12,19 @@
 
 namespace gbx {
 
-static int bits_for(int64_t v) {  // smallest b with 2^b > v
-    int b = 0;
-    while (b < 62 && ((int64_t)1 << b) <= v) ++b;
+static int bits_for(int64_t v) {  // smallest b >= 1 with 2^b > v
+    int b = 1;
+    while (b < 31 && ((int64_t)1 << b) <= v) ++b;
     return b;
 }
 
+// A dropped self-loop's key is `none`, all ones in 2b bits: the largest key.  It is no valid
+// pair's then -- the pair of ones is (n - 1, n - 1) at most, a self-loop -- and without the
+// drop no key is invalid.
 __global__ void make_keys_kernel(const int32_t* __restrict__ src, const int32_t* __restrict__ dst, int64_t m,
                                  int32_t n, int b, int symmetrize, int drop_self, int reverse,
                                  unsigned long long* __restrict__ keys, int32_t* status) {
-    const unsigned long long sentinel = ~0ull;
+    const unsigned long long none = (1ull << (2 * b)) - 1ull;
     for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < m; e += (int64_t)gridDim.x * blockDim.x) {
         int32_t u = src[e], v = dst[e];
         if (reverse) {
@@ -29,7 +32,7 @@ __global__ void make_keys_kernel(const int32_t* __restrict__ src, const int32_t*
             u = v;
             v = t;
         }
-        unsigned long long k0 = sentinel, k1 = sentinel;
+        unsigned long long k0 = none, k1 = none;
         if (u < 0 || u >= n || v < 0 || v >= n) {
             atomicCAS(status + ST_BADINDEX, -1, (int)(e < INT32_MAX ? e : INT32_MAX));
         } else if (!(drop_self && u == v)) {
@@ -41,146 +44,186 @@ __global__ void make_keys_kernel(const int32_t* __restrict__ src, const int32_t*
     }
 }
 
-// keep[k] = 1 if key k is valid and differs from key k-1.
-__global__ void mark_unique_kernel(const unsigned long long* __restrict__ keys, int64_t K, int32_t* __restrict__ keep) {
-    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < K; k += (int64_t)gridDim.x * blockDim.x) {
-        const unsigned long long x = keys[k];
-        keep[k] = (x != ~0ull) && (k == 0 || keys[k - 1] != x) ? 1 : 0;
+// The sorted keys a thread owns (kUniqItems consecutive ones) and which of them are kept: valid
+// and different from the one before.
+constexpr int kUniqThreads = 256;
+constexpr int kUniqItems = 8;
+constexpr int kUniqTile = kUniqThreads * kUniqItems;
+
+__device__ __forceinline__ uint32_t load_unique(const unsigned long long* __restrict__ keys, int64_t K,
+                                                unsigned long long none, int64_t i0, unsigned long long (&x)[kUniqItems],
+                                                unsigned long long& prev) {
+    prev = i0 > 0 && i0 <= K ? keys[i0 - 1] : ~0ull;
+    if (i0 + kUniqItems <= K) {
+#pragma unroll
+        for (int t = 0; t < kUniqItems / 2; ++t) {
+            const ulonglong2 y = reinterpret_cast<const ulonglong2*>(keys + i0)[t];
+            x[2 * t] = y.x;
+            x[2 * t + 1] = y.y;
+        }
+    } else {
+#pragma unroll
+        for (int t = 0; t < kUniqItems; ++t) x[t] = i0 + t < K ? keys[i0 + t] : none;
+    }
+    uint32_t keep = 0u;
+    unsigned long long p = prev;
+#pragma unroll
+    for (int t = 0; t < kUniqItems; ++t) {
+        if (i0 + t < K && x[t] != none && x[t] != p) keep |= 1u << t;
+        p = x[t];
+    }
+    return keep;
+}
+
+// counts[b] = keys kept in tile b.  (none: ~0 when every key is valid)
+__global__ void __launch_bounds__(kUniqThreads)
+    count_unique_kernel(const unsigned long long* __restrict__ keys, int64_t K, unsigned long long none,
+                        int32_t* __restrict__ counts) {
+    __shared__ uint32_t part[kUniqThreads / 32];
+    unsigned long long x[kUniqItems], prev;
+    const int64_t i0 = ((int64_t)blockIdx.x * kUniqThreads + threadIdx.x) * kUniqItems;
+    const uint32_t c = __reduce_add_sync(0xffffffffu, (uint32_t)__popc(load_unique(keys, K, none, i0, x, prev)));
+    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = c;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        uint32_t s = 0;
+        for (int w = 0; w < kUniqThreads / 32; ++w) s += part[w];
+        counts[blockIdx.x] = (int32_t)s;
     }
 }
 
-__global__ void emit_csr_kernel(const unsigned long long* __restrict__ keys, int64_t K, const int32_t* __restrict__ keep,
-                                const int32_t* __restrict__ pos, int b, int32_t* __restrict__ col,
-                                int32_t* __restrict__ rows) {
-    const unsigned long long mask = (1ull << b) - 1ull;
-    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < K; k += (int64_t)gridDim.x * blockDim.x) {
-        if (!keep[k]) continue;
-        const unsigned long long x = keys[k];
-        col[pos[k]] = (int32_t)(x & mask);
-        rows[pos[k]] = (int32_t)(x >> b);
+// The kept keys' columns, and row_ptr[r] = first position whose row is >= r: the first key of
+// a row writes its own entry and those of the empty rows before it, the last key those after it.
+__global__ void __launch_bounds__(kUniqThreads)
+    emit_csr_kernel(const unsigned long long* __restrict__ keys, int64_t K, unsigned long long none,
+                    const int32_t* __restrict__ before, int b, int32_t n, int32_t nnz, int32_t* __restrict__ col,
+                    int32_t* __restrict__ row_ptr) {
+    __shared__ uint32_t part[kUniqThreads / 32];
+    __shared__ int32_t tile[kUniqTile];  // the tile's columns, so that they leave coalesced
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    unsigned long long x[kUniqItems], prev;
+    const int64_t i0 = ((int64_t)blockIdx.x * kUniqThreads + threadIdx.x) * kUniqItems;
+    const uint32_t keep = load_unique(keys, K, none, i0, x, prev);
+    const uint32_t inc = warp_inclusive_sum((uint32_t)__popc(keep));
+    if (lane == 31) part[wid] = inc;
+    __syncthreads();
+    const uint32_t base = (uint32_t)before[blockIdx.x];
+    uint32_t at = inc - (uint32_t)__popc(keep), kept = 0;
+#pragma unroll
+    for (int w = 0; w < kUniqThreads / 32; ++w) {
+        at += w < wid ? part[w] : 0u;
+        kept += part[w];
     }
-}
-
-// row_ptr[r] = first position whose row is >= r (rows are sorted).
-__global__ void row_ptr_kernel(const int32_t* __restrict__ rows, int64_t nnz, int32_t n, int32_t* __restrict__ row_ptr) {
-    for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p <= nnz; p += (int64_t)gridDim.x * blockDim.x) {
-        const int32_t hi = p < nnz ? rows[p] : n;
-        const int32_t lo = p == 0 ? -1 : rows[p - 1];
-        for (int32_t r = lo + 1; r <= hi; ++r) row_ptr[r] = (int32_t)p;
+    const unsigned long long cmask = (1ull << b) - 1ull;
+    int32_t row = prev == ~0ull && i0 == 0 ? -1 : (int32_t)(prev >> b);
+#pragma unroll
+    for (int t = 0; t < kUniqItems; ++t) {
+        if (!((keep >> t) & 1u)) continue;
+        const int32_t r = (int32_t)(x[t] >> b);
+        for (int32_t q = row + 1; q <= r; ++q) row_ptr[q] = (int32_t)(base + at);
+        row = r;
+        tile[at++] = (int32_t)(x[t] & cmask);
+        if ((int32_t)(base + at) == nnz)  // the last key
+            for (int32_t q = r + 1; q <= n; ++q) row_ptr[q] = nnz;
     }
+    __syncthreads();
+    for (uint32_t i = threadIdx.x; i < kept; i += kUniqThreads) col[base + i] = tile[i];
 }
 
-__global__ void first_neighbour_kernel(const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
-                                       int32_t n, int32_t* __restrict__ first) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        first[i] = row_ptr[i + 1] > row_ptr[i] ? col[row_ptr[i]] : -1;
-}
-
-// next[i] = entries 1..4 of row i (-1 past the row's end).
-__global__ void next_neighbours_kernel(const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
-                                       int32_t n, int4* __restrict__ next) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const int32_t b = row_ptr[i], d = row_ptr[i + 1] - b;
-        next[i] = make_int4(d > 1 ? col[b + 1] : -1, d > 2 ? col[b + 2] : -1, d > 3 ? col[b + 3] : -1,
-                            d > 4 ? col[b + 4] : -1);
+// What the kernels read of each row beside the CSR: its first entry, entries 1..4 (-1 past the
+// row's end), whether it has any entry and whether it has two, and the longest row's length.
+__global__ void __launch_bounds__(256)
+    row_heads_kernel(const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col, int32_t n,
+                     int32_t* __restrict__ first, int4* __restrict__ next, uint32_t* __restrict__ nz,
+                     uint32_t* __restrict__ multi, int32_t* longest) {
+    const int lane = threadIdx.x & 31;
+    int32_t most = 0;
+    for (int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x - lane; i0 < n; i0 += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t i = i0 + lane;
+        int32_t d = 0;
+        if (i < n) {
+            const int32_t b = row_ptr[i];
+            d = row_ptr[i + 1] - b;
+            first[i] = d > 0 ? col[b] : -1;
+            next[i] = make_int4(d > 1 ? col[b + 1] : -1, d > 2 ? col[b + 2] : -1, d > 3 ? col[b + 3] : -1,
+                                d > 4 ? col[b + 4] : -1);
+        }
+        const uint32_t w1 = __ballot_sync(0xffffffffu, d >= 1), w2 = __ballot_sync(0xffffffffu, d >= 2);
+        if (lane == 0) {
+            nz[i0 >> 5] = w1;
+            multi[i0 >> 5] = w2;
+        }
+        most = max(most, d);
     }
-}
-
-// bm bit i set iff row i has at least min_len entries.
-__global__ void nonzero_rows_kernel(const int32_t* __restrict__ row_ptr, int32_t n, int32_t min_len,
-                                    uint32_t* __restrict__ bm) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t nw32 = ((int64_t)n + 31) & ~(int64_t)31;
-    if (i - (threadIdx.x & 31) >= nw32) return;
-    const bool nz = i < n && row_ptr[i + 1] - row_ptr[i] >= min_len;
-    const uint32_t word = __ballot_sync(0xffffffffu, nz);
-    if ((threadIdx.x & 31) == 0) bm[i >> 5] = word;
-}
-
-// *out = the length of the longest row (*out starts at 0).
-__global__ void max_row_kernel(const int32_t* __restrict__ row_ptr, int32_t n, int32_t* out) {
-    int32_t m = 0;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        m = max(m, row_ptr[i + 1] - row_ptr[i]);
-    m = __reduce_max_sync(0xffffffffu, m);
-    if ((threadIdx.x & 31) == 0) atomicMax(out, m);
+    most = __reduce_max_sync(0xffffffffu, most);
+    if (lane == 0 && longest && most > 0) atomicMax(longest, most);
 }
 
 static unsigned grid_for(int64_t work) { return (unsigned)std::max<int64_t>(1, std::min<int64_t>((work + 255) / 256, 152 * 32)); }
 
-// Sort the K keys and produce CSR (row_ptr, col) in freshly allocated device memory.
-static gbx_status keys_to_csr(unsigned long long* keys, unsigned long long* alt, int64_t K, int32_t n, int b,
-                              int32_t** row_ptr_out, int32_t** col_out, int64_t* nnz_out, cudaStream_t s) {
+// Temporaries of a build, one allocation: cudaMalloc and cudaFree take about 0.1 ms together
+// whatever the size, the stream-ordered pool gives its memory back at every synchronisation
+// and takes 1.2 ms for these 540 MB.
+struct BuildTemp {
+    void* p = nullptr;
+    ~BuildTemp() {
+        if (p) cudaFree(p);
+    }
+};
+
+// Sorts the K keys and produces the CSR: row_ptr (given) and col (allocated here).  counts
+// needs an int per tile of kUniqTile keys and one more, and room for the scan of those.
+static gbx_status keys_to_csr(unsigned long long* keys, unsigned long long* alt, int64_t K, int32_t n, int b, bool drop,
+                              int32_t* sort_tmp, int32_t* counts, const int32_t* status, int32_t* row_ptr,
+                              int32_t** col_out, int64_t* nnz_out, cudaStream_t s) {
     unsigned long long* k1 = keys;
     unsigned long long* k2 = alt;
-    GBX_TRY(radix_sort_u64(&k1, &k2, K, 2 * b, s));
-    // k2 is free now; reuse it as keep flags + positions (2K + 1 int32 fit in K + 1 uint64)
-    int32_t* keep = reinterpret_cast<int32_t*>(k2);
-    int32_t* pos = keep + K;
-    int32_t* tmp = nullptr;
-    GBX_CUDA_TRY(cudaMallocAsync((void**)&tmp, sizeof(int32_t) * scan_tmp_ints(K), s));
-    mark_unique_kernel<<<grid_for(K), 256, 0, s>>>(k1, K, keep);
-    gbx_status st = exclusive_scan_i32(keep, pos, K, nullptr, tmp, s);
-    int32_t nnz32 = 0;
-    if (st == GBX_OK) {
-        const cudaError_t e1 = cudaMemcpyAsync(&nnz32, pos + K, sizeof(int32_t), cudaMemcpyDeviceToHost, s);
-        const cudaError_t e2 = cudaStreamSynchronize(s);
-        if (e1 != cudaSuccess || e2 != cudaSuccess) {
-            cudaFreeAsync(tmp, s);
-            GBX_CUDA_TRY(e1 != cudaSuccess ? e1 : e2);
-        }
+    const unsigned long long none = drop ? (1ull << (2 * b)) - 1ull : ~0ull;
+    const int64_t tiles = (K + kUniqTile - 1) / kUniqTile;
+    int32_t nnz32 = 0, bad = -1;
+    if (K > 0) {
+        GBX_TRY(radix_sort_u64(&k1, &k2, K, 2 * b, sort_tmp, s));
+        count_unique_kernel<<<(unsigned)tiles, kUniqThreads, 0, s>>>(k1, K, none, counts);
+        GBX_TRY(exclusive_scan_i32(counts, counts, tiles, nullptr, counts + tiles + 1, s));
+        GBX_CUDA_TRY(cudaMemcpyAsync(&nnz32, counts + tiles, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
     }
-    cudaFreeAsync(tmp, s);
-    if (st != GBX_OK) return st;
+    GBX_CUDA_TRY(cudaMemcpyAsync(&bad, status + ST_BADINDEX, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+    GBX_CUDA_TRY(cudaStreamSynchronize(s));
+    if (bad >= 0) {
+        set_error("edge " + std::to_string(bad) + " has an endpoint outside [0, n)");
+        return GBX_ERR_INVALID_INDEX;
+    }
     const int64_t nnz = (uint32_t)nnz32;  // K < 2^32 entries; counts below 2^31 checked below
     GBX_CHECK(nnz < ((int64_t)1 << 31), GBX_ERR_OVERFLOW, "graph has 2^31 or more stored edges");
-    int32_t* row_ptr = nullptr;
     int32_t* col = nullptr;
-    int32_t* rows = nullptr;
-    GBX_CUDA_TRY(cudaMalloc((void**)&row_ptr, sizeof(int32_t) * ((size_t)n + 1)));
-    cudaError_t e = cudaMalloc((void**)&col, sizeof(int32_t) * (size_t)std::max<int64_t>(nnz, 1));
-    if (e == cudaSuccess) e = cudaMallocAsync((void**)&rows, sizeof(int32_t) * (size_t)std::max<int64_t>(nnz, 1), s);
-    if (e != cudaSuccess) {
-        cudaFree(row_ptr);
-        if (col) cudaFree(col);
-        GBX_CUDA_TRY(e);
-    }
-    emit_csr_kernel<<<grid_for(K), 256, 0, s>>>(k1, K, keep, pos, b, col, rows);
-    row_ptr_kernel<<<grid_for(nnz + 1), 256, 0, s>>>(rows, nnz, n, row_ptr);
-    cudaFreeAsync(rows, s);
-    e = cudaGetLastError();
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    if (e != cudaSuccess) {
-        cudaFree(row_ptr);
-        cudaFree(col);
-        GBX_CUDA_TRY(e);
-    }
-    *row_ptr_out = row_ptr;
-    *col_out = col;
+    GBX_CUDA_TRY(cudaMalloc((void**)&col, sizeof(int32_t) * (size_t)(nnz + kColPad)));
+    *col_out = col;  // the graph's from here on
     *nnz_out = nnz;
+    if (nnz > 0)
+        emit_csr_kernel<<<(unsigned)tiles, kUniqThreads, 0, s>>>(k1, K, none, counts, b, n, (int32_t)nnz, col, row_ptr);
+    else
+        GBX_CUDA_TRY(cudaMemsetAsync(row_ptr, 0, sizeof(int32_t) * ((size_t)n + 1), s));
+    GBX_CUDA_TRY(cudaGetLastError());
     return GBX_OK;
 }
+
+// Hands out 256-byte aligned parts of one allocation: first with base NULL for the size, then again.
+struct Carve {
+    char* base = nullptr;
+    size_t used = 0;
+    template <typename T>
+    T* take(size_t count) {
+        T* r = reinterpret_cast<T*>(base + used);
+        used += (sizeof(T) * count + 255) & ~(size_t)255;
+        return r;
+    }
+};
 
 void workspace_release(Workspace& w) {
     auto f = [](void* p) {
         if (p) cudaFree(p);
     };
-    for (auto& p : w.bm) f(p);
-    for (int i = 0; i < 2; ++i) {
-        f(w.q[i]);
-        f(w.qp[i]);
-        f(w.qd[i]);
-    }
-    f(w.list);
-    f(w.scan_tmp);
-    f(w.ctr);
-    f(w.bar);
-    f(w.trace);
-    f(w.status);
-    f(w.flag);
-    f(w.handoff);
-    f(w.mx_bm[0]);
-    f(w.mx_ctr);
+    f(w.slab);
     f(w.msV);
     for (auto& p : w.msF) f(p);
     f(w.msP);
@@ -196,18 +239,9 @@ static void graph_release(Graph* g) {
     auto f = [](void* p) {
         if (p) cudaFree(p);
     };
-    if (g->in_ptr != g->out_ptr) f(g->in_ptr);
     if (g->in_col != g->out_col) f(g->in_col);
-    f(g->out_ptr);
     f(g->out_col);
-    f(g->nz_in);
-    if (g->multi_out != g->multi_in) f(g->multi_out);
-    f(g->multi_in);
-    if (g->nz_out != g->nz_in) f(g->nz_out);
-    if (g->first_out != g->first_in) f(g->first_out);
-    f(g->first_in);
-    if (g->next_out != g->next_in) f(g->next_out);
-    f(g->next_in);
+    f(g->slab);
     if (g->in_val != g->out_val) f(g->in_val);
     f(g->out_val);
     f(g->nzr_in);
@@ -223,40 +257,48 @@ static void graph_release(Graph* g) {
     delete g;
 }
 
-static gbx_status workspace_alloc_all(Workspace& w, int32_t n) {
+// The parts of a workspace for n vertices; those that start out zero come first (*zero bytes).
+static void workspace_carve(Workspace& w, int32_t n, Carve& c, size_t* zero) {
     const size_t nw = (size_t)(n + 31) / 32 + 1;
     const size_t nn = (size_t)n + 1;
-    for (auto& p : w.bm) GBX_CUDA_TRY(cudaMalloc((void**)&p, sizeof(uint32_t) * nw));
-    for (int i = 0; i < 2; ++i) {
-        GBX_CUDA_TRY(cudaMalloc((void**)&w.q[i], sizeof(int32_t) * nn));
-        GBX_CUDA_TRY(cudaMalloc((void**)&w.qp[i], sizeof(int32_t) * nn));
-        GBX_CUDA_TRY(cudaMalloc((void**)&w.qd[i], sizeof(int32_t) * nn));
-    }
-    GBX_CUDA_TRY(cudaMalloc((void**)&w.list, sizeof(int32_t) * nn));
-    GBX_CUDA_TRY(cudaMalloc((void**)&w.scan_tmp, sizeof(int32_t) * scan_tmp_ints((int64_t)nn)));
-    GBX_CUDA_TRY(cudaMalloc((void**)&w.ctr, sizeof(LevelCtr) * 4));
-    GBX_CUDA_TRY(cudaMalloc((void**)&w.bar, sizeof(GridBar)));
-    GBX_CUDA_TRY(cudaMemset(w.bar, 0, sizeof(GridBar)));
-    GBX_CUDA_TRY(cudaMalloc((void**)&w.trace, sizeof(LevelRec) * kTraceCap));
-    GBX_CUDA_TRY(cudaMalloc((void**)&w.status, sizeof(int32_t) * ST_WORDS));
-    GBX_CUDA_TRY(cudaMemset(w.status, 0, sizeof(int32_t) * ST_WORDS));
-    GBX_CUDA_TRY(cudaMalloc((void**)&w.flag, sizeof(int32_t) * 64));
-    GBX_CUDA_TRY(cudaMemset(w.flag, 0, sizeof(int32_t) * 64));
-    GBX_CUDA_TRY(cudaMalloc((void**)&w.handoff, sizeof(ClHandoff)));
-    GBX_CUDA_TRY(cudaMalloc((void**)&w.mx_bm[0], sizeof(uint32_t) * 3 * nw));
-    GBX_CUDA_TRY(cudaMemset(w.mx_bm[0], 0, sizeof(uint32_t) * 3 * nw));
+    w.bar = c.take<GridBar>(1);
+    w.status = c.take<int32_t>(ST_WORDS);
+    w.flag = c.take<int32_t>(64);
+    w.mx_ctr = c.take<LevelCtr>(1);
+    w.mx_bm[0] = c.take<uint32_t>(3 * nw);
     w.mx_bm[1] = w.mx_bm[0] + nw;
     w.mx_bm[2] = w.mx_bm[1] + nw;
-    GBX_CUDA_TRY(cudaMalloc((void**)&w.mx_ctr, sizeof(LevelCtr)));
-    GBX_CUDA_TRY(cudaMemset(w.mx_ctr, 0, sizeof(LevelCtr)));
+    *zero = c.used;
+    for (auto& p : w.bm) p = c.take<uint32_t>(nw);
+    for (int i = 0; i < 2; ++i) {
+        w.q[i] = c.take<int32_t>(nn);
+        w.qp[i] = c.take<int32_t>(nn);
+        w.qd[i] = c.take<int32_t>(nn);
+    }
+    w.list = c.take<int32_t>(nn);
+    w.scan_tmp = c.take<int32_t>(scan_tmp_ints((int64_t)nn));
+    w.ctr = c.take<LevelCtr>(4);
+    w.trace = c.take<LevelRec>(kTraceCap);
+    w.handoff = c.take<ClHandoff>(1);
+}
+
+static gbx_status workspace_alloc_all(Workspace& w, int32_t n, cudaStream_t s) {
+    Carve c;
+    size_t zero = 0;
+    workspace_carve(w, n, c, &zero);
+    GBX_CUDA_TRY(cudaMalloc(&w.slab, c.used));
+    c.base = static_cast<char*>(w.slab);
+    c.used = 0;
+    workspace_carve(w, n, c, &zero);
+    GBX_CUDA_TRY(cudaMemsetAsync(w.slab, 0, zero, s));
     w.n_cap = n;  // only once every buffer exists
     return GBX_OK;
 }
 
 // All or nothing: a failed allocation releases what was allocated, so no half-built
 // workspace (one that claims capacity n but holds null buffers) is ever left behind.
-gbx_status workspace_alloc(Workspace& w, int32_t n) {
-    const gbx_status st = workspace_alloc_all(w, n);
+gbx_status workspace_alloc(Workspace& w, int32_t n, cudaStream_t s) {
+    const gbx_status st = workspace_alloc_all(w, n, s);
     if (st != GBX_OK) workspace_release(w);
     return st;
 }
@@ -271,101 +313,74 @@ static gbx_status build_impl(Graph* g, int32_t n, int64_t m, const int32_t* src,
     g->nwords = (n + 31) / 32;
     g->symmetric = sym;
     g->drop_self_loops = drop;
-    GBX_TRY(workspace_alloc(g->ws, n));
+    GBX_TRY(workspace_alloc(g->ws, n, s));
 
     const int64_t K = sym ? 2 * m : m;
     GBX_CHECK(K < ((int64_t)1 << 32), GBX_ERR_OVERFLOW, "too many edge entries (2^32 or more)");
-    const int b = bits_for(n);  // 2^b > n - 1 and the all-ones pattern is never a vertex pair
+    const int b = bits_for((int64_t)n - 1);
 
-    // device copies of the edge list
+    // the arrays whose size follows from n
+    for (int pass = 0; pass < 2; ++pass) {
+        Carve c;
+        c.base = static_cast<char*>(g->slab);
+        g->out_ptr = c.take<int32_t>((size_t)n + 1);
+        g->in_ptr = sym ? g->out_ptr : c.take<int32_t>((size_t)n + 1);
+        g->nz_in = c.take<uint32_t>((size_t)g->nwords + 1);
+        g->multi_in = c.take<uint32_t>((size_t)g->nwords + 1);
+        g->first_in = c.take<int32_t>((size_t)n + 1);
+        g->next_in = c.take<int4>((size_t)n + 1);
+        g->nz_out = sym ? g->nz_in : c.take<uint32_t>((size_t)g->nwords + 1);
+        g->multi_out = sym ? g->multi_in : c.take<uint32_t>((size_t)g->nwords + 1);
+        g->first_out = sym ? g->first_in : c.take<int32_t>((size_t)n + 1);
+        g->next_out = sym ? g->next_in : c.take<int4>((size_t)n + 1);
+        if (pass == 0) GBX_CUDA_TRY(cudaMalloc(&g->slab, c.used));
+    }
+
+    // temporaries: two key buffers, the sort's and the deduplication's scratch, a device copy of a host edge list
+    const bool on_host = !(flags & GBX_DEVICE_EDGES) && m > 0;
+    const int64_t tiles = (K + kUniqTile - 1) / kUniqTile;
+    BuildTemp temp;
+    unsigned long long* keys = nullptr;
+    unsigned long long* alt = nullptr;
+    int32_t* sort_tmp = nullptr;
+    int32_t* counts = nullptr;
+    int32_t* own = nullptr;
+    for (int pass = 0; pass < 2; ++pass) {
+        Carve c;
+        c.base = static_cast<char*>(temp.p);
+        keys = c.take<unsigned long long>((size_t)K + 1);
+        alt = c.take<unsigned long long>((size_t)K + 1);
+        sort_tmp = c.take<int32_t>(radix_tmp_ints(K));
+        counts = c.take<int32_t>((size_t)tiles + 1 + scan_tmp_ints(tiles));
+        own = c.take<int32_t>(on_host ? 2 * (size_t)m : 0);
+        if (pass == 0) GBX_CUDA_TRY(cudaMalloc(&temp.p, c.used));
+    }
     const int32_t* dsrc = src;
     const int32_t* ddst = dst;
-    int32_t* own = nullptr;
-    if (!(flags & GBX_DEVICE_EDGES) && m > 0) {
-        GBX_CUDA_TRY(cudaMallocAsync((void**)&own, sizeof(int32_t) * 2 * (size_t)m, s));
+    if (on_host) {
         GBX_CUDA_TRY(cudaMemcpyAsync(own, src, sizeof(int32_t) * (size_t)m, cudaMemcpyHostToDevice, s));
         GBX_CUDA_TRY(cudaMemcpyAsync(own + m, dst, sizeof(int32_t) * (size_t)m, cudaMemcpyHostToDevice, s));
         dsrc = own;
         ddst = own + m;
     }
-    unsigned long long* keys = nullptr;
-    unsigned long long* alt = nullptr;
-    const size_t kbytes = sizeof(unsigned long long) * (size_t)(K + 1);  // + 1: keep flags and positions reuse it
-    cudaError_t e = cudaMallocAsync((void**)&keys, kbytes, s);
-    if (e == cudaSuccess) e = cudaMallocAsync((void**)&alt, kbytes, s);
-    if (e != cudaSuccess) {
-        if (own) cudaFreeAsync(own, s);
-        if (keys) cudaFreeAsync(keys, s);
-        GBX_CUDA_TRY(e);
-    }
-    gbx_status st = GBX_OK;
-    int32_t bad = -1;
-    auto cleanup = [&]() {
-        cudaFreeAsync(keys, s);
-        cudaFreeAsync(alt, s);
-        if (own) cudaFreeAsync(own, s);
-    };
     GBX_CUDA_TRY(cudaMemsetAsync(g->ws.status + ST_BADINDEX, 0xff, sizeof(int32_t), s));
     if (m > 0) make_keys_kernel<<<grid_for(m), 256, 0, s>>>(dsrc, ddst, m, n, b, sym, drop, 0, keys, g->ws.status);
-    e = cudaMemcpyAsync(&bad, g->ws.status + ST_BADINDEX, sizeof(int32_t), cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    if (e != cudaSuccess) {
-        cleanup();
-        GBX_CUDA_TRY(e);
-    }
-    if (bad >= 0) {
-        cleanup();
-        set_error("edge " + std::to_string(bad) + " has an endpoint outside [0, n)");
-        return GBX_ERR_INVALID_INDEX;
-    }
-    st = keys_to_csr(keys, alt, K, n, b, &g->out_ptr, &g->out_col, &g->nnz, s);
-    if (st == GBX_OK && !sym) {
+    GBX_TRY(keys_to_csr(keys, alt, K, n, b, drop != 0, sort_tmp, counts, g->ws.status, g->out_ptr, &g->out_col, &g->nnz, s));
+    if (sym) {
+        g->in_col = g->out_col;
+    } else {
         // A^T: the same entries with row and column exchanged
         if (m > 0) make_keys_kernel<<<grid_for(m), 256, 0, s>>>(dsrc, ddst, m, n, b, 0, drop, 1, keys, g->ws.status);
         int64_t nnz_t = 0;
-        st = keys_to_csr(keys, alt, K, n, b, &g->in_ptr, &g->in_col, &nnz_t, s);
-        if (st == GBX_OK && nnz_t != g->nnz) {
-            set_error("internal: transpose has a different edge count");
-            st = GBX_ERR_CUDA;
-        }
-    } else if (st == GBX_OK) {
-        g->in_ptr = g->out_ptr;
-        g->in_col = g->out_col;
-    }
-    cleanup();
-    if (st != GBX_OK) return st;
-    GBX_CUDA_TRY(cudaMalloc((void**)&g->nz_in, sizeof(uint32_t) * ((size_t)g->nwords + 1)));
-    const int64_t nw32 = ((int64_t)n + 31) & ~(int64_t)31;
-    nonzero_rows_kernel<<<div_up(nw32, 256), 256, 0, s>>>(g->in_ptr, n, 1, g->nz_in);
-    GBX_CUDA_TRY(cudaMalloc((void**)&g->multi_in, sizeof(uint32_t) * ((size_t)g->nwords + 1)));
-    nonzero_rows_kernel<<<div_up(nw32, 256), 256, 0, s>>>(g->in_ptr, n, 2, g->multi_in);
-    if (sym) {
-        g->nz_out = g->nz_in;
-        g->multi_out = g->multi_in;
-    } else {
-        GBX_CUDA_TRY(cudaMalloc((void**)&g->multi_out, sizeof(uint32_t) * ((size_t)g->nwords + 1)));
-        nonzero_rows_kernel<<<div_up(nw32, 256), 256, 0, s>>>(g->out_ptr, n, 2, g->multi_out);
-        GBX_CUDA_TRY(cudaMalloc((void**)&g->nz_out, sizeof(uint32_t) * ((size_t)g->nwords + 1)));
-        nonzero_rows_kernel<<<div_up(nw32, 256), 256, 0, s>>>(g->out_ptr, n, 1, g->nz_out);
-    }
-    GBX_CUDA_TRY(cudaMalloc((void**)&g->first_in, sizeof(int32_t) * ((size_t)n + 1)));
-    first_neighbour_kernel<<<grid_for(n), 256, 0, s>>>(g->in_ptr, g->in_col, n, g->first_in);
-    if (sym) {
-        g->first_out = g->first_in;
-    } else {
-        GBX_CUDA_TRY(cudaMalloc((void**)&g->first_out, sizeof(int32_t) * ((size_t)n + 1)));
-        first_neighbour_kernel<<<grid_for(n), 256, 0, s>>>(g->out_ptr, g->out_col, n, g->first_out);
-    }
-    GBX_CUDA_TRY(cudaMalloc((void**)&g->next_in, sizeof(int4) * ((size_t)n + 1)));
-    next_neighbours_kernel<<<grid_for(n), 256, 0, s>>>(g->in_ptr, g->in_col, n, g->next_in);
-    if (sym) {
-        g->next_out = g->next_in;
-    } else {
-        GBX_CUDA_TRY(cudaMalloc((void**)&g->next_out, sizeof(int4) * ((size_t)n + 1)));
-        next_neighbours_kernel<<<grid_for(n), 256, 0, s>>>(g->out_ptr, g->out_col, n, g->next_out);
+        GBX_TRY(keys_to_csr(keys, alt, K, n, b, drop != 0, sort_tmp, counts, g->ws.status, g->in_ptr, &g->in_col, &nnz_t, s));
+        GBX_CHECK(nnz_t == g->nnz, GBX_ERR_CUDA, "internal: transpose has a different edge count");
     }
     int32_t* const longest = g->ws.flag + 10;  // zero since the workspace was made
-    max_row_kernel<<<grid_for(n), 256, 0, s>>>(g->out_ptr, n, longest);
+    row_heads_kernel<<<grid_for(n), 256, 0, s>>>(g->out_ptr, g->out_col, n, g->first_out, g->next_out, g->nz_out,
+                                                 g->multi_out, longest);
+    if (!sym)
+        row_heads_kernel<<<grid_for(n), 256, 0, s>>>(g->in_ptr, g->in_col, n, g->first_in, g->next_in, g->nz_in,
+                                                     g->multi_in, nullptr);
     GBX_CUDA_TRY(cudaGetLastError());
     GBX_CUDA_TRY(cudaMemcpyAsync(&g->max_out_degree, longest, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
     GBX_CUDA_TRY(cudaStreamSynchronize(s));

