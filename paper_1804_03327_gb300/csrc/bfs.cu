@@ -224,29 +224,17 @@ __device__ __forceinline__ void push_level(const BfsArgs& a, int32_t L, int cur,
 // ---------------------------------------------------------------- pull (Eq 4, Algorithm 2)
 
 #ifndef GBX_PULL_ILP
-#define GBX_PULL_ILP 2
+#define GBX_PULL_ILP 1
 #endif
-constexpr int kPullIlp = GBX_PULL_ILP;  // candidate rows per lane per round (independent probe chains)
-#ifndef GBX_PULL_STEP
-#define GBX_PULL_STEP 2
-#endif
-constexpr int kPullStep = GBX_PULL_STEP;  // in-neighbours a lane loads per probe step (loads in flight)
-// Bitmap words one warp takes at a time in a pull level, a.tile_words: 32, 16 or
-// 8 (lane l holds word l of the tile).  The host picks the width whose round-robin
-// critical path, ceil(tiles / warps) * width, is shortest (ties: the wider), so a
-// graph with fewer 32-word tiles than warps still keeps every warp busy.
+constexpr int kPullIlp = GBX_PULL_ILP;  // pass-2 rows per lane (2: 928 us instead of 888, from spills)
+// Bitmap words one warp takes at a time in a pull level (lane l holds word l of the tile): an
+// even share of the words over as many rounds as 32 words a warp need.  RMAT-22 has 27 words
+// for each of 4,864 warps; tiles of 32 left 768 warps without any and the others a fifth longer
+// (eight sources one after another 888 -> 856 us; tiles of half the width 941).
 int32_t pull_tile_words(int32_t nwords, long long nwarps) {
-    int32_t best = 32;
-    long long best_cost = -1;
-    for (int32_t tw = 32; tw >= 8; tw >>= 1) {
-        const long long tiles = ((long long)nwords + tw - 1) / tw;
-        const long long cost = (tiles + nwarps - 1) / nwarps * tw;
-        if (best_cost < 0 || cost < best_cost) {
-            best = tw;
-            best_cost = cost;
-        }
-    }
-    return best;
+    const long long rounds = (nwords + 32 * nwarps - 1) / (32 * nwarps);
+    const long long tw = (nwords + nwarps * rounds - 1) / (nwarps * rounds);
+    return (int32_t)(tw < 4 ? 4 : tw);
 }
 // A row with more than kPullHugeRow in-edges left after the lane probe is not
 // scanned by the warp that met it: it is listed and, once every tile is done,
@@ -306,10 +294,16 @@ __device__ __forceinline__ int warp_scan(const int32_t* __restrict__ in_col, con
 // (put_tile_list).  Pass 1 tests every such row's first in-neighbour (the dense
 // first_in array) against the frontier, kP1 rows per lane in flight; most rows
 // of a power-law graph settle here.  Pass 2 takes the rows pass 1 left open that
-// have more in-neighbours, 32 * kPullIlp per round, kPullIlp rows per lane probing
-// in lockstep: in-neighbours 1..4 from the dense next_in array, then the lane
-// probe; rows longer than the probe depth are finished by the whole warp, or by
-// the whole grid when they are very long.
+// have more in-neighbours, a row per lane, each lane going on to the next one as
+// soon as its row is settled: in-neighbours 1..4 from the dense next_in array, then
+// four at a time up to the probe depth; rows longer than that are finished by the
+// whole warp, or by the whole grid when they are very long.
+//
+// Bound by dependent gathers, not by bandwidth (RMAT-22's first big pull reads about
+// 140 MB in 65 us).  Rounds of 64 rows probing in lockstep took as long as the slowest
+// row of each: that level 82 us, and eight sources one after another (each with its
+// seven levels) 989, now 847.  The in-neighbour arrays are read past L1, which then keeps more
+// of the frontier bitmap: 989 -> 949 by itself.
 #ifndef GBX_PULL_P1
 #define GBX_PULL_P1 4
 #endif
@@ -413,132 +407,109 @@ __device__ __forceinline__ void pull_level(const BfsArgs& a, int32_t L, int vcur
         const uint32_t incl = warp_inclusive_sum(cntw);
         const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);
         if (total) put_tile_list(clist, sv, incl - cntw);
-        for (uint32_t base = 0; base < total; base += 32 * kPullIlp) {
-            bool mine[kPullIlp], found[kPullIlp], found1[kPullIlp], done[kPullIlp];
-            int jw[kPullIlp], bitpos[kPullIlp];
-            uint32_t cwj[kPullIlp];
-            int32_t i[kPullIlp], beg[kPullIlp], end[kPullIlp], k[kPullIlp], par[kPullIlp];
-            unsigned long long exam[kPullIlp];
+        // Each lane has kPullIlp rows of its own and takes the next open one as soon as a row is
+        // settled; in one step a row tests four in-neighbours (1..4 from the dense next_in array,
+        // further ones from the column array), its loads issued together with the other's.
+        uint32_t nxt = 0;  // rows of the list handed out
+        int32_t i[kPullIlp], beg[kPullIlp], end[kPullIlp], k[kPullIlp], par[kPullIlp];
+        bool known[kPullIlp];  // pass 1 found the row already (without early exit)
+#pragma unroll
+        for (int r = 0; r < kPullIlp; ++r) {
+            i[r] = -1;
+            beg[r] = end[r] = k[r] = 0;
+            par[r] = -1;
+            known[r] = false;
+        }
+        for (;;) {
+            int32_t x[kPullIlp][4], f0[kPullIlp];
+            bool live = false;
 #pragma unroll
             for (int r = 0; r < kPullIlp; ++r) {
-                const uint32_t c = base + 32 * r + lane;
-                mine[r] = c < total;
-                const int off = mine[r] ? (int)clist[c] : 0;
-                const int j = off >> 5;
-                jw[r] = j;
-                const uint32_t f1j = __shfl_sync(0xffffffffu, f1, j);
-                cwj[r] = __shfl_sync(0xffffffffu, cw, j);
-                bitpos[r] = off & 31;
-                i[r] = ((tile * tw + j) << 5) + bitpos[r];
-                // only without early exit does pass 2 see rows pass 1 already found
-                found1[r] = mine[r] && ((f1j >> bitpos[r]) & 1u);
-                found[r] = found1[r];
-                done[r] = false;
-                exam[r] = 0;
-            }
-            int4 nx[kPullIlp];
-#pragma unroll
-            for (int r = 0; r < kPullIlp; ++r) {
-                beg[r] = mine[r] ? __ldg(a.in_ptr + i[r]) : 0;
-                end[r] = mine[r] ? __ldg(a.in_ptr + i[r] + 1) : 0;
-                par[r] = (mine[r] && (!two_pass || found1[r])) ? __ldg(a.first_in + i[r]) : -1;
-                nx[r] = mine[r] ? __ldg(a.next_in + i[r]) : make_int4(-1, -1, -1, -1);
-            }
-#pragma unroll
-            for (int r = 0; r < kPullIlp; ++r) {
-                k[r] = beg[r] + 1;  // the first in-neighbour is examined (by pass 1, or right here)
-                if (!two_pass && mine[r]) {
-                    exam[r] = 1;
-                    if (bit_test(tbm, par[r])) {  // a candidate has in-edges: par holds its first
-                        found[r] = true;
-                        done[r] = a.early_exit != 0;
-                    } else {
+                const uint32_t need = __ballot_sync(0xffffffffu, i[r] < 0);
+                bool fresh = false;
+                if (need != 0u && nxt < total) {
+                    const uint32_t c = nxt + __popc(need & lanemask_lt());
+                    fresh = i[r] < 0 && c < total;
+                    const int off = fresh ? (int)clist[c] : 0;
+                    const uint32_t f1j = __shfl_sync(0xffffffffu, f1, off >> 5);
+                    nxt += __popc(need);
+                    if (fresh) {
+                        i[r] = ((tile * tw) << 5) + off;
                         par[r] = -1;
+                        known[r] = (f1j >> (off & 31)) & 1u;
                     }
                 }
-            }
-            // in-neighbours 1..4 from the dense next-entries array (one 16-byte load, four probes
-            // in flight); the first hit in row order is the parent
+                live |= i[r] >= 0;
+                f0[r] = -1;
 #pragma unroll
-            for (int r = 0; r < kPullIlp; ++r) {
-                if (!mine[r] || done[r]) continue;
-                const bool h0 = nx[r].x >= 0 && bit_test(tbm, nx[r].x);
-                const bool h1 = nx[r].y >= 0 && bit_test(tbm, nx[r].y);
-                const bool h2 = nx[r].z >= 0 && bit_test(tbm, nx[r].z);
-                const bool h3 = nx[r].w >= 0 && bit_test(tbm, nx[r].w);
-                const int nv = (nx[r].x >= 0) + (nx[r].y >= 0) + (nx[r].z >= 0) + (nx[r].w >= 0);
-                const int hit = h0 ? 0 : (h1 ? 1 : (h2 ? 2 : (h3 ? 3 : -1)));
-                if (hit >= 0 && !found[r]) {
-                    found[r] = true;
-                    par[r] = hit == 0 ? nx[r].x : (hit == 1 ? nx[r].y : (hit == 2 ? nx[r].z : nx[r].w));
-                }
-                const bool stop = hit >= 0 && a.early_exit;
-                const int used = stop ? hit + 1 : nv;
-                exam[r] += (unsigned long long)used;
-                k[r] += used;
-                done[r] = stop;
-            }
-            // lane probes: up to a.probe in-neighbours per row, kPullStep at a time, both rows in lockstep
-            for (int it = 0; it < (a.probe + kPullStep - 1) / kPullStep; ++it) {
-                int32_t jj[kPullIlp][kPullStep];
-                int32_t cnt[kPullIlp];
-                bool act[kPullIlp];
-#pragma unroll
-                for (int r = 0; r < kPullIlp; ++r) {
+                for (int t = 0; t < 4; ++t) x[r][t] = -1;
+                if (fresh) {
+                    const int4 nx = ld_stream(a.next_in + i[r]);
+                    x[r][0] = nx.x;
+                    x[r][1] = nx.y;
+                    x[r][2] = nx.z;
+                    x[r][3] = nx.w;
+                    beg[r] = __ldg(a.in_ptr + i[r]);
+                    end[r] = __ldg(a.in_ptr + i[r] + 1);
+                    if (!two_pass || known[r]) f0[r] = __ldg(a.first_in + i[r]);
+                    k[r] = beg[r] + 1;  // the first in-neighbour is examined (by pass 1, or right here)
+                } else if (i[r] >= 0) {
                     const int32_t lim = end[r] < beg[r] + a.probe ? end[r] : beg[r] + a.probe;
-                    act[r] = mine[r] && !done[r] && k[r] < lim;
-                    cnt[r] = act[r] ? (lim - k[r] < kPullStep ? lim - k[r] : kPullStep) : 0;
 #pragma unroll
-                    for (int t = 0; t < kPullStep; ++t) jj[r][t] = t < cnt[r] ? __ldg(a.in_col + k[r] + t) : 0;
-                }
-                bool any = false;
-#pragma unroll
-                for (int r = 0; r < kPullIlp; ++r) any |= act[r];
-                if (!any) break;
-#pragma unroll
-                for (int r = 0; r < kPullIlp; ++r) {
-                    if (!act[r]) continue;
-                    int hit = -1;
-#pragma unroll
-                    for (int t = kPullStep - 1; t >= 0; --t)
-                        if (t < cnt[r] && bit_test(tbm, jj[r][t])) hit = t;
-                    if (hit >= 0 && !found[r]) {
-                        found[r] = true;
-                        par[r] = jj[r][0];
-#pragma unroll
-                        for (int t = 1; t < kPullStep; ++t)
-                            if (hit == t) par[r] = jj[r][t];
-                        if (a.early_exit) {
-                            exam[r] += (unsigned long long)(hit + 1);
-                            k[r] += hit + 1;
-                            done[r] = true;
-                            continue;
-                        }
-                    }
-                    exam[r] += (unsigned long long)cnt[r];
-                    k[r] += cnt[r];
+                    for (int t = 0; t < 4; ++t) x[r][t] = k[r] + t < lim ? ld_stream(a.in_col + k[r] + t) : -1;
                 }
             }
-            // rows longer than the lane probe: the whole warp scans them (32, then 128 edges a step),
-            // or lists them for the grid-wide phase when more than kPullHugeRow are left
+            if (!__any_sync(0xffffffffu, live)) break;
+            bool hit0[kPullIlp];
+            int hit[kPullIlp], nv[kPullIlp];
+#pragma unroll
+            for (int r = 0; r < kPullIlp; ++r) {  // every probe of the step in flight before the first is used
+                hit0[r] = !two_pass && f0[r] >= 0 && bit_test(tbm, f0[r]);
+                bool h[4];
+                nv[r] = 0;
+#pragma unroll
+                for (int t = 0; t < 4; ++t) {
+                    h[t] = x[r][t] >= 0 && bit_test(tbm, x[r][t]);
+                    nv[r] += x[r][t] >= 0 ? 1 : 0;
+                }
+                hit[r] = h[0] ? 0 : (h[1] ? 1 : (h[2] ? 2 : (h[3] ? 3 : -1)));
+            }
 #pragma unroll
             for (int r = 0; r < kPullIlp; ++r) {
-                uint32_t pend = __ballot_sync(0xffffffffu, mine[r] && !done[r] && k[r] < end[r]);
+                bool done = false;
+                if (i[r] >= 0) {
+                    if (f0[r] >= 0) {  // a new row: its first in-neighbour
+                        if (!two_pass) acc.exam += 1;
+                        if (hit0[r] || known[r]) par[r] = f0[r];
+                        done = hit0[r] && a.early_exit;
+                    }
+                    if (!done) {
+                        if (hit[r] >= 0 && par[r] < 0)
+                            par[r] = hit[r] == 0 ? x[r][0] : (hit[r] == 1 ? x[r][1] : (hit[r] == 2 ? x[r][2] : x[r][3]));
+                        done = hit[r] >= 0 && a.early_exit;
+                        const int used = done ? hit[r] + 1 : nv[r];
+                        acc.exam += (uint32_t)used;
+                        k[r] += used;
+                    }
+                }
+                // rows longer than the lane probe: the whole warp scans them (32, then 128 edges a step),
+                // or lists them for the grid-wide phase when more than kPullHugeRow are left
+                uint32_t pend =
+                    __ballot_sync(0xffffffffu, i[r] >= 0 && !done && k[r] >= beg[r] + a.probe && k[r] < end[r]);
                 while (pend) {
                     const int t = __ffs(pend) - 1;
                     pend &= pend - 1;
                     int32_t kk = __shfl_sync(0xffffffffu, k[r], t);
                     const int32_t ee = __shfl_sync(0xffffffffu, end[r], t);
-                    bool tf = __shfl_sync(0xffffffffu, found[r], t);
                     int32_t tp = __shfl_sync(0xffffffffu, par[r], t);
-                    unsigned long long tx = 0;
+                    uint32_t tx = 0;
                     if (kHuge && ee - kk > kPullHugeRow) {
                         const int32_t row = __shfl_sync(0xffffffffu, i[r], t);
                         if (lane == 0) {
                             const unsigned long long nch = (unsigned long long)((ee - kk + kPullChunk - 1) / kPullChunk);
                             const unsigned long long old = atomicAdd(&st.cout->huge, (nch << 32) | 1ull);
                             const uint32_t slot = (uint32_t)old;
-                            hr.row[slot] = tf ? ~row : row;
+                            hr.row[slot] = tp >= 0 ? ~row : row;
                             hr.k[slot] = kk;
                             hr.base[slot] = (int32_t)(old >> 32);
                             hr.first[slot] = INT32_MAX;
@@ -551,30 +522,29 @@ __device__ __forceinline__ void pull_level(const BfsArgs& a, int32_t L, int vcur
                         const int pos = step == 32 ? warp_scan<1>(a.in_col, tbm, kk, ee, &jf)
                                                    : warp_scan<4>(a.in_col, tbm, kk, ee, &jf);
                         if (pos < step) {
-                            if (!tf) {
-                                tf = true;
-                                tp = jf;
-                            }
+                            if (tp < 0) tp = jf;
                             if (a.early_exit) {
-                                tx += (unsigned long long)(pos + 1);
+                                tx += (uint32_t)(pos + 1);
                                 break;
                             }
                         }
-                        tx += (unsigned long long)(ee - kk < step ? ee - kk : step);
+                        tx += (uint32_t)(ee - kk < step ? ee - kk : step);
                     }
                     if (lane == t) {
-                        found[r] = tf;
                         par[r] = tp;
-                        exam[r] += tx;
+                        acc.exam += tx;
+                        done = true;
                     }
                 }
-            }
-#pragma unroll
-            for (int r = 0; r < kPullIlp; ++r) {
+                done |= i[r] >= 0 && k[r] >= end[r];
                 // new: found here, not by pass 1, and not visited before (rows without masking may be)
-                const bool isnew = found[r] && !found1[r] && !((cwj[r] >> bitpos[r]) & 1u);
+                bool isnew = done && par[r] >= 0 && !known[r];
+                if (!a.masking) {
+                    const uint32_t cwj = __shfl_sync(0xffffffffu, cw, isnew ? (i[r] >> 5) - tile * tw : 0);
+                    isnew = isnew && !((cwj >> (i[r] & 31)) & 1u);
+                }
                 if (isnew) {
-                    atomicOr(snew + jw[r], 1u << bitpos[r]);
+                    atomicOr(snew + ((i[r] >> 5) - tile * tw), 1u << (i[r] & 31));
                     a.depth[i[r]] = L + 1;
                     if (a.parent) a.parent[i[r]] = par[r];
                     const int32_t od = a.symmetric ? end[r] - beg[r]
@@ -583,8 +553,8 @@ __device__ __forceinline__ void pull_level(const BfsArgs& a, int32_t L, int vcur
                     acc.mf += (uint32_t)od;
                     acc.indeg += (uint32_t)(end[r] - beg[r]);
                 }
-                acc.exam += exam[r];
                 if (append) st.put(isnew, i[r]);
+                if (done) i[r] = -1;
             }
         }
         __syncwarp();

@@ -253,6 +253,33 @@ __device__ __forceinline__ unsigned long long ld_volatile_u64(const unsigned lon
     return *(const volatile unsigned long long*)p;
 }
 
+// Loads of arrays that are read once, kept out of L1 so that what is gathered beside them stays
+// there.
+__device__ __forceinline__ int32_t ld_stream(const int32_t* p) {
+    int32_t v;
+    asm("ld.global.nc.L1::no_allocate.s32 %0, [%1];" : "=r"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ float ld_stream(const float* p) {
+    float v;
+    asm("ld.global.nc.L1::no_allocate.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ int4 ld_stream(const int4* p) {
+    int4 v;
+    asm("ld.global.nc.L1::no_allocate.v4.s32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+                 : "l"(p));
+    return v;
+}
+__device__ __forceinline__ float4 ld_stream(const float4* p) {
+    float4 v;
+    asm("ld.global.nc.L1::no_allocate.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+                 : "l"(p));
+    return v;
+}
+
 // atomic min of a binary32 value: non-negative floats order like their int bits
 // and negative ones in reverse of their unsigned bits, so the two halves use
 // atomicMin (int) and atomicMax (unsigned).  Returns the previous value.  NaN is

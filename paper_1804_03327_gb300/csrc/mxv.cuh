@@ -39,21 +39,13 @@ struct PullSmem {
     int nlong, hit;
 };
 
-// Bitmap words a warp takes at a time, 32 .. 4: the width whose round-robin critical path
-// over the grid's warps is shortest (ties: the wider).  A tile of 32 words (1,024 rows)
-// leaves most of 9,728 warps without any on a graph of a million rows.
+// Bitmap words a warp takes at a time: an even share of the words over as many rounds as 32
+// words a warp need.  Tiles of 32 words (1,024 rows) leave most warps without any on a graph
+// of a million rows.
 inline int32_t mxv_tile_words(int32_t nwords, long long nwarps) {
-    int32_t best = 32;
-    long long best_cost = -1;
-    for (int32_t tw = 32; tw >= 4; tw >>= 1) {
-        const long long tiles = ((long long)nwords + tw - 1) / tw;
-        const long long cost = (tiles + nwarps - 1) / nwarps * tw;
-        if (best_cost < 0 || cost < best_cost) {
-            best = tw;
-            best_cost = cost;
-        }
-    }
-    return best;
+    const long long rounds = (nwords + 32 * nwarps - 1) / (32 * nwarps);
+    const long long tw = (nwords + nwarps * rounds - 1) / (nwarps * rounds);
+    return (int32_t)(tw < 2 ? 2 : tw);
 }
 
 // The row-based matvec alone (mxv.cu), for the allocation-free entry point; kMxvThreads a block.
