@@ -20,7 +20,8 @@
 namespace gbx {
 
 constexpr int kMpUnroll = 4;          // entries a lane has in flight
-constexpr int32_t kMpChunk = 1024;    // entries of a deferred row a warp takes at a time
+constexpr int32_t kMpChunk = 512;     // entries of a deferred row a warp takes at a time
+constexpr int32_t kMpLongSteps = 4;   // steps left beyond which a row is deferred
 
 struct MpArgs {
     int32_t n, nwords;
@@ -61,6 +62,7 @@ __device__ __forceinline__ Stage mp_stage(const MpArgs& a, StageBuf* sb, Acc* ac
 // The mask as a bitmap; u's finite entries as the push queue (dir == PUSH) or as a bitmap and
 // their number (AUTO); w = +inf where a push without accumulation starts from that.
 __global__ void __launch_bounds__(kMxvThreads) mp_prep_kernel(const __grid_constant__ MpArgs a) {
+    pdl_begin();
     __shared__ StageBuf sb[kMxvThreads / 32];
     __shared__ unsigned long long bsm[kMxvThreads / 32];
     __shared__ unsigned long long csm[kMxvThreads / 32][4];
@@ -137,21 +139,22 @@ __device__ __forceinline__ void mp_push(const MpArgs& a) {
 
 // Pull: groups of a.group lanes take a row each, kMpUnroll entries a lane in flight, and go on to
 // the next row as soon as their own is done.  A warp's row offsets come 32 rows at a time,
-// the next 32 loaded ahead.  A row with more than 64 steps left is deferred: mp_last_kernel
-// spreads its chunks over all warps.
+// the next 32 loaded ahead.  A row with more than kMpLongSteps left is deferred:
+// mp_last_kernel spreads its chunks over all warps.
 //
 // Bound by the gathers of u (4 bytes of a 32-byte L2 sector per entry).  A lane per row of up to
 // 32 entries, one load at a time, and a warp for each longer row had taken 316 us on a
 // directed graph of 700,001 rows and 11.2M entries whose longest rows hold tens of thousands
-// (the whole call 358 us, now 141).  The group is 8 lanes from 12 entries a row on, 4 from 6, else 1: rows shorter
+// (the whole call 358 us, now 93; rows deferred after 8 steps 95, after 16 102, after 64
+// 132).  The group is 8 lanes from 12 entries a row on, 4 from 6, else 1: rows shorter
 // than the group's step leave lanes idle, longer ones take several dependent steps.
-__device__ __forceinline__ void mp_pull(const MpArgs& a) {
+__device__ __forceinline__ void mp_pull(const MpArgs& a, uint8_t* list) {
     const int lane = threadIdx.x & 31;
     const int G = a.group, sub = lane & (G - 1), first = lane & ~(G - 1);
     const int32_t nwarps = (int32_t)((gridDim.x * kMxvThreads) >> 5);
     const int32_t ntiles = a.nwords;
     int32_t tile = (int32_t)((blockIdx.x * kMxvThreads + threadIdx.x) >> 5);
-    const int32_t kLong = 64 * kMpUnroll * G;
+    const int32_t kLong = kMpLongSteps * kMpUnroll * G;
     // a tile's rows: lane l holds row 32 tile + l
     auto load = [&](int32_t t, int32_t& b, int32_t& e) {
         const int64_t i = ((int64_t)t << 5) + lane;
@@ -164,44 +167,44 @@ __device__ __forceinline__ void mp_pull(const MpArgs& a) {
     int32_t b0, e0, b1, e1;
     load(tile, b0, e0);
     load(tile + nwarps, b1, e1);
-    int32_t base = -1;   // first row of the tile in b0 / e0 that is being handed out
-    uint32_t open = 0;   // its rows not yet handed out
+    int32_t base = -1;        // first row of the tile in b0 / e0
+    int open = 0, next = 0;   // its rows with entries (list: their lanes), and how many are handed out
+    bool fresh = true;        // the tile has not been looked at
     int32_t v = -1, k = 0, end = 0;
     float m = INFINITY;
     for (;;) {
         const uint32_t need = __ballot_sync(0xffffffffu, v < 0 && sub == 0);
-        if (need && !open && tile < ntiles) {  // the next tile; its rows without entries are settled here
-            open = __ballot_sync(0xffffffffu, e0 > b0);
-            base = tile << 5;
-            if (e0 == b0 && base + lane < a.n && !a.accum) a.w[base + lane] = INFINITY;
-        }
-        if (need && open) {
-            // the r-th group without a row takes the r-th open one
-            const int r = __popc(need & ((1u << first) - 1u));
-            const int nth = (int)__fns(open, 0, r + 1);
-            const bool got = v < 0 && nth >= 0 && nth < 32;
-            const int32_t nb = __shfl_sync(0xffffffffu, b0, got ? nth : 0);
-            const int32_t ne = __shfl_sync(0xffffffffu, e0, got ? nth : 0);
-            const uint32_t taken = __ballot_sync(0xffffffffu, got && sub == 0);
-            if (got) {
-                v = base + nth;
-                k = nb;
-                end = ne;
-                m = INFINITY;
-            }
-            for (int c = __popc(taken); c > 0; --c) open &= open - 1;
-            if (!open) {
+        if (need && next == open && tile < ntiles) {
+            if (!fresh) {
                 tile += nwarps;
                 b0 = b1;
                 e0 = e1;
                 load(tile + nwarps, b1, e1);
             }
-        } else if (need && tile < ntiles) {  // a tile without open rows
-            tile += nwarps;
-            b0 = b1;
-            e0 = e1;
-            load(tile + nwarps, b1, e1);
-            if (__popc(need) * G == 32) continue;
+            fresh = false;
+            base = tile << 5;
+            const uint32_t with = __ballot_sync(0xffffffffu, e0 > b0);  // none past the last tile
+            __syncwarp();
+            if (e0 > b0) list[__popc(with & lanemask_lt())] = (uint8_t)lane;
+            __syncwarp();
+            open = __popc(with);
+            next = 0;
+            // rows without entries (or that do not pass) are settled here
+            if (tile < ntiles && e0 == b0 && base + lane < a.n && !a.accum) a.w[base + lane] = INFINITY;
+        }
+        if (need && next < open) {
+            const int r = next + __popc(need & ((1u << first) - 1u));  // the group's place among those without a row
+            const bool got = v < 0 && r < open;
+            const int from = got ? (int)list[r] : 0;
+            const int32_t nb = __shfl_sync(0xffffffffu, b0, from);
+            const int32_t ne = __shfl_sync(0xffffffffu, e0, from);
+            if (got) {
+                v = base + from;
+                k = nb;
+                end = ne;
+                m = INFINITY;
+            }
+            next = min(open, next + __popc(need));
         }
         if (__ballot_sync(0xffffffffu, v >= 0) == 0u) {
             if (tile >= ntiles) break;
@@ -252,10 +255,11 @@ __device__ __forceinline__ void mp_pull(const MpArgs& a) {
 
 // Pull, push, or -- AUTO found u sparse -- the queue (and w = +inf) for mp_push_kernel.
 __global__ void __launch_bounds__(kMxvThreads, 6) mp_main_kernel(const __grid_constant__ MpArgs a) {
+    pdl_begin();
     __shared__ StageBuf sb[kMxvThreads / 32];
     __shared__ unsigned long long bsm[kMxvThreads / 32];
     if (mp_dir(a) == GBX_DIR_PULL) {
-        mp_pull(a);
+        mp_pull(a, reinterpret_cast<uint8_t*>(sb + (threadIdx.x >> 5)));
     } else if (a.dir == GBX_DIR_PUSH) {
         mp_push(a);
     } else {
@@ -280,11 +284,13 @@ __global__ void __launch_bounds__(kMxvThreads, 6) mp_main_kernel(const __grid_co
 }
 
 __global__ void __launch_bounds__(kMxvThreads) mp_push_kernel(const __grid_constant__ MpArgs a) {
+    pdl_begin();
     if (mp_dir(a) == GBX_DIR_PUSH) mp_push(a);
 }
 
 // The chunks of the rows a pull deferred, and the scratch left zero for the next call.
 __global__ void __launch_bounds__(kMxvThreads) mp_last_kernel(const __grid_constant__ MpArgs a) {
+    pdl_begin();
     const int lane = threadIdx.x & 31;
     const int64_t gtid = (int64_t)blockIdx.x * kMxvThreads + threadIdx.x, gs = (int64_t)gridDim.x * kMxvThreads;
     const unsigned long long huge = a.ctr->huge;
@@ -356,13 +362,12 @@ gbx_status mxv_minplus(Graph* G, float* w, const MxvVec& mask, const float* u, c
     const unsigned small = std::max(1u, std::min(div_up(a.n, kMxvThreads), (unsigned)G->num_sms * 4u));
     GBX_TRY(mxv_scratch(G, s));
     G->ws.mx_dirty = true;  // until every kernel of the call is issued
-    mp_prep_kernel<<<small, kMxvThreads, 0, s>>>(a);
+    GBX_TRY(pdl_launch(mp_prep_kernel, small, a, false, s));
     if (!a.nothing) {
-        mp_main_kernel<<<grid, kMxvThreads, 0, s>>>(a);
-        if (a.dir == GBX_DIR_AUTO) mp_push_kernel<<<grid, kMxvThreads, 0, s>>>(a);
+        GBX_TRY(pdl_launch(mp_main_kernel, grid, a, true, s));
+        if (a.dir == GBX_DIR_AUTO) GBX_TRY(pdl_launch(mp_push_kernel, grid, a, true, s));
     }
-    mp_last_kernel<<<small, kMxvThreads, 0, s>>>(a);
-    GBX_CUDA_TRY(cudaGetLastError());
+    GBX_TRY(pdl_launch(mp_last_kernel, small, a, true, s));
     G->ws.mx_dirty = false;
     return GBX_OK;
 }

@@ -17,9 +17,9 @@
 // with its degree prefix; mxv_main_kernel pulls or pushes, by a decision each block takes
 // from the count of u; the output kernels write w and leave the scratch bitmaps zero for the
 // next call.  A small call is bound by its launches: the separate conversions, scans and
-// decisions of 17 captured launches took 42 us for a sparse step of 100 vertices on RMAT-20
-// (and a capture for every new set of buffers); now 22 us, launched directly (a first
-// call on new buffers 172 -> 55 us).
+// decisions of 17 captured launches took 38 us for a sparse step of 100 vertices on RMAT-20
+// (and a capture for every new set of buffers); now 16 us, launched directly (a first
+// call on new buffers 154 -> 46 us).
 #include <algorithm>
 
 #include "frontier.cuh"
@@ -29,20 +29,21 @@
 namespace gbx {
 
 constexpr int kMxvProbe = 16;
-constexpr int kMxvLaneRow = 32;
 
 // Row-based matvec over the rows the mask lets through (Eq 2 / Eq 4).  A warp
-// takes a tile of a.tile_words result words (at most 32: 1,024 rows), lists the passing nonempty rows in
-// shared memory (each lane its word's rows, at its prefix of the words' counts)
-// and computes them 64 per round, two rows per lane probing in lockstep: the
-// first entry of a row comes from the dense first-entry array when one is given
-// (one coalesced read instead of a random sector), entries 1..4 from the dense
-// next-entries array (one 16-byte read), then up to kMxvProbe entries four at a
-// time; longer rows are finished by the whole warp 128 entries at a time, and those
-// with more than kMxvLongRow left by the whole block after its tiles.  With
-// early exit a row stops at its first hit (Section 5.3); the result is the same
-// either way.
-constexpr int kMxvIlp = 2;
+// takes a tile of a.tile_words result words (at most 32: 1,024 rows) and lists the
+// passing nonempty rows in shared memory (each lane its word's rows, at its prefix of
+// the words' counts).  A fuller tile first tests every row's entry 0 from the dense
+// first-entry array (one coalesced read instead of a random sector); then a lane takes
+// a row at a time: entries 1..4 from the dense next-entries array (one 16-byte read),
+// then up to kMxvProbe entries four at a time.  Longer rows are finished by the whole
+// warp 128 entries at a time, and those with more than kMxvLongRow left by the whole
+// block after its tiles.  With early exit a row stops at its first hit (Section 5.3); the
+// result is the same either way.
+//
+// Bound by dependent gathers: RMAT-22 with half its rows masked and a fifth of its vertices in
+// u reads 124 MB.  Rounds of 64 rows in lockstep took as long as their slowest row: the
+// call 59.7 us, now 51.3 (and 102.6 with 17 launches and tiles of 32 words).
 constexpr int kMxvP1 = 4;  // first-pass rows per lane per round
 
 // The rows of a tile whose bits are set in the lane words m (lane l: word l), in
@@ -124,7 +125,7 @@ __device__ __forceinline__ void mxv_pull(const PullArgs& a, PullSmem& sm) {
         const uint32_t cnt0 = __popc(cand0);
         const uint32_t incl0 = warp_inclusive_sum(cnt0);
         const uint32_t total0 = __shfl_sync(0xffffffffu, incl0, 31);
-        const bool two_pass = first != nullptr && total0 > 32u * kMxvIlp;
+        const bool two_pass = first != nullptr && total0 > 64u;
         if (two_pass) {
             mxv_tile_list(list, cand0, incl0 - cnt0);
             for (uint32_t base = 0; base < total0; base += 32 * kMxvP1) {
@@ -153,153 +154,123 @@ __device__ __forceinline__ void mxv_pull(const PullArgs& a, PullSmem& sm) {
         const uint32_t incl = warp_inclusive_sum(cntw);
         const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);
         if (total) mxv_tile_list(list, cand, incl - cntw);
-        for (uint32_t base = 0; base < total; base += 32 * kMxvIlp) {
-            bool mine[kMxvIlp], found[kMxvIlp], done[kMxvIlp];
-            int jw[kMxvIlp], bitpos[kMxvIlp];
-            uint32_t f1w[kMxvIlp];
-            int32_t k[kMxvIlp], end[kMxvIlp], beg[kMxvIlp], f0[kMxvIlp];
-#pragma unroll
-            for (int r = 0; r < kMxvIlp; ++r) {
-                const uint32_t c = base + 32 * r + lane;
-                mine[r] = c < total;
-                const int off = mine[r] ? (int)list[c] : 0;
-                const int j = off >> 5;
-                jw[r] = j;
-                f1w[r] = __shfl_sync(0xffffffffu, f1, j);
-                bitpos[r] = off & 31;
-                found[r] = false;
-                done[r] = false;
-            }
-            int4 nx[kMxvIlp];
-#pragma unroll
-            for (int r = 0; r < kMxvIlp; ++r) {
-                const int32_t i = ((w0 + jw[r]) << 5) + bitpos[r];
-                beg[r] = mine[r] ? ptr[i] : 0;
-                end[r] = mine[r] ? ptr[i + 1] : 0;
-                f0[r] = (mine[r] && !two_pass) ? (first ? first[i] : -2) : -1;
-                nx[r] = (mine[r] && next) ? next[i] : make_int4(-1, -1, -1, -1);
-            }
-#pragma unroll
-            for (int r = 0; r < kMxvIlp; ++r) {
-                if (!mine[r]) continue;
-                k[r] = beg[r] + 1;
-                if (two_pass) {  // the first entry was examined (and counted) by the first pass
-                    found[r] = (f1w[r] >> bitpos[r]) & 1u;  // only without early exit can it be set here
-                    continue;
-                }
-                rows += 1;
-                if (f0[r] == -2) f0[r] = col[beg[r]];  // no first-entry array: read the row's first entry
-                exam += 1;
-                if (bit_test(ubm, f0[r])) {
-                    found[r] = true;
-                    done[r] = early_exit != 0;
+        // a row per lane, each lane going on to the next one as soon as its row is settled
+        uint32_t nxt = 0;  // rows of the list handed out
+        int32_t i = -1, beg = 0, end = 0, k = 0;
+        bool found = false;
+        for (;;) {
+            const uint32_t need = __ballot_sync(0xffffffffu, i < 0);
+            int32_t x[4] = {-1, -1, -1, -1}, f0 = -1;
+            bool fresh = false;
+            if (need != 0u && nxt < total) {
+                const uint32_t c = nxt + __popc(need & lanemask_lt());
+                fresh = i < 0 && c < total;
+                const int off = fresh ? (int)list[c] : 0;
+                const uint32_t f1j = __shfl_sync(0xffffffffu, f1, off >> 5);
+                nxt += __popc(need);
+                if (fresh) {
+                    i = (w0 << 5) + off;
+                    found = two_pass && ((f1j >> (off & 31)) & 1u);  // only without early exit can it be set here
                 }
             }
-            // entries 1..4 from the dense next-entries array (one 16-byte read, four probes in flight)
-#pragma unroll
-            for (int r = 0; r < kMxvIlp; ++r) {
-                if (!mine[r] || done[r] || !next) continue;
-                const bool h0 = nx[r].x >= 0 && bit_test(ubm, nx[r].x);
-                const bool h1 = nx[r].y >= 0 && bit_test(ubm, nx[r].y);
-                const bool h2 = nx[r].z >= 0 && bit_test(ubm, nx[r].z);
-                const bool h3 = nx[r].w >= 0 && bit_test(ubm, nx[r].w);
-                const int nv = (nx[r].x >= 0) + (nx[r].y >= 0) + (nx[r].z >= 0) + (nx[r].w >= 0);
-                const int hit = h0 ? 0 : (h1 ? 1 : (h2 ? 2 : (h3 ? 3 : -1)));
-                if (hit >= 0) found[r] = true;
-                const bool stop = hit >= 0 && early_exit;
-                const int used = stop ? hit + 1 : nv;
-                exam += (unsigned long long)used;
-                k[r] += used;
-                done[r] = stop;
-            }
-            // a lane scans rows of up to kMxvLaneRow entries itself; longer rows get kMxvProbe
-            // entries here and the rest from the whole warp below
-            while (true) {
-                int32_t jj[kMxvIlp][4];
-                int32_t cnt[kMxvIlp];
-                bool act[kMxvIlp];
-#pragma unroll
-                for (int r = 0; r < kMxvIlp; ++r) {
-                    const int32_t span = end[r] - beg[r] <= kMxvLaneRow ? kMxvLaneRow : kMxvProbe;
-                    const int32_t lim = end[r] < beg[r] + span ? end[r] : beg[r] + span;
-                    act[r] = mine[r] && !done[r] && k[r] < lim;
-                    cnt[r] = act[r] ? (lim - k[r] < 4 ? lim - k[r] : 4) : 0;
-#pragma unroll
-                    for (int t = 0; t < 4; ++t) jj[r][t] = t < cnt[r] ? col[k[r] + t] : 0;
+            if (!__any_sync(0xffffffffu, i >= 0)) break;
+            if (fresh) {
+                beg = __ldg(ptr + i);
+                end = __ldg(ptr + i + 1);
+                if (next) {
+                    const int4 nx = ld_stream(next + i);
+                    x[0] = nx.x;
+                    x[1] = nx.y;
+                    x[2] = nx.z;
+                    x[3] = nx.w;
                 }
-                if (!__any_sync(0xffffffffu, act[0] || act[1])) break;
+                k = beg + 1;
+                if (!two_pass) {
+                    rows += 1;
+                    exam += 1;
+                    f0 = first ? __ldg(first + i) : __ldg(col + beg);
+                }
+            }
+            if (i >= 0 && !(fresh && next)) {
+                const int32_t lim = end < beg + kMxvProbe ? end : beg + kMxvProbe;
 #pragma unroll
-                for (int r = 0; r < kMxvIlp; ++r) {
-                    if (!act[r]) continue;
-                    int hit = -1;
+                for (int t = 0; t < 4; ++t) x[t] = k + t < lim ? ld_stream(col + k + t) : -1;
+            }
+            const bool hit0 = f0 >= 0 && bit_test(ubm, f0);
+            bool h[4];
+            int nv = 0;
 #pragma unroll
-                    for (int t = 3; t >= 0; --t)
-                        if (t < cnt[r] && bit_test(ubm, jj[r][t])) hit = t;
-                    if (hit >= 0) {
-                        found[r] = true;
-                        if (early_exit) {
-                            exam += (unsigned long long)(hit + 1);
-                            k[r] += hit + 1;
-                            done[r] = true;
-                            continue;
-                        }
+            for (int t = 0; t < 4; ++t) {
+                h[t] = x[t] >= 0 && bit_test(ubm, x[t]);
+                nv += x[t] >= 0 ? 1 : 0;
+            }
+            bool done = false;
+            if (i >= 0) {
+                found |= hit0;
+                done = hit0 && early_exit;
+                if (!done) {
+                    const int hit = h[0] ? 0 : (h[1] ? 1 : (h[2] ? 2 : (h[3] ? 3 : -1)));
+                    found |= hit >= 0;
+                    done = hit >= 0 && early_exit;
+                    const int used = done ? hit + 1 : nv;
+                    exam += (unsigned long long)used;
+                    k += used;
+                }
+                done |= k >= end;
+            }
+            // past the lane probe: the whole warp, or the whole block once its tiles are done
+            const bool past = i >= 0 && !done && k >= beg + kMxvProbe;
+            if (past && end - k > kMxvLongRow) {
+                const int slot = atomicAdd(&sm.nlong, 1);
+                if (slot < kMxvLongs) {
+                    sm.longs[slot] = make_int2(i, k);
+                    done = true;  // a found row keeps its bit
+                }
+            }
+            uint32_t pend = __ballot_sync(0xffffffffu, past && !done);
+            while (pend) {
+                const int t = __ffs(pend) - 1;
+                pend &= pend - 1;
+                int32_t kk = __shfl_sync(0xffffffffu, k, t);
+                const int32_t ee = __shfl_sync(0xffffffffu, end, t);
+                bool tf = __shfl_sync(0xffffffffu, found, t);
+                unsigned long long tx = 0;
+                // 128 entries per round (four independent loads per lane)
+                for (; kk < ee; kk += 128) {
+                    int32_t jq[4];
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        const int32_t idx = kk + 32 * q + lane;
+                        jq[q] = idx < ee ? col[idx] : -1;
                     }
-                    exam += (unsigned long long)cnt[r];
-                    k[r] += cnt[r];
-                }
-            }
+                    bool stop = false;
 #pragma unroll
-            for (int r = 0; r < kMxvIlp; ++r) {
-                if (mine[r] && !done[r] && end[r] - k[r] > kMxvLongRow) {
-                    // left to the whole block once its tiles are done (a found row keeps its bit
-                    // from the probe)
-                    const int slot = atomicAdd(&sm.nlong, 1);
-                    if (slot < kMxvLongs) {
-                        sm.longs[slot] = make_int2(((w0 + jw[r]) << 5) + bitpos[r], k[r]);
-                        done[r] = true;
-                    }
-                }
-                uint32_t pend = __ballot_sync(0xffffffffu, mine[r] && !done[r] && k[r] < end[r]);
-                while (pend) {
-                    const int t = __ffs(pend) - 1;
-                    pend &= pend - 1;
-                    int32_t kk = __shfl_sync(0xffffffffu, k[r], t);
-                    const int32_t ee = __shfl_sync(0xffffffffu, end[r], t);
-                    bool tf = __shfl_sync(0xffffffffu, found[r], t);
-                    unsigned long long tx = 0;
-                    // 128 entries per round (four independent loads per lane)
-                    for (; kk < ee; kk += 128) {
-                        int32_t jq[4];
-#pragma unroll
-                        for (int q = 0; q < 4; ++q) {
-                            const int32_t idx = kk + 32 * q + lane;
-                            jq[q] = idx < ee ? col[idx] : -1;
-                        }
-                        bool stop = false;
-#pragma unroll
-                        for (int q = 0; q < 4; ++q) {
-                            if (stop) break;
-                            const uint32_t hb = __ballot_sync(0xffffffffu, jq[q] >= 0 && bit_test(ubm, jq[q]));
-                            const int32_t left = ee - (kk + 32 * q);
-                            if (left <= 0) break;
-                            if (hb) {
-                                tf = true;
-                                if (early_exit) {
-                                    tx += (unsigned long long)__ffs(hb);
-                                    stop = true;
-                                    break;
-                                }
-                            }
-                            tx += (unsigned long long)(left < 32 ? left : 32);
-                        }
+                    for (int q = 0; q < 4; ++q) {
                         if (stop) break;
+                        const uint32_t hb = __ballot_sync(0xffffffffu, jq[q] >= 0 && bit_test(ubm, jq[q]));
+                        const int32_t left = ee - (kk + 32 * q);
+                        if (left <= 0) break;
+                        if (hb) {
+                            tf = true;
+                            if (early_exit) {
+                                tx += (unsigned long long)__ffs(hb);
+                                stop = true;
+                                break;
+                            }
+                        }
+                        tx += (unsigned long long)(left < 32 ? left : 32);
                     }
-                    if (lane == t) {
-                        found[r] = tf;
-                        exam += tx;
-                    }
+                    if (stop) break;
                 }
-                if (found[r]) atomicOr(hits + jw[r], 1u << bitpos[r]);
+                if (lane == t) {
+                    found = tf;
+                    exam += tx;
+                    done = true;
+                }
+            }
+            if (done) {
+                if (found) atomicOr(hits + ((i >> 5) - w0), 1u << (i & 31));
+                i = -1;
             }
         }
         __syncwarp();
@@ -375,6 +346,7 @@ __device__ __forceinline__ void mxv_stage_words(Stage& st, uint32_t mine, int32_
 }
 
 __global__ void __launch_bounds__(kMxvThreads) mxv_prep_kernel(const __grid_constant__ MxvArgs a) {
+    pdl_begin();
     __shared__ StageBuf sb[kMxvThreads / 32];
     __shared__ unsigned long long bsm[kMxvThreads / 32];
     __shared__ unsigned long long csm[kMxvThreads / 32][4];
@@ -475,6 +447,7 @@ __device__ __forceinline__ void mxv_push(const MxvArgs& a) {
 
 // Pull, push, or -- a dense u that AUTO found sparse -- the queue for mxv_push_kernel.
 __global__ void __launch_bounds__(kMxvThreads, 4) mxv_main_kernel(const __grid_constant__ MxvArgs a) {
+    pdl_begin();
     union MainSmem {
         PullSmem pull;
         StageBuf sb[kMxvThreads / 32];
@@ -497,6 +470,7 @@ __global__ void __launch_bounds__(kMxvThreads, 4) mxv_main_kernel(const __grid_c
 }
 
 __global__ void __launch_bounds__(kMxvThreads) mxv_push_kernel(const __grid_constant__ MxvArgs a) {
+    pdl_begin();
     if (mxv_dir(a) == GBX_DIR_PUSH) mxv_push(a);
 }
 
@@ -514,6 +488,7 @@ __device__ __forceinline__ uint32_t mxv_take_word(const MxvArgs& a, int32_t w) {
 // One thread per word writes its 32 bytes (two 16-byte stores where w is aligned), ORing in the
 // old values when accumulating.
 __global__ void __launch_bounds__(kMxvThreads) mxv_dense_kernel(const __grid_constant__ MxvArgs a) {
+    pdl_begin();
     uint8_t* out = static_cast<uint8_t*>(const_cast<void*>(a.w.data));
     const bool vec = (reinterpret_cast<uintptr_t>(out) & 15u) == 0;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -550,6 +525,7 @@ __global__ void __launch_bounds__(kMxvThreads) mxv_dense_kernel(const __grid_con
 
 // Set bits of each block's words (a.per consecutive words a thread).
 __global__ void __launch_bounds__(kMxvThreads) mxv_count_kernel(const __grid_constant__ MxvArgs a) {
+    pdl_begin();
     __shared__ int32_t part[kMxvThreads / 32];
     const int64_t w0 = ((int64_t)blockIdx.x * kMxvThreads + threadIdx.x) * a.per;
     uint32_t c = 0;
@@ -567,6 +543,7 @@ __global__ void __launch_bounds__(kMxvThreads) mxv_count_kernel(const __grid_con
 
 // The sorted list of the set bits: a block's place is the sum of the blocks before it.
 __global__ void __launch_bounds__(kMxvThreads) mxv_list_kernel(const __grid_constant__ MxvArgs a) {
+    pdl_begin();
     __shared__ uint32_t part[2][kMxvThreads / 32];
     int32_t* out = static_cast<int32_t*>(const_cast<void*>(a.w.data));
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
@@ -739,21 +716,21 @@ static gbx_status mxv_bool(Graph* G, gbx_vector* w, const gbx_vector* mask, cons
                                   std::max(mask && mask->format == GBX_SPARSE ? std::min(mask->capacity, G->n) : 0,
                                            p.accum ? G->n : 0));
     const unsigned prep_blocks = std::max(1u, std::min(div_up(most, kMxvThreads), (unsigned)G->num_sms * 4u));
-    mxv_prep_kernel<<<prep_blocks, kMxvThreads, 0, s>>>(a);
+    GBX_TRY(pdl_launch(mxv_prep_kernel, prep_blocks, a, false, s));
     if (!a.nothing) {
-        mxv_main_kernel<<<main_blocks, kMxvThreads, 0, s>>>(a);
-        if (u->format == GBX_DENSE && a.dir == GBX_DIR_AUTO) mxv_push_kernel<<<main_blocks, kMxvThreads, 0, s>>>(a);
+        GBX_TRY(pdl_launch(mxv_main_kernel, main_blocks, a, true, s));
+        if (u->format == GBX_DENSE && a.dir == GBX_DIR_AUTO)
+            GBX_TRY(pdl_launch(mxv_push_kernel, main_blocks, a, true, s));
     }
     if (w->format == GBX_DENSE) {
         const unsigned blocks = std::max(1u, std::min(div_up(a.nwords, kMxvThreads), (unsigned)G->num_sms * 16u));
-        mxv_dense_kernel<<<blocks, kMxvThreads, 0, s>>>(a);
+        GBX_TRY(pdl_launch(mxv_dense_kernel, blocks, a, true, s));
     } else {
         a.per = std::max(4, (int)(((int64_t)a.nwords + kMxvThreads * 4096ll - 1) / (kMxvThreads * 4096ll)));
         const unsigned blocks = div_up(a.nwords, (int64_t)kMxvThreads * a.per);
-        mxv_count_kernel<<<blocks, kMxvThreads, 0, s>>>(a);
-        mxv_list_kernel<<<blocks, kMxvThreads, 0, s>>>(a);
+        GBX_TRY(pdl_launch(mxv_count_kernel, blocks, a, true, s));
+        GBX_TRY(pdl_launch(mxv_list_kernel, blocks, a, true, s));
     }
-    GBX_CUDA_TRY(cudaGetLastError());
     G->ws.mx_dirty = false;
     G->ws.last_stream = s;
     return GBX_OK;

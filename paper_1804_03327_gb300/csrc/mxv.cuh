@@ -51,6 +51,31 @@ inline int32_t mxv_tile_words(int32_t nwords, long long nwarps) {
 // The row-based matvec alone (mxv.cu), for the allocation-free entry point; kMxvThreads a block.
 __global__ void mxv_pull_kernel(PullArgs a);
 
+// The kernels of one call depend on one another and each is short: a later one is launched
+// while the one before still runs (programmatic dependent launch), its blocks take their
+// places as soon as every block of that one has started, and pdl_begin waits there until
+// the one before has ended and its writes are visible.  Saves about 2 us of the 4 between
+// two dependent launches.
+__device__ __forceinline__ void pdl_begin() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+template <typename A>
+gbx_status pdl_launch(void (*fn)(A), unsigned blocks, const A& a, bool dependent, cudaStream_t s) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(blocks);
+    cfg.blockDim = dim3(kMxvThreads);
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = dependent ? 1 : 0;
+    GBX_CUDA_TRY(cudaLaunchKernelEx(&cfg, fn, a));
+    return GBX_OK;
+}
+
 // What gbx_mxv reads, as bitmaps and queues (mxv.cu).
 struct MxvVec {
     int32_t format;  // GBX_DENSE, GBX_SPARSE or GBX_DENSE_F32; -1: none
