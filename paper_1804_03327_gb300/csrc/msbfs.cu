@@ -751,7 +751,8 @@ struct IdStage {
 // barrier; the prefix search, the queue's row starts, the probe of D and the degrees of the
 // flush are off it, and one atomic per block instead of one per warp reserves the list slots.
 // A level 11.7 -> 8.5 us on the whole GPU (the batch 23.8 -> 18.4 ms); on the quarter that a
-// server slot gets 14 -> 11 us.
+// server slot gets 14 -> 11 us, and to 10.2 with the clearing of the level before last off the
+// chain, too.
 constexpr int kMsMeshIlp = 4;
 constexpr int32_t kMsMeshDegree = 32;  // longest row of a mesh
 
@@ -1120,12 +1121,19 @@ __global__ void __launch_bounds__(kMsThreads, kOcc) ms_bfs_kernel(const __grid_c
         }
         Acc acc;
         Stage st{&mem.warp[wib].stage, 0, cout, a.ids[r1], a.qp[p1], a.qd[p1], a.out_ptr, a.in_ptr, 1, 0, &acc};
-        ms_clear_prev<WL>(a, a.ids[r2], prev_count, a.Fb[r2], a.Tb[r2]);
+        if (!kMesh) ms_clear_prev<WL>(a, a.ids[r2], prev_count, a.Fb[r2], a.Tb[r2]);
         const MsLong lr{a.tlist, a.qp[p0], a.qd[p0]};  // a pull level does not read the queue's prefix
         if (dir == GBX_DIR_PUSH) {
             if (kMesh) {
+                // the words of level L - 1's list are cleared here, their ids loaded before the push so that
+                // nothing waits for them
+                const long long c1 = gtid + gstride;
+                const int32_t v0 = gtid < prev_count ? a.ids[r2][gtid] : -1, v1 = c1 < prev_count ? a.ids[r2][c1] : -1;
                 IdStage ist{&mem.warp[wib].stage, 0, cout, a.ids[r1]};
                 ms_push_mesh(a, L, a.ids[r0], qcount, a.Fb[r0], a.Fb[r1], row_mem, ist, stage_sum, acc);
+                if (v0 >= 0) a.Fb[r2][v0] = 0ull;
+                if (v1 >= 0) a.Fb[r2][v1] = 0ull;
+                for (long long k = c1 + gstride; k < prev_count; k += gstride) a.Fb[r2][a.ids[r2][k]] = 0ull;
             } else if (WL == 1) {
                 ms_push_one(a, L, a.ids[r0], a.qp[p0], a.qd[p0], qcount, qedges, a.Fb[r0], a.Fb[r1], st,
                             stage_sum, acc);
@@ -1138,6 +1146,7 @@ __global__ void __launch_bounds__(kMsThreads, kOcc) ms_bfs_kernel(const __grid_c
                 ms_finalize<WL>(a, L, a.tlist, (uint32_t)lvl[5], a.Fb[r1], a.Tb[r1], st, stage_sum, acc);
             }
         } else {
+            if (kMesh) ms_clear_prev<WL>(a, a.ids[r2], prev_count, a.Fb[r2], a.Tb[r2]);
             const bool one = a.W <= WL * a.group;  // one chunk of words: long rows can be deferred
             for (int32_t c0 = 0; c0 < a.W; c0 += WL * a.group)
                 ms_pull<WL>(a, L, c0, a.Fb[r1], a.Tb[r1], mem.warp[wib].open_list, lr, one, st, stage_sum, acc);
