@@ -111,9 +111,9 @@ gbx_status exclusive_scan_i32(const int32_t* in, int32_t* out, int64_t count_max
 // One pass per 8-bit digit: the tiles' digit counts, their scan, and a scatter that orders each
 // tile in shared memory first, so that a digit's keys leave as one run of consecutive
 // addresses (16 keys on average) instead of one address per lane.  The keys' traffic is three
-// times 8 bytes a key and pass; the scatter is bound by its ranking (the matches of a warp's
-// digits and the counters' round trips).  A scatter of 33.5M 64-bit keys took 155-384 us
-// straight from registers, 180-250 through shared memory with the matches issued ahead of the
+// times 8 bytes a key and pass; the scatter is bound by its ranking (comparing a warp's digits
+// and the counters' round trips in shared memory).  A scatter of 33.5M 64-bit keys took 155-384 us
+// straight from registers, 170-235 through shared memory with the comparisons issued ahead of the
 // counting (275-317 with 256 threads of 16 keys); 79 us are its two streams at the copy rate.
 constexpr int kSortThreads = 512;
 constexpr int kSortWarps = kSortThreads / 32;
@@ -140,6 +140,18 @@ __global__ void __launch_bounds__(kSortThreads) radix_hist_kernel(const K* __res
     if (threadIdx.x < 256) hist[(int64_t)threadIdx.x * nblocks + blockIdx.x] = (int32_t)cnt[threadIdx.x];
 }
 
+// The lanes whose 9-bit value equals this lane's.  Nine votes: a match instruction goes through
+// the same pipe as the shared memory that the ranking keeps busy (3 % of the sort).
+__device__ __forceinline__ uint32_t same_digit(uint32_t d) {
+    uint32_t same = 0xffffffffu;
+#pragma unroll
+    for (int b = 0; b < 9; ++b) {
+        const uint32_t set = __ballot_sync(0xffffffffu, (d >> b) & 1u);
+        same &= ((d >> b) & 1u) ? set : ~set;
+    }
+    return same;
+}
+
 // Stable: a warp takes 256 consecutive keys of the tile, and keys are ranked by (warp, round,
 // lane), i.e. by input order.
 template <typename K>
@@ -161,7 +173,7 @@ __global__ void __launch_bounds__(kSortThreads, 2) radix_scatter_kernel(const K*
     for (int r = 0; r < kSortRounds; ++r) key[r] = first + 32 * r < count ? in[base + first + 32 * r] : K(0);
 #pragma unroll
     for (int r = 0; r < kSortRounds; ++r)  // 256: past the end
-        peers[r] = __match_any_sync(0xffffffffu, first + 32 * r < count ? (uint32_t)(key[r] >> shift) & 255u : 256u);
+        peers[r] = same_digit(first + 32 * r < count ? (uint32_t)(key[r] >> shift) & 255u : 256u);
     __syncthreads();
     uint16_t rank[kSortRounds];
 #pragma unroll
