@@ -270,7 +270,7 @@ static void workspace_carve(Workspace& w, int32_t n, Carve& c, size_t* zero) {
     w.mx_bm[2] = w.mx_bm[1] + nw;
     *zero = c.used;
     for (auto& p : w.bm) p = c.take<uint32_t>(nw);
-    for (int i = 0; i < 2; ++i) {
+    for (int i = 0; i < 2; ++i) {  // one after another: the batched BFS on meshes uses the three as one list
         w.q[i] = c.take<int32_t>(nn);
         w.qp[i] = c.take<int32_t>(nn);
         w.qd[i] = c.take<int32_t>(nn);

@@ -77,6 +77,11 @@ struct MsArgs {
     int32_t* status;
     float alpha;
     int32_t mode, trace_cap, symmetric, probe;
+    // kMesh: every level pushes, and a vertex may be listed more than once: lists 0 and 1 alternate (ids[0]
+    // and ids[1], from entry more_from on more[]), as do Fb[0] and Fb[1]
+    int32_t never_pull;
+    uint32_t more_from;
+    int32_t* more[2];
     int32_t group;  // warp lanes that hold a vertex's words (a power of two)
     unsigned long long timeout_ns;
 };
@@ -744,17 +749,25 @@ __device__ __forceinline__ void ms_push_one(const MsArgs& a, int32_t L, const in
     st.flush_block<kMsThreads / 32>(bsm);
 }
 
+// A list of vertices in two pieces of memory: entries [0, cap) and the rest.
+struct IdList {
+    int32_t* first;
+    int32_t* rest;
+    uint32_t cap;
+    __device__ __forceinline__ int32_t& at(uint32_t i) const { return i < cap ? first[i] : rest[i - cap]; }
+};
+
 // A level's next active list without degrees: vertices staged per warp, published with one
 // atomic per full stage and one per block at the end.
 struct IdStage {
     StageBuf* sb;
     int cnt;  // warp-uniform
     LevelCtr* cout;
-    int32_t* ids;
+    IdList ids;
 
     __device__ __forceinline__ void write(unsigned long long at) {
         __syncwarp();
-        for (int i = threadIdx.x & 31; i < cnt; i += 32) ids[(uint32_t)at + i] = sb->v[i];
+        for (int i = threadIdx.x & 31; i < cnt; i += 32) ids.at((uint32_t)at + i) = sb->v[i];
         __syncwarp();
         cnt = 0;
     }
@@ -827,9 +840,14 @@ __device__ __forceinline__ bool ms_mesh_gain(const MsArgs& a, int32_t L, int32_t
 }
 
 // rows: the output rows' addresses (shared memory).
-__device__ __forceinline__ void ms_push_mesh(const MsArgs& a, int32_t L, const int32_t* ids, uint32_t qcount,
-                                             const unsigned long long* Fc, unsigned long long* Fn, char* const* rows,
-                                             IdStage& st, unsigned long long* bsm, Acc& acc) {
+// once: v is listed by the first edge that gains a lane there, which the word of F_next tells it
+// (a round trip before the list).  Else every edge that gains one lists v -- 7 % more entries on
+// the grid, where a vertex has 1.07 new lanes a level -- and whoever takes an entry takes its
+// lanes with it, leaving F_cur zero (which needs no clearing later) and nothing for the others;
+// those entries are counted (exam, indeg: their number and degrees).
+__device__ __forceinline__ void ms_push_mesh(const MsArgs& a, int32_t L, const IdList& ids, uint32_t qcount,
+                                             unsigned long long* Fc, unsigned long long* Fn, char* const* rows,
+                                             bool once, IdStage& st, unsigned long long* bsm, Acc& acc) {
     constexpr int K = kMsMeshIlp;
     const int lane = threadIdx.x & 31, j = lane & 3;
     const uint32_t gwarp = (uint32_t)((blockIdx.x * kMsThreads + threadIdx.x) >> 5);
@@ -847,7 +865,7 @@ __device__ __forceinline__ void ms_push_mesh(const MsArgs& a, int32_t L, const i
 #pragma unroll
         for (int k = 0; k < K; ++k) {
             const uint32_t o = 8u * k + (lane >> 2);
-            u[k] = o < per && base + o < qcount ? ids[base + o] : -1;
+            u[k] = o < per && base + o < qcount ? ids.at((uint32_t)base + o) : -1;
         }
 #pragma unroll
         for (int k = 0; k < K; ++k) acc.mf += (uint32_t)(db[k] - da[k]);
@@ -856,7 +874,10 @@ __device__ __forceinline__ void ms_push_mesh(const MsArgs& a, int32_t L, const i
             w[k] = -1;
             f[k] = 0ull;
             if (u[k] < 0) continue;
-            f[k] = Fc[u[k]];
+            if (once)
+                f[k] = Fc[u[k]];
+            else if (j == 0)
+                f[k] = atomicExch(Fc + u[k], 0ull);
             if (j == 0) {
                 w[k] = __ldg(a.first_out + u[k]);
             } else if (j < 3) {
@@ -867,10 +888,31 @@ __device__ __forceinline__ void ms_push_mesh(const MsArgs& a, int32_t L, const i
                 more |= x.y >= 0;
             }
         }
+        if (!once) {
+#pragma unroll
+            for (int k = 0; k < K; ++k) {
+                f[k] = __shfl_sync(0xffffffffu, f[k], lane & ~3);
+                if (u[k] >= 0 && f[k] == 0ull) {  // listed before
+                    if (j == 0) {
+                        acc.exam += 1;
+                        acc.indeg += (uint32_t)(__ldg(a.out_ptr + u[k] + 1) - __ldg(a.out_ptr + u[k]));
+                    }
+                    u[k] = w[k] = -1;
+                }
+            }
+        }
 #pragma unroll
         for (int k = 0; k < K; ++k) old[k] = w[k] >= 0 ? atomicOr(a.V + w[k], f[k]) : ~0ull;
+        if (once) {
 #pragma unroll
-        for (int k = 0; k < K; ++k) was[k] = (f[k] & ~old[k]) ? atomicOr(Fn + w[k], f[k] & ~old[k]) : ~0ull;
+            for (int k = 0; k < K; ++k) was[k] = (f[k] & ~old[k]) ? atomicOr(Fn + w[k], f[k] & ~old[k]) : ~0ull;
+        } else {
+#pragma unroll
+            for (int k = 0; k < K; ++k) {
+                was[k] = 0ull;
+                if (f[k] & ~old[k]) atomicOr(Fn + w[k], f[k] & ~old[k]);  // a reduction
+            }
+        }
 #pragma unroll
         for (int k = 0; k < K; ++k) {
             const bool first = ms_mesh_gain(a, L, w[k], f[k], old[k], was[k], rows, acc);
@@ -893,7 +935,7 @@ __device__ __forceinline__ void ms_push_mesh(const MsArgs& a, int32_t L, const i
                         v = __ldg(a.out_col + x);
                         const unsigned long long o = atomicOr(a.V + v, f[k]);
                         const unsigned long long p = (f[k] & ~o) ? atomicOr(Fn + v, f[k] & ~o) : ~0ull;
-                        first = ms_mesh_gain(a, L, v, f[k], o, p, rows, acc);
+                        first = ms_mesh_gain(a, L, v, f[k], o, once ? p : 0ull, rows, acc);
                         if (first) acc.mf += (uint32_t)(__ldg(a.out_ptr + v + 1) - __ldg(a.out_ptr + v));
                     }
                     st.put(first, v);
@@ -1163,6 +1205,7 @@ __global__ void __launch_bounds__(kMsThreads, kOcc) ms_bfs_kernel(const __grid_c
         // direction for the whole batch: pull once the active edges exceed alpha * nnz
         int dir = a.mode;
         if (dir == GBX_DIR_AUTO) dir = (double)qedges > (double)a.alpha * (double)a.nnz ? GBX_DIR_PULL : GBX_DIR_PUSH;
+        if (kMesh && a.never_pull) dir = GBX_DIR_PUSH;
         if (a.depth16 && L + 1 > 32767) {
             if (gtid == 0) atomicCAS(a.status + ST_ERROR, 0, (int)GBX_ERR_OVERFLOW);
             return;
@@ -1173,15 +1216,23 @@ __global__ void __launch_bounds__(kMsThreads, kOcc) ms_bfs_kernel(const __grid_c
         const MsLong lr{a.tlist, a.qp[p0], a.qd[p0]};  // a pull level does not read the queue's prefix
         if (dir == GBX_DIR_PUSH) {
             if (kMesh) {
-                // the words of level L - 1's list are cleared here, their ids loaded before the push so that
-                // nothing waits for them
-                const long long c1 = gtid + gstride;
-                const int32_t v0 = gtid < prev_count ? a.ids[r2][gtid] : -1, v1 = c1 < prev_count ? a.ids[r2][c1] : -1;
-                IdStage ist{&mem.warp[wib].stage, 0, cout, a.ids[r1]};
-                ms_push_mesh(a, L, a.ids[r0], qcount, a.Fb[r0], a.Fb[r1], row_mem, ist, stage_sum, acc);
-                if (v0 >= 0) a.Fb[r2][v0] = 0ull;
-                if (v1 >= 0) a.Fb[r2][v1] = 0ull;
-                for (long long k = c1 + gstride; k < prev_count; k += gstride) a.Fb[r2][a.ids[r2][k]] = 0ull;
+                if (a.never_pull) {
+                    const IdList now{a.ids[L & 1], a.more[L & 1], a.more_from};
+                    IdStage ist{&mem.warp[wib].stage, 0, cout, IdList{a.ids[p1], a.more[p1], a.more_from}};
+                    ms_push_mesh(a, L, now, qcount, a.Fb[p0], a.Fb[p1], row_mem, false, ist, stage_sum, acc);
+                } else {
+                    // the words of level L - 1's list are cleared here, their ids loaded before the push so that
+                    // nothing waits for them
+                    const long long c1 = gtid + gstride;
+                    const int32_t v0 = gtid < prev_count ? a.ids[r2][gtid] : -1;
+                    const int32_t v1 = c1 < prev_count ? a.ids[r2][c1] : -1;
+                    IdStage ist{&mem.warp[wib].stage, 0, cout, IdList{a.ids[r1], nullptr, 0xffffffffu}};
+                    ms_push_mesh(a, L, IdList{a.ids[r0], nullptr, 0xffffffffu}, qcount, a.Fb[r0], a.Fb[r1], row_mem,
+                                 true, ist, stage_sum, acc);
+                    if (v0 >= 0) a.Fb[r2][v0] = 0ull;
+                    if (v1 >= 0) a.Fb[r2][v1] = 0ull;
+                    for (long long k = c1 + gstride; k < prev_count; k += gstride) a.Fb[r2][a.ids[r2][k]] = 0ull;
+                }
             } else if (WL == 1) {
                 ms_push_one(a, L, a.ids[r0], a.qp[p0], a.qd[p0], qcount, qedges, a.Fb[r0], a.Fb[r1], st,
                             stage_sum, acc);
@@ -1199,13 +1250,14 @@ __global__ void __launch_bounds__(kMsThreads, kOcc) ms_bfs_kernel(const __grid_c
             for (int32_t c0 = 0; c0 < a.W; c0 += WL * a.group)
                 ms_pull<WL>(a, L, c0, a.Fb[r1], a.Tb[r1], mem.warp[wib].open_list, lr, one, st, stage_sum, acc);
         }
-        block_add_counts<kMsThreads / 32>(acc_mem, acc.n_new, acc.mf, acc.exam, 0ull, &cout->n_new, &cout->mf_new,
-                                          &cout->e_exam, nullptr);
+        block_add_counts<kMsThreads / 32>(acc_mem, acc.n_new, acc.mf, acc.exam, kMesh ? acc.indeg : 0ull, &cout->n_new,
+                                          &cout->mf_new, &cout->e_exam, kMesh ? &cout->indeg_new : nullptr);
         if (!grid_barrier(barc, gridDim.x, bar_round, a.status, a.timeout_ns)) return;
         if (threadIdx.x == 0) {
             lvl[0] = ld_volatile_u64(&cout->n_new);
             lvl[1] = ld_volatile_u64(&cout->mf_new);
             lvl[2] = ld_volatile_u64(&cout->huge);
+            if (kMesh) lvl[5] = ld_volatile_u64(&cout->indeg_new);
             lvl[3] = ld_volatile_u64(&cout->e_exam);
             lvl[4] = ld_volatile_u64(&cout->q);
         }
@@ -1247,6 +1299,11 @@ __global__ void __launch_bounds__(kMsThreads, kOcc) ms_bfs_kernel(const __grid_c
             r.e_exam = dir == GBX_DIR_PULL ? (long long)lvl[3] : -1;
             r.n_new = n_new;
             r.mf_new = (long long)lvl[1];
+            if (kMesh && a.never_pull) {  // without the entries that were listed again
+                r.nf -= (long long)lvl[3];
+                r.mf -= (long long)lvl[5];
+                if (L > 0) a.trace[L - 1].mf_new = r.mf;
+            }
             const unsigned long long now = global_timer_ns();
             r.t_ns = (long long)(now - t_mark);
             t_mark = now;
@@ -1384,6 +1441,14 @@ gbx_status ms_run(Graph* G, Workspace& w, int32_t S, const int32_t* src_dev, voi
     const bool lean = blocks <= 1 && d.blocks_per_sm >= kMsOccLean && cw <= 2;
     const int cap = lean ? 0 : d.blocks_per_sm;
     gbx_status st;
+    // A threshold of one and more never pulls: at most every edge is active.  A level lists at most one
+    // vertex per edge; the queue arrays q, qp and qd of one side lie one after another (workspace_carve)
+    // and the third lane buffer, not needed then, holds n more entries of each of two lists.
+    a.never_pull = G->nnz <= 4ll * G->n && G->n <= (1 << 30) &&
+                   (d.direction == GBX_DIR_PUSH || (d.direction == GBX_DIR_AUTO && d.alpha >= 1.0f));
+    a.more_from = 3u * (uint32_t)G->n;
+    a.more[0] = reinterpret_cast<int32_t*>(w.msF[2]);
+    a.more[1] = a.more[0] + G->n;
     a.group = 1;
     while (2 * a.group < W && a.group < 32) a.group *= 2;
     if (W > 1)

@@ -80,4 +80,9 @@ def test_mesh_batches(w, h, S, k):
             for b in range(min(S, 16)):
                 assert np.array_equal(got[b], want[int(srcs[b])]), (direction, b)
             assert tr["n_new"].sum() == np.sum(got > 0) and np.all(tr["mf"][1:] == tr["mf_new"][:-1])
+            # the active vertices of a level, each once however often it was listed
+            deg = np.diff(og.out_ptr)
+            active = [(got == level).any(axis=0) & (deg > 0) for level in range(len(tr))]
+            assert [int(x) for x in tr["nf"]] == [int(x.sum()) for x in active]
+            assert [int(x) for x in tr["mf"]] == [int(deg[x].sum()) for x in active]
     g.free()
