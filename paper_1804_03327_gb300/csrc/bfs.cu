@@ -960,6 +960,7 @@ static gbx_status bfs_geometry(Graph* G) {
                          (const void*)bfs_kernel<false, false, true>};
     int per_sm = 1 << 30;
     for (const void* fn : fns) {
+        GBX_TRY(prefer_l1(fn, kBfsMinBlocks));
         int b = 0;
         GBX_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, fn, kBfsThreads, 0));
         per_sm = b < per_sm ? b : per_sm;

@@ -1369,6 +1369,11 @@ int64_t ms_scratch_bytes(int32_t n, int32_t S) {
 
 template <int WL, int kOcc, bool kMesh = false>
 static gbx_status ms_launch(Graph* G, const MsArgs& a0, int blocks, int per_sm_cap, cudaStream_t s) {
+    const uint32_t which = 32u << (WL == 2 ? kOcc - kMsOcc : 2 + (kMesh ? 2 : kOcc - kMsOcc));
+    if (!(G->l1_set & which)) {
+        GBX_TRY(prefer_l1((const void*)ms_bfs_kernel<WL, kOcc, kMesh>, kOcc));
+        G->l1_set |= which;
+    }
     int per_sm = 0;
     GBX_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ms_bfs_kernel<WL, kOcc, kMesh>, kMsThreads, 0));
     GBX_CHECK(per_sm >= 1, GBX_ERR_CUDA, "batched BFS kernel cannot be resident");

@@ -710,6 +710,10 @@ static gbx_status mxv_bool(Graph* G, gbx_vector* w, const gbx_vector* mask, cons
     p.tile_words = mxv_tile_words(a.nwords, (long long)main_blocks * (kMxvThreads / 32));
     p.early_exit = a.early_exit;
     p.stats = a.stats;
+    if (!(G->l1_set & 1024u)) {
+        GBX_TRY(prefer_l1((const void*)mxv_main_kernel, 4));
+        G->l1_set |= 1024u;
+    }
     GBX_TRY(mxv_scratch(G, s));
     G->ws.mx_dirty = true;  // until every kernel of the call is issued
     const int32_t most = std::max(std::max(a.nwords, u->format == GBX_SPARSE ? std::min(u->capacity, G->n) : 0),

@@ -173,8 +173,8 @@ constexpr int kSpullStep = 32 * kSpullVec;     // in-edges per warp and step
 static_assert(kSpullStep == 128, "a step's row starts fit four 32-bit words, one per group of eight lanes");
 // Finished rows wait in a ring of kSpullRing (row entry, minimum) pairs: fewer than
 // 32 are left after a write-out and one step adds at most kSpullStep.
-constexpr int kSpullRing = 256;
-static_assert(kSpullRing >= 31 + kSpullStep && (kSpullRing & (kSpullRing - 1)) == 0, "pull ring size");
+constexpr int kSpullRing = 160;
+static_assert(kSpullRing >= 31 + kSpullStep, "pull ring size");
 
 struct SpullSmem {
     uint32_t occ[4];            // row starts of the step, one bit per edge
@@ -229,7 +229,7 @@ __device__ __forceinline__ void sssp_pull_queue(SpullSmem& sm, uint32_t& tail, b
                                                 float m) {
     const uint32_t b = __ballot_sync(0xffffffffu, take);
     if (take)
-        sm.ring[(tail + __popc(b & lanemask_lt())) & (kSpullRing - 1)] =
+        sm.ring[(tail + __popc(b & lanemask_lt())) % kSpullRing] =
             make_int2(own ? kr : ~kr, __float_as_int(m));
     tail += __popc(b);
 }
@@ -242,7 +242,7 @@ __device__ __forceinline__ void sssp_pull_drain(const SsspArgs& a, int32_t L, Sp
     __syncwarp();
     while (tail - head >= least) {
         if ((uint32_t)lane < tail - head) {
-            const int2 e = sm.ring[(head + lane) & (kSpullRing - 1)];
+            const int2 e = sm.ring[(head + lane) % kSpullRing];
             sssp_pull_commit(a, L, e.x >= 0 ? e.x : ~e.x, __int_as_float(e.y), e.x >= 0, acc);
         }
         head += tail - head < 32u ? tail - head : 32u;
@@ -546,6 +546,11 @@ extern "C" gbx_status gbx_sssp(gbx_graph* g, int32_t source, float* dist, const 
         GBX_TRY(sssp_cluster_launch(G, source, dist, s));
         w.last_stream = s;
         w.last_traced = 0;
+    }
+    const uint32_t which = lean ? (d.trace ? 1u : 2u) : (cluster ? 4u : (d.trace ? 8u : 16u));
+    if (!(G->l1_set & which)) {
+        GBX_TRY(prefer_l1(fn, lean ? kSsspOccLean : kSsspOcc));
+        G->l1_set |= which;
     }
     int per_sm = 0;
     GBX_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kSsspThreads, 0));

@@ -64,7 +64,7 @@ def test_mesh_batches(w, h, S, k):
     arrays, up to the 32 that make a mesh), in every direction, int16 and int32 rows."""
     n, s, d = synth.grid_edges(w, h, p_delete=0.02, seed=h)
     if k:
-        n = w * h + 40
+        n = min(w * h, 2500) + 40
         s = np.repeat(np.arange(n, dtype=np.int32), k)
         d = ((s + np.tile(np.arange(1, k + 1, dtype=np.int32), n)) % n).astype(np.int32)
     og, g = oracle.graph(n, s, d), gbx.graph_build(n, s, d)
