@@ -1219,7 +1219,7 @@ def run_ours(args):
                    "l2": "inputs larger than L2 (0.5 GB CSR, 64 distinct depth+parent pairs per step); no flush",
                    "parallelism": f"replicas x{world}, sources sharded by rank"},
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
-                     "frac": achieved / peak, "traffic": traffic, "kernel": "bfs_kernel<false, false>",
+                     "frac": achieved / peak, "traffic": traffic, "kernel": "bfs_kernel<false, false, false>",
                      "peak_kind": f"{peak_kind} (MEASURED_PEAKS.json hbm_gbs copy bandwidth)",
                      "bytes_per_launch": mean_bytes, "launch_ms": mean_launch_s * 1e3,
                      "frac_of_nominal_7900": achieved / 7900.0},

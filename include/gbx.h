@@ -285,8 +285,12 @@ gbx_status gbx_mxv_pull_noalloc(int32_t n, const int32_t* row_ptr, const int32_t
  * Breadth-first search from `source` (Algorithm 1): every level runs the
  * masked matvec f <- A^T f .* !v in the direction the descriptor selects
  * (AUTO: start in push, switch per desc->heuristic after every level, decided
- * on the device).  The whole level loop runs in one persistent cooperative
- * kernel, so no level costs a host round trip.
+ * on the device).  The level loop runs in one persistent cooperative kernel, so
+ * no level costs a host round trip.  On a graph whose rows have at most 32
+ * entries, or a tiny one, an untraced run under the ratio rule that is not forced
+ * to pull starts in one thread-block cluster, which pushes while the frontier is
+ * small, in a launch of its own before that kernel; the kernel takes over where
+ * the cluster stopped (and returns at once if it finished).
  * Outputs (device, int32[n], caller-owned): depth[v] = hops from the source
  * (depth[source] = 0, unreached = -1); parent (may be NULL): parent[source] =
  * source, parent[v] = some in-neighbour u of v with depth[u] = depth[v] - 1,
@@ -344,8 +348,8 @@ gbx_status gbx_bfs_trace(gbx_graph* g, gbx_level* levels, int32_t cap, int32_t* 
  * untraced run that is not forced to pull relaxes the vertices near the source
  * first instead of all improved ones (the distances are the same).
  * A negative cycle ends in GBX_ERR_OVERFLOW after n iterations (reported by
- * gbx_graph_sync).  One persistent cooperative launch, asynchronous on
- * `stream`; desc->blocks_per_sm >= 3 selects a register-lean build at three
+ * gbx_graph_sync).  One persistent cooperative launch (after the cluster's, where
+ * near vertices go first), asynchronous on `stream`; desc->blocks_per_sm >= 3 selects a register-lean build at three
  * blocks per SM (faster on long push iterations over skewed graphs, slower with
  * pull iterations; GBX_TUNE_SSSP times both).  Errors: NULL_POINTER, INVALID_INDEX, INVALID_VALUE (no weights,
  * desc fields), NOT_SUPPORTED (push_sort), CUDA.

@@ -359,23 +359,6 @@ struct PushCursorT {
         k += (int32_t)before;
     }
 
-    // The entry of each lane's edge slots of the step [base, base + kStep) (qp must
-    // be strictly ascending: no entry without edges); the cursor moves on to the
-    // entry of the step's last edge.  A slot at or past the end of the last entry's
-    // edges maps to the last entry.
-    __device__ __forceinline__ void locate(const int32_t* qp, uint32_t qcount, int32_t base, int32_t (&kk)[I]) {
-        const int lane = threadIdx.x & 31;
-        uint32_t occ[I];
-        occupancy(qp, qcount, base, occ);
-        uint32_t before = 0;
-#pragma unroll
-        for (int t = 0; t < I; ++t) {
-            kk[t] = k + (int32_t)(before + __popc(occ[t] & (0xffffffffu >> (31 - lane))));
-            before += __popc(occ[t]);
-        }
-        k += (int32_t)before;
-    }
-
     __device__ __forceinline__ PushStepT<I> gather(const int32_t* out_col, const int32_t* q, const int32_t* qp,
                                                const int32_t* qd, uint32_t qcount, int32_t base, int32_t e1) {
         const int lane = threadIdx.x & 31;
