@@ -44,6 +44,12 @@ constexpr int kMxvProbe = 16;
 // Bound by dependent gathers: RMAT-22 with half its rows masked and a fifth of its vertices in
 // u reads 124 MB.  Rounds of 64 rows in lockstep took as long as their slowest row: the
 // call 59.7 us, now 51.3 (and 102.6 with 17 launches and tiles of 32 words).
+//
+// A tile's words lie ntiles apart, not side by side: the unvisited rows of a mesh are one band of
+// the numbering, which would be the work of a few warps (the 2048 x 2048 grid's BFS levels pulled at
+// 40, 60 and 80 % of the levels 61.5, 51 and 30 us, so 40, 25 and 17).  A warp then reads its words'
+// masks from as many sectors; the RMAT-22 call 50.6 -> 51.8 us.  Pieces of 4 words side by side:
+// 45, 29, 19 and 51.8.
 constexpr int kMxvP1 = 4;  // first-pass rows per lane per round
 
 // The rows of a tile whose bits are set in the lane words m (lane l: word l), in
@@ -114,7 +120,9 @@ __device__ __forceinline__ void mxv_pull(const PullArgs& a, PullSmem& sm) {
     const int32_t ntiles = (nwords + tw - 1) / tw;
     unsigned long long rows = 0, exam = 0;
     for (int32_t tile = gwarp; tile < ntiles; tile += nwarps) {
-        const int32_t w0 = tile * tw, w = w0 + lane;
+        const int32_t w = tile + lane * ntiles;
+        // the row of an entry of the list
+        auto row_at = [&](int off) { return ((tile + (off >> 5) * ntiles) << 5) + (off & 31); };
         const bool wok = lane < tw && w < nwords;
         const uint32_t cand0 = wok ? ((a.pass ? a.pass[w] ^ a.invert : 0xffffffffu) & a.nz[w]) : 0u;
         hits[lane] = 0u;
@@ -129,20 +137,20 @@ __device__ __forceinline__ void mxv_pull(const PullArgs& a, PullSmem& sm) {
         if (two_pass) {
             mxv_tile_list(list, cand0, incl0 - cnt0);
             for (uint32_t base = 0; base < total0; base += 32 * kMxvP1) {
-                int32_t i[kMxvP1], f0[kMxvP1];
+                int32_t off[kMxvP1], f0[kMxvP1];
 #pragma unroll
                 for (int r = 0; r < kMxvP1; ++r) {
                     const uint32_t c = base + 32 * r + lane;
-                    i[r] = c < total0 ? (w0 << 5) + (int)list[c] : -1;
+                    off[r] = c < total0 ? (int)list[c] : -1;
                 }
 #pragma unroll
-                for (int r = 0; r < kMxvP1; ++r) f0[r] = i[r] >= 0 ? first[i[r]] : -1;
+                for (int r = 0; r < kMxvP1; ++r) f0[r] = off[r] >= 0 ? first[row_at(off[r])] : -1;
 #pragma unroll
                 for (int r = 0; r < kMxvP1; ++r) {
-                    if (i[r] < 0) continue;
+                    if (off[r] < 0) continue;
                     rows += 1;
                     exam += 1;
-                    if (bit_test(ubm, f0[r])) atomicOr(hits + ((i[r] >> 5) - w0), 1u << (i[r] & 31));
+                    if (bit_test(ubm, f0[r])) atomicOr(hits + (off[r] >> 5), 1u << (off[r] & 31));
                 }
             }
             __syncwarp();
@@ -156,7 +164,7 @@ __device__ __forceinline__ void mxv_pull(const PullArgs& a, PullSmem& sm) {
         if (total) mxv_tile_list(list, cand, incl - cntw);
         // a row per lane, each lane going on to the next one as soon as its row is settled
         uint32_t nxt = 0;  // rows of the list handed out
-        int32_t i = -1, beg = 0, end = 0, k = 0;
+        int32_t i = -1, at = 0, beg = 0, end = 0, k = 0;  // row, its place in the tile
         bool found = false;
         for (;;) {
             const uint32_t need = __ballot_sync(0xffffffffu, i < 0);
@@ -169,7 +177,8 @@ __device__ __forceinline__ void mxv_pull(const PullArgs& a, PullSmem& sm) {
                 const uint32_t f1j = __shfl_sync(0xffffffffu, f1, off >> 5);
                 nxt += __popc(need);
                 if (fresh) {
-                    i = (w0 << 5) + off;
+                    i = row_at(off);
+                    at = off;
                     found = two_pass && ((f1j >> (off & 31)) & 1u);  // only without early exit can it be set here
                 }
             }
@@ -269,7 +278,7 @@ __device__ __forceinline__ void mxv_pull(const PullArgs& a, PullSmem& sm) {
                 }
             }
             if (done) {
-                if (found) atomicOr(hits + ((i >> 5) - w0), 1u << (i & 31));
+                if (found) atomicOr(hits + (at >> 5), 1u << (at & 31));
                 i = -1;
             }
         }
