@@ -181,7 +181,8 @@ typedef struct {
     int32_t pull_probe;      /* BFS pull: in-neighbours one lane scans before its warp takes the row over
                                 (0 = default: 16 single-source, 8 batched; otherwise 4..1024).  Batched:
                                 a row still open after four times as many is shared by the grid */
-    int32_t blocks_per_sm;   /* BFS and SSSP kernels: persistent blocks per SM (0 = as many as fit).
+    int32_t blocks_per_sm;   /* BFS and SSSP kernels: persistent blocks per SM (0 = as many as fit;
+                                gbx_bfs: one on a small graph, where that is faster).
                                 gbx_bfs_batch and gbx_sssp: 1 or 2 caps the default build (two per
                                 SM); 3 or more selects a register-lean build at three per SM (batches:
                                 at most 128 sources run alone; server batches keep the default build) */

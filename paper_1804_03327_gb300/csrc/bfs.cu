@@ -20,6 +20,8 @@
 // GrB_assign of line 7 (depth stamp) and the GrB_reduce of line 9 (frontier
 // count) are fused into the level; levels are separated by a bounded grid
 // barrier instead of kernel launches.
+#include <algorithm>
+
 #include <atomic>
 
 #include "bfs_cluster.cuh"
@@ -227,6 +229,10 @@ __device__ __forceinline__ void push_level(const BfsArgs& a, int32_t L, int cur,
 #define GBX_PULL_ILP 1
 #endif
 constexpr int kPullIlp = GBX_PULL_ILP;  // pass-2 rows per lane (2: 928 us instead of 888, from spills)
+// Stored entries up to which a search left to its default runs one block per SM.  One and two, us a
+// source: edge factor 4: 12K vertices 46 and 51, 300K 61 and 67, 1M (8M entries) 66 and 68, 2M (16M)
+// 96 and 94; edge factor 16: 30K 42 and 46, 300K (9M) 57 and 60, 600K (18M) 73 and 72, 1M 91 and 85.
+constexpr long long kBfsSmallEntries = 12ll << 20;
 // Bitmap words one warp takes at a time in a pull level (lane l holds word l of the tile): an
 // even share of the words over as many rounds as 32 words a warp need.  RMAT-22 has 27 words
 // for each of 4,864 warps; tiles of 32 left 768 warps without any and the others a fifth longer
@@ -1031,7 +1037,10 @@ static gbx_status launch_bfs(Graph* G, int32_t source, int32_t* depth, int32_t* 
         if (complete) return GBX_OK;
         fn = (const void*)bfs_kernel<false, false, true>;
     }
-    const int per_sm = d.blocks_per_sm > 0 && d.blocks_per_sm < G->bfs_blocks ? d.blocks_per_sm : G->bfs_blocks;
+    // a small graph's levels are short and their barriers and counters cheaper with half the blocks
+    const int wanted = d.blocks_per_sm > 0 ? d.blocks_per_sm
+                       : !huge && !cluster && G->nnz <= kBfsSmallEntries ? 1 : G->bfs_blocks;
+    const int per_sm = std::min(wanted, G->bfs_blocks);
     a.tile_words = pull_tile_words(G->nwords, (long long)per_sm * G->num_sms * (kBfsThreads / 32));
     GBX_CUDA_TRY(cudaLaunchCooperativeKernel(fn, dim3(per_sm * G->num_sms), dim3(kBfsThreads), args, 0, s));
     G->ws.bar_parity ^= 1u;

@@ -83,3 +83,19 @@ def test_cluster_bfs(name):
     gbx.graph_sync(g)
     assert np.array_equal(depth.cpu().numpy(), want[0])
     g.free()
+
+
+@pytest.mark.parametrize("blocks", [0, 1, 2])
+@pytest.mark.parametrize("scale,ef", [(14, 16), (19, 12), (20, 16)])
+def test_grid_size(scale, ef, blocks):
+    """The whole grid with one and with two blocks per SM, on both sides of the size where the default changes."""
+    n, s, d = rmat(scale, ef)
+    og, g = oracle.graph(n, s, d), gbx.graph_build(n, s, d)
+    src = int(s[0])
+    want, _, _ = oracle.bfs(og, src)
+    depth = torch.empty(n, dtype=torch.int32, device="cuda")
+    parent = torch.empty(n, dtype=torch.int32, device="cuda")
+    gbx.bfs(g, src, depth, parent, gbx.desc_init(blocks_per_sm=blocks))
+    gbx.graph_sync(g)
+    assert np.array_equal(depth.cpu().numpy(), want)
+    assert_valid_parents(og.out_ptr, og.out_col, want, parent.cpu().numpy(), src)
