@@ -409,6 +409,10 @@ __device__ __forceinline__ void record_words(const MsArgs& a, int32_t v, int32_t
 // ---------------------------------------------------------------- pull level
 
 constexpr int kMsUnroll = 4;        // in-neighbours a group ORs per step (loads in flight)
+// On a graph with at most a word of rows per warp a lane's walk of up to 96 in-edges is what a pull level
+// takes: there the warp takes a row over after a.probe of them when more than kMsFewRow are left (5 to 45
+// sources on 3K to 20K vertices: 134-196 -> 123-183 us; 36 sources on 125K 197 -> 182).
+constexpr int32_t kMsFewRow = 24;
 constexpr int32_t kMsLongRow = 64;   // in-edges left after the probe beyond which a row is deferred
 // Steps of a whole warp on a row before it is deferred, with one word (128 in-neighbours a step):
 // at a level whose lanes are mostly covered that settles the row without the chain of a
@@ -457,6 +461,8 @@ __device__ __forceinline__ void ms_pull(const MsArgs& a, int32_t L, int32_t c0, 
     Words<WL> lm;
 #pragma unroll
     for (int j = 0; j < WL; ++j) lm.x[j] = wok ? lane_mask(a.S, w + j) : 0ull;
+    const bool few = WL == 1 && a.nwords <= nwarps;  // a word per warp at most: a level lasts as long as a row
+    const int32_t own = few ? a.probe : 4 * a.probe, most = few ? kMsFewRow : kMsLongRow;
     for (long long wb = gwarp; wb < a.nwords; wb += 32ll * nwarps) {
         const long long tw = wb + (long long)lane * nwarps;
         uint32_t m = tw < a.nwords ? (a.nz_in[tw] & ~a.D[tw]) : 0u;
@@ -481,7 +487,7 @@ __device__ __forceinline__ void ms_pull(const MsArgs& a, int32_t L, int32_t c0, 
                     v = (int32_t)((wb + (long long)(off >> 5) * nwarps) << 5) + (int32_t)(off & 31u);
                     k = __ldg(a.in_ptr + v);
                     end = __ldg(a.in_ptr + v + 1);
-                    lim = end - k > 4 * a.probe + kMsLongRow ? k + 4 * a.probe : end;
+                    lim = end - k > own + most ? k + own : end;
                     sink = !a.symmetric && __ldg(a.out_ptr + v + 1) == __ldg(a.out_ptr + v);
                     unv = wok ? ld_words<WL>(a.V + (size_t)v * a.W + w) : zero_words<WL>();
 #pragma unroll
