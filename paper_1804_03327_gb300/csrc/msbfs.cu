@@ -1450,7 +1450,10 @@ gbx_status ms_run(Graph* G, Workspace& w, int32_t S, const int32_t* src_dev, voi
     // the lean build only when this batch has the GPU to itself: concurrent cooperative
     // grids of one register budget tile the SMs exactly, mixed budgets need not
     const bool lean = blocks <= 1 && d.blocks_per_sm >= kMsOccLean && cw <= 2;
-    const int cap = lean ? 0 : d.blocks_per_sm;
+    // few vertices: barriers among half the blocks are cheaper (8K vertices, 436 sources 515 -> 423 us, 45
+    // sources 171 -> 149; 20K, 516 sources 622 -> 563, 38 sources 183 -> 171; 125K, 36 sources 182 -> 186)
+    const bool small = blocks <= 1 && d.blocks_per_sm == 0 && G->n <= 32768;
+    const int cap = lean ? 0 : small ? 1 : d.blocks_per_sm;
     gbx_status st;
     // A threshold of one and more never pulls: at most every edge is active.  A level lists at most one
     // vertex per edge; the queue arrays q, qp and qd of one side lie one after another (workspace_carve)
