@@ -266,18 +266,17 @@ struct HugeRows {
     int32_t* first;  // smallest edge index with a hit found so far (INT32_MAX: none)
 };
 
-// One warp-wide scan of in_col[kk, kk + 32 * kT) against tbm (kT loads in
-// flight per lane).  Returns the position of the first edge whose source is in
+// One warp-wide scan of in_col[kk, kk + 32 * kT), at most `left` entries, against tbm (kT
+// loads in flight per lane; a position past a row's end need not fit 32 bits).  Returns the position of the first edge whose source is in
 // tbm (32 * kT if none in range) and that source in *jf.
 template <int kT>
 __device__ __forceinline__ int warp_scan(const int32_t* __restrict__ in_col, const uint32_t* tbm, int32_t kk,
-                                         int32_t ee, int32_t* jf) {
+                                         int32_t left, int32_t* jf) {
     const int lane = threadIdx.x & 31;
     int32_t j[kT];
 #pragma unroll
     for (int t = 0; t < kT; ++t) {
-        const int32_t idx = kk + 32 * t + lane;
-        j[t] = idx < ee ? __ldg(in_col + idx) : -1;
+        j[t] = 32 * t + lane < left ? __ldg(in_col + kk + 32 * t + lane) : -1;
     }
     uint32_t b[kT];
 #pragma unroll
@@ -460,9 +459,9 @@ __device__ __forceinline__ void pull_level(const BfsArgs& a, int32_t L, int vcur
                     if (!two_pass || known[r]) f0[r] = __ldg(a.first_in + i[r]);
                     k[r] = beg[r] + 1;  // the first in-neighbour is examined (by pass 1, or right here)
                 } else if (i[r] >= 0) {
-                    const int32_t lim = end[r] < beg[r] + a.probe ? end[r] : beg[r] + a.probe;
+                    const int32_t own = min(end[r] - beg[r], a.probe) - (k[r] - beg[r]);  // left to the lane
 #pragma unroll
-                    for (int t = 0; t < 4; ++t) x[r][t] = k[r] + t < lim ? ld_stream(a.in_col + k[r] + t) : -1;
+                    for (int t = 0; t < 4; ++t) x[r][t] = t < own ? ld_stream(a.in_col + k[r] + t) : -1;
                 }
             }
             if (!__any_sync(0xffffffffu, live)) break;
@@ -501,18 +500,18 @@ __device__ __forceinline__ void pull_level(const BfsArgs& a, int32_t L, int vcur
                 // rows longer than the lane probe: the whole warp scans them (32, then 128 edges a step),
                 // or lists them for the grid-wide phase when more than kPullHugeRow are left
                 uint32_t pend =
-                    __ballot_sync(0xffffffffu, i[r] >= 0 && !done && k[r] >= beg[r] + a.probe && k[r] < end[r]);
+                    __ballot_sync(0xffffffffu, i[r] >= 0 && !done && k[r] - beg[r] >= a.probe && k[r] < end[r]);
                 while (pend) {
                     const int t = __ffs(pend) - 1;
                     pend &= pend - 1;
                     int32_t kk = __shfl_sync(0xffffffffu, k[r], t);
-                    const int32_t ee = __shfl_sync(0xffffffffu, end[r], t);
+                    int32_t left = __shfl_sync(0xffffffffu, end[r], t) - kk;
                     int32_t tp = __shfl_sync(0xffffffffu, par[r], t);
                     uint32_t tx = 0;
-                    if (kHuge && ee - kk > kPullHugeRow) {
+                    if (kHuge && left > kPullHugeRow) {
                         const int32_t row = __shfl_sync(0xffffffffu, i[r], t);
                         if (lane == 0) {
-                            const unsigned long long nch = (unsigned long long)((ee - kk + kPullChunk - 1) / kPullChunk);
+                            const unsigned long long nch = (unsigned long long)((left - 1) / kPullChunk + 1);
                             const unsigned long long old = atomicAdd(&st.cout->huge, (nch << 32) | 1ull);
                             const uint32_t slot = (uint32_t)old;
                             hr.row[slot] = tp >= 0 ? ~row : row;
@@ -520,13 +519,13 @@ __device__ __forceinline__ void pull_level(const BfsArgs& a, int32_t L, int vcur
                             hr.base[slot] = (int32_t)(old >> 32);
                             hr.first[slot] = INT32_MAX;
                         }
-                        kk = ee;
+                        left = 0;
                     }
                     // 32 edges first (an early hit then costs no wider read), then 128 at a time
-                    for (int step = 32; kk < ee; kk += step, step = 128) {
+                    for (int step = 32; left > 0; kk += step, left -= step, step = 128) {
                         int32_t jf = 0;
-                        const int pos = step == 32 ? warp_scan<1>(a.in_col, tbm, kk, ee, &jf)
-                                                   : warp_scan<4>(a.in_col, tbm, kk, ee, &jf);
+                        const int pos = step == 32 ? warp_scan<1>(a.in_col, tbm, kk, left, &jf)
+                                                   : warp_scan<4>(a.in_col, tbm, kk, left, &jf);
                         if (pos < step) {
                             if (tp < 0) tp = jf;
                             if (a.early_exit) {
@@ -534,7 +533,7 @@ __device__ __forceinline__ void pull_level(const BfsArgs& a, int32_t L, int vcur
                                 break;
                             }
                         }
-                        tx += (uint32_t)(ee - kk < step ? ee - kk : step);
+                        tx += (uint32_t)(left < step ? left : step);
                     }
                     if (lane == t) {
                         par[r] = tp;
@@ -601,7 +600,7 @@ __device__ GBX_PULL_HUGE_INLINE void pull_huge(const BfsArgs& a, int32_t L, int 
         const int32_t i = known ? ~code : code;
         const int32_t rend = __ldg(a.in_ptr + i + 1);
         const int32_t beg = hr.k[e] + (c - hr.base[e]) * kPullChunk;
-        const int32_t end = rend - beg < kPullChunk ? rend : beg + kPullChunk;
+        const int32_t len = rend - beg < kPullChunk ? rend - beg : kPullChunk;
         if (a.early_exit) {
             const int32_t fk = ld_volatile_i32(hr.first + e);
             if (exact_exam ? fk < beg : fk != INT32_MAX) continue;
@@ -611,18 +610,18 @@ __device__ GBX_PULL_HUGE_INLINE void pull_huge(const BfsArgs& a, int32_t L, int 
         bool hit = false;
         int32_t par = -1, hit_at = 0;
         unsigned long long ex = 0;
-        for (int32_t kk = beg; kk < end; kk += 128) {
+        for (int32_t o = 0; o < len; o += 128) {
             int32_t jf = 0;
-            const int pos = warp_scan<4>(a.in_col, tbm, kk, end, &jf);
+            const int pos = warp_scan<4>(a.in_col, tbm, beg + o, len - o, &jf);
             if (pos < 128) {
                 if (!hit) {
                     hit = true;
                     par = jf;
-                    hit_at = kk + pos;
+                    hit_at = beg + o + pos;
                 }
                 if (a.early_exit) break;
             }
-            ex += (unsigned long long)(end - kk < 128 ? end - kk : 128);
+            ex += (unsigned long long)(len - o < 128 ? len - o : 128);
         }
         bool isnew = false;
         int32_t od = 0;

@@ -215,15 +215,15 @@ __device__ __forceinline__ void mp_pull(const MpArgs& a, uint8_t* list) {
         float x[kMpUnroll];
 #pragma unroll
         for (int t = 0; t < kMpUnroll; ++t) {
-            const int32_t e = k + sub + G * t;
-            const bool in = v >= 0 && e < end;
-            c[t] = in ? __ldg(a.pull_col + e) : -1;
-            x[t] = in ? __ldg(a.pull_val + e) : INFINITY;
+            const int32_t o = sub + G * t;
+            const bool in = v >= 0 && o < end - k;  // (a position past the row's end need not fit 32 bits)
+            c[t] = in ? __ldg(a.pull_col + k + o) : -1;
+            x[t] = in ? __ldg(a.pull_val + k + o) : INFINITY;
         }
 #pragma unroll
         for (int t = 0; t < kMpUnroll; ++t)
             if (c[t] >= 0) m = fminf(m, x[t] + __ldg(a.u + c[t]));
-        k += G * kMpUnroll;
+        k = end - k > G * kMpUnroll ? k + G * kMpUnroll : end;
         const bool done = v >= 0 && k >= end;
         const bool defer = v >= 0 && end - k > kLong;
         if (!__any_sync(0xffffffffu, done || defer)) continue;
@@ -300,16 +300,16 @@ __global__ void __launch_bounds__(kMxvThreads) mp_last_kernel(const __grid_const
         const int32_t v = a.q[1][h];
         const int32_t rend = __ldg(a.pull_ptr + v + 1);
         const int32_t beg = a.qp[1][h] + (int32_t)(c - a.qd[1][h]) * kMpChunk;
-        const int32_t end = rend - beg < kMpChunk ? rend : beg + kMpChunk;
+        const int32_t len = rend - beg < kMpChunk ? rend - beg : kMpChunk;
         float m = INFINITY;
-        for (int32_t k = beg + lane; k < end; k += 32 * kMpUnroll) {
+        for (int32_t o = lane; o < len; o += 32 * kMpUnroll) {
             int32_t j[kMpUnroll];
             float x[kMpUnroll];
 #pragma unroll
             for (int t = 0; t < kMpUnroll; ++t) {
-                const bool in = k + 32 * t < end;
-                j[t] = in ? __ldg(a.pull_col + k + 32 * t) : -1;
-                x[t] = in ? __ldg(a.pull_val + k + 32 * t) : INFINITY;
+                const bool in = o + 32 * t < len;
+                j[t] = in ? __ldg(a.pull_col + beg + o + 32 * t) : -1;
+                x[t] = in ? __ldg(a.pull_val + beg + o + 32 * t) : INFINITY;
             }
 #pragma unroll
             for (int t = 0; t < kMpUnroll; ++t)

@@ -496,7 +496,7 @@ __device__ __forceinline__ void ms_pull(const MsArgs& a, int32_t L, int32_t c0, 
                         ac.x[j] = 0ull;
                     }
 #pragma unroll
-                    for (int t = 0; t < kMsUnroll; ++t) u[t] = k + t < end ? __ldg(a.in_col + k + t) : -1;
+                    for (int t = 0; t < kMsUnroll; ++t) u[t] = t < end - k ? __ldg(a.in_col + k + t) : -1;
                 }
                 next += __popc(need);
             }
@@ -506,9 +506,9 @@ __device__ __forceinline__ void ms_pull(const MsArgs& a, int32_t L, int32_t c0, 
             for (int t = 0; t < kMsUnroll; ++t)
                 x[t] = u[t] >= 0 && wok ? ld_words<WL>(a.V + (size_t)u[t] * a.W + w) : zero_words<WL>();
             const int32_t left = end - k;
-            k += kMsUnroll;
+            k = left > kMsUnroll ? k + kMsUnroll : end;  // (a position past the row's end need not fit 32 bits)
 #pragma unroll
-            for (int t = 0; t < kMsUnroll; ++t) u[t] = v >= 0 && k + t < end ? __ldg(a.in_col + k + t) : -1;
+            for (int t = 0; t < kMsUnroll; ++t) u[t] = v >= 0 && t < end - k ? __ldg(a.in_col + k + t) : -1;
             bool cov = true;
 #pragma unroll
             for (int j = 0; j < WL; ++j) {
@@ -532,14 +532,14 @@ __device__ __forceinline__ void ms_pull(const MsArgs& a, int32_t L, int32_t c0, 
                     at.x[j] = __shfl_sync(0xffffffffu, ac.x[j], t0 + gr.sub);
                 }
                 const int32_t step = kMsUnroll * (32 / gr.size);
-                const int32_t stop = et - kt > kMsScan * step ? kt + kMsScan * step : et;
-                int32_t kk = kt;
+                const int32_t len = et - kt > kMsScan * step ? kMsScan * step : et - kt;
+                int32_t at_k = 0;
                 bool all = false;
-                while (kk < stop && !all) {
+                while (at_k < len && !all) {
                     int32_t uu[kMsUnroll];
-                    const int32_t kg = kk + kMsUnroll * (gr.first / gr.size);
+                    const int32_t kg = at_k + kMsUnroll * (gr.first / gr.size);
 #pragma unroll
-                    for (int t = 0; t < kMsUnroll; ++t) uu[t] = kg + t < stop ? __ldg(a.in_col + kg + t) : -1;
+                    for (int t = 0; t < kMsUnroll; ++t) uu[t] = kg + t < len ? __ldg(a.in_col + kt + kg + t) : -1;
                     Words<WL> y[kMsUnroll];
 #pragma unroll
                     for (int t = 0; t < kMsUnroll; ++t)
@@ -553,14 +553,14 @@ __device__ __forceinline__ void ms_pull(const MsArgs& a, int32_t L, int32_t c0, 
                         c &= (at.x[j] & ut.x[j]) == ut.x[j];
                     }
                     all = __all_sync(0xffffffffu, c);
-                    kk += step;
+                    at_k += step;
                 }
                 if (gr.first == t0) {
                     ac = at;
-                    k = kk;
-                    done = all || kk >= et;
+                    k = et - kt > at_k ? kt + at_k : et;
+                    done = all || k >= et;
                     put_off = !done;
-                    if (gr.sub == 0) acc.exam += chunks256 * (uint32_t)((kk < et ? kk : et) - kt);
+                    if (gr.sub == 0) acc.exam += chunks256 * (uint32_t)(k - kt);
                 }
             }
             Words<WL> nw;
@@ -634,7 +634,7 @@ __device__ __forceinline__ void ms_pull_long(const MsArgs& a, unsigned long long
         const int32_t v = lr.row[e];
         const int32_t rend = __ldg(a.in_ptr + v + 1);
         const int32_t beg = lr.k[e] + (c - lr.base[e]) * kMsChunk;
-        const int32_t end = rend - beg < kMsChunk ? rend : beg + kMsChunk;
+        const int32_t len = rend - beg < kMsChunk ? rend - beg : kMsChunk;
         const size_t iv = (size_t)v * a.W + w;
         Words<WL> unv = zero_words<WL>(), ac = zero_words<WL>();
         if (wok) {
@@ -644,24 +644,24 @@ __device__ __forceinline__ void ms_pull_long(const MsArgs& a, unsigned long long
                 unv.x[j] = ~(vis.x[j] | __ldcg(Fn + iv + j)) & lane_mask(a.S, w + j);
         }
         if (!__any_sync(0xffffffffu, unv.any())) continue;
-        int32_t k0 = beg;
+        int32_t k0 = 0;
         const int32_t kofs = kMsUnroll * (gr.first / gr.size);
         int32_t u[kMsUnroll];  // the group's in-neighbours of this step; the next step's are loaded meanwhile
 #pragma unroll
-        for (int t = 0; t < kMsUnroll; ++t) u[t] = k0 + kofs + t < end ? __ldg(a.in_col + k0 + kofs + t) : -1;
-        while (k0 < end) {
+        for (int t = 0; t < kMsUnroll; ++t) u[t] = kofs + t < len ? __ldg(a.in_col + beg + kofs + t) : -1;
+        while (k0 < len) {
             Words<WL> x[kMsUnroll];
 #pragma unroll
             for (int t = 0; t < kMsUnroll; ++t)
                 x[t] = u[t] >= 0 && wok ? ld_words<WL>(a.V + (size_t)u[t] * a.W + w) : zero_words<WL>();
             k0 += step;
 #pragma unroll
-            for (int t = 0; t < kMsUnroll; ++t) u[t] = k0 + kofs + t < end ? __ldg(a.in_col + k0 + kofs + t) : -1;
+            for (int t = 0; t < kMsUnroll; ++t) u[t] = k0 + kofs + t < len ? __ldg(a.in_col + beg + k0 + kofs + t) : -1;
 #pragma unroll
             for (int j = 0; j < WL; ++j)
 #pragma unroll
                 for (int t = 0; t < kMsUnroll; ++t) ac.x[j] |= x[t].x[j];
-            if (k0 < end && ((k0 - beg) & (kMsCheck - 1)) != 0) continue;
+            if (k0 < len && (k0 & (kMsCheck - 1)) != 0) continue;
             bool cov = true;
 #pragma unroll
             for (int j = 0; j < WL; ++j) {
@@ -670,7 +670,7 @@ __device__ __forceinline__ void ms_pull_long(const MsArgs& a, unsigned long long
             }
             if (__all_sync(0xffffffffu, cov)) break;
         }
-        if ((threadIdx.x & 31) == 0) acc.exam += chunks256 * (uint32_t)((k0 < end ? k0 : end) - beg);
+        if ((threadIdx.x & 31) == 0) acc.exam += chunks256 * (uint32_t)(k0 < len ? k0 : len);
         if (gr.first == 0)
 #pragma unroll
             for (int j = 0; j < WL; ++j)
@@ -929,16 +929,16 @@ __device__ __forceinline__ void ms_push_mesh(const MsArgs& a, int32_t L, const I
         if (__any_sync(0xffffffffu, more)) {  // rows of more than four entries: the rest, four lanes each
 #pragma unroll
             for (int k = 0; k < K; ++k) {
-                int32_t x = 0, end = 0;
+                int32_t beg = 0, deg = 0;
                 if (u[k] >= 0) {
-                    x = __ldg(a.out_ptr + u[k]) + 4 + j;
-                    end = __ldg(a.out_ptr + u[k] + 1);
+                    beg = __ldg(a.out_ptr + u[k]);
+                    deg = __ldg(a.out_ptr + u[k] + 1) - beg;
                 }
-                for (; __any_sync(0xffffffffu, x < end); x += 4) {
+                for (int32_t x = 4 + j; __any_sync(0xffffffffu, x < deg); x += 4) {
                     bool first = false;
                     int32_t v = 0;
-                    if (x < end) {
-                        v = __ldg(a.out_col + x);
+                    if (x < deg) {
+                        v = __ldg(a.out_col + beg + x);
                         const unsigned long long o = atomicOr(a.V + v, f[k]);
                         const unsigned long long p = (f[k] & ~o) ? atomicOr(Fn + v, f[k] & ~o) : ~0ull;
                         first = ms_mesh_gain(a, L, v, f[k], o, once ? p : 0ull, rows, acc);

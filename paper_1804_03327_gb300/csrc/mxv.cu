@@ -76,13 +76,14 @@ __device__ __forceinline__ void mxv_long_rows(const PullArgs& a, PullSmem& sm, u
         const int32_t i = sm.longs[h].x, beg = sm.longs[h].y, end = a.ptr[i + 1];
         if (threadIdx.x == 0) sm.hit = 0;
         __syncthreads();
-        for (int32_t k0 = beg + 512 * wib; k0 < end; k0 += 512 * (kMxvThreads / 32)) {
+        // (offsets from beg and entries left: positions past a row's end need not fit 32 bits)
+        for (int64_t o = 512 * wib; o < end - beg; o += 512 * (kMxvThreads / 32)) {
             if (a.early_exit && *(volatile int*)&sm.hit) break;
-            const int32_t k1 = end - k0 > 512 ? k0 + 512 : end;
-            for (int32_t kk = k0; kk < k1; kk += 128) {
+            const int32_t k0 = beg + (int32_t)o, len = end - k0 < 512 ? end - k0 : 512;
+            for (int32_t kk = 0; kk < len; kk += 128) {
                 int32_t j[4];
 #pragma unroll
-                for (int q = 0; q < 4; ++q) j[q] = kk + 32 * q + lane < k1 ? a.col[kk + 32 * q + lane] : -1;
+                for (int q = 0; q < 4; ++q) j[q] = kk + 32 * q + lane < len ? a.col[k0 + kk + 32 * q + lane] : -1;
                 bool hit = false;
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
@@ -201,9 +202,9 @@ __device__ __forceinline__ void mxv_pull(const PullArgs& a, PullSmem& sm) {
                 }
             }
             if (i >= 0 && !(fresh && next)) {
-                const int32_t lim = end < beg + kMxvProbe ? end : beg + kMxvProbe;
+                const int32_t own = (end - beg < kMxvProbe ? end - beg : kMxvProbe) - (k - beg);  // left to the lane
 #pragma unroll
-                for (int t = 0; t < 4; ++t) x[t] = k + t < lim ? ld_stream(col + k + t) : -1;
+                for (int t = 0; t < 4; ++t) x[t] = t < own ? ld_stream(col + k + t) : -1;
             }
             const bool hit0 = f0 >= 0 && bit_test(ubm, f0);
             bool h[4];
@@ -228,7 +229,7 @@ __device__ __forceinline__ void mxv_pull(const PullArgs& a, PullSmem& sm) {
                 done |= k >= end;
             }
             // past the lane probe: the whole warp, or the whole block once its tiles are done
-            const bool past = i >= 0 && !done && k >= beg + kMxvProbe;
+            const bool past = i >= 0 && !done && k - beg >= kMxvProbe;
             if (past && end - k > kMxvLongRow) {
                 const int slot = atomicAdd(&sm.nlong, 1);
                 if (slot < kMxvLongs) {
@@ -240,24 +241,21 @@ __device__ __forceinline__ void mxv_pull(const PullArgs& a, PullSmem& sm) {
             while (pend) {
                 const int t = __ffs(pend) - 1;
                 pend &= pend - 1;
-                int32_t kk = __shfl_sync(0xffffffffu, k, t);
-                const int32_t ee = __shfl_sync(0xffffffffu, end, t);
+                const int32_t kk = __shfl_sync(0xffffffffu, k, t);
+                int32_t ahead = __shfl_sync(0xffffffffu, end, t) - kk;  // entries left
                 bool tf = __shfl_sync(0xffffffffu, found, t);
                 unsigned long long tx = 0;
                 // 128 entries per round (four independent loads per lane)
-                for (; kk < ee; kk += 128) {
+                for (int64_t o = kk; ahead > 0; o += 128, ahead -= 128) {
                     int32_t jq[4];
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        const int32_t idx = kk + 32 * q + lane;
-                        jq[q] = idx < ee ? col[idx] : -1;
-                    }
+                    for (int q = 0; q < 4; ++q) jq[q] = 32 * q + lane < ahead ? col[o + 32 * q + lane] : -1;
                     bool stop = false;
 #pragma unroll
                     for (int q = 0; q < 4; ++q) {
                         if (stop) break;
                         const uint32_t hb = __ballot_sync(0xffffffffu, jq[q] >= 0 && bit_test(ubm, jq[q]));
-                        const int32_t left = ee - (kk + 32 * q);
+                        const int32_t left = ahead - 32 * q;
                         if (left <= 0) break;
                         if (hb) {
                             tf = true;

@@ -238,15 +238,15 @@ __global__ void __launch_bounds__(kSpThreads, 1) sssp_cluster_kernel(const __gri
                 sp_relax(a, sm, np, f, base, live && w >= 0, w, x + len, T);
                 const uint32_t mm = __ballot_sync(0xffffffffu, more);
                 if (mm) {
-                    int32_t k = 0, end = 0;
+                    int32_t beg = 0, deg = 0;
                     if ((mm >> (lane | (kSpLanes - 1))) & 1u) {
-                        k = __ldg(a.ptr + u) + kSpLanes + j;
-                        end = __ldg(a.ptr + u + 1);
+                        beg = __ldg(a.ptr + u);
+                        deg = __ldg(a.ptr + u + 1) - beg;
                     }
-                    for (; __any_sync(0xffffffffu, k < end); k += kSpLanes) {
-                        const bool in = k < end;
-                        const int32_t v = in ? __ldg(a.col + k) : 0;
-                        const float d = in ? x + __ldg(a.val + k) : 0.0f;
+                    for (int32_t k = kSpLanes + j; __any_sync(0xffffffffu, k < deg); k += kSpLanes) {
+                        const bool in = k < deg;
+                        const int32_t v = in ? __ldg(a.col + beg + k) : 0;
+                        const float d = in ? x + __ldg(a.val + beg + k) : 0.0f;
                         sp_relax(a, sm, np, f, base, in, v, d, T);
                     }
                 }
