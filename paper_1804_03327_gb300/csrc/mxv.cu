@@ -78,7 +78,8 @@ __device__ __forceinline__ void mxv_long_rows(const PullArgs& a, PullSmem& sm, u
         __syncthreads();
         // (offsets from beg and entries left: positions past a row's end need not fit 32 bits)
         for (int64_t o = 512 * wib; o < end - beg; o += 512 * (kMxvThreads / 32)) {
-            if (a.early_exit && *(volatile int*)&sm.hit) break;
+            // the whole warp stops or goes on: another warp, or its own lane 0, may just be writing the word
+            if (a.early_exit && __any_sync(0xffffffffu, *(volatile int*)&sm.hit)) break;
             const int32_t k0 = beg + (int32_t)o, len = end - k0 < 512 ? end - k0 : 512;
             for (int32_t kk = 0; kk < len; kk += 128) {
                 int32_t j[4];
