@@ -319,7 +319,15 @@ constexpr int32_t kSpMeshDegree = 32;
 gbx_status sssp_cluster_prepare(Graph* G, cudaStream_t s) {
     G->sp_step = -1.0f;
     if (G->max_out_degree > kSpMeshDegree || G->nnz == 0) return GBX_OK;
-    if (!G->sp_rec) GBX_CUDA_TRY(cudaMalloc(&G->sp_rec, 32 * (size_t)G->n));
+    if (!G->sp_rec) {
+        const cudaError_t e = cudaMalloc(&G->sp_rec, 32 * (size_t)G->n);
+        if (e == cudaErrorMemoryAllocation) {  // the weights are in; searches run on the whole grid
+            G->sp_rec = nullptr;
+            cudaGetLastError();
+            return GBX_OK;
+        }
+        GBX_CUDA_TRY(e);
+    }
     int4* rcol = static_cast<int4*>(G->sp_rec);
     const unsigned grid = std::min<unsigned>(div_up(G->n, 256), (unsigned)G->num_sms * 8u);
     sp_records_kernel<<<grid, 256, 0, s>>>(G->out_ptr, G->out_col, G->out_val, G->n, rcol,

@@ -86,3 +86,34 @@ def test_weights_replaced_by_negative_ones():
         else:  # with negative weights the rounding depends on the schedule
             assert np.allclose(dist.cpu().numpy(), want, rtol=1e-4)
     g.free()
+
+
+def test_weights_without_memory_for_the_mesh_records():
+    """The records only make searches faster: weights are accepted where there is no room for them."""
+    n = 8_000_000  # weights and row list: 128 MB, the records: 256 MB
+    s = torch.arange(n - 1, dtype=torch.int32, device="cuda")
+    w = torch.ones(n - 1, dtype=torch.float32, device="cuda")
+    small = gbx.graph_build(3, s[:2].contiguous(), (s[:2] + 1).contiguous())
+    gbx.graph_set_weights(small, s[:2].contiguous(), (s[:2] + 1).contiguous(), w[:2].contiguous())  # kernels loaded
+    # a path of 1,000 vertices among pairs, so that the whole grid has few iterations
+    d = torch.where((s < 1000) | (s % 2 == 0), s + 1, s)
+    g = gbx.graph_build(n, s, d)
+    dist = torch.empty(n, dtype=torch.float32, device="cuda")
+    want = np.full(n, np.inf, np.float32)
+    want[:1002] = np.arange(1002)
+    gbx.sssp(small, 0, torch.empty(3, dtype=torch.float32, device="cuda"))
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    free, _ = torch.cuda.mem_get_info()
+    held = torch.empty(free - (200 << 20), dtype=torch.uint8, device="cuda")
+    for room in (False, True):
+        if room:
+            del held
+            torch.cuda.empty_cache()
+        gbx.graph_set_weights(g, s, d, w)
+        dist.fill_(-1.0)
+        gbx.sssp(g, 0, dist)
+        gbx.graph_sync(g)
+        assert np.array_equal(dist.cpu().numpy(), want)
+    g.free()
+    small.free()
