@@ -189,8 +189,14 @@ __device__ __forceinline__ void mp_pull(const MpArgs& a, uint8_t* list) {
             __syncwarp();
             open = __popc(with);
             next = 0;
-            // rows without entries (or that do not pass) are settled here
-            if (tile < ntiles && e0 == b0 && base + lane < a.n && !a.accum) a.w[base + lane] = INFINITY;
+            // rows without entries (or that do not pass) are settled here; min(NaN, +inf) is +inf where a
+            // row passes
+            if (tile < ntiles && e0 == b0 && base + lane < a.n) {
+                if (!a.accum)
+                    a.w[base + lane] = INFINITY;
+                else if (mp_pass(a, base + lane) && isnan(a.w[base + lane]))
+                    a.w[base + lane] = INFINITY;
+            }
         }
         if (need && next < open) {
             const int r = next + __popc(need & ((1u << first) - 1u));  // the group's place among those without a row

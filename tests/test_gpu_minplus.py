@@ -231,3 +231,24 @@ def test_sssp_pull_chunk_borders(shape):
             gbx.graph_sync(g)
             assert np.array_equal(dist.cpu().numpy(), want), (shape, src, desc.direction, desc.alpha)
     g.free()
+
+
+@pytest.mark.parametrize("direction", [gbx.DIR_AUTO, gbx.DIR_PULL])
+def test_accumulating_pull_takes_nan_as_no_value(direction):
+    """min(NaN, x) = x: a row that passes the mask loses a NaN in w also where it has no entries."""
+    n = 100
+    s = np.arange(0, 40, dtype=np.int32)
+    d = (s + 50).astype(np.int32)  # rows 50 .. 89 have an entry, the others none
+    wgt = np.full(len(s), 2.0, np.float32)
+    g = gbx.graph_build(n, s, d, symmetrize=False)
+    gbx.graph_set_weights(g, s, d, wgt)
+    u = np.full(n, 1.0, np.float32)
+    m = (np.arange(n) % 3 != 0).astype(np.uint8)
+    old = np.where(np.arange(n) % 2 == 0, np.float32(np.nan), np.float32(5.0))
+    w, m_d, u_d = torch.from_numpy(old.copy()).cuda(), torch.from_numpy(m).cuda(), torch.from_numpy(u).cuda()
+    gbx.mxv(gbx.dense_f32(w), gbx.dense(m_d), gbx.MIN_PLUS_F32, g, gbx.dense_f32(u_d),
+            gbx.desc_init(accum=1, direction=direction, alpha=0.0))
+    t = np.where((np.arange(n) >= 50) & (np.arange(n) < 90), np.float32(3.0), np.float32(np.inf))
+    want = np.where(m != 0, np.fmin(old, t), old)
+    assert np.array_equal(w.cpu().numpy(), want, equal_nan=True)
+    g.free()
