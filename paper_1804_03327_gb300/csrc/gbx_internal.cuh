@@ -20,6 +20,7 @@ uint64_t wait_timeout_ns();
     do {                                                                                                  \
         cudaError_t err__ = (expr);                                                                       \
         if (err__ != cudaSuccess) {                                                                       \
+            (void)cudaGetLastError(); /* reported by this call, not again by the next one's checks */     \
             ::gbx::set_error(std::string(#expr) + ": " + cudaGetErrorString(err__) + " (" + __FILE__ + ":" + \
                              std::to_string(__LINE__) + ")");                                             \
             return err__ == cudaErrorMemoryAllocation ? GBX_ERR_OUT_OF_MEMORY : GBX_ERR_CUDA;             \

@@ -46,3 +46,21 @@ def test_build_and_weights(n, m, kind):
                 assert np.array_equal(gbx.graph_weights(g, False), og.out_val)
                 assert np.array_equal(gbx.graph_weights(g, True), og.in_val)
             g.free()
+
+
+def test_a_build_that_found_no_memory_leaves_the_next_one_alone():
+    n, s, d = 30_000_000, np.zeros(1, np.int32), np.ones(1, np.int32)  # some 2.5 GB
+    gbx.graph_build(10, s, d).free()
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    free, _ = torch.cuda.mem_get_info()
+    held = torch.empty(free - (300 << 20), dtype=torch.uint8, device="cuda")
+    with pytest.raises(gbx.GbxError):
+        gbx.graph_build(n, s, d)
+    g = gbx.graph_build(10, s, d)
+    depth = torch.empty(10, dtype=torch.int32, device="cuda")
+    gbx.bfs(g, 0, depth)
+    gbx.graph_sync(g)
+    assert depth.tolist() == [0, 1] + [-1] * 8
+    del held
+    g.free()
