@@ -28,7 +28,7 @@ struct MpArgs {
     MxvVec mask;
     uint32_t invert;
     int32_t accum, dir, group;
-    float alpha;
+    int32_t push_most;  // finite entries of u up to which AUTO pushes
     const float* u;
     float* w;
     const int32_t* pull_ptr;
@@ -48,7 +48,7 @@ struct MpArgs {
 
 __device__ __forceinline__ int mp_dir(const MpArgs& a) {
     if (a.dir != GBX_DIR_AUTO) return a.dir;
-    return (double)(int32_t)a.ctr->n_new / (double)a.n <= (double)a.alpha ? GBX_DIR_PUSH : GBX_DIR_PULL;
+    return (int32_t)a.ctr->n_new <= a.push_most ? GBX_DIR_PUSH : GBX_DIR_PULL;
 }
 
 __device__ __forceinline__ bool mp_pass(const MpArgs& a, int32_t i) {
@@ -346,7 +346,7 @@ gbx_status mxv_minplus(Graph* G, float* w, const MxvVec& mask, const float* u, c
     a.accum = d.accum ? 1 : 0;
     a.dir = d.direction;
     a.group = G->nnz > 12ll * G->n ? 8 : (G->nnz > 6ll * G->n ? 4 : 1);
-    a.alpha = d.alpha;
+    a.push_most = mxv_push_most(G->n, d.alpha);
     a.u = u;
     a.w = w;
     a.pull_ptr = d.transpose ? G->in_ptr : G->out_ptr;

@@ -309,7 +309,7 @@ struct MxvArgs {
     MxvVec u, mask, w;
     uint32_t invert;  // the mask's complement: all ones
     int32_t accum, dir, early_exit;
-    float alpha;
+    int32_t push_most;  // nonzeros of u up to which AUTO pushes
     PullArgs pull;
     const int32_t* push_ptr;
     const int32_t* push_col;
@@ -328,11 +328,10 @@ struct MxvArgs {
     MxvStats* stats;
 };
 
-// AUTO: push when nnz(u)/n <= alpha (input sparsity), else pull (Section 6.3).
 __device__ __forceinline__ int mxv_dir(const MxvArgs& a) {
     if (a.dir != GBX_DIR_AUTO) return a.dir;
     const int32_t c = a.u.format == GBX_SPARSE ? *a.u.count : (int32_t)a.ctr->n_new;
-    return (double)c / (double)a.n <= (double)a.alpha ? GBX_DIR_PUSH : GBX_DIR_PULL;
+    return c <= a.push_most ? GBX_DIR_PUSH : GBX_DIR_PULL;
 }
 
 // A queue of the columns a push expands: vertex, exclusive prefix of the columns' lengths, column
@@ -687,7 +686,7 @@ static gbx_status mxv_bool(Graph* G, gbx_vector* w, const gbx_vector* mask, cons
     a.invert = d.mask_complement ? 0xffffffffu : 0u;
     a.accum = d.accum ? 1 : 0;
     a.dir = d.direction;
-    a.alpha = d.alpha;
+    a.push_most = mxv_push_most(G->n, d.alpha);
     a.early_exit = d.early_exit ? 1 : 0;
     a.stats = d.trace ? reinterpret_cast<MxvStats*>(G->ws.ctr + 3) : nullptr;
     a.push_ptr = d.transpose ? G->out_ptr : G->in_ptr;

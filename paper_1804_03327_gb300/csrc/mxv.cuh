@@ -76,6 +76,18 @@ gbx_status pdl_launch(void (*fn)(A), unsigned blocks, const A& a, bool dependent
     return GBX_OK;
 }
 
+// AUTO pushes while count / n <= alpha (input sparsity, Section 6.3): the largest such count.  The
+// division is the host's: binary64 is slow here, and every thread of a kernel dividing took 8 of the
+// 12 us of an otherwise empty one.
+inline int32_t mxv_push_most(int32_t n, float alpha) {
+    const double a = (double)alpha;
+    if (a * (double)n >= 2147483647.0) return INT32_MAX;
+    int32_t c = (int32_t)(a * (double)n);
+    while (c < INT32_MAX && (double)(c + 1) / (double)n <= a) ++c;
+    while (c > 0 && (double)c / (double)n > a) --c;
+    return c;
+}
+
 // What gbx_mxv reads, as bitmaps and queues (mxv.cu).
 struct MxvVec {
     int32_t format;  // GBX_DENSE, GBX_SPARSE or GBX_DENSE_F32; -1: none

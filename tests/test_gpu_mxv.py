@@ -241,3 +241,28 @@ def test_push_sort_is_mxv_only():
     with pytest.raises(gbx.GbxError) as e:
         gbx.mxv(gbx.dense(t), None, gbx.LOR_LAND, g, gbx.dense(torch.zeros_like(t)), gbx.desc_init(push_sort=2))
     assert e.value.status == gbx.ERR_INVALID_VALUE
+
+
+@pytest.mark.parametrize("n", [1, 3, 7, 100, 1021])
+def test_auto_switches_at_the_quotient(n):
+    """AUTO pushes while nnz(u) / n <= alpha, the division in binary64 and alpha a binary32 number:
+    alpha on both sides of every quotient."""
+    s = np.arange(n, dtype=np.int32)
+    g = gbx.graph_build(n, s, (s + 1) % n, symmetrize=False)
+    w, w_d = torch.empty(n, dtype=torch.int32, device="cuda"), torch.empty(n, dtype=torch.uint8, device="cuda")
+    wn = torch.zeros(1, dtype=torch.int32, device="cuda")
+    for c in sorted({0, 1, n // 3, n // 2, n - 1, n}):
+        ids = torch.arange(max(c, 1), dtype=torch.int32, device="cuda")
+        cnt = torch.tensor([c], dtype=torch.int32, device="cuda")
+        bits = torch.zeros(n, dtype=torch.uint8, device="cuda")
+        bits[:c] = 1
+        q = np.float32(c / n)
+        for alpha in {np.nextafter(q, np.float32(-1)), q, np.nextafter(q, np.float32(2)), np.float32(1e30)}:
+            if alpha < 0:
+                continue
+            push = c / n <= float(alpha)
+            for u, out in ((gbx.sparse(ids, cnt, n), gbx.sparse(w, wn, n)), (gbx.dense(bits), gbx.dense(w_d))):
+                gbx.mxv(out, None, gbx.LOR_LAND, g, u, gbx.desc_init(alpha=float(alpha), trace=1))
+                st = gbx.mxv_stats(g)
+                assert (st["rows"] == 0) == (push or n == 1) and st["u_nnz"] == (c if push else 0), (c, alpha, st)
+    g.free()
