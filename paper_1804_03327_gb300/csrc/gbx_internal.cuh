@@ -182,6 +182,7 @@ struct Graph {
     int bfs_blocks = 0;  // BFS launch geometry
     int cluster_blocks = 0;  // ... blocks of the cluster kernel (0: not asked yet, -1: none fits)
     int32_t max_out_degree = 0;
+    int32_t max_in_degree = 0;
     // SSSP on meshes (sssp_cluster.cu), made with the weights
     void* sp_rec = nullptr;     // records of the first four out-edges: int4[n], float4[n]
     float sp_step = -1.0f;      // step of the near-far threshold (negative: not used)

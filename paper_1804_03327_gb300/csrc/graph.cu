@@ -156,7 +156,7 @@ __global__ void __launch_bounds__(256)
         most = max(most, d);
     }
     most = __reduce_max_sync(0xffffffffu, most);
-    if (lane == 0 && longest && most > 0) atomicMax(longest, most);
+    if (lane == 0 && most > 0) atomicMax(longest, most);
 }
 
 static unsigned grid_for(int64_t work) { return (unsigned)std::max<int64_t>(1, std::min<int64_t>((work + 255) / 256, 152 * 32)); }
@@ -375,15 +375,18 @@ static gbx_status build_impl(Graph* g, int32_t n, int64_t m, const int32_t* src,
         GBX_TRY(keys_to_csr(keys, alt, K, n, b, drop != 0, sort_tmp, counts, g->ws.status, g->in_ptr, &g->in_col, &nnz_t, s));
         GBX_CHECK(nnz_t == g->nnz, GBX_ERR_CUDA, "internal: transpose has a different edge count");
     }
-    int32_t* const longest = g->ws.flag + 10;  // zero since the workspace was made
+    int32_t* const longest = g->ws.flag + 10;  // of the out-rows and of the in-rows: zero since the workspace was made
     row_heads_kernel<<<grid_for(n), 256, 0, s>>>(g->out_ptr, g->out_col, n, g->first_out, g->next_out, g->nz_out,
                                                  g->multi_out, longest);
     if (!sym)
         row_heads_kernel<<<grid_for(n), 256, 0, s>>>(g->in_ptr, g->in_col, n, g->first_in, g->next_in, g->nz_in,
-                                                     g->multi_in, nullptr);
+                                                     g->multi_in, longest + 1);
     GBX_CUDA_TRY(cudaGetLastError());
-    GBX_CUDA_TRY(cudaMemcpyAsync(&g->max_out_degree, longest, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+    int32_t most[2] = {0, 0};
+    GBX_CUDA_TRY(cudaMemcpyAsync(most, longest, sizeof(most), cudaMemcpyDeviceToHost, s));
     GBX_CUDA_TRY(cudaStreamSynchronize(s));
+    g->max_out_degree = most[0];
+    g->max_in_degree = sym ? most[0] : most[1];
     return GBX_OK;
 }
 
