@@ -46,8 +46,14 @@ constexpr int kClNear = 1024;                       // ... of which with neighbo
 constexpr int kClBmWords = 15360;                   // bitmap words a block holds (n up to 7.8M in 16 blocks)
 constexpr int kClAhead = 2 * kClPerRound;            // block share up to which neighbours are loaded ahead
 constexpr int kClShareWhole = 16;                   // queue length from which a small graph's levels are shared
-// The frontier size at which the cluster hands over to the grid.
+// The frontier at which the cluster hands over to the grid: the edges of that many average rows, at
+// most kClMaxFrontier vertices.  The cluster takes about 5,000 edges a microsecond, a grid-wide
+// level 8 to 10 us.  Random 16-regular graph of 30,000 vertices: 62 us, on the grid alone 79, with
+// 24,576 vertices as the only limit 155; 126 x 126 x 126 grid 2.61 ms, 2.70 and 2.86.  48K edges: 2.49
+// there, but a ring of 500,000 vertices with one edge in a thousand rewired 1.87 ms instead of 1.33;
+// 96K and 128K: 2.87 on the 3-D grid.  2-D grids keep below it (a 2000 x 2000 one 5.58 ms with all).
 constexpr int kClMaxFrontier = 24576;
+constexpr int64_t kClMaxEdges = 64 * 1024;
 
 struct ClArgs {
     int32_t n, nwords, source;
@@ -64,6 +70,7 @@ struct ClArgs {
     int32_t* status;
     int32_t fill;   // initialise the outputs and the bitmap here (else cl_fill_kernel did)
     int32_t whole;  // the graph fits: never hand over
+    int32_t max_frontier;  // ... else above this many vertices
     unsigned long long timeout_ns;
     int32_t shared_bm;  // the visited bitmap is in shared memory (block r: words w with w mod blocks = r)
 };
@@ -342,7 +349,7 @@ __global__ void __launch_bounds__(kClThreads, 1) bfs_cluster_kernel(const __grid
             return;
         }
         int32_t inc = 0;  // the blocks' queues one after another: where each one ends
-        if (!a.whole && (total > kClMaxFrontier || most > kClCap)) {
+        if (!a.whole && (total > a.max_frontier || most > kClCap)) {
             // hand over: the queues one after another (the spilled entries are listed already)
             cluster_barrier();  // every claim is in the bitmap
             if (ld_volatile_i32(&sm.abort)) return;
@@ -415,9 +422,11 @@ static gbx_status cl_geometry(Graph* G) {
 }
 
 // Which searches start in the cluster: those of graphs whose levels stay small.
-//  - no row longer than kClMeshDegree (grids, meshes, roads): frontiers grow by a bounded
-//    factor and there are many levels.  A graph with hubs reaches most of its vertices in a
-//    few levels, which need the whole GPU: RMAT-22 takes 107 us there.
+//  - no row longer than kClMeshDegree.  On grids, meshes and roads there are many small levels.  A
+//    graph of short rows whose frontier grows fast (random regular, small world) is handed
+//    over after a few levels, each still cheaper here: 16 entries a row 63 us for 10,000 vertices
+//    (82 on the grid alone), 80 for 100,000 (109), 91 for 500,000 (96), 235 for 2M (247).  A graph with
+//    hubs reaches most of its vertices in a few levels, which need the whole GPU: RMAT-22 takes 107 us.
 //  - a graph that one block's queue holds (n <= kClCap) with few entries: every level is
 //    small.  RMAT-10 (edge factor 16) takes 25 us here and 44 there, 8,192 vertices of edge
 //    factor 4 37 and 55; at 105K entries the two are even (7,000 vertices of edge factor 16,
@@ -456,6 +465,7 @@ gbx_status cluster_bfs_launch(Graph* G, int32_t source, int32_t* depth, int32_t*
     a.ho = G->ws.handoff;
     a.status = G->ws.status;
     a.whole = cl_tiny(G) ? 1 : 0;
+    a.max_frontier = (int32_t)std::min<int64_t>(kClMaxFrontier, kClMaxEdges * G->n / std::max<int64_t>(G->nnz, 1));
     a.timeout_ns = wait_timeout_ns();
     a.fill = G->n <= (1 << 16) ? 1 : 0;  // 16 blocks write 0.5 MB faster than a launch takes
     const int32_t bm_words = (G->nwords + G->cluster_blocks - 1) / G->cluster_blocks;

@@ -23,3 +23,16 @@ def assert_valid_parents(out_ptr, out_col, depth, parent, source):
     for a, b, pp, vv in zip(starts, ends, p, v):
         k = np.searchsorted(col[a:b], vv)
         assert k < b - a and col[a + k] == vv, f"no edge {pp} -> {vv}"
+
+
+def assert_valid_parents_large(n, pairs, depth, parent, source):
+    """The same for many vertices, without a loop: pairs = (from, to) of the graph's edges."""
+    depth, parent = np.asarray(depth), np.asarray(parent)
+    assert parent[source] == source and np.all(parent[depth < 0] == -1)
+    v = np.flatnonzero(depth >= 0)
+    v = v[v != source]
+    p = parent[v].astype(np.int64)
+    assert np.all((p >= 0) & (p < n)) and np.all(depth[p] == depth[v] - 1)
+    keys = np.unique(pairs[0].astype(np.int64) * n + pairs[1])
+    at = np.searchsorted(keys, p * n + v)
+    assert np.all(keys[np.minimum(at, len(keys) - 1)] == p * n + v)
