@@ -31,7 +31,15 @@ constexpr int kSpThreads = 512;
 constexpr int kSpLanes = 4;                         // lanes per vertex, one neighbour of its record each
 constexpr int kSpPerRound = kSpThreads / kSpLanes;  // vertices a block takes at a time
 constexpr int kSpCap = 6144;                        // near queue entries a block holds
-constexpr int32_t kSpMaxNear = 32768;               // near vertices at which the grid takes over
+// The near queue at which the grid takes over: the edges of that many average rows, at most
+// kSpMaxNear vertices.  A phase of the cluster takes its edges' time on 16 SMs, the hand-over pulls
+// every row.  With 32,768 vertices as the only limit the random 16-regular graph of 30,000 vertices took
+// 170 us (the grid alone 127, now 118); with 128K edges and no share of the entries the 8-regular
+// one of 2M 738 (688, 689), and the 126 x 126 x 126 grid 10.1 ms (13.0, 5.6): it was handed over at its
+// widest.  16K and 32K edges take 2-D grids off the cluster too early (777K vertices 21.5 ms, not 3.7).
+constexpr int32_t kSpMaxNear = 32768;
+constexpr int64_t kSpMaxEdges = 96 * 1024;
+constexpr int64_t kSpMaxShare = 80;  // ... and this fraction of the stored entries
 // T first moves on by this many mean weights; the step is doubled while the near queue keeps
 // below kSpFew vertices from one move to the next (a phase then has idle lanes, and moves cost
 // phases of their own) and halved when it exceeds kSpMany (vertices would improve too often).
@@ -49,7 +57,7 @@ struct SpArgs {
     float* dist;
     int32_t* farv[2];  // far piles: vertices ...
     float* fard[2];    // ... and the distance each was put there with; block r's part is [r seg, r seg + seg)
-    int32_t seg;
+    int32_t seg, max_near;
     float step;
     ClHandoff* ho;
     int32_t* status;
@@ -154,10 +162,10 @@ __global__ void __launch_bounds__(kSpThreads, 1) sssp_cluster_kernel(const __gri
         const int32_t total = (int32_t)__reduce_add_sync(0xffffffffu, (uint32_t)c);
         const bool over = __any_sync(0xffffffffu, fc < 0);  // a far pile overflowed
         const bool far = __any_sync(0xffffffffu, fc > 0);
-        if (over || total > kSpMaxNear || (total == 0 && !far)) {
+        if (over || total > a.max_near || (total == 0 && !far)) {
             if (rank == 0 && t == 0) {
                 // handed over: the distances are those of paths; the grid's pull iterations finish them
-                a.ho->done = over || total > kSpMaxNear ? 0 : 1;
+                a.ho->done = over || total > a.max_near ? 0 : 1;
                 a.status[ST_LEVELS] = ph;
             }
             cluster_barrier();  // no block leaves while another may still write to its shared memory
@@ -312,8 +320,10 @@ __global__ void __launch_bounds__(256) sp_stats_kernel(const float* __restrict__
     }
 }
 
-// Which searches run here: rows of at most kSpMeshDegree entries (frontiers stay short; a graph
-// with hubs reaches most of its vertices in a few iterations of the whole GPU).
+// Which searches run here: rows of at most kSpMeshDegree entries.  On meshes the near queue stays
+// short; random regular graphs and small worlds (10K to 2M vertices, 4 to 16 entries a row, integer
+// and real weights) are handed over early and take 0.31 to 1.04 of the grid's time.  A graph with
+// hubs reaches most of its vertices in a few iterations of the whole GPU.
 constexpr int32_t kSpMeshDegree = 32;
 
 gbx_status sssp_cluster_prepare(Graph* G, cudaStream_t s) {
@@ -368,6 +378,8 @@ gbx_status sssp_cluster_launch(Graph* G, int32_t source, float* dist, cudaStream
         a.fard[i] = reinterpret_cast<float*>(G->ws.qp[i]);
     }
     a.seg = G->n / G->sp_cluster_blocks;
+    a.max_near = (int32_t)std::min<int64_t>(
+        kSpMaxNear, (kSpMaxEdges + G->nnz / kSpMaxShare) * G->n / std::max<int64_t>(G->nnz, 1));
     a.step = G->sp_step;
     a.ho = G->ws.handoff;
     a.status = G->ws.status;

@@ -68,3 +68,22 @@ def test_bfs_across_the_handover(name):
             assert np.array_equal(got, want), src
             assert_valid_parents_large(n, pairs, got, parent.cpu().numpy(), src)
     g.free()
+
+
+@pytest.mark.parametrize("name", sorted(CASES))
+@pytest.mark.parametrize("integer", [0, 1])
+def test_sssp_across_the_handover(name, integer):
+    make, sym = CASES[name]
+    n, s, d = make()
+    r = np.random.default_rng(11)
+    w = (r.integers(1, 65, len(s)) if integer else r.random(len(s)) * 0.9 + 0.1).astype(np.float32)
+    og = oracle.graph_weighted(n, s, d, w, symmetrize=sym)
+    g = gbx.graph_build(n, s, d, symmetrize=sym)
+    gbx.graph_set_weights(g, s, d, w)
+    want = oracle.sssp(og, n // 3)[0]
+    for direction in (gbx.DIR_AUTO, gbx.DIR_PUSH):
+        dist = torch.full((n,), -1.0, dtype=torch.float32, device="cuda")
+        gbx.sssp(g, n // 3, dist, gbx.desc_init(direction=direction))
+        gbx.graph_sync(g)
+        assert np.array_equal(dist.cpu().numpy(), want), direction
+    g.free()
