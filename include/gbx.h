@@ -515,9 +515,11 @@ gbx_status gbx_server_stats(gbx_server* s, int64_t* queued, int32_t* in_flight, 
 /* Wait for batches in flight and release the server (not the graphs). */
 gbx_status gbx_server_destroy(gbx_server* s);
 
-/* Upper bound, in nanoseconds, of every device-side wait in this library (the
- * persistent kernels' grid barriers).  When it runs out the kernel records
- * GBX_ERR_TIMEOUT and returns.  Default 5e9.  Process-wide. */
+/* Upper bound, in nanoseconds, of the polling device-side waits of this library: the
+ * persistent kernels' grid barriers, and the exchange of counts that ends a level of a
+ * thread-block cluster.  When it runs out the kernel records GBX_ERR_TIMEOUT and returns.
+ * The clusters' hardware barrier has no limit of its own: it ends because every block reaches
+ * it, one whose wait ran out included.  Default 5e9.  Process-wide. */
 gbx_status gbx_set_wait_timeout_ns(uint64_t ns);
 
 /* Failure-detection self-test: runs the persistent kernels' bounded grid
@@ -527,6 +529,10 @@ gbx_status gbx_set_wait_timeout_ns(uint64_t ns);
  * error, BFS kernels on g see it at their first barrier and return at once.
  * Asynchronous on `stream`.  Causes no GPU fault. */
 gbx_status gbx_selftest_barrier_timeout(gbx_graph* g, uint64_t timeout_ns, void* stream);
+/* The same for the thread-block clusters that gbx_bfs (GBX_TUNE_BFS) and gbx_sssp (GBX_TUNE_SSSP)
+ * start in: one block withholds what it found, so that every block's wait for it runs out after
+ * timeout_ns and all of them leave.  NOT_SUPPORTED where searches on g do not start in a cluster. */
+gbx_status gbx_selftest_cluster_timeout(gbx_graph* g, int32_t which, uint64_t timeout_ns, void* stream);
 
 #ifdef __cplusplus
 }

@@ -27,6 +27,7 @@
 #include "bfs_cluster.cuh"
 #include "frontier.cuh"
 #include "gbx_internal.cuh"
+#include "sssp_cluster.cuh"
 
 namespace gbx {
 
@@ -1071,6 +1072,17 @@ extern "C" gbx_status gbx_selftest_barrier_timeout(gbx_graph* g, uint64_t timeou
     G->ws.bar_parity ^= 1u;
     GBX_CUDA_TRY(cudaGetLastError());
     G->ws.last_stream = (cudaStream_t)stream;
+    return GBX_OK;
+}
+
+extern "C" gbx_status gbx_selftest_cluster_timeout(gbx_graph* g, int32_t which, uint64_t timeout_ns, void* stream) {
+    clear_error();
+    GBX_TRY(check_graph(g));
+    GBX_CHECK(which == GBX_TUNE_BFS || which == GBX_TUNE_SSSP, GBX_ERR_INVALID_VALUE, "GBX_TUNE_BFS or GBX_TUNE_SSSP");
+    Graph* G = as_impl(g);
+    cudaStream_t s = (cudaStream_t)stream;
+    GBX_TRY(which == GBX_TUNE_BFS ? cluster_bfs_selftest(G, timeout_ns, s) : sssp_cluster_selftest(G, timeout_ns, s));
+    G->ws.last_stream = s;
     return GBX_OK;
 }
 

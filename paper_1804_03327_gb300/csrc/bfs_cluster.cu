@@ -296,6 +296,8 @@ __device__ __forceinline__ void cl_take(const ClArgs& a, ClSmem& sm, const ClSha
     }
 }
 
+// kWithhold: block 1 keeps its queue length to itself, so that every block's wait runs out.
+template <bool kWithhold>
 __global__ void __launch_bounds__(kClThreads, 1) bfs_cluster_kernel(const __grid_constant__ ClArgs a) {
     extern __shared__ __align__(16) unsigned char raw[];
     ClSmem& sm = *reinterpret_cast<ClSmem*>(raw);
@@ -399,7 +401,7 @@ __global__ void __launch_bounds__(kClThreads, 1) bfs_cluster_kernel(const __grid
             __syncthreads();
         }
         // this block's queue length to every block, theirs from them
-        if (t < C)
+        if (t < C && !(kWithhold && rank == 1))
             st_async(remote_smem(&sm.counts[np][rank], (uint32_t)t), sm.cnt[np], remote_smem(&sm.bar[np], (uint32_t)t));
         if (t == 0) mbar_expect(&sm.bar[np], 4u * (uint32_t)C);
         last = total;
@@ -418,7 +420,7 @@ static size_t cl_smem(int32_t bm_words) { return sizeof(ClSmem) + sizeof(uint32_
 
 static gbx_status cl_geometry(Graph* G) {
     if (G->cluster_blocks != 0) return GBX_OK;
-    return cluster_fit((const void*)bfs_cluster_kernel, kClThreads, cl_smem(kClBmWords), &G->cluster_blocks);
+    return cluster_fit((const void*)bfs_cluster_kernel<false>, kClThreads, cl_smem(kClBmWords), &G->cluster_blocks);
 }
 
 // Which searches start in the cluster: those of graphs whose levels stay small.
@@ -447,9 +449,7 @@ gbx_status cluster_bfs_wanted(Graph* G, const gbx_desc& d, bool* wanted) {
     return GBX_OK;
 }
 
-gbx_status cluster_bfs_launch(Graph* G, int32_t source, int32_t* depth, int32_t* parent, cudaStream_t s,
-                              bool* complete) {
-    ClArgs a;
+static void cluster_bfs_args(Graph* G, int32_t source, int32_t* depth, int32_t* parent, ClArgs& a, int32_t* bm_words) {
     a.n = G->n;
     a.nwords = G->nwords;
     a.source = source;
@@ -468,8 +468,16 @@ gbx_status cluster_bfs_launch(Graph* G, int32_t source, int32_t* depth, int32_t*
     a.max_frontier = (int32_t)std::min<int64_t>(kClMaxFrontier, kClMaxEdges * G->n / std::max<int64_t>(G->nnz, 1));
     a.timeout_ns = wait_timeout_ns();
     a.fill = G->n <= (1 << 16) ? 1 : 0;  // 16 blocks write 0.5 MB faster than a launch takes
-    const int32_t bm_words = (G->nwords + G->cluster_blocks - 1) / G->cluster_blocks;
-    a.shared_bm = bm_words <= kClBmWords ? 1 : 0;
+    *bm_words = (G->nwords + G->cluster_blocks - 1) / G->cluster_blocks;
+    a.shared_bm = *bm_words <= kClBmWords ? 1 : 0;
+    if (!a.shared_bm) *bm_words = 0;
+}
+
+gbx_status cluster_bfs_launch(Graph* G, int32_t source, int32_t* depth, int32_t* parent, cudaStream_t s,
+                              bool* complete) {
+    ClArgs a;
+    int32_t bm_words = 0;
+    cluster_bfs_args(G, source, depth, parent, a, &bm_words);
     *complete = a.whole != 0;
     if (!a.fill) {
         const unsigned blocks = std::min<unsigned>(div_up(G->n, 512 * 4), (unsigned)G->num_sms * 4u);
@@ -477,9 +485,28 @@ gbx_status cluster_bfs_launch(Graph* G, int32_t source, int32_t* depth, int32_t*
         GBX_CUDA_TRY(cudaGetLastError());
     }
     void* args[] = {&a};
-    GBX_TRY(cluster_launch((const void*)bfs_cluster_kernel, G->cluster_blocks, kClThreads,
-                           cl_smem(a.shared_bm ? bm_words : 0), args, s));
+    GBX_TRY(cluster_launch((const void*)bfs_cluster_kernel<false>, G->cluster_blocks, kClThreads, cl_smem(bm_words), args,
+                           s));
     return GBX_OK;
+}
+
+gbx_status cluster_bfs_selftest(Graph* G, uint64_t timeout_ns, cudaStream_t s) {
+    bool wanted = false;
+    gbx_desc d;
+    gbx_desc_init(&d);
+    GBX_TRY(cluster_bfs_wanted(G, d, &wanted));
+    GBX_CHECK(wanted, GBX_ERR_NOT_SUPPORTED, "searches on this graph do not start in a cluster");
+    const void* fn = (const void*)bfs_cluster_kernel<true>;
+    int blocks = 0;
+    GBX_TRY(cluster_fit(fn, kClThreads, cl_smem(kClBmWords), &blocks));
+    GBX_CHECK(blocks == G->cluster_blocks, GBX_ERR_NOT_SUPPORTED, "the cluster does not fit");
+    ClArgs a;
+    int32_t bm_words = 0;
+    cluster_bfs_args(G, 0, G->ws.qp[0], nullptr, a, &bm_words);
+    a.fill = 1;
+    a.timeout_ns = timeout_ns;
+    void* args[] = {&a};
+    return cluster_launch(fn, blocks, kClThreads, cl_smem(bm_words), args, s);
 }
 
 }  // namespace gbx

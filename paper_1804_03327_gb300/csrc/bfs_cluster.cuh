@@ -15,6 +15,10 @@ gbx_status cluster_bfs_wanted(Graph* G, const gbx_desc& d, bool* wanted);
 gbx_status cluster_bfs_launch(Graph* G, int32_t source, int32_t* depth, int32_t* parent, cudaStream_t s,
                               bool* complete);
 
+// One launch in which a block withholds its queue length: every block's wait runs out after
+// timeout_ns.
+gbx_status cluster_bfs_selftest(Graph* G, uint64_t timeout_ns, cudaStream_t s);
+
 // out[i] = fill for all i < n except out[special] = special_value; 16-byte stores when aligned.
 __device__ __forceinline__ void fill_i32(int32_t* out, int32_t n, int32_t fill, int32_t special, int32_t special_value,
                                          long long gtid, long long gstride) {

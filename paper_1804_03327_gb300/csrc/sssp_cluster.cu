@@ -124,6 +124,8 @@ __device__ __forceinline__ void sp_relax(const SpArgs& a, SpSmem& sm, int np, in
     sp_far(a, sm, f, base, lowered && !(d <= T), v, d);
 }
 
+// kWithhold: block 1 keeps its counts to itself, so that every block's wait runs out.
+template <bool kWithhold>
 __global__ void __launch_bounds__(kSpThreads, 1) sssp_cluster_kernel(const __grid_constant__ SpArgs a) {
     extern __shared__ __align__(16) unsigned char raw[];
     SpSmem& sm = *reinterpret_cast<SpSmem*>(raw);
@@ -261,7 +263,7 @@ __global__ void __launch_bounds__(kSpThreads, 1) sssp_cluster_kernel(const __gri
             }
         }
         __syncthreads();
-        if (t < C * SP_WORDS) {
+        if (t < C * SP_WORDS && !(kWithhold && rank == 1)) {
             const int to = t / SP_WORDS, what = t - to * SP_WORDS;
             const int32_t v = what == SP_NEAR ? min(sm.cnt[np], kSpCap)
                               : what == SP_FAR ? (sm.lost ? -1 : sm.fcnt[f])
@@ -358,13 +360,12 @@ gbx_status sssp_cluster_wanted(Graph* G, const gbx_desc& d, bool* wanted) {
     *wanted = false;
     if (d.trace || d.direction == GBX_DIR_PULL || !(G->sp_step >= 0.0f)) return GBX_OK;
     if (G->sp_cluster_blocks == 0)
-        GBX_TRY(cluster_fit((const void*)sssp_cluster_kernel, kSpThreads, sizeof(SpSmem), &G->sp_cluster_blocks));
+        GBX_TRY(cluster_fit((const void*)sssp_cluster_kernel<false>, kSpThreads, sizeof(SpSmem), &G->sp_cluster_blocks));
     *wanted = G->sp_cluster_blocks > 0;
     return GBX_OK;
 }
 
-gbx_status sssp_cluster_launch(Graph* G, int32_t source, float* dist, cudaStream_t s) {
-    SpArgs a;
+static void sssp_cluster_args(Graph* G, int32_t source, float* dist, SpArgs& a) {
     a.n = G->n;
     a.source = source;
     a.ptr = G->out_ptr;
@@ -384,10 +385,36 @@ gbx_status sssp_cluster_launch(Graph* G, int32_t source, float* dist, cudaStream
     a.ho = G->ws.handoff;
     a.status = G->ws.status;
     a.timeout_ns = wait_timeout_ns();
+}
+
+gbx_status sssp_cluster_launch(Graph* G, int32_t source, float* dist, cudaStream_t s) {
+    SpArgs a;
+    sssp_cluster_args(G, source, dist, a);
     sp_fill_kernel<<<std::min<unsigned>(div_up(G->n, 512), (unsigned)G->num_sms * 4u), 512, 0, s>>>(dist, G->n, source);
     GBX_CUDA_TRY(cudaGetLastError());
     void* args[] = {&a};
-    return cluster_launch((const void*)sssp_cluster_kernel, G->sp_cluster_blocks, kSpThreads, sizeof(SpSmem), args, s);
+    return cluster_launch((const void*)sssp_cluster_kernel<false>, G->sp_cluster_blocks, kSpThreads, sizeof(SpSmem), args,
+                          s);
+}
+
+gbx_status sssp_cluster_selftest(Graph* G, uint64_t timeout_ns, cudaStream_t s) {
+    bool wanted = false;
+    gbx_desc d;
+    gbx_desc_init(&d);
+    GBX_TRY(sssp_cluster_wanted(G, d, &wanted));
+    GBX_CHECK(wanted, GBX_ERR_NOT_SUPPORTED, "searches on this graph do not start in a cluster (or it has no weights)");
+    const void* fn = (const void*)sssp_cluster_kernel<true>;
+    int blocks = 0;
+    GBX_TRY(cluster_fit(fn, kSpThreads, sizeof(SpSmem), &blocks));
+    GBX_CHECK(blocks == G->sp_cluster_blocks, GBX_ERR_NOT_SUPPORTED, "the cluster does not fit");
+    SpArgs a;
+    float* const dist = reinterpret_cast<float*>(G->ws.qd[0]);
+    sssp_cluster_args(G, 0, dist, a);
+    a.timeout_ns = timeout_ns;
+    sp_fill_kernel<<<std::min<unsigned>(div_up(G->n, 512), (unsigned)G->num_sms * 4u), 512, 0, s>>>(dist, G->n, 0);
+    GBX_CUDA_TRY(cudaGetLastError());
+    void* args[] = {&a};
+    return cluster_launch(fn, blocks, kSpThreads, sizeof(SpSmem), args, s);
 }
 
 }  // namespace gbx

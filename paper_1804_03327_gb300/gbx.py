@@ -55,6 +55,7 @@ EXPORTED = [
     "gbx_last_error", "gbx_status_string", "gbx_version", "gbx_graph_build", "gbx_graph_free", "gbx_graph_info",
     "gbx_graph_csr", "gbx_graph_copy_csr", "gbx_graph_sync", "gbx_desc_init", "gbx_mxv", "gbx_mxv_stats",
     "gbx_bfs", "gbx_bfs_host", "gbx_bfs_trace", "gbx_set_wait_timeout_ns", "gbx_selftest_barrier_timeout",
+    "gbx_selftest_cluster_timeout",
     "gbx_mxv_pull_noalloc", "gbx_bfs_batch", "gbx_bfs_batch_trace",
     "gbx_server_config_init", "gbx_server_create", "gbx_server_add_graph", "gbx_server_graph_lanes",
     "gbx_server_submit", "gbx_server_poll", "gbx_server_stats", "gbx_server_destroy", "gbx_autotune",
@@ -139,6 +140,7 @@ def load():
                 "gbx_bfs_trace": (ctypes.c_int, [p, ctypes.POINTER(Level), i32, ctypes.POINTER(i32)]),
                 "gbx_set_wait_timeout_ns": (ctypes.c_int, [u64]),
                 "gbx_selftest_barrier_timeout": (ctypes.c_int, [p, u64, p]),
+                "gbx_selftest_cluster_timeout": (ctypes.c_int, [p, i32, u64, p]),
                 "gbx_mxv_pull_noalloc": (ctypes.c_int, [i32, p, p, p, p, i32, i32, p, p]),
                 "gbx_bfs_batch": (ctypes.c_int, [p, p, i32, p, i32, ctypes.POINTER(Desc), p]),
                 "gbx_bfs_batch_trace": (ctypes.c_int, [p, ctypes.POINTER(Level), i32, ctypes.POINTER(i32)]),
@@ -207,6 +209,11 @@ def desc_init(**fields) -> Desc:
 def selftest_barrier_timeout(g: "Graph", timeout_ns: int, stream=None):
     _check(load().gbx_selftest_barrier_timeout(g.handle, int(timeout_ns), _stream_ptr(stream)),
            "gbx_selftest_barrier_timeout")
+
+
+def selftest_cluster_timeout(g: "Graph", which: int, timeout_ns: int, stream=None):
+    _check(load().gbx_selftest_cluster_timeout(g.handle, int(which), int(timeout_ns), _stream_ptr(stream)),
+           "gbx_selftest_cluster_timeout")
 
 
 def set_wait_timeout_ns(ns: int):
