@@ -141,7 +141,7 @@ __device__ __forceinline__ void record_depth(const MsArgs& a, int32_t v, int32_t
 // and each row's 128 entries leave together: four entries of a lane are one 8- or
 // 16-byte store where the rows allow it (aligned, a full group), else four stores whose
 // 32 lanes are consecutive.  Lanes never visited get -1; lanes found at depth 16 or more
-// were stored when found and are left alone (emit_rows_mixed).
+// were stored when found and are left alone (emit_rows).
 //
 // Bound by the stores: S rows of n entries, written once, many rows at a time.  With 32
 // vertices a warp (one 64- or 128-byte piece of a row per store, ten instructions an
@@ -167,26 +167,23 @@ __device__ __forceinline__ char* depth_row(const MsArgs& a, int32_t b) {
     return static_cast<char*>(a.depth) + (size_t)b * (size_t)a.n * (a.depth16 ? 2u : 4u);
 }
 
-// One group's half word when some lane of it was found at depth 16 or more, or is its own
-// source: entry by entry, a row's 32 consecutive entries per store.
-__device__ __noinline__ void emit_rows_mixed(const MsArgs& a, int32_t g, int32_t h, int nrows) {
-    for (int j = 0; j < kEmitV; ++j) {
-        const int32_t v = g * kEmitTile + 32 * j + (threadIdx.x & 31);
-        if (v >= a.n) continue;
-        const size_t iw = (size_t)v * a.W * 2 + h;
-        const uint32_t vis = reinterpret_cast<const uint32_t*>(a.V)[iw];
-        uint32_t p[kMsPlanes];
+// Rows [b0, b1) of half word h for 32 consecutive vertices, a lane each: entry by entry, a row's
+// 32 entries per store.  Lanes found at depth 16 or more were stored when found.
+__device__ __noinline__ void emit_rows(const MsArgs& a, int32_t v, int32_t h, int b0, int b1) {
+    if (v >= a.n) return;
+    const size_t iw = (size_t)v * a.W * 2 + h;
+    const uint32_t vis = reinterpret_cast<const uint32_t*>(a.V)[iw];
+    uint32_t p[kMsPlanes];
 #pragma unroll
-        for (int q = 0; q < kMsPlanes; ++q) p[q] = reinterpret_cast<const uint32_t*>(a.P[q])[iw];
-        for (int b = 0; b < nrows; ++b) {
-            int32_t d = -1;
-            if ((vis >> b) & 1u) {
-                d = (int32_t)(((p[0] >> b) & 1u) | (((p[1] >> b) & 1u) << 1) | (((p[2] >> b) & 1u) << 2) |
-                              (((p[3] >> b) & 1u) << 3));
-                if (d == 0 && __ldg(a.src + 32 * h + b) != v) continue;  // deep: already stored
-            }
-            store_depth(a, 32 * h + b, v, d);
+    for (int q = 0; q < kMsPlanes; ++q) p[q] = reinterpret_cast<const uint32_t*>(a.P[q])[iw];
+    for (int b = b0; b < b1; ++b) {
+        int32_t d = -1;
+        if ((vis >> b) & 1u) {
+            d = (int32_t)(((p[0] >> b) & 1u) | (((p[1] >> b) & 1u) << 1) | (((p[2] >> b) & 1u) << 2) |
+                          (((p[3] >> b) & 1u) << 3));
+            if (d == 0 && __ldg(a.src + 32 * h + b) != v) continue;  // deep: already stored
         }
+        store_depth(a, 32 * h + b, v, d);
     }
 }
 
@@ -262,8 +259,23 @@ __device__ __forceinline__ void emit_depths(const MsArgs& a, uint32_t* smem) {
     const int32_t per = kStaged ? 2 * kEmitWords : 1;
     const int32_t ntile = (nhalf + per - 1) / per;
     const long long items = (long long)ngroups * ntile;
+    const long long nwarps = ((long long)gridDim.x * kMsThreads) >> 5;
+    if ((long long)ngroups * nhalf < nwarps) {
+        // fewer pieces than warps: 32 vertices and as few rows as keep every warp busy, at least 4 (1,000
+        // vertices, what a batch takes beside its levels: 20 sources 40 -> 25 us, 100 sources 56 -> 25)
+        const int32_t nv = (a.n + 31) >> 5;
+        int rows = 32;
+        while (rows > 4 && (long long)nv * nhalf * (64 / rows) <= nwarps) rows >>= 1;
+        const int32_t parts = 32 / rows;
+        for (long long it = (long long)wib * gridDim.x + blockIdx.x; it < (long long)nv * nhalf * parts; it += nwarps) {
+            const int32_t r = (int32_t)(it % parts), i = (int32_t)(it / parts), h = i % nhalf;
+            const int b1 = a.S - 32 * h < (r + 1) * rows ? a.S - 32 * h : (r + 1) * rows;
+            emit_rows(a, 32 * (i / nhalf) + lane, h, r * rows, b1);
+        }
+        return;
+    }
     const long long first = kStaged ? blockIdx.x : (((long long)blockIdx.x * kMsThreads + threadIdx.x) >> 5);
-    const long long nstep = kStaged ? gridDim.x : (((long long)gridDim.x * kMsThreads) >> 5);
+    const long long nstep = kStaged ? gridDim.x : nwarps;
     for (long long it = first; it < items; it += nstep) {
         const int32_t g = (int32_t)(it / ntile);
         const int32_t h0 = (int32_t)(it - (long long)g * ntile) * per;
@@ -312,8 +324,8 @@ __device__ __forceinline__ void emit_depths(const MsArgs& a, uint32_t* smem) {
             }
             deep |= e.vis[j] & ~(e.p[0][j] | e.p[1][j] | e.p[2][j] | e.p[3][j]);
         }
-        if (__any_sync(0xffffffffu, deep != 0u))
-            emit_rows_mixed(a, g, h, nrows);
+        if (__any_sync(0xffffffffu, deep != 0u))  // or a lane's own source
+            for (int j = 0; j < kEmitV; ++j) emit_rows(a, g * kEmitTile + 32 * j + lane, h, 0, nrows);
         else
             emit_half(a, e, row, nrows, v, wide);
     }
