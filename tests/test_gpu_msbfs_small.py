@@ -39,3 +39,28 @@ def test_output_rows(n, S):
     s, d = np.concatenate([p[:-1], e[0]]), np.concatenate([p[1:], e[1]])
     for dtype, shift in ((torch.int16, 0), (torch.int16, 3), (torch.int32, 0), (torch.int32, 1)):
         check(n, s, d, True, S, [gbx.desc_init()], dtype, distinct=8, shift=shift, seed=S)
+
+
+@pytest.mark.parametrize("alpha", [0.0, 1e-9, 0.01, 0.25, 0.5, 0.999, 1.0, 1e30, float("inf")])
+def test_direction_is_the_edge_quotient(alpha):
+    """AUTO pulls once the active edges exceed alpha * nnz, the product in binary64."""
+    n, s, d = synth.rmat_edges(9, 8, seed=5)
+    og, g = oracle.graph(n, s, d), gbx.graph_build(n, s, d)
+    srcs = synth.sources(n, s, d, 7, seed=2).astype(np.int32)
+    depth = torch.empty((7, n), dtype=torch.int32, device="cuda")
+    gbx.bfs_batch(g, srcs, depth, gbx.desc_init(alpha=alpha))
+    gbx.graph_sync(g)
+    for b, v in enumerate(srcs):
+        assert np.array_equal(depth[b].cpu().numpy(), oracle.bfs(og, int(v))[0])
+    tr = gbx.bfs_batch_trace(g)
+    pull = tr["mf"].astype(np.float64) > np.float64(np.float32(alpha)) * np.float64(og.nnz)
+    assert np.array_equal(tr["direction"] == gbx.DIR_PULL, pull)
+    # alpha a quotient of binary32 that a level meets exactly
+    for mf in set(int(x) for x in tr["mf"]):
+        for a in (np.float32(mf / og.nnz), np.nextafter(np.float32(mf / og.nnz), np.float32(0))):
+            gbx.bfs_batch(g, srcs, depth, gbx.desc_init(alpha=float(a)))
+            gbx.graph_sync(g)
+            t = gbx.bfs_batch_trace(g)
+            assert np.array_equal(t["direction"] == gbx.DIR_PULL,
+                                  t["mf"].astype(np.float64) > np.float64(a) * np.float64(og.nnz))
+    g.free()
