@@ -47,7 +47,7 @@ constexpr int kMsThreads = 512;
 // chooses it (blocks_per_sm >= 3) and the autotuner times both.
 constexpr int kMsOcc = 2;
 constexpr int kMsOccLean = 3;
-constexpr int kMsProbe = 8;  // default a.probe: a long row is deferred after four times as many in-neighbours
+constexpr int kMsProbe = 8;  // default a.probe; with two words and more a long row is deferred after four times as many
 constexpr int kMsPlanes = 4;  // depth bit planes: bit p of depths below 16
 
 struct MsArgs {
@@ -58,8 +58,8 @@ struct MsArgs {
     const int32_t* in_ptr;
     const int32_t* in_col;
     const uint32_t* nz_in;
-    const int32_t* first_out;
-    const int4* next_out;
+    const int32_t* first_in;
+    const int4* next_in;
     unsigned long long* V;
     unsigned long long* Fb[3];  // rotating found-lane buffers
     unsigned long long* P[4];   // depth bit planes (see record_depth)
@@ -424,17 +424,12 @@ __device__ __forceinline__ void record_words(const MsArgs& a, int32_t v, int32_t
 // ---------------------------------------------------------------- pull level
 
 constexpr int kMsUnroll = 4;        // in-neighbours a group ORs per step (loads in flight)
-// On a graph with at most a word of rows per warp a lane's walk of up to 96 in-edges is what a pull level
-// takes: there the warp takes a row over after a.probe of them when more than kMsFewRow are left (5 to 45
-// sources on 3K to 20K vertices: 134-196 -> 123-183 us; 36 sources on 125K 197 -> 182).
-constexpr int32_t kMsFewRow = 24;
 constexpr int32_t kMsLongRow = 64;   // in-edges left after the probe beyond which a row is deferred
 // Steps of a whole warp on a row before it is deferred, with one word (128 in-neighbours a step):
-// at a level whose lanes are mostly covered that settles the row without the chain of a
-// deferred chunk (RMAT-21, 64 sources: 797 us without, 748 with 2 steps, 738 with 4, 730 with
-// 8).  Wide batches look at 16 in-neighbours a step, so the row would hold up its warp (RMAT-20,
-// 1,000 sources: 3.7 -> 4.0 ms).
-constexpr int kMsScan = 8;
+// a deferred row costs two more grid barriers and the chain of its chunks, 11 us.  RMAT graphs of
+// 300,000, 600,000 and 2M vertices (20, 20 and 64 sources): 170, 276 and 725 us with 8 steps, 161, 285
+// and 726 with 16.
+constexpr int kMsScan = 16;
 constexpr int32_t kMsChunk = 512;   // in-edges of a deferred row a warp takes at a time
 constexpr int32_t kMsCheck = 128;   // ... between two tests whether they cover the row (a power of two)
 
@@ -446,9 +441,54 @@ struct MsLong {
     int32_t* base;
 };
 
-// Every vertex with an unvisited lane ORs V of its in-neighbours (V as of the level's
-// start), kMsUnroll at a time, until all its unvisited lanes are covered.  A warp lists
-// the open vertices of 32 of its bitmap words in shared memory and its groups take them
+// Leaves the rows v of the lanes with `take`, from in-edge k on (left of them), to the grid; all lanes call.
+__device__ __forceinline__ void ms_defer(const MsLong& lr, bool take, int32_t v, int32_t k, int32_t left,
+                                         LevelCtr* cout) {
+    const uint32_t dm = __ballot_sync(0xffffffffu, take);
+    const uint32_t nch = take ? (uint32_t)(left - 1) / kMsChunk + 1u : 0u;
+    const uint32_t inc = warp_inclusive_sum(nch);
+    const uint32_t tot = __shfl_sync(0xffffffffu, inc, 31);
+    unsigned long long old = 0ull;
+    if ((threadIdx.x & 31) == 0)
+        old = atomicAdd(&cout->huge, ((unsigned long long)tot << 32) | (unsigned long long)__popc(dm));
+    old = __shfl_sync(0xffffffffu, old, 0);
+    if (take) {
+        const uint32_t slot = (uint32_t)old + __popc(dm & lanemask_lt());
+        lr.row[slot] = v;
+        lr.k[slot] = k;
+        lr.base[slot] = (int32_t)((uint32_t)(old >> 32) + inc - nch);
+    }
+}
+
+// A row of a pull level is settled: the lane's new words nw of vertex v (unv: the lanes v missed
+// before).  F_next is zero before the level: only words with new lanes are written.
+template <int WL>
+__device__ __forceinline__ void ms_settle(const MsArgs& a, int32_t L, int32_t v, int32_t w, bool sink,
+                                          const Words<WL>& nw, const Words<WL>& unv, const Words<WL>& lm,
+                                          unsigned long long* Fn, Acc& acc) {
+    if (!nw.any()) return;
+    const size_t iv = (size_t)v * a.W + w;
+    if (sink) {
+        // nobody's in-neighbour: no other row reads its V, and it never joins the active list
+        Words<WL> t = ld_words<WL>(a.V + iv);
+#pragma unroll
+        for (int j = 0; j < WL; ++j) t.x[j] |= nw.x[j];
+        st_words<WL>(a.V + iv, t);
+    } else {
+        st_words<WL>(Fn + iv, nw);
+    }
+    Words<WL> was;
+#pragma unroll
+    for (int j = 0; j < WL; ++j) {
+        acc.n_new += (uint32_t)__popcll(nw.x[j]);
+        was.x[j] = ~unv.x[j] & lm.x[j];
+    }
+    record_words<WL>(a, v, w, nw, was, L + 1);
+}
+
+// Two words and more: every vertex with an unvisited lane ORs V of its in-neighbours (V as of
+// the level's start), kMsUnroll at a time, until all its unvisited lanes are covered.  A warp
+// lists the open vertices of 32 of its bitmap words in shared memory and its groups take them
 // one after another, each going on to the next as soon as its own is settled, so a long
 // row holds up nobody else's.  A row that is still open after 4 a.probe in-neighbours with
 // more than kMsLongRow left is deferred: its chunks are spread over all warps
@@ -459,8 +499,8 @@ struct MsLong {
 // pull level of the RMAT-20 batch of 1,000 sources 7.1 ms: every gather touched 32 rows at
 // once and a hub row held one warp for milliseconds.  Now 0.76 ms (31.4M in-neighbours x
 // 128 B, 5.3 TB/s).  kMsLongRow 64, 128 and 512 give that level 0.76, 0.78 and 1.0 ms;
-// deferring after 8 instead of 32 in-neighbours costs the RMAT-21 batch of 64 5 %, and
-// kMsChunk 256 instead of 512 6 % (more of a row's chunks run before one covers it).
+// kMsChunk 256 instead of 512 cost the RMAT-21 batch of 64 6 % (more of a row's chunks run before
+// one covers it).
 template <int WL>
 __device__ __forceinline__ void ms_pull(const MsArgs& a, int32_t L, int32_t c0, unsigned long long* Fn, uint32_t* Tn,
                                         uint16_t* list, const MsLong& lr, bool defer, Stage& st,
@@ -476,17 +516,21 @@ __device__ __forceinline__ void ms_pull(const MsArgs& a, int32_t L, int32_t c0, 
     Words<WL> lm;
 #pragma unroll
     for (int j = 0; j < WL; ++j) lm.x[j] = wok ? lane_mask(a.S, w + j) : 0ull;
-    const bool few = WL == 1 && a.nwords <= nwarps;  // a word per warp at most: a level lasts as long as a row
-    const int32_t own = few ? a.probe : 4 * a.probe, most = few ? kMsFewRow : kMsLongRow;
+    const int32_t own = 4 * a.probe;
     for (long long wb = gwarp; wb < a.nwords; wb += 32ll * nwarps) {
         const long long tw = wb + (long long)lane * nwarps;
-        uint32_t m = tw < a.nwords ? (a.nz_in[tw] & ~a.D[tw]) : 0u;
+        const uint32_t m = tw < a.nwords ? (a.nz_in[tw] & ~a.D[tw]) : 0u;
         const uint32_t cnt = __popc(m);
         const uint32_t incl = warp_inclusive_sum(cnt);
         const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);
         if (total == 0u) continue;
         __syncwarp();
-        for (uint32_t at = incl - cnt; m; m &= m - 1) list[at++] = (uint16_t)((lane << 5) + __ffs(m) - 1);
+        // a word's rows at a time, a lane per row (a warp has a few words only on all but huge graphs)
+        for (uint32_t wm = __ballot_sync(0xffffffffu, m != 0u); wm; wm &= wm - 1) {
+            const int j = __ffs(wm) - 1;
+            const uint32_t word = __shfl_sync(0xffffffffu, m, j), at = __shfl_sync(0xffffffffu, incl - cnt, j);
+            if ((word >> lane) & 1u) list[at + __popc(word & lanemask_lt())] = (uint16_t)((j << 5) + lane);
+        }
         __syncwarp();
         uint32_t next = 0;
         int32_t v = -1, k = 0, end = 0, lim = 0;
@@ -502,7 +546,7 @@ __device__ __forceinline__ void ms_pull(const MsArgs& a, int32_t L, int32_t c0, 
                     v = (int32_t)((wb + (long long)(off >> 5) * nwarps) << 5) + (int32_t)(off & 31u);
                     k = __ldg(a.in_ptr + v);
                     end = __ldg(a.in_ptr + v + 1);
-                    lim = end - k > own + most ? k + own : end;
+                    lim = end - k > own + kMsLongRow ? k + own : end;
                     sink = !a.symmetric && __ldg(a.out_ptr + v + 1) == __ldg(a.out_ptr + v);
                     unv = wok ? ld_words<WL>(a.V + (size_t)v * a.W + w) : zero_words<WL>();
 #pragma unroll
@@ -521,7 +565,7 @@ __device__ __forceinline__ void ms_pull(const MsArgs& a, int32_t L, int32_t c0, 
             for (int t = 0; t < kMsUnroll; ++t)
                 x[t] = u[t] >= 0 && wok ? ld_words<WL>(a.V + (size_t)u[t] * a.W + w) : zero_words<WL>();
             const int32_t left = end - k;
-            k = left > kMsUnroll ? k + kMsUnroll : end;  // (a position past the row's end need not fit 32 bits)
+            k = left > kMsUnroll ? k + kMsUnroll : end;
 #pragma unroll
             for (int t = 0; t < kMsUnroll; ++t) u[t] = v >= 0 && t < end - k ? __ldg(a.in_col + k + t) : -1;
             bool cov = true;
@@ -533,99 +577,118 @@ __device__ __forceinline__ void ms_pull(const MsArgs& a, int32_t L, int32_t c0, 
             }
             const bool covered = gr.all(cov);
             if (v >= 0 && gr.sub == 0) acc.exam += chunks256 * (uint32_t)(left < kMsUnroll ? left : kMsUnroll);
-            bool done = v >= 0 && (covered || k >= end);
-            bool put_off = defer && v >= 0 && !done && k >= lim && lim != end;
+            const bool done = v >= 0 && (covered || k >= end);
+            const bool put_off = defer && v >= 0 && !done && k >= lim && lim != end;
             if (!__any_sync(0xffffffffu, done || put_off)) continue;
-            // one word: the whole warp looks at the row's next in-neighbours first, kMsScan steps of 128
-            for (uint32_t pm = WL == 1 ? __ballot_sync(0xffffffffu, put_off) : 0u; pm; pm &= pm - 1) {
-                const int t0 = __ffs(pm) - 1;  // the row's group starts at this lane
-                const int32_t kt = __shfl_sync(0xffffffffu, k, t0), et = __shfl_sync(0xffffffffu, end, t0);
-                Words<WL> ut, at;
-#pragma unroll
-                for (int j = 0; j < WL; ++j) {
-                    ut.x[j] = __shfl_sync(0xffffffffu, unv.x[j], t0 + gr.sub);
-                    at.x[j] = __shfl_sync(0xffffffffu, ac.x[j], t0 + gr.sub);
-                }
-                const int32_t step = kMsUnroll * (32 / gr.size);
-                const int32_t len = et - kt > kMsScan * step ? kMsScan * step : et - kt;
-                int32_t at_k = 0;
-                bool all = false;
-                while (at_k < len && !all) {
-                    int32_t uu[kMsUnroll];
-                    const int32_t kg = at_k + kMsUnroll * (gr.first / gr.size);
-#pragma unroll
-                    for (int t = 0; t < kMsUnroll; ++t) uu[t] = kg + t < len ? __ldg(a.in_col + kt + kg + t) : -1;
-                    Words<WL> y[kMsUnroll];
-#pragma unroll
-                    for (int t = 0; t < kMsUnroll; ++t)
-                        y[t] = uu[t] >= 0 && wok ? ld_words<WL>(a.V + (size_t)uu[t] * a.W + w) : zero_words<WL>();
-                    bool c = true;
-#pragma unroll
-                    for (int j = 0; j < WL; ++j) {
-#pragma unroll
-                        for (int t = 0; t < kMsUnroll; ++t) at.x[j] |= y[t].x[j];
-                        for (int o = gr.size; o < 32; o <<= 1) at.x[j] |= __shfl_xor_sync(0xffffffffu, at.x[j], o);
-                        c &= (at.x[j] & ut.x[j]) == ut.x[j];
-                    }
-                    all = __all_sync(0xffffffffu, c);
-                    at_k += step;
-                }
-                if (gr.first == t0) {
-                    ac = at;
-                    k = et - kt > at_k ? kt + at_k : et;
-                    done = all || k >= et;
-                    put_off = !done;
-                    if (gr.sub == 0) acc.exam += chunks256 * (uint32_t)(k - kt);
-                }
-            }
             Words<WL> nw;
 #pragma unroll
             for (int j = 0; j < WL; ++j) nw.x[j] = done || put_off ? ac.x[j] & unv.x[j] : 0ull;
             const bool any_new = gr.any(nw.any());
             const bool full = gr.all(!done || (nw.x[0] == unv.x[0] && nw.x[WL - 1] == unv.x[WL - 1]));
-            // F_next is zero before the level: only words with new lanes are written
-            if (nw.any()) {
-                const size_t iv = (size_t)v * a.W + w;
-                if (done && sink) {
-                    // nobody's in-neighbour: no other row reads its V, and it never joins the active list
-                    Words<WL> t = ld_words<WL>(a.V + iv);
-#pragma unroll
-                    for (int j = 0; j < WL; ++j) t.x[j] |= nw.x[j];
-                    st_words<WL>(a.V + iv, t);
-                } else {
-                    st_words<WL>(Fn + iv, nw);
-                }
-                if (done) {
-#pragma unroll
-                    for (int j = 0; j < WL; ++j) acc.n_new += (uint32_t)__popcll(nw.x[j]);
-                    Words<WL> was;
-#pragma unroll
-                    for (int j = 0; j < WL; ++j) was.x[j] = ~unv.x[j] & lm.x[j];
-                    record_words<WL>(a, v, w, nw, was, L + 1);
-                }
-            }
+            if (done)
+                ms_settle<WL>(a, L, v, w, sink, nw, unv, lm, Fn, acc);
+            else if (nw.any())
+                st_words<WL>(Fn + (size_t)v * a.W + w, nw);
             bool take = done && gr.sub == 0 && any_new && !sink;
             if (done && sink && full && one && gr.sub == 0) atomicOr(a.D + (v >> 5), 1u << (v & 31));
             if (!one && take) take = !(atomicOr(Tn + (v >> 5), 1u << (v & 31)) & (1u << (v & 31)));
             st.put(take, v);
-            const uint32_t dm = __ballot_sync(0xffffffffu, put_off && gr.sub == 0);
-            if (dm) {
-                const uint32_t nch = put_off && gr.sub == 0 ? (uint32_t)(end - k + kMsChunk - 1) / kMsChunk : 0u;
-                const uint32_t inc = warp_inclusive_sum(nch);
-                const uint32_t tot = __shfl_sync(0xffffffffu, inc, 31);
-                unsigned long long old = 0ull;
-                if (lane == 0)
-                    old = atomicAdd(&st.cout->huge, ((unsigned long long)tot << 32) | (unsigned long long)__popc(dm));
-                old = __shfl_sync(0xffffffffu, old, 0);
-                if (put_off && gr.sub == 0) {
-                    const uint32_t slot = (uint32_t)old + __popc(dm & lanemask_lt());
-                    lr.row[slot] = v;
-                    lr.k[slot] = k;
-                    lr.base[slot] = (int32_t)((uint32_t)(old >> 32) + inc - nch);
-                }
-            }
+            if (__any_sync(0xffffffffu, put_off)) ms_defer(lr, put_off && gr.sub == 0, v, k, end - k, st.cout);
             if (done || put_off) v = -1;
         }
+    }
+    st.flush_block<kMsThreads / 32>(bsm);
+}
+
+// The pull with one word: a lane per row of the warp's bitmap word, the first five in-neighbours
+// from the dense arrays, then up to a.probe more, four at a time, or all if kMsOwnRow more end the
+// row; the rows still open are taken by the whole warp one after another, kMsScan steps each, and
+// what is open then is deferred.  Rows of a mesh (kMesh: at most kMsMeshDegree entries) are left
+// to their lanes.
+//
+// Bound by its instructions where the rows are short: handing rows out to lanes as ms_pull does took
+// 710M instructions and 1.85 ms for the 46 x 46 x 46 grid and 64 sources, so 1.32 ms; the first pull
+// level of an RMAT graph of 300,000 vertices and 20 sources 68 us, so 39.  Without kMsOwnRow a
+// random graph of 100,000 vertices and 16 edges each 193 us, with 16 or 24 152.
+constexpr int32_t kMsOwnRow = 24;
+
+template <bool kMesh>
+__device__ __forceinline__ void ms_pull_one(const MsArgs& a, int32_t L, unsigned long long* Fn, const MsLong& lr,
+                                            Stage& st, unsigned long long* bsm, Acc& acc) {
+    const int lane = threadIdx.x & 31;
+    const int gwarp = (int)((blockIdx.x * kMsThreads + threadIdx.x) >> 5);
+    const int nwarps = (int)((gridDim.x * kMsThreads) >> 5);
+    const unsigned long long full0 = lane_mask(a.S, 0);
+    for (int32_t tile = gwarp; tile < a.nwords; tile += nwarps) {
+        const uint32_t m = a.nz_in[tile] & ~a.D[tile];
+        if (m == 0u) continue;
+        const int32_t v = (tile << 5) + lane;
+        unsigned long long ac = 0ull, unv = 0ull;
+        int32_t beg = 0, left = 0, k = 0;  // the row: where it starts, its length, in-neighbours looked at
+        bool sink = false;
+        if ((m >> lane) & 1u) {
+            const int4 x = __ldg(a.next_in + v);
+            const int32_t u[5] = {__ldg(a.first_in + v), x.x, x.y, x.z, x.w};
+            beg = __ldg(a.in_ptr + v);
+            left = __ldg(a.in_ptr + v + 1) - beg;
+            if (!kMesh) sink = !a.symmetric && __ldg(a.out_ptr + v + 1) == __ldg(a.out_ptr + v);
+            unv = ~a.V[v] & full0;
+#pragma unroll
+            for (int t = 0; t < 5; ++t) ac |= u[t] >= 0 ? a.V[u[t]] : 0ull;
+            const int32_t lim = kMesh || left <= 5 + a.probe + kMsOwnRow ? left : 5 + a.probe;
+            for (k = 5; k < lim && (ac & unv) != unv; k += kMsUnroll) {
+                int32_t y[kMsUnroll];
+#pragma unroll
+                for (int t = 0; t < kMsUnroll; ++t) y[t] = k + t < left ? __ldg(a.in_col + beg + k + t) : -1;
+#pragma unroll
+                for (int t = 0; t < kMsUnroll; ++t) ac |= y[t] >= 0 ? a.V[y[t]] : 0ull;
+            }
+            k = min(k, left);
+            acc.exam += (uint32_t)k;
+        }
+        bool open = !kMesh && k < left && (ac & unv) != unv;
+        if (!kMesh) {
+            for (uint32_t pm = __ballot_sync(0xffffffffu, open); pm; pm &= pm - 1) {
+                const int t0 = __ffs(pm) - 1;
+                const int32_t kt = __shfl_sync(0xffffffffu, beg + k, t0), lt = __shfl_sync(0xffffffffu, left - k, t0);
+                const unsigned long long ut = __shfl_sync(0xffffffffu, unv, t0);
+                unsigned long long at = __shfl_sync(0xffffffffu, ac, t0);
+                const int32_t len = lt > kMsScan * 32 * kMsUnroll ? kMsScan * 32 * kMsUnroll : lt;
+                int32_t o = 0;
+                for (; o < len && (at & ut) != ut; o += 32 * kMsUnroll) {
+                    int32_t y[kMsUnroll];
+#pragma unroll
+                    for (int t = 0; t < kMsUnroll; ++t)
+                        y[t] = o + 32 * t + lane < len ? __ldg(a.in_col + kt + o + 32 * t + lane) : -1;
+                    unsigned long long z = 0ull;
+#pragma unroll
+                    for (int t = 0; t < kMsUnroll; ++t) z |= y[t] >= 0 ? a.V[y[t]] : 0ull;
+                    at |= ((unsigned long long)__reduce_or_sync(0xffffffffu, (uint32_t)(z >> 32)) << 32) |
+                          __reduce_or_sync(0xffffffffu, (uint32_t)z);
+                }
+                if (lane == t0) {
+                    ac = at;
+                    acc.exam += (uint32_t)min(o, len);
+                    k += min(o, lt);
+                    open = k < left && (ac & unv) != unv;
+                }
+            }
+        }
+        const unsigned long long nw = ac & unv;
+        if (nw) {
+            if (sink && !open)  // nobody's in-neighbour: no other row reads its V, and it never joins the active list
+                a.V[v] |= nw;
+            else
+                Fn[v] = nw;  // zero before the level
+            if (!open) {
+                acc.n_new += (uint32_t)__popcll(nw);
+                record_depth(a, v, 0, nw, L + 1, false);
+            }
+        }
+        if (!kMesh && sink && !open && nw == unv) atomicOr(a.D + (v >> 5), 1u << (v & 31));
+        st.put(nw != 0ull && !open && !sink, v);
+        if (!kMesh && __any_sync(0xffffffffu, open))
+            ms_defer(lr, open, v, beg + k, left - k, st.cout);
     }
     st.flush_block<kMsThreads / 32>(bsm);
 }
@@ -905,11 +968,11 @@ __device__ __forceinline__ void ms_push_mesh(const MsArgs& a, int32_t L, const I
             else if (j == 0)
                 f[k] = atomicExch(Fc + u[k], 0ull);
             if (j == 0) {
-                w[k] = __ldg(a.first_out + u[k]);
+                w[k] = __ldg(a.first_in + u[k]);
             } else if (j < 3) {
-                w[k] = __ldg(reinterpret_cast<const int32_t*>(a.next_out + u[k]) + (j - 1));
+                w[k] = __ldg(reinterpret_cast<const int32_t*>(a.next_in + u[k]) + (j - 1));
             } else {
-                const int2 x = __ldg(reinterpret_cast<const int2*>(a.next_out + u[k]) + 1);
+                const int2 x = __ldg(reinterpret_cast<const int2*>(a.next_in + u[k]) + 1);
                 w[k] = x.x;
                 more |= x.y >= 0;
             }
@@ -1271,10 +1334,16 @@ __global__ void __launch_bounds__(kMsThreads, kOcc) ms_bfs_kernel(const __grid_c
                 ms_finalize<WL>(a, L, a.tlist, (uint32_t)lvl[5], a.Fb[r1], a.Tb[r1], st, stage_sum, acc);
             }
         } else {
-            if (kMesh) ms_clear_prev<WL>(a, a.ids[r2], prev_count, a.Fb[r2], a.Tb[r2]);
-            const bool one = a.W <= WL * a.group;  // one chunk of words: long rows can be deferred
-            for (int32_t c0 = 0; c0 < a.W; c0 += WL * a.group)
-                ms_pull<WL>(a, L, c0, a.Fb[r1], a.Tb[r1], mem.warp[wib].open_list, lr, one, st, stage_sum, acc);
+            if (kMesh) {
+                ms_clear_prev<WL>(a, a.ids[r2], prev_count, a.Fb[r2], a.Tb[r2]);
+                ms_pull_one<true>(a, L, a.Fb[r1], lr, st, stage_sum, acc);
+            } else if (WL == 1) {
+                ms_pull_one<false>(a, L, a.Fb[r1], lr, st, stage_sum, acc);
+            } else {
+                const bool one = a.W <= WL * a.group;  // one chunk of words: long rows can be deferred
+                for (int32_t c0 = 0; c0 < a.W; c0 += WL * a.group)
+                    ms_pull<WL>(a, L, c0, a.Fb[r1], a.Tb[r1], mem.warp[wib].open_list, lr, one, st, stage_sum, acc);
+            }
         }
         block_add_counts<kMsThreads / 32>(acc_mem, acc.n_new, acc.mf, acc.exam, kMesh ? acc.indeg : 0ull, &cout->n_new,
                                           &cout->mf_new, &cout->e_exam, kMesh ? &cout->indeg_new : nullptr);
@@ -1288,7 +1357,7 @@ __global__ void __launch_bounds__(kMsThreads, kOcc) ms_bfs_kernel(const __grid_c
             lvl[4] = ld_volatile_u64(&cout->q);
         }
         __syncthreads();
-        if (dir == GBX_DIR_PULL && lvl[2] != 0ull) {  // the level deferred long rows: the grid takes them now
+        if (!kMesh && dir == GBX_DIR_PULL && lvl[2] != 0ull) {  // the level deferred long rows: the grid takes them now
             const uint32_t rows = (uint32_t)lvl[2];
             Acc acc2;
             Stage st2{&mem.warp[wib].stage, 0, cout, a.ids[r1], a.qp[p1], a.qd[p1], a.out_ptr, a.in_ptr, 1, 0, &acc2};
@@ -1435,8 +1504,8 @@ gbx_status ms_run(Graph* G, Workspace& w, int32_t S, const int32_t* src_dev, voi
     a.in_ptr = G->in_ptr;
     a.in_col = G->in_col;
     a.nz_in = G->nz_in;
-    a.first_out = G->first_out;
-    a.next_out = G->next_out;
+    a.first_in = G->first_in;
+    a.next_in = G->next_in;
     a.V = w.msV;
     for (int k = 0; k < 3; ++k) a.Fb[k] = w.msF[k];
     for (int k = 0; k < kMsPlanes; ++k) a.P[k] = w.msP + (size_t)k * (size_t)G->n * (size_t)W;

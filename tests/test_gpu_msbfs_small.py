@@ -64,3 +64,25 @@ def test_direction_is_the_edge_quotient(alpha):
             assert np.array_equal(t["direction"] == gbx.DIR_PULL,
                                   t["mf"].astype(np.float64) > np.float64(a) * np.float64(og.nnz))
     g.free()
+
+
+def hubs(n, directed, seed):
+    """Random edges with some rows of in-degree around the five dense entries, the lane's share and the
+    24 more it takes, a few hundred, and thousands (beyond the warp's 2,048); directed: sinks too."""
+    r = np.random.default_rng(seed)
+    s, d = [r.integers(0, n // 2, 2 * n)], [r.integers(0, n, 2 * n)]
+    for k, deg in enumerate([4, 5, 6, 12, 13, 14, 36, 37, 38, 40, 300, 700, 2060, 2100, min(n - 1, 9000), n // 2]):
+        deg = min(deg, n // 2)
+        d.append(np.full(deg, n - 1 - 7 * k % n if k % 2 else 3 + 5 * k % n))
+        s.append(r.permutation(n // 2)[:deg])
+    return n, np.concatenate(s).astype(np.int32), np.concatenate(d).astype(np.int32), not directed
+
+
+@pytest.mark.parametrize("n", [97, 3000, 20011, 50021, 160001])
+@pytest.mark.parametrize("directed", [False, True])
+@pytest.mark.parametrize("S", [1, 20, 64])
+def test_one_word(n, directed, S):
+    n, s, d, sym = hubs(n, directed, n)
+    descs = [gbx.desc_init(), gbx.desc_init(direction=gbx.DIR_PULL), gbx.desc_init(alpha=0.2, pull_probe=4),
+             gbx.desc_init(direction=gbx.DIR_PULL, pull_probe=100), gbx.desc_init(blocks_per_sm=3)]
+    check(n, s, d, sym, S, descs, distinct=min(S, 12))
