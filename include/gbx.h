@@ -179,8 +179,9 @@ typedef struct {
     int32_t operand_reuse;   /* BFS pull tests "visited" instead of "in frontier" (Section 5.4; default 1) */
     int32_t trace;           /* BFS: record per-level statistics (see gbx_bfs_trace) */
     int32_t pull_probe;      /* BFS pull: in-neighbours one lane scans before its warp takes the row over
-                                (0 = default: 16 single-source, 8 batched; otherwise 4..1024).  Batched:
-                                a row still open after four times as many is shared by the grid */
+                                (0 = default: 16 single-source, 8 batched; otherwise 4..1024).  Batches of
+                                more than 64 sources: a row still open after four times as many is shared
+                                by the grid (on a small graph: by its block after so many) */
     int32_t blocks_per_sm;   /* BFS and SSSP kernels: persistent blocks per SM (0 = as many as fit;
                                 gbx_bfs: one on a small graph, where that is faster).
                                 gbx_bfs_batch and gbx_sssp: 1 or 2 caps the default build (two per

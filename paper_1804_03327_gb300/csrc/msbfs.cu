@@ -86,6 +86,7 @@ struct MsArgs {
     uint32_t more_from;
     int32_t* more[2];
     int32_t group;  // warp lanes that hold a vertex's words (a power of two)
+    int32_t team;   // warp lanes per row of a pull (ms_pull_few); 0: ms_pull
     unsigned long long timeout_ns;
 };
 
@@ -693,6 +694,187 @@ __device__ __forceinline__ void ms_pull_one(const MsArgs& a, int32_t L, unsigned
     st.flush_block<kMsThreads / 32>(bsm);
 }
 
+// A block's open rows of a pull level on a small graph: those with up to kMsFewWarp in-neighbours
+// left from the front of row, longer ones from its back, those with more than kMsFewBlock in most.
+// (20,000 vertices, 64 sources: listed after 2, 4 and 8 steps 129, 130 and 138 us; a warp each from
+// 96, 256 and 1,024 left 128, 129 and 133.)
+constexpr int32_t kMsFewWarp = 256;
+constexpr int32_t kMsFewBlock = 2048;
+constexpr int kMsFewSteps = 2;  // steps of a row's team before it is listed
+constexpr int kMsFewMost = 32;  // rows of most (further ones are taken as longer)
+struct MsFew {
+    int32_t row[kMsThreads], most[kMsFewMost];
+    int32_t cnt[3];
+    unsigned long long acc[64];
+};
+
+// ORs V of the in-neighbours [k, end) of a row into ac, team lanes (a power of two, at least the
+// group's) taking kMsUnroll a group and step, until what it misses (unv) is covered or `stop` is
+// reached.  All lanes of the warp call; row < 0: nothing to do.  Returns whether it is covered.
+template <int WL>
+__device__ __forceinline__ bool ms_team_scan(const MsArgs& a, const Group& gr, int team, int32_t row, int32_t& k,
+                                             int32_t end, int32_t stop, const Words<WL>& unv, Words<WL>& ac) {
+    const int lane = threadIdx.x & 31, tg = (lane & (team - 1)) / gr.size, step = kMsUnroll * (team / gr.size);
+    const uint32_t tmask = (team == 32 ? 0xffffffffu : (1u << team) - 1u) << (lane & ~(team - 1));
+    const int32_t w = WL * gr.sub;
+    bool covered = false;
+    int32_t u[kMsUnroll];  // the in-neighbours of this step; the next step's are loaded meanwhile
+#pragma unroll
+    for (int t = 0; t < kMsUnroll; ++t)
+        u[t] = row >= 0 && kMsUnroll * tg + t < end - k ? __ldg(a.in_col + k + kMsUnroll * tg + t) : -1;
+    while (__any_sync(0xffffffffu, row >= 0 && !covered && k < stop)) {
+        const bool go = row >= 0 && !covered && k < stop;
+        Words<WL> x[kMsUnroll];
+#pragma unroll
+        for (int t = 0; t < kMsUnroll; ++t)
+            x[t] = go && u[t] >= 0 && w < a.W ? ld_words<WL>(a.V + (size_t)u[t] * a.W + w) : zero_words<WL>();
+        if (go) k = end - k > step ? k + step : end;
+#pragma unroll
+        for (int t = 0; t < kMsUnroll; ++t)
+            u[t] = go && kMsUnroll * tg + t < end - k ? __ldg(a.in_col + k + kMsUnroll * tg + t) : -1;
+        bool cov = true;
+#pragma unroll
+        for (int j = 0; j < WL; ++j) {
+#pragma unroll
+            for (int t = 0; t < kMsUnroll; ++t) ac.x[j] |= x[t].x[j];
+            for (int o = gr.size; o < team; o <<= 1) ac.x[j] |= __shfl_xor_sync(0xffffffffu, ac.x[j], o);
+            cov &= (ac.x[j] & unv.x[j]) == unv.x[j];
+        }
+        const bool all = (__ballot_sync(0xffffffffu, cov) & tmask) == tmask;
+        covered |= go && all;
+    }
+    return covered;
+}
+
+// The pull on a small graph: every row its own team of a.team lanes, spread over the blocks.  A
+// level then lasts as long as its longest row, and ms_pull with its deferred rows (two more
+// grid barriers and a finalising pass) as long as several: rows still open after kMsFewSteps
+// steps are listed by the block and taken by as many lanes as there are for each, by a warp
+// each, or by the whole block.
+//
+// Batches on RMAT graphs with ms_pull and so: 1,000 vertices, 100 sources 208 and 102 us (a level 35 and
+// 10.5); 6,000 vertices, 100 sources 328 and 152; 20,000, 64 sources 175 and 125; 1,000, 700 sources 449
+// and 171.
+template <int WL>
+__device__ __forceinline__ void ms_pull_few(const MsArgs& a, int32_t L, unsigned long long* Fn, MsFew& few, Stage& st,
+                                            unsigned long long* bsm, Acc& acc) {
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    const Group gr(a.group);
+    const int32_t w = WL * gr.sub;
+    const bool wok = w < a.W;
+    const uint32_t chunks256 = (uint32_t)(a.W + 3) >> 2;
+    Words<WL> lm;
+#pragma unroll
+    for (int j = 0; j < WL; ++j) lm.x[j] = wok ? lane_mask(a.S, w + j) : 0ull;
+    struct Row {
+        int32_t k, end;
+        bool sink;
+        Words<WL> unv, ac;
+    };
+    auto open = [&](int32_t v) {
+        Row r{0, 0, false, zero_words<WL>(), zero_words<WL>()};
+        if (v >= 0) {
+            r.k = __ldg(a.in_ptr + v);
+            r.end = __ldg(a.in_ptr + v + 1);
+            r.sink = !a.symmetric && __ldg(a.out_ptr + v + 1) == __ldg(a.out_ptr + v);
+            if (wok) r.unv = ld_words<WL>(a.V + (size_t)v * a.W + w);
+#pragma unroll
+            for (int j = 0; j < WL; ++j) r.unv.x[j] = ~r.unv.x[j] & lm.x[j];
+        }
+        return r;
+    };
+    // the row's first group writes what is new; all lanes call (v < 0: nothing)
+    auto settle = [&](int32_t v, const Row& r, bool first_group) {
+        Words<WL> nw;
+        const bool mine = v >= 0 && first_group;
+#pragma unroll
+        for (int j = 0; j < WL; ++j) nw.x[j] = mine ? r.ac.x[j] & r.unv.x[j] : 0ull;
+        const bool any_new = gr.any(nw.any());
+        const bool full = gr.all(nw.x[0] == r.unv.x[0] && nw.x[WL - 1] == r.unv.x[WL - 1]);
+        ms_settle<WL>(a, L, v, w, r.sink, nw, r.unv, lm, Fn, acc);
+        const bool lead = mine && gr.sub == 0;
+        if (lead && r.sink && full) atomicOr(a.D + (v >> 5), 1u << (v & 31));
+        st.put(lead && any_new && !r.sink, v);
+    };
+    if (threadIdx.x < 3) few.cnt[threadIdx.x] = 0;
+    __syncthreads();
+    {
+        const int team = a.team;
+        const long long id = (((long long)wib * gridDim.x + blockIdx.x) * 32 + lane) / team;
+        int32_t v = id < a.n ? (int32_t)id : -1;
+        if (v >= 0 && !(((a.nz_in[v >> 5] & ~a.D[v >> 5]) >> (v & 31)) & 1u)) v = -1;
+        Row r = open(v);
+        const int32_t beg = r.k, own = max(a.probe, kMsFewSteps * kMsUnroll * (team / gr.size));
+        const bool leader = (lane & (team - 1)) == 0;
+        const bool list = r.end - beg > (team == 32 ? own + kMsFewBlock : 2 * own);
+        const bool covered = ms_team_scan<WL>(a, gr, team, v, r.k, r.end, list ? beg + own : r.end, r.unv, r.ac);
+        if (v >= 0 && leader) acc.exam += chunks256 * (uint32_t)(r.k - beg);
+        const bool done = covered || r.k >= r.end;
+        if (v >= 0 && !done && leader) {
+            const int32_t left = r.end - r.k;
+            const int at = left > kMsFewBlock ? atomicAdd(&few.cnt[2], 1) : kMsFewMost;
+            if (at < kMsFewMost)
+                few.most[at] = v;
+            else if (left > kMsFewWarp)
+                few.row[kMsThreads - 1 - atomicAdd(&few.cnt[1], 1)] = v;
+            else
+                few.row[atomicAdd(&few.cnt[0], 1)] = v;
+        }
+        settle(done ? v : -1, r, (lane & (team - 1)) < gr.size);
+    }
+    __syncthreads();
+    // listed rows are read from their start: what their team found is not kept
+    for (int part = 0; part < 2; ++part) {
+        const int32_t count = few.cnt[part];
+        int team = 32;
+        while (part == 0 && team > max(8, gr.size) && count * team > kMsThreads) team >>= 1;
+        for (int32_t h0 = wib * (32 / team); h0 < count; h0 += kMsThreads / team) {
+            const int32_t h = h0 + lane / team;
+            const int32_t v = h < count ? few.row[part ? kMsThreads - 1 - h : h] : -1;
+            Row r = open(v);
+            const int32_t beg = r.k;
+            ms_team_scan<WL>(a, gr, team, v, r.k, r.end, r.end, r.unv, r.ac);
+            if (v >= 0 && (lane & (team - 1)) == 0) acc.exam += chunks256 * (uint32_t)(r.k - beg);
+            settle(v, r, (lane & (team - 1)) < gr.size);
+        }
+    }
+    const int32_t most = min(few.cnt[2], kMsFewMost);
+    for (int32_t h = 0; h < most; ++h) {
+        const int32_t v = few.most[h];
+        Row r = open(v);
+        const int32_t piece = 4 * kMsUnroll * (32 / gr.size), first = r.k;  // in-neighbours a warp takes at a time
+        if ((int)threadIdx.x < a.W) few.acc[threadIdx.x] = 0ull;
+        __syncthreads();
+        for (int32_t o = wib * piece; o < r.end - first; o += piece * (kMsThreads / 32)) {
+            r.k = first + o;
+            const int32_t e = r.end - r.k < piece ? r.end : r.k + piece;
+            const int32_t beg = r.k;
+            ms_team_scan<WL>(a, gr, 32, v, r.k, e, e, r.unv, r.ac);
+            if (lane == 0) acc.exam += chunks256 * (uint32_t)(r.k - beg);
+            // with what the other warps have found meanwhile
+            if (wok) {
+#pragma unroll
+                for (int j = 0; j < WL; ++j) {
+                    if (gr.first == 0 && r.ac.x[j]) atomicOr(few.acc + w + j, r.ac.x[j]);
+                    r.ac.x[j] |= *(volatile unsigned long long*)(few.acc + w + j);
+                }
+            }
+            bool cov = true;
+#pragma unroll
+            for (int j = 0; j < WL; ++j) cov &= (r.ac.x[j] & r.unv.x[j]) == r.unv.x[j];
+            if (__all_sync(0xffffffffu, cov)) break;
+        }
+        __syncthreads();
+        if (wib == h % (kMsThreads / 32)) {
+#pragma unroll
+            for (int j = 0; j < WL; ++j) r.ac.x[j] = wok ? few.acc[w + j] : 0ull;
+            settle(v, r, gr.first == 0);
+        }
+        __syncthreads();
+    }
+    st.flush_block<kMsThreads / 32>(bsm);
+}
+
 // The deferred rows' chunks, round-robin over the warps: the groups of a warp take
 // kMsUnroll in-neighbours each per step, their results are ORed together and folded into
 // F_next (which already holds what the probe found).  A chunk of a row that is covered by
@@ -1207,6 +1389,7 @@ __global__ void __launch_bounds__(kMsThreads, kOcc) ms_bfs_kernel(const __grid_c
         uint32_t emit[WL == 2 ? kEmitSmem / 4 : 1];
     };
     __shared__ __align__(16) BlockMem mem;
+    __shared__ MsFew few_mem;
     __shared__ unsigned long long stage_sum[kMsThreads / 32];  // per-warp queue ranges of a block flush
     __shared__ unsigned long long lvl[6];
     __shared__ unsigned long long acc_mem[kMsThreads / 32][4];
@@ -1337,6 +1520,8 @@ __global__ void __launch_bounds__(kMsThreads, kOcc) ms_bfs_kernel(const __grid_c
             if (kMesh) {
                 ms_clear_prev<WL>(a, a.ids[r2], prev_count, a.Fb[r2], a.Tb[r2]);
                 ms_pull_one<true>(a, L, a.Fb[r1], lr, st, stage_sum, acc);
+            } else if (a.team) {
+                ms_pull_few<WL>(a, L, a.Fb[r1], few_mem, st, stage_sum, acc);
             } else if (WL == 1) {
                 ms_pull_one<false>(a, L, a.Fb[r1], lr, st, stage_sum, acc);
             } else {
@@ -1476,6 +1661,13 @@ static gbx_status ms_launch(Graph* G, const MsArgs& a0, int blocks, int per_sm_c
     const int full = per_sm * G->num_sms;
     const int nb = blocks > 1 ? (full / blocks > 0 ? full / blocks : 1) : full;  // a 1/blocks share of the GPU
     MsArgs a = a0;
+    // a team of lanes for every row where there are as many; with one word four a row, since a lane walks
+    // short rows well by itself (80,000 vertices, 20 sources: 108 us with a lane or two a row, 103
+    // without; 40,000: 101 and 99; 20,000 and 64 sources, four: 131 and 132)
+    const long long lanes = (long long)nb * kMsThreads;
+    a.team = 0;
+    if (a.W <= WL * a.group && (WL == 1 ? 4ll : (long long)a.group) * a.n <= lanes)
+        for (a.team = a.group; a.team < 32 && 2ll * a.team * a.n <= lanes;) a.team *= 2;
     void* args[] = {&a};
     GBX_CUDA_TRY(cudaLaunchCooperativeKernel((const void*)ms_bfs_kernel<WL, kOcc, kMesh>, dim3(nb), dim3(kMsThreads), args, 0,
                                              s));

@@ -73,7 +73,7 @@ def hubs(n, directed, seed):
     s, d = [r.integers(0, n // 2, 2 * n)], [r.integers(0, n, 2 * n)]
     for k, deg in enumerate([4, 5, 6, 12, 13, 14, 36, 37, 38, 40, 300, 700, 2060, 2100, min(n - 1, 9000), n // 2]):
         deg = min(deg, n // 2)
-        d.append(np.full(deg, n - 1 - 7 * k % n if k % 2 else 3 + 5 * k % n))
+        d.append(np.full(deg, (n - 1 - 7 * k) % n if k % 2 else (3 + 5 * k) % n))
         s.append(r.permutation(n // 2)[:deg])
     return n, np.concatenate(s).astype(np.int32), np.concatenate(d).astype(np.int32), not directed
 
@@ -86,3 +86,25 @@ def test_one_word(n, directed, S):
     descs = [gbx.desc_init(), gbx.desc_init(direction=gbx.DIR_PULL), gbx.desc_init(alpha=0.2, pull_probe=4),
              gbx.desc_init(direction=gbx.DIR_PULL, pull_probe=100), gbx.desc_init(blocks_per_sm=3)]
     check(n, s, d, sym, S, descs, distinct=min(S, 12))
+
+
+@pytest.mark.parametrize("S", [20, 64, 100, 200, 300, 700, 2100, 4100])
+@pytest.mark.parametrize("n,directed", [(3, False), (90, True), (2999, True), (9001, False), (19001, True),
+                                        (40009, False), (90001, True)])
+def test_teams(n, directed, S):
+    """Teams of 4 to 32 lanes a row and none (too many vertices for the words), one to 66 words."""
+    if n * S > 40_000_000:
+        pytest.skip("the same forms as with fewer sources")
+    n, s, d, sym = hubs(n, directed, n + S)
+    descs = [gbx.desc_init(), gbx.desc_init(direction=gbx.DIR_PULL), gbx.desc_init(alpha=0.1, blocks_per_sm=3)]
+    check(n, s, d, sym, S, descs, distinct=min(S, 10))
+
+
+@pytest.mark.parametrize("S", [3, 130])
+@pytest.mark.parametrize("n,deg", [(6000, 2400), (4000, 600)])
+def test_long_rows_only(n, deg, S):
+    """Every row is long: more in a block than it takes together (32), and none for the lanes alone."""
+    v = np.arange(n, dtype=np.int64)
+    s = ((v[:, None] + 1 + np.arange(deg)) % n).reshape(-1).astype(np.int32)
+    d = np.repeat(v, deg).astype(np.int32)
+    check(n, s, d, False, S, [gbx.desc_init(direction=gbx.DIR_PULL), gbx.desc_init()], distinct=3)
