@@ -1392,11 +1392,15 @@ __global__ void __launch_bounds__(kMsThreads, kOcc) ms_bfs_kernel(const __grid_c
     __shared__ MsFew few_mem;
     __shared__ unsigned long long stage_sum[kMsThreads / 32];  // per-warp queue ranges of a block flush
     __shared__ unsigned long long lvl[6];
+    // of the level under way: its queue (entries, out-edges), the entries of the one before, the pairs found by
+    // that one and when it ended; kept here rather than in every thread's registers
+    __shared__ unsigned long long now_q, now_pairs, now_mark;
+    __shared__ uint32_t now_prev;
     __shared__ unsigned long long acc_mem[kMsThreads / 32][4];
     const int wib = threadIdx.x >> 5;
     unsigned int* barc = a.bar->count + a.bar_parity;
     unsigned int bar_round = 0;
-    unsigned long long t_mark = gtid == 0 ? global_timer_ns() : 0ull;
+    if (threadIdx.x == 0) now_mark = global_timer_ns();
     // ---- init: V = F_k = 0, depth planes = 0, D = T_k = 0 (the output rows are written at the end)
     const size_t nw_total = (size_t)a.n * (size_t)a.W;
     for (size_t i = gtid; i < nw_total; i += gstride) {
@@ -1461,11 +1465,12 @@ __global__ void __launch_bounds__(kMsThreads, kOcc) ms_bfs_kernel(const __grid_c
     }
     __shared__ char* row_mem[kMesh ? 64 : 1];  // the output rows' addresses
     if (kMesh && threadIdx.x < 64) row_mem[threadIdx.x] = depth_row(a, (int)threadIdx.x < a.S ? threadIdx.x : 0);
-    if (threadIdx.x == 0) lvl[4] = ld_volatile_u64(&a.ctr[0].q);
+    if (threadIdx.x == 0) {
+        now_q = ld_volatile_u64(&a.ctr[0].q);
+        now_pairs = (unsigned long long)a.S;
+        now_prev = 0u;
+    }
     if (!grid_barrier(barc, gridDim.x, bar_round, a.status, a.timeout_ns)) return;
-    unsigned long long qv = lvl[4];
-    uint32_t prev_count = 0;  // size of the active list of level L - 1
-    long long pairs = a.S;
     for (int32_t L = 0;; ++L) {
         const int r0 = L % 3, r1 = (L + 1) % 3, r2 = (L + 2) % 3, p0 = L & 1, p1 = p0 ^ 1;
         LevelCtr* cout = a.ctr + ((L + 1) % 3);
@@ -1473,7 +1478,8 @@ __global__ void __launch_bounds__(kMsThreads, kOcc) ms_bfs_kernel(const __grid_c
             LevelCtr z = {};
             a.ctr[(L + 2) % 3] = z;
         }
-        const uint32_t qcount = (uint32_t)qv, qedges = (uint32_t)(qv >> 32);  // active vertices, their out-edges
+        const uint32_t qcount = (uint32_t)now_q, qedges = (uint32_t)(now_q >> 32);  // active vertices, their out-edges
+        const uint32_t prev_count = now_prev;  // entries of the list of level L - 1
         // direction for the whole batch: pull once the active edges exceed alpha * nnz
         int dir = a.mode;
         if (dir == GBX_DIR_AUTO) dir = qedges > a.push_most ? GBX_DIR_PULL : GBX_DIR_PUSH;
@@ -1560,12 +1566,10 @@ __global__ void __launch_bounds__(kMsThreads, kOcc) ms_bfs_kernel(const __grid_c
             }
             __syncthreads();
         }
-        qv = lvl[4];
-        if (kMesh && dir == GBX_DIR_PUSH) qv |= lvl[1] << 32;  // a mesh push lists without the degrees
         if (dir == GBX_DIR_PULL) {
             // V |= F for the vertices the pull found (their new lanes were kept apart so the
             // level read V as it was before it started)
-            ms_pull_commit<WL>(a, a.ids[r1], (uint32_t)qv, a.Fb[r1]);
+            ms_pull_commit<WL>(a, a.ids[r1], (uint32_t)lvl[4], a.Fb[r1]);
             if (!grid_barrier(barc, gridDim.x, bar_round, a.status, a.timeout_ns)) return;
         }
         const long long n_new = (long long)lvl[0];
@@ -1573,9 +1577,9 @@ __global__ void __launch_bounds__(kMsThreads, kOcc) ms_bfs_kernel(const __grid_c
             LevelRec r;
             r.direction = dir;
             r.level = L;
-            r.nf = (long long)qcount;
-            r.mf = (long long)qedges;
-            r.mu = pairs;
+            r.nf = (long long)(uint32_t)now_q;
+            r.mf = (long long)(now_q >> 32);
+            r.mu = (long long)now_pairs;
             r.e_exam = dir == GBX_DIR_PULL ? (long long)lvl[3] : -1;
             r.n_new = n_new;
             r.mf_new = (long long)lvl[1];
@@ -1585,8 +1589,8 @@ __global__ void __launch_bounds__(kMsThreads, kOcc) ms_bfs_kernel(const __grid_c
                 if (L > 0) a.trace[L - 1].mf_new = r.mf;
             }
             const unsigned long long now = global_timer_ns();
-            r.t_ns = (long long)(now - t_mark);
-            t_mark = now;
+            r.t_ns = (long long)(now - now_mark);
+            now_mark = now;
             a.trace[L] = r;
         }
         if (n_new == 0) {
@@ -1601,8 +1605,12 @@ __global__ void __launch_bounds__(kMsThreads, kOcc) ms_bfs_kernel(const __grid_c
             if (gtid == 0) atomicCAS(a.status + ST_ERROR, 0, (int)GBX_ERR_OVERFLOW);
             return;
         }
-        pairs = n_new;
-        prev_count = qcount;
+        if (threadIdx.x == 0) {
+            now_prev = (uint32_t)now_q;
+            now_pairs = lvl[0];
+            now_q = lvl[4] | (kMesh && dir == GBX_DIR_PUSH ? lvl[1] << 32 : 0ull);  // a mesh push lists without the degrees
+        }
+        __syncthreads();
     }
 }
 
