@@ -430,11 +430,12 @@ static gbx_status cl_geometry(Graph* G) {
 //    (82 on the grid alone), 80 for 100,000 (109), 91 for 500,000 (96), 235 for 2M (247).  A graph with
 //    hubs reaches most of its vertices in a few levels, which need the whole GPU: RMAT-22 takes 107 us.
 //  - a graph that one block's queue holds (n <= kClCap) with few entries: every level is
-//    small.  RMAT-10 (edge factor 16) takes 25 us here and 44 there, 8,192 vertices of edge
-//    factor 4 37 and 55; at 105K entries the two are even (7,000 vertices of edge factor 16,
-//    directed: 48.5 and 46.7).
+//    small.  RMAT-10 (edge factor 16) takes 25 us here and 41 on the grid (one block per SM).  Of 112 RMAT
+//    graphs (500 to 8,000 vertices, edge factors 2 to 24, directed and not) all 89 of up to 72K
+//    entries are faster here (69-72K: 41-43 us and 43-45), and of those with 74K to 95K the grid is:
+//    4,000 vertices of edge factor 12 43.7 and 41.4, of 16 49.2 and 42.0.
 constexpr int32_t kClMeshDegree = 32;
-constexpr int64_t kClTinyEntries = 96 * 1024;
+constexpr int64_t kClTinyEntries = 72 * 1024;
 
 static bool cl_tiny(const Graph* G) { return G->n <= kClCap && G->nnz <= kClTinyEntries; }
 

@@ -87,3 +87,25 @@ def test_sssp_across_the_handover(name, integer):
         gbx.graph_sync(g)
         assert np.array_equal(dist.cpu().numpy(), want), direction
     g.free()
+
+
+@pytest.mark.parametrize("n", [300, 8192, 8193])
+@pytest.mark.parametrize("entries", [72 * 1024 - 2, 72 * 1024, 72 * 1024 + 2])
+def test_bfs_around_the_size_of_a_whole_search(n, entries):
+    r = np.random.default_rng(entries)
+    key = np.unique(r.integers(0, n, 200000).astype(np.int64) * n + r.integers(0, n, 200000))
+    s, d = key // n, key % n
+    keep = r.permutation(np.flatnonzero(s < d))[: entries // 2]
+    s, d = s[keep].astype(np.int32), d[keep].astype(np.int32)
+    g = gbx.graph_build(n, s, d)
+    assert g.info()[1] == min(entries, 2 * len(s))
+    og = oracle.graph(n, s, d)
+    for src in (int(s[0]), int(d[-1])):
+        depth = torch.empty(n, dtype=torch.int32, device="cuda")
+        parent = torch.empty(n, dtype=torch.int32, device="cuda")
+        gbx.bfs(g, src, depth, parent)
+        gbx.graph_sync(g)
+        got = depth.cpu().numpy()
+        assert np.array_equal(got, oracle.bfs(og, src)[0])
+        assert_valid_parents_large(n, (np.concatenate([s, d]), np.concatenate([d, s])), got, parent.cpu().numpy(), src)
+    g.free()
