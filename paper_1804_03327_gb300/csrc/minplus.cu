@@ -22,7 +22,8 @@ namespace gbx {
 
 constexpr int kMpUnroll = 4;          // entries a lane has in flight
 constexpr int32_t kMpChunk = 512;     // entries of a deferred row a warp takes at a time
-constexpr int32_t kMpLongSteps = 4;   // steps left beyond which a row is deferred
+constexpr int32_t kMpLongSteps = 4;   // steps left beyond which a row is deferred ...
+constexpr int32_t kMpWarpSteps = 16;  // ... with a whole warp to a row
 
 struct MpArgs {
     int32_t n, nwords;
@@ -41,7 +42,7 @@ struct MpArgs {
     const float* push_val;
     uint32_t* ubm;
     uint32_t* pass;
-    LevelCtr* ctr;  // q: the push queue; n_new: finite entries of u; huge: deferred rows and their chunks
+    LevelCtr* ctr;  // q: the push queue; n_new: finite entries of u
     int32_t* q[2];  // [0] the push queue, [1] deferred rows: row, next entry, prefix of the chunk counts
     int32_t* qp[2];
     int32_t* qd[2];
@@ -49,6 +50,8 @@ struct MpArgs {
     const uint8_t* bytes;  // the dense mask, where the pull reads it as it is
     int32_t shorts;        // every row is short: a lane each
     int32_t dirty;         // the bitmaps have been written
+    unsigned long long* huge;  // deferred rows and their chunks; zero when the pull starts
+    int32_t longest;       // entries left beyond which a row is deferred
 };
 
 __device__ __forceinline__ int mp_dir(const MpArgs& a) {
@@ -57,8 +60,12 @@ __device__ __forceinline__ int mp_dir(const MpArgs& a) {
 }
 
 __device__ __forceinline__ bool mp_pass(const MpArgs& a, int32_t i) {
-    if (a.bytes) return (a.bytes[i] != 0) != (a.invert != 0u);
     return a.mask.format < 0 || (((a.pass[i >> 5] ^ a.invert) >> (i & 31)) & 1u);
+}
+
+// ... of a pull, which may read the mask's bytes
+__device__ __forceinline__ bool mp_pull_pass(const MpArgs& a, int32_t i) {
+    return a.bytes ? (a.bytes[i] != 0) != (a.invert != 0u) : mp_pass(a, i);
 }
 
 __device__ __forceinline__ Stage mp_stage(const MpArgs& a, StageBuf* sb, Acc* acc) {
@@ -74,6 +81,7 @@ __global__ void __launch_bounds__(kMxvThreads) mp_prep_kernel(const __grid_const
     __shared__ unsigned long long csm[kMxvThreads / 32][4];
     const int lane = threadIdx.x & 31;
     const int64_t gtid = (int64_t)blockIdx.x * kMxvThreads + threadIdx.x, gs = (int64_t)gridDim.x * kMxvThreads;
+    if (gtid == 0) *a.huge = 0ull;
     if (a.mask.format == GBX_DENSE) {
         for (int64_t w = gtid; w < a.nwords; w += gs)
             a.pass[w] = pack_word(static_cast<const uint8_t*>(a.mask.data), a.n, (int32_t)w);
@@ -144,7 +152,7 @@ __device__ __forceinline__ void mp_push(const MpArgs& a) {
 
 // Pull: groups of a.group lanes take a row each, kMpUnroll entries a lane in flight, and go on to
 // the next row as soon as their own is done.  A warp's row offsets come 32 rows at a time,
-// the next 32 loaded ahead.  A row with more than kMpLongSteps left is deferred:
+// the next 32 loaded ahead.  A row with more than a.longest entries left is deferred:
 // mp_last_kernel spreads its chunks over all warps.
 //
 // Bound by the gathers of u (4 bytes of a 32-byte L2 sector per entry).  A lane per row of up to
@@ -152,19 +160,20 @@ __device__ __forceinline__ void mp_push(const MpArgs& a) {
 // directed graph of 700,001 rows and 11.2M entries whose longest rows hold tens of thousands
 // (the whole call 358 us, now 93; rows deferred after 8 steps 95, after 16 102, after 64
 // 132).  The group is 8 lanes from 12 entries a row on, 4 from 6, else 1: rows shorter
-// than the group's step leave lanes idle, longer ones take several dependent steps.
+// than the group's step leave lanes idle, longer ones take several dependent steps.  On small graphs
+// it grows to a warp while a quarter of the lanes are enough, and a row of up to 2,176 entries is not
+// deferred then: 3,537 vertices and 24 edges each 11.2 us with a launch for the deferred rows, so 7.6.
 __device__ __forceinline__ void mp_pull(const MpArgs& a, uint8_t* list) {
     const int lane = threadIdx.x & 31;
     const int G = a.group, sub = lane & (G - 1), first = lane & ~(G - 1);
     const int32_t nwarps = (int32_t)((gridDim.x * kMxvThreads) >> 5);
     const int32_t R = a.rows, ntiles = (a.n + R - 1) / R;
     int32_t tile = (int32_t)((blockIdx.x * kMxvThreads + threadIdx.x) >> 5);
-    const int32_t kLong = kMpLongSteps * kMpUnroll * G;
     // a tile's rows: lane l holds row R tile + l
     auto load = [&](int32_t t, int32_t& b, int32_t& e) {
         const int64_t i = (int64_t)t * R + lane;
         b = e = 0;
-        if (t < ntiles && lane < R && i < a.n && mp_pass(a, (int32_t)i)) {
+        if (t < ntiles && lane < R && i < a.n && mp_pull_pass(a, (int32_t)i)) {
             b = __ldg(a.pull_ptr + i);
             e = __ldg(a.pull_ptr + i + 1);
         }
@@ -199,7 +208,7 @@ __device__ __forceinline__ void mp_pull(const MpArgs& a, uint8_t* list) {
             if (tile < ntiles && e0 == b0 && lane < R && base + lane < a.n) {
                 if (!a.accum)
                     a.w[base + lane] = INFINITY;
-                else if (mp_pass(a, base + lane) && isnan(a.w[base + lane]))
+                else if (mp_pull_pass(a, base + lane) && isnan(a.w[base + lane]))
                     a.w[base + lane] = INFINITY;
             }
         }
@@ -236,7 +245,7 @@ __device__ __forceinline__ void mp_pull(const MpArgs& a, uint8_t* list) {
             if (c[t] >= 0) m = fminf(m, x[t] + __ldg(a.u + c[t]));
         k = end - k > G * kMpUnroll ? k + G * kMpUnroll : end;
         const bool done = v >= 0 && k >= end;
-        const bool defer = v >= 0 && end - k > kLong;
+        const bool defer = v >= 0 && end - k > a.longest;
         if (!__any_sync(0xffffffffu, done || defer)) continue;
         float t = m;
         for (int o = 1; o < G; o <<= 1) t = fminf(t, __shfl_xor_sync(0xffffffffu, t, o));
@@ -251,7 +260,7 @@ __device__ __forceinline__ void mp_pull(const MpArgs& a, uint8_t* list) {
             const uint32_t tot = __shfl_sync(0xffffffffu, inc, 31);
             unsigned long long old = 0ull;
             if (lane == 0)
-                old = atomicAdd(&a.ctr->huge, ((unsigned long long)tot << 32) | (unsigned long long)__popc(dm));
+                old = atomicAdd(a.huge, ((unsigned long long)tot << 32) | (unsigned long long)__popc(dm));
             old = __shfl_sync(0xffffffffu, old, 0);
             if (defer && sub == 0) {
                 const uint32_t slot = (uint32_t)old + __popc(dm & lanemask_lt());
@@ -272,7 +281,7 @@ constexpr int32_t kMpShortRow = 32;
 __device__ __forceinline__ void mp_pull_short(const MpArgs& a) {
     for (int64_t i = (int64_t)blockIdx.x * kMxvThreads + threadIdx.x; i < a.n; i += (int64_t)gridDim.x * kMxvThreads) {
         float t = INFINITY;
-        if (!mp_pass(a, (int32_t)i)) {
+        if (!mp_pull_pass(a, (int32_t)i)) {
             if (a.accum) continue;
         } else {
             const int32_t beg = __ldg(a.pull_ptr + i), len = __ldg(a.pull_ptr + i + 1) - beg;
@@ -337,7 +346,7 @@ __global__ void __launch_bounds__(kMxvThreads) mp_last_kernel(const __grid_const
     pdl_begin();
     const int lane = threadIdx.x & 31;
     const int64_t gtid = (int64_t)blockIdx.x * kMxvThreads + threadIdx.x, gs = (int64_t)gridDim.x * kMxvThreads;
-    const unsigned long long huge = a.ctr->huge;
+    const unsigned long long huge = *a.huge;
     const int32_t entries = (int32_t)(uint32_t)huge, chunks = (int32_t)(huge >> 32);
     for (int64_t c = gtid >> 5; c < chunks; c += gs >> 5) {
         const int32_t h = warp_find_entry(a.qd[1], entries, c);
@@ -363,16 +372,21 @@ __global__ void __launch_bounds__(kMxvThreads) mp_last_kernel(const __grid_const
         for (int o = 16; o > 0; o >>= 1) m = fminf(m, __shfl_xor_sync(0xffffffffu, m, o));
         if (lane == 0 && m < a.w[v]) atomic_min_f32(a.w + v, m);
     }
-    for (int64_t w = a.dirty ? gtid : a.nwords; w < a.nwords; w += gs) {
-        a.ubm[w] = 0u;
-        if (a.mask.format >= 0) a.pass[w] = 0u;
+    if (a.dirty) {
+        for (int64_t w = gtid; w < a.nwords; w += gs) {
+            a.ubm[w] = 0u;
+            if (a.mask.format >= 0) a.pass[w] = 0u;
+        }
+        if (gtid == 0) {
+            a.ctr->q = 0ull;
+            a.ctr->n_new = 0ull;
+        }
+        return;
     }
-    // the last block to have read the number of deferred rows clears it
+    // nothing clears the number before the next such call: the last block to have read it does
     __syncthreads();
     if (threadIdx.x == 0 && atomicAdd(&a.ctr->list, 1ull) == gridDim.x - 1) {
-        a.ctr->q = 0ull;
-        a.ctr->n_new = 0ull;
-        a.ctr->huge = 0ull;
+        *a.huge = 0ull;
         a.ctr->list = 0ull;
     }
 }
@@ -388,7 +402,7 @@ gbx_status mxv_minplus(Graph* G, float* w, const MxvVec& mask, const float* u, c
     a.accum = d.accum ? 1 : 0;
     a.dir = d.direction;
     a.group = G->nnz > 12ll * G->n ? 8 : (G->nnz > 6ll * G->n ? 4 : 1);
-    a.push_most = mxv_push_most(G->n, d.alpha);
+    a.push_most = a.dir == GBX_DIR_AUTO ? mxv_push_most(G->n, d.alpha) : 0;
     a.u = u;
     a.w = w;
     a.pull_ptr = d.transpose ? G->in_ptr : G->out_ptr;
@@ -411,8 +425,13 @@ gbx_status mxv_minplus(Graph* G, float* w, const MxvVec& mask, const float* u, c
     a.bytes = direct && mask.format == GBX_DENSE ? static_cast<const uint8_t*>(mask.data) : nullptr;
     a.shorts = a.group == 1 && longest <= kMpShortRow;
     a.dirty = direct ? 0 : 1;
-    const bool deferring = !a.shorts && longest > (kMpLongSteps + 1) * kMpUnroll * a.group;
+    a.huge = direct ? &G->ws.mx_ctr->mf_new : &G->ws.mx_ctr->huge;
     const unsigned full = (unsigned)G->num_sms * 6u;
+    const long long lanes = (long long)full * kMxvThreads;
+    if (!a.shorts)
+        while (a.group < 32 && 4ll * a.group * a.n <= lanes) a.group *= 2;
+    a.longest = kMpUnroll * a.group * (a.group == 32 ? kMpWarpSteps : kMpLongSteps);
+    const bool deferring = !a.shorts && longest > a.longest + kMpUnroll * a.group;
     // 5,000 vertices of 30 entries (157 warps of 32 rows): 18.5 us, with 4 rows a warp and one launch fewer 12.3
     a.rows = 32;
     while (a.rows * a.group > 32 && (long long)a.n * 2 < (long long)a.rows * full * (kMxvThreads / 32)) a.rows /= 2;

@@ -686,7 +686,7 @@ static gbx_status mxv_bool(Graph* G, gbx_vector* w, const gbx_vector* mask, cons
     a.invert = d.mask_complement ? 0xffffffffu : 0u;
     a.accum = d.accum ? 1 : 0;
     a.dir = d.direction;
-    a.push_most = mxv_push_most(G->n, d.alpha);
+    a.push_most = a.dir == GBX_DIR_AUTO ? mxv_push_most(G->n, d.alpha) : 0;
     a.early_exit = d.early_exit ? 1 : 0;
     a.stats = d.trace ? reinterpret_cast<MxvStats*>(G->ws.ctr + 3) : nullptr;
     a.push_ptr = d.transpose ? G->out_ptr : G->in_ptr;

@@ -14,7 +14,7 @@ torch = pytest.importorskip("torch")
 N = 3001
 
 
-def graph(k, longest):
+def graph(k, longest, N=N):
     """Every vertex has edges to the k next ones; vertex 5 has `longest` in-edges from elsewhere."""
     s = np.repeat(np.arange(N, dtype=np.int32), k)
     d = ((s + np.tile(np.arange(1, k + 1, dtype=np.int32), N)) % N).astype(np.int32)
@@ -27,8 +27,8 @@ def graph(k, longest):
 @pytest.mark.parametrize("k,longest", [(4, 3), (4, 20), (4, 21), (4, 32), (4, 33), (4, 512 + 4), (4, 2000),
                                        (8, 80), (8, 81), (8, 700), (16, 160), (16, 161), (16, 2500), (30, 0)])
 @pytest.mark.parametrize("transpose", [0, 1])
-def test_row_lengths(k, longest, transpose):
-    s, d = graph(k, longest)
+def test_row_lengths(k, longest, transpose, N=N):
+    s, d = graph(k, longest, N)
     rng = np.random.default_rng(k)
     val = rng.random(len(s)).astype(np.float32)
     og = oracle.graph_weighted(N, s, d, val, symmetrize=False)
@@ -49,3 +49,11 @@ def test_row_lengths(k, longest, transpose):
                                   alpha=0.01))
             assert np.array_equal(w.cpu().numpy(), want), (masked, complement, accum, direction)
     g.free()
+
+
+@pytest.mark.parametrize("n", [5003, 14401, 60001])
+@pytest.mark.parametrize("k,longest", [(4, 20), (4, 21), (4, 33), (4, 600), (7, 80), (7, 81), (16, 160), (16, 161),
+                                       (16, 320), (16, 321), (5, 640), (5, 2176), (5, 2177), (5, 4000)])
+def test_row_lengths_by_group_width(n, k, longest):
+    """More vertices: fewer lanes a row."""
+    test_row_lengths(k, longest, 1, n)
