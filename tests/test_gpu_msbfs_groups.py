@@ -86,3 +86,26 @@ def test_mesh_batches(w, h, S, k):
             assert [int(x) for x in tr["nf"]] == [int(x.sum()) for x in active]
             assert [int(x) for x in tr["mf"]] == [int(deg[x].sum()) for x in active]
     g.free()
+
+
+@pytest.mark.parametrize("k", [1, 2, 5, 12])
+@pytest.mark.parametrize("dtype", [torch.int16, torch.int32])
+def test_lists_beyond_the_queue_arrays(k, dtype):
+    """Disjoint complete graphs of five vertices, every vertex a source: nnz = 4 n, and every edge lists its
+    end at the first level, 4 n entries where the queue arrays hold 3 n."""
+    a, b = np.triu_indices(5, 1)
+    n = 5 * k
+    s = (np.arange(k)[:, None] * 5 + a).reshape(-1).astype(np.int32)
+    d = (np.arange(k)[:, None] * 5 + b).reshape(-1).astype(np.int32)
+    g = gbx.graph_build(n, s, d)
+    assert g.info()[1] == 4 * n
+    depth = torch.full((n, n), 55, dtype=dtype, device="cuda")
+    v = np.arange(n)
+    want = np.where(v[:, None] // 5 == v // 5, 1, -1) + np.where(v[:, None] == v, -1, 0)
+    for _ in range(3):
+        gbx.bfs_batch(g, v.astype(np.int32), depth, gbx.desc_init(alpha=1e30))
+        gbx.graph_sync(g)
+        assert np.array_equal(depth.cpu().numpy(), want)
+        tr = gbx.bfs_batch_trace(g)
+        assert [int(x) for x in tr["nf"]] == [n, n] and [int(x) for x in tr["n_new"]] == [4 * n, 0]
+    g.free()
