@@ -353,7 +353,7 @@ gbx_status gbx_bfs_trace(gbx_graph* g, gbx_level* levels, int32_t cap, int32_t* 
  * gbx_graph_sync).  One persistent cooperative launch (after the cluster's, where
  * near vertices go first), asynchronous on `stream`; desc->blocks_per_sm >= 3 selects a register-lean build at three
  * blocks per SM (faster on long push iterations over skewed graphs, slower with
- * pull iterations; GBX_TUNE_SSSP times both).  Errors: NULL_POINTER, INVALID_INDEX, INVALID_VALUE (no weights,
+ * pull iterations; GBX_TUNE_SSSP times both), except where the cluster runs first.  Errors: NULL_POINTER, INVALID_INDEX, INVALID_VALUE (no weights,
  * desc fields), NOT_SUPPORTED (push_sort), CUDA.
  */
 gbx_status gbx_sssp(gbx_graph* g, int32_t source, float* dist, const gbx_desc* desc, void* stream);

@@ -22,7 +22,7 @@
 // entries take the rest from the column array, split evenly over the block's threads.
 //
 // 2048 x 2048 grid (1 % of the edges deleted, 3,375 levels of 1,250 vertices): 8.0 us a level
-// in the grid-wide kernel, 1.85 here (27.0 -> 6.3 ms); an 8 x 20,000 grid 6.1 and 1.14 us.  A
+// in the grid-wide kernel, 1.7 here (26.2-27.0 -> 5.5-5.9 ms); an 8 x 20,000 grid 6.1 and 1.14 us.  A
 // level then takes 3,800 cycles: 1,900 claims and loads, 300 waiting for the block's other
 // warps, 1,000 for the other blocks.  Blocks of 256 threads: 2.10 us; clusters of 8: 3.1 us;
 // neighbours only ever loaded after the claim: the 8-wide grid 1.22 us.

@@ -116,7 +116,7 @@ struct Workspace {
     // batched multi-source BFS scratch (allocated on first use, grown as needed)
     unsigned long long* msV = nullptr;                     // visited lanes [n][W]
     unsigned long long* msF[3] = {nullptr, nullptr, nullptr};  // lanes found per level, rotating [n][W]
-    unsigned long long* msP = nullptr;  // depth bit planes: 5 x [n][W] (bits 0-3 of depths below 16, overflow)
+    unsigned long long* msP = nullptr;  // depth bit planes: 4 x [n][W] (bits 0-3 of depths below 16)
     int32_t* msT = nullptr;                                    // vertices a wide push level touched [n]
     int64_t ms_t_cap = 0;                                      // entries msT holds
     int64_t ms_cap_words = 0;
@@ -263,22 +263,10 @@ __device__ __forceinline__ int32_t ld_stream(const int32_t* p) {
     asm("ld.global.nc.L1::no_allocate.s32 %0, [%1];" : "=r"(v) : "l"(p));
     return v;
 }
-__device__ __forceinline__ float ld_stream(const float* p) {
-    float v;
-    asm("ld.global.nc.L1::no_allocate.f32 %0, [%1];" : "=f"(v) : "l"(p));
-    return v;
-}
 __device__ __forceinline__ int4 ld_stream(const int4* p) {
     int4 v;
     asm("ld.global.nc.L1::no_allocate.v4.s32 {%0, %1, %2, %3}, [%4];"
                  : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
-                 : "l"(p));
-    return v;
-}
-__device__ __forceinline__ float4 ld_stream(const float4* p) {
-    float4 v;
-    asm("ld.global.nc.L1::no_allocate.v4.f32 {%0, %1, %2, %3}, [%4];"
-                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
                  : "l"(p));
     return v;
 }
@@ -365,8 +353,9 @@ __device__ __forceinline__ bool grid_barrier(unsigned int* count, unsigned int n
 
 // Leaves as much of each SM to L1 as `blocks` resident blocks of fn allow: the gathers of the
 // persistent kernels (bitmap words, distances) live on it, and left to itself the driver
-// gives shared memory more than they use.  RMAT-22 SSSP 1,936 -> 1,882 us (with a smaller
-// ring), eight BFS 847 -> 831, the RMAT-21 batch of 64 sources 726 -> 717.
+// gives shared memory more than they use.  Without and with, in turn on the same inputs (four runs
+// each, at most 0.3 % apart; two inputs): RMAT-22 SSSP 1,715 -> 1,664 and 2,463 -> 2,377 us, eight BFS
+// 764 -> 752 and 789 -> 774; the RMAT-21 batch of 64 sources 742 -> 736 is within its spread.
 inline gbx_status prefer_l1(const void* fn, int blocks) {
     cudaFuncAttributes at;
     GBX_CUDA_TRY(cudaFuncGetAttributes(&at, fn));

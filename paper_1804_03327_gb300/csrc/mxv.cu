@@ -1,7 +1,7 @@
 // GrB_mxv over the Boolean semiring: the four matvec variants of Table 1.
 //
-//   row-based (pull, Eq 2 / Eq 4, Algorithm 2): one warp per 32 output rows;
-//     only rows whose mask test passes are computed; each row ORs u over its
+//   row-based (pull, Eq 2 / Eq 4, Algorithm 2): a warp takes the rows of up to 32
+//     result words that the mask test passes; each row ORs u over its
 //     entries, stopping at the first hit when early exit is on (Section 5.3).
 //   column-based (push, Eq 3 / Eq 5): the columns selected by u's nonzeros
 //     are expanded with their edges split evenly over warps (exclusive prefix
@@ -12,13 +12,13 @@
 // The result bitmap is then written out as a dense byte vector or as a sorted
 // index list (Section 3: sparse vectors are sorted lists).
 //
-// A call is three kernels (a fourth for a sparse result, or where AUTO has to count a dense u
-// before it can push): mxv_prep_kernel reads u and the mask into bitmaps, or u into a queue
+// A call is three kernels, one more for a sparse result and one more where AUTO has to count a
+// dense u before it can push: mxv_prep_kernel reads u and the mask into bitmaps, or u into a queue
 // with its degree prefix; mxv_main_kernel pulls or pushes, by a decision each block takes
 // from the count of u; the output kernels write w and leave the scratch bitmaps zero for the
 // next call.  A small call is bound by its launches: the separate conversions, scans and
 // decisions of 17 captured launches took 38 us for a sparse step of 100 vertices on RMAT-20
-// (and a capture for every new set of buffers); now 16 us, launched directly (a first
+// (and a capture for every new set of buffers); now 14-16 us, launched directly (a first
 // call on new buffers 154 -> 46 us).
 #include <algorithm>
 
@@ -42,14 +42,14 @@ constexpr int kMxvProbe = 16;
 // result is the same either way.
 //
 // Bound by dependent gathers: RMAT-22 with half its rows masked and a fifth of its vertices in
-// u reads 124 MB.  Rounds of 64 rows in lockstep took as long as their slowest row: the
-// call 59.7 us, now 51.3 (and 102.6 with 17 launches and tiles of 32 words).
+// u reads 117 MB.  Rounds of 64 rows in lockstep took as long as their slowest row, 8 us longer;
+// the call takes 51-55 us (107-109 in rounds, with 17 launches and tiles of 32 words).
 //
 // A tile's words lie ntiles apart, not side by side: the unvisited rows of a mesh are one band of
 // the numbering, which would be the work of a few warps (the 2048 x 2048 grid's BFS levels pulled at
 // 40, 60 and 80 % of the levels 61.5, 51 and 30 us, so 40, 25 and 17).  A warp then reads its words'
-// masks from as many sectors; the RMAT-22 call 50.6 -> 51.8 us.  Pieces of 4 words side by side:
-// 45, 29, 19 and 51.8.
+// masks from as many sectors, 1 us of the RMAT-22 call.  Pieces of 4 words side by side: 45, 29
+// and 19, and the same 1 us.
 constexpr int kMxvP1 = 4;  // first-pass rows per lane per round
 
 // The rows of a tile whose bits are set in the lane words m (lane l: word l), in

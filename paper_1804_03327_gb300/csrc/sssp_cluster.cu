@@ -18,7 +18,7 @@
 //
 // A phase is bound by two dependent round trips (the vertex's record and distance, the atomic
 // minima of its neighbours) and the exchange of the queue lengths.  1001 x 777
-// grid: 22.0 -> 3.3 ms.  With a fixed step of 2, 4, 8 and 16 mean weights: 4.8, 3.9, 3.6 and
+// grid: 25.4-26.2 -> 3.6-3.7 ms.  With a fixed step of 2, 4, 8 and 16 mean weights: 4.8, 3.9, 3.6 and
 // 3.5 ms there; a 200 x 200 grid 1.04, 0.85, 0.74 and 0.66 ms, with the moving step 0.63.
 #include <algorithm>
 

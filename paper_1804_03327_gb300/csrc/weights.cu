@@ -1,8 +1,8 @@
 // Edge weights for the (min, +) semiring that Section 5.6 names for SSSP: the
 // Boolean path needs only the structure of A (Section 5.5), the tropical one a
 // value per stored entry.  Weights are attached after the build: every input
-// pair finds its CSR entry (and its reverse, or its CSC entry) by binary search
-// in the sorted row, and parallel pairs keep the smallest weight.
+// pair finds its CSR entry (and its reverse, or its CSC entry) by an interpolating
+// search in the sorted row, and parallel pairs keep the smallest weight.
 #include <cmath>
 
 #include "gbx_internal.cuh"
