@@ -55,12 +55,15 @@ def test_a_build_that_found_no_memory_leaves_the_next_one_alone():
     torch.cuda.empty_cache()
     free, _ = torch.cuda.mem_get_info()
     held = torch.empty(free - (300 << 20), dtype=torch.uint8, device="cuda")
-    with pytest.raises(gbx.GbxError):
-        gbx.graph_build(n, s, d)
-    g = gbx.graph_build(10, s, d)
-    depth = torch.empty(10, dtype=torch.int32, device="cuda")
-    gbx.bfs(g, 0, depth)
-    gbx.graph_sync(g)
-    assert depth.tolist() == [0, 1] + [-1] * 8
-    del held
-    g.free()
+    try:
+        with pytest.raises(gbx.GbxError):
+            gbx.graph_build(n, s, d)
+        g = gbx.graph_build(10, s, d)
+        depth = torch.empty(10, dtype=torch.int32, device="cuda")
+        gbx.bfs(g, 0, depth)
+        gbx.graph_sync(g)
+        assert depth.tolist() == [0, 1] + [-1] * 8
+        g.free()
+    finally:  # the memory goes back to the device, not only to the allocator's cache
+        del held
+        torch.cuda.empty_cache()

@@ -106,14 +106,18 @@ def test_weights_without_memory_for_the_mesh_records():
     torch.cuda.empty_cache()
     free, _ = torch.cuda.mem_get_info()
     held = torch.empty(free - (200 << 20), dtype=torch.uint8, device="cuda")
-    for room in (False, True):
-        if room:
-            del held
-            torch.cuda.empty_cache()
-        gbx.graph_set_weights(g, s, d, w)
-        dist.fill_(-1.0)
-        gbx.sssp(g, 0, dist)
-        gbx.graph_sync(g)
-        assert np.array_equal(dist.cpu().numpy(), want)
+    try:
+        for room in (False, True):
+            if room:
+                held = None
+                torch.cuda.empty_cache()
+            gbx.graph_set_weights(g, s, d, w)
+            dist.fill_(-1.0)
+            gbx.sssp(g, 0, dist)
+            gbx.graph_sync(g)
+            assert np.array_equal(dist.cpu().numpy(), want)
+    finally:  # the memory goes back to the device, not only to the allocator's cache
+        held = None
+        torch.cuda.empty_cache()
     g.free()
     small.free()
