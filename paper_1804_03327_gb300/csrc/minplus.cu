@@ -150,10 +150,44 @@ __device__ __forceinline__ void mp_push(const MpArgs& a) {
     }
 }
 
+// The minimum over entries [beg, beg + len) of a row, by a warp.
+__device__ __forceinline__ float mp_chunk(const MpArgs& a, int32_t beg, int32_t len) {
+    float m = INFINITY;
+    for (int32_t o = threadIdx.x & 31; o < len; o += 32 * kMpUnroll) {
+        int32_t j[kMpUnroll];
+        float x[kMpUnroll];
+#pragma unroll
+        for (int t = 0; t < kMpUnroll; ++t) {
+            const bool in = o + 32 * t < len;
+            j[t] = in ? __ldg(a.pull_col + beg + o + 32 * t) : -1;
+            x[t] = in ? __ldg(a.pull_val + beg + o + 32 * t) : INFINITY;
+        }
+#pragma unroll
+        for (int t = 0; t < kMpUnroll; ++t)
+            if (j[t] >= 0) m = fminf(m, x[t] + __ldg(a.u + j[t]));
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) m = fminf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    return m;
+}
+
+// The long rows of a small graph a block finishes itself (mp_pull<true>): no launch for them.  A pull of
+// 50,000 rows that a mask lets 1 % of through, 9.8-12.3 us with that launch, takes 7.5; one of 5,000
+// rows 12.3, now 10.3.  A block that meets more than kMpLongs leaves the rest to the groups that have them.
+// Above 58,000 rows (fewer than four lanes each) a block meets too many: 388,799 rows, 4 directed
+// edges each, 30 us with the launch and 48 without.
+constexpr int kMpLongs = 64;
+constexpr int32_t kMpBlockRow = 16384;
+struct MpLong {
+    int2 row[kMpLongs];  // row, next entry
+    float part[kMxvThreads / 32];
+    int count;
+};
+
 // Pull: groups of a.group lanes take a row each, kMpUnroll entries a lane in flight, and go on to
 // the next row as soon as their own is done.  A warp's row offsets come 32 rows at a time,
 // the next 32 loaded ahead.  A row with more than a.longest entries left is deferred:
-// mp_last_kernel spreads its chunks over all warps.
+// mp_last_kernel spreads its chunks over all warps, or (kBlock) the block's warps take them in the end.
 //
 // Bound by the gathers of u (4 bytes of a 32-byte L2 sector per entry).  A lane per row of up to
 // 32 entries, one load at a time, and a warp for each longer row had taken 316 us on a
@@ -163,7 +197,12 @@ __device__ __forceinline__ void mp_push(const MpArgs& a) {
 // than the group's step leave lanes idle, longer ones take several dependent steps.  On small graphs
 // it grows to a warp while a quarter of the lanes are enough, and a row of up to 2,176 entries is not
 // deferred then: 3,537 vertices and 24 edges each 11.2 us with a launch for the deferred rows, so 7.6.
-__device__ __forceinline__ void mp_pull(const MpArgs& a, uint8_t* list) {
+template <bool kBlock>
+__device__ __forceinline__ void mp_pull(const MpArgs& a, uint8_t* list, MpLong& lo) {
+    if constexpr (kBlock) {
+        if (threadIdx.x == 0) lo.count = 0;
+        __syncthreads();
+    }
     const int lane = threadIdx.x & 31;
     const int G = a.group, sub = lane & (G - 1), first = lane & ~(G - 1);
     const int32_t nwarps = (int32_t)((gridDim.x * kMxvThreads) >> 5);
@@ -245,7 +284,14 @@ __device__ __forceinline__ void mp_pull(const MpArgs& a, uint8_t* list) {
             if (c[t] >= 0) m = fminf(m, x[t] + __ldg(a.u + c[t]));
         k = end - k > G * kMpUnroll ? k + G * kMpUnroll : end;
         const bool done = v >= 0 && k >= end;
-        const bool defer = v >= 0 && end - k > a.longest;
+        bool defer = v >= 0 && end - k > a.longest;
+        if (kBlock && __any_sync(0xffffffffu, defer)) {  // to the block, as long as its list has room
+            int slot = kMpLongs;
+            if (defer && sub == 0) slot = atomicAdd(&lo.count, 1);
+            slot = __shfl_sync(0xffffffffu, slot, first);
+            defer = defer && slot < kMpLongs;
+            if (defer && sub == 0) lo.row[slot] = make_int2(v, k);
+        }
         if (!__any_sync(0xffffffffu, done || defer)) continue;
         float t = m;
         for (int o = 1; o < G; o <<= 1) t = fminf(t, __shfl_xor_sync(0xffffffffu, t, o));
@@ -253,7 +299,7 @@ __device__ __forceinline__ void mp_pull(const MpArgs& a, uint8_t* list) {
             if (a.accum) t = fminf(t, a.w[v]);
             a.w[v] = t;
         }
-        const uint32_t dm = __ballot_sync(0xffffffffu, defer && sub == 0);
+        const uint32_t dm = kBlock ? 0u : __ballot_sync(0xffffffffu, defer && sub == 0);
         if (dm) {
             const uint32_t nch = defer && sub == 0 ? (uint32_t)(end - k + kMpChunk - 1) / kMpChunk : 0u;
             const uint32_t inc = warp_inclusive_sum(nch);
@@ -270,6 +316,25 @@ __device__ __forceinline__ void mp_pull(const MpArgs& a, uint8_t* list) {
             }
         }
         if (done || defer) v = -1;
+    }
+    if constexpr (!kBlock) return;
+    // the block's long rows, one after another, its warps taking kMpChunk entries at a time
+    __syncthreads();
+    const int wib = threadIdx.x >> 5, count = min(lo.count, kMpLongs);
+    for (int h = 0; h < count; ++h) {
+        const int32_t row = lo.row[h].x, beg = lo.row[h].y, len = __ldg(a.pull_ptr + row + 1) - beg;
+        float least = INFINITY;
+        for (int32_t o = kMpChunk * wib; o < len; o += kMpChunk * (kMxvThreads / 32))
+            least = fminf(least, mp_chunk(a, beg + o, len - o < kMpChunk ? len - o : kMpChunk));
+        if (lane == 0) lo.part[wib] = least;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            least = a.w[row];
+#pragma unroll
+            for (int x = 0; x < kMxvThreads / 32; ++x) least = fminf(least, lo.part[x]);
+            a.w[row] = least;
+        }
+        __syncthreads();
     }
 }
 
@@ -304,15 +369,17 @@ __device__ __forceinline__ void mp_pull_short(const MpArgs& a) {
 }
 
 // Pull, push, or -- AUTO found u sparse -- the queue (and w = +inf) for mp_push_kernel.
+template <bool kBlock>
 __global__ void __launch_bounds__(kMxvThreads, 6) mp_main_kernel(const __grid_constant__ MpArgs a) {
     pdl_begin();
     __shared__ StageBuf sb[kMxvThreads / 32];
     __shared__ unsigned long long bsm[kMxvThreads / 32];
+    __shared__ MpLong longs;
     if (mp_dir(a) == GBX_DIR_PULL) {
         if (a.shorts)
             mp_pull_short(a);
         else
-            mp_pull(a, reinterpret_cast<uint8_t*>(sb + (threadIdx.x >> 5)));
+            mp_pull<kBlock>(a, reinterpret_cast<uint8_t*>(sb + (threadIdx.x >> 5)), longs);
     } else if (a.dir == GBX_DIR_PUSH) {
         mp_push(a);
     } else {
@@ -354,22 +421,7 @@ __global__ void __launch_bounds__(kMxvThreads) mp_last_kernel(const __grid_const
         const int32_t rend = __ldg(a.pull_ptr + v + 1);
         const int32_t beg = a.qp[1][h] + (int32_t)(c - a.qd[1][h]) * kMpChunk;
         const int32_t len = rend - beg < kMpChunk ? rend - beg : kMpChunk;
-        float m = INFINITY;
-        for (int32_t o = lane; o < len; o += 32 * kMpUnroll) {
-            int32_t j[kMpUnroll];
-            float x[kMpUnroll];
-#pragma unroll
-            for (int t = 0; t < kMpUnroll; ++t) {
-                const bool in = o + 32 * t < len;
-                j[t] = in ? __ldg(a.pull_col + beg + o + 32 * t) : -1;
-                x[t] = in ? __ldg(a.pull_val + beg + o + 32 * t) : INFINITY;
-            }
-#pragma unroll
-            for (int t = 0; t < kMpUnroll; ++t)
-                if (j[t] >= 0) m = fminf(m, x[t] + __ldg(a.u + j[t]));
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) m = fminf(m, __shfl_xor_sync(0xffffffffu, m, o));
+        const float m = mp_chunk(a, beg, len);
         if (lane == 0 && m < a.w[v]) atomic_min_f32(a.w + v, m);
     }
     if (a.dirty) {
@@ -384,6 +436,7 @@ __global__ void __launch_bounds__(kMxvThreads) mp_last_kernel(const __grid_const
         return;
     }
     // nothing clears the number before the next such call: the last block to have read it does
+    if (huge == 0ull) return;
     __syncthreads();
     if (threadIdx.x == 0 && atomicAdd(&a.ctr->list, 1ull) == gridDim.x - 1) {
         *a.huge = 0ull;
@@ -431,7 +484,8 @@ gbx_status mxv_minplus(Graph* G, float* w, const MxvVec& mask, const float* u, c
     if (!a.shorts)
         while (a.group < 32 && 4ll * a.group * a.n <= lanes) a.group *= 2;
     a.longest = kMpUnroll * a.group * (a.group == 32 ? kMpWarpSteps : kMpLongSteps);
-    const bool deferring = !a.shorts && longest > a.longest + kMpUnroll * a.group;
+    const bool block = direct && !a.shorts && longest <= kMpBlockRow && 4ll * a.n <= lanes;
+    const bool deferring = !a.shorts && !block && longest > a.longest + kMpUnroll * a.group;
     // 5,000 vertices of 30 entries (157 warps of 32 rows): 18.5 us, with 4 rows a warp and one launch fewer 12.3
     a.rows = 32;
     while (a.rows * a.group > 32 && (long long)a.n * 2 < (long long)a.rows * full * (kMxvThreads / 32)) a.rows /= 2;
@@ -441,7 +495,7 @@ gbx_status mxv_minplus(Graph* G, float* w, const MxvVec& mask, const float* u, c
     G->ws.mx_dirty = true;  // until every kernel of the call is issued
     if (!direct) GBX_TRY(pdl_launch(mp_prep_kernel, small, a, false, s));
     if (!a.nothing) {
-        GBX_TRY(pdl_launch(mp_main_kernel, grid, a, !direct, s));
+        GBX_TRY(pdl_launch(block ? mp_main_kernel<true> : mp_main_kernel<false>, grid, a, !direct, s));
         if (a.dir == GBX_DIR_AUTO) GBX_TRY(pdl_launch(mp_push_kernel, grid, a, true, s));
     }
     if (!direct || deferring) GBX_TRY(pdl_launch(mp_last_kernel, small, a, true, s));

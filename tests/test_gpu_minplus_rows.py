@@ -57,3 +57,34 @@ def test_row_lengths(k, longest, transpose, N=N):
 def test_row_lengths_by_group_width(n, k, longest):
     """More vertices: fewer lanes a row."""
     test_row_lengths(k, longest, 1, n)
+
+
+@pytest.mark.parametrize("longest", [2000, 16384, 16385, 24000])
+@pytest.mark.parametrize("visited", [0.0, 0.9])
+def test_many_long_rows(longest, visited):
+    """More long rows in one block than it keeps (neighbouring rows), and rows around the length from
+    which they are left to the grid."""
+    n, hubs = 40000, 700
+    r = np.random.default_rng(longest)
+    lengths = np.full(hubs, 300)
+    lengths[::50] = longest
+    d = np.repeat(np.arange(hubs), lengths)
+    s = np.concatenate([r.permutation(np.arange(hubs, n))[:x] for x in lengths])
+    s, d = s.astype(np.int32), d.astype(np.int32)
+    val = r.random(len(s)).astype(np.float32)
+    og = oracle.graph_weighted(n, s, d, val, symmetrize=False)
+    g = gbx.graph_build(n, s, d, symmetrize=False)
+    gbx.graph_set_weights(g, s, d, val)
+    u = np.where(r.random(n) < 0.02, (r.random(n) * 9).astype(np.float32), np.float32(np.inf))
+    m = (r.random(n) < visited).astype(np.uint8)
+    old = (r.random(n) * 3).astype(np.float32)
+    u_d, m_d = torch.from_numpy(u).cuda(), torch.from_numpy(m).cuda()
+    for accum in (0, 1):
+        want = oracle.mxv_minplus(n, n, og.out_ptr, og.out_col, og.out_val, u.astype(np.float64), m, transpose=True,
+                                  complement=True, accum=bool(accum), w_old=old.astype(np.float64)).astype(np.float32)
+        for _ in range(2):
+            w = torch.from_numpy(old.copy()).cuda()
+            gbx.mxv(gbx.dense_f32(w), gbx.dense(m_d), gbx.MIN_PLUS_F32, g, gbx.dense_f32(u_d),
+                    gbx.desc_init(direction=gbx.DIR_PULL, mask_complement=1, accum=accum))
+            assert np.array_equal(w.cpu().numpy(), want), accum
+    g.free()
