@@ -192,7 +192,7 @@ struct MpLong {
 // Bound by the gathers of u (4 bytes of a 32-byte L2 sector per entry).  A lane per row of up to
 // 32 entries, one load at a time, and a warp for each longer row had taken 316 us on a
 // directed graph of 700,001 rows and 11.2M entries whose longest rows hold tens of thousands
-// (the whole call 373-382 us, now 83-90; rows deferred after 8, 16 and 64 steps 2, 9 and 39 us
+// (the whole call 373-382 us, now 82-90; rows deferred after 8, 16 and 64 steps 2, 9 and 39 us
 // more).  The group is 8 lanes from 12 entries a row on, 4 from 6, else 1: rows shorter
 // than the group's step leave lanes idle, longer ones take several dependent steps.  On small graphs
 // it grows to a warp while a quarter of the lanes are enough, and a row of up to 2,176 entries is not
